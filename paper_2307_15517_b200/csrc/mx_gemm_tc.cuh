@@ -218,12 +218,14 @@ __device__ __forceinline__ void store_mxint_chunk(const TcParams &p, int row, in
 // the fragment shape (two loads of 16 lanes) and stored from registers; four neighbouring lanes write one 32-byte
 // sector.  The staging of the tiled store costs the pair kernel shared-memory bandwidth, which is what bounds its
 // main loop (see the header of mx_gemm_tc2.cuh).  taddr = the warp's lane quarter and the chunk's first column.
-__device__ __forceinline__ void store_f32_frag(const TcParams &p, uint32_t taddr, int rows0, int n, int tb, int lane)
+__device__ __forceinline__ void load_f32_frag(uint32_t taddr, uint32_t (&r)[2][16])
 {
-    uint32_t r[2][16];
     ptx::tmem_ld_16x256b_x4(taddr, r[0]);
     ptx::tmem_ld_16x256b_x4(taddr + (16u << 16), r[1]);
     ptx::tmem_ld_wait();
+}
+__device__ __forceinline__ void store_f32_frag_regs(const TcParams &p, const uint32_t (&r)[2][16], int rows0, int n, int tb, int lane)
+{
     if (n >= p.N || rows0 >= p.M) return;                  // warp-uniform
     float *y = p.y + (int64_t)tb * p.y_batch;
     const int cq = 2 * (lane & 3);
@@ -247,6 +249,13 @@ __device__ __forceinline__ void store_f32_frag(const TcParams &p, uint32_t taddr
                 else *dst = v.x;
             }
         }
+}
+
+__device__ __forceinline__ void store_f32_frag(const TcParams &p, uint32_t taddr, int rows0, int n, int tb, int lane)
+{
+    uint32_t r[2][16];
+    load_f32_frag(taddr, r);
+    store_f32_frag_regs(p, r, rows0, n, tb, lane);
 }
 
 // fp32 epilogue of one lane: r holds 32 consecutive outputs (columns n .. n + 31) of row `row`; the

@@ -7,6 +7,7 @@
 #include <stdio.h>
 #include <string.h>
 
+#include <atomic>
 #include <map>
 #include <mutex>
 #include <tuple>
@@ -18,11 +19,13 @@
 #include "mx_gemm_simt.cuh"
 #include "mx_gemm_tc.cuh"
 #include "mx_gemm_tc2.cuh"
+#include "mx_gemm_rec.cuh"
 #include "mx_gemm_tc8.cuh"
 #include "mx_gemm_tcx.cuh"
 #include "mx_gemv_stream.cuh"
 #include "mx_glue.cuh"
 #include "mx_quantize.cuh"
+#include "mx_records.cuh"
 
 namespace {
 
@@ -44,6 +47,7 @@ struct DeviceInfo {
     bool tc2_attr_set[2] = {false, false};
     bool tcx_attr_set = false;
     bool tc8_attr_set = false;
+    bool rec_attr_set[2] = {false, false};
     bool attn_attr_set[2] = {false, false};
 };
 DeviceInfo g_dev[MAX_DEVICES];
@@ -392,6 +396,8 @@ mx_status_t encode_bf16_rows(CUtensorMap *tm, const void *base, int64_t rows, in
     return MX_OK;
 }
 
+size_t tc_workspace(int64_t M, int64_t N, int64_t K);
+
 struct QuantizedOut {            // MXInt result of the tensor-core product (see TcParams::yq_mant)
     uint8_t *mant = nullptr;
     uint8_t *exps = nullptr;
@@ -704,6 +710,220 @@ mx_status_t run_tc8(const void *a_mant, const uint8_t *a_exp, const mx_format_t 
                        (const uint8_t *)sfa, (const uint8_t *)sfw, (int)chunks_a, (int)chunks_w));
     MX_CUDA(cudaGetLastError());
     return MX_OK;
+}
+
+// ---- block-scaled product on records (mx_records.cuh, mx_gemm_rec.cuh) ------------------------------
+struct RecLayout {
+    int panels_a, panels_w, kblocks, kgroups;
+    size_t a_elems, a_sf, a_sfw, w_elems, w_sf, w_sfw, flag, bytes;      // offsets into the workspace, total size
+};
+int even_up(int v) { return (v + 1) & ~1; }
+RecLayout rec_layout(int64_t M, int64_t N, int64_t K)
+{
+    RecLayout l;
+    l.panels_a = (int)((M + mx::REC_ROWS - 1) / mx::REC_ROWS);
+    l.panels_w = (int)((N + mx::REC_ROWS - 1) / mx::REC_ROWS);
+    l.kblocks = (int)((K + mx::REC_K - 1) / mx::REC_K);
+    l.kgroups = (l.kblocks + 3) / 4;
+    size_t off = 0;
+    l.a_elems = off; off += (size_t)l.panels_a * l.kblocks * mx::REC_BYTES;
+    l.a_sf = off; off += (size_t)even_up(l.panels_a) * l.kgroups * mx::REC_SF_BYTES;
+    l.a_sfw = off; off += (size_t)even_up(l.panels_a) * l.kblocks * mx::REC_SFW_BYTES;
+    l.w_elems = off; off += (size_t)l.panels_w * l.kblocks * mx::REC_BYTES;
+    l.w_sf = off; off += (size_t)even_up(l.panels_w) * l.kgroups * mx::REC_SF_BYTES;
+    l.w_sfw = off; off += (size_t)even_up(l.panels_w) * l.kblocks * mx::REC_SFW_BYTES;
+    l.flag = off; off += 256;
+    l.bytes = off;
+    return l;
+}
+
+// Calls that take the block-scaled product: mantissas that E4M3 holds, container form on both sides, whole groups of
+// 32 along K, and sizes where it is the faster one.  Whole calls, 4-bit, block 16, against the bf16 path (us): the
+// pair tile costs more to start and drain than one CTA's, which short reductions into narrow results do not earn back
+// (256 x 768 x 768 12.9 against 11.5, 512 x 2048 x 1024 13.4 / 13.1); from K = 2048 on it wins everywhere (24 x 256 x
+// 2048 14.7 / 15.4, 2048^3 22.2 / 24.1, 512 x 6144 x 4096 34.2 / 62.5), and so do weights of 3 M elements, whose operand
+// form is half as large (256 x 6144 x 512 12.2 / 13.8; 64 x 4096 x 512, 2 M, 10.9 / 9.9).
+bool rec_fits(const mx_format_t &fa, const mx_format_t &fw, int64_t M, int64_t N, int64_t K)
+{
+    if (fa.elem_bits > 5 || fw.elem_bits > 5 || fa.packing || fw.packing || (K % 32) != 0) return false;
+    if (K < 2048 && N * K < 3 * (1 << 20)) return false;
+    const RecLayout l = rec_layout(M, N, K);
+    if ((int64_t)l.panels_a * l.kblocks * 16 > INT32_MAX / 2 || (int64_t)l.panels_w * l.kblocks * 16 > INT32_MAX / 2) return false;
+    return l.bytes <= tc_workspace(M, N, K);             // the workspace the caller was told to bring
+}
+
+mx::RecOut rec_out(const RecLayout &l, uint8_t *ws, bool weights, uint64_t tag)
+{
+    mx::RecOut o;
+    o.elems = ws + (weights ? l.w_elems : l.a_elems);
+    o.sf = ws + (weights ? l.w_sf : l.a_sf);
+    o.sf_wide = ws + (weights ? l.w_sfw : l.a_sfw);
+    o.panels = weights ? l.panels_w : l.panels_a;
+    o.panels_sf = even_up(o.panels);
+    o.kblocks = l.kblocks;
+    o.flag = reinterpret_cast<unsigned long long *>(ws + l.flag);
+    o.tag = tag;
+    return o;
+}
+
+mx::RecPacked rec_packed(const void *mant, const uint8_t *exps, const mx_format_t &f, int64_t rows, int64_t K)
+{
+    mx::RecPacked p;
+    p.mant = static_cast<const uint8_t *>(mant); p.exps = exps;
+    p.rows = rows; p.K = K;
+    p.block = f.block; p.w = f.elem_bits; p.row_shift = f.block_rows == 2 ? 1 : 0;
+    return p;
+}
+
+// A tag no other call of this process has; an old flag word equal to it costs speed only.
+uint64_t next_rec_tag()
+{
+    static std::atomic<uint64_t> calls{0};
+    return (calls.fetch_add(1, std::memory_order_relaxed) + 1) * 0x9E3779B97F4A7C15ull;
+}
+
+// `rows` rows of `words` (at most 256) 32-bit words, box of `box_rows` of them (contiguous in shared memory).
+mx_status_t encode_words(CUtensorMap *tm, const void *base, int words, int64_t rows, int box_rows)
+{
+    mx_status_t s = ensure_encoder();
+    if (s != MX_OK) return s;
+    const MapKey key = std::make_tuple(4, base, rows, (int64_t)box_rows, (int64_t)words, (int64_t)0, (int64_t)0);
+    if (cached_map(key, tm)) return MX_OK;
+    const cuuint64_t dims[2] = {(cuuint64_t)words, (cuuint64_t)rows};
+    const cuuint64_t strides[1] = {(cuuint64_t)words * 4};
+    const cuuint32_t box[2] = {(cuuint32_t)words, (cuuint32_t)box_rows};
+    const cuuint32_t estr[2] = {1, 1};
+    const CUresult r = g_encode_tiled(tm, CU_TENSOR_MAP_DATA_TYPE_UINT32, 2, const_cast<void *>(base), dims, strides, box, estr,
+                                      CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
+                                      CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+    if (r != CUDA_SUCCESS) {
+        snprintf(t_cuda_error, sizeof(t_cuda_error), "cuTensorMapEncodeTiled (records) failed (%d)", (int)r);
+        return MX_ERR_CUDA;
+    }
+    remember_map(key, *tm);
+    return MX_OK;
+}
+
+mx_status_t launch_rec(const RecLayout &l, uint8_t *ws, uint64_t tag, int64_t M, int64_t N, int64_t K, const float *bias,
+                       float *y, int64_t ldy, const QuantizedOut *yq, DeviceInfo &d, cudaStream_t st, const EpiTail &et)
+{
+    using Cfg = mx::RecCfg;
+    mx::RecMaps tm;
+    const int sa = even_up(l.panels_a), sw = even_up(l.panels_w);
+    constexpr int SF_WORDS = (int)mx::REC_SF_BYTES / 4, SFW_WORDS = (int)mx::REC_SFW_BYTES / 4;
+    const struct { CUtensorMap *map; size_t at; int words; int64_t rows; int box; } maps[] = {
+        {&tm.a, l.a_elems, 256, (int64_t)l.panels_a * l.kblocks * 16, 16},
+        {&tm.w, l.w_elems, 256, (int64_t)l.panels_w * l.kblocks * 16, 16},
+        {&tm.sa, l.a_sf, SF_WORDS, (int64_t)sa * l.kgroups, 1},
+        {&tm.sw, l.w_sf, SF_WORDS, (int64_t)sw * l.kgroups, 2},
+        {&tm.sa_wide, l.a_sfw, SFW_WORDS, (int64_t)sa * l.kblocks, 1},
+        {&tm.sw_wide, l.w_sfw, SFW_WORDS, (int64_t)sw * l.kblocks, 2},
+    };
+    mx_status_t s = MX_OK;
+    for (const auto &m : maps) {
+        s = encode_words(m.map, ws + m.at, m.words, m.rows, m.box);
+        if (s != MX_OK) return s;
+    }
+    tm.y = tm.a;
+    const bool tma_store = !yq && (ldy % 4) == 0 && (N % 4) == 0;       // see launch_tc
+    if (tma_store) {
+        s = encode_f32_out(&tm.y, y, M, N, ldy);
+        if (s != MX_OK) return s;
+    }
+    s = et.any() ? smem_attr_once(d.rec_attr_set[1], mx::gemm_rec_kernel<true>, (int)Cfg::SMEM_BYTES)
+                 : smem_attr_once(d.rec_attr_set[0], mx::gemm_rec_kernel<false>, (int)Cfg::SMEM_BYTES);
+    if (s != MX_OK) return s;
+    mx::TcParams p{};
+    p.y = y;
+    p.bias = et.any() ? nullptr : bias;
+    p.ex_bias = et.any() ? bias : nullptr;
+    p.relu = et.relu;
+    p.residual = et.residual;
+    p.ldr = et.ldr;
+    p.ldy = ldy;
+    p.M = (int)M;
+    p.N = (int)N;
+    p.K = (int)K;
+    p.tiles_m = (l.panels_a + 1) / 2;
+    p.tiles_n = (l.panels_w + 1) / 2;
+    p.status = d.status;
+    p.tma_store = tma_store ? 1 : 0;
+    p.frag_store = frag_store_ok(yq != nullptr, et.any(), y, ldy, 0) ? 1 : 0;
+    p.batch = 1;
+    p.yq_mant = yq ? yq->mant : nullptr;
+    p.yq_exp = yq ? yq->exps : nullptr;
+    p.yq_nonfinite = yq ? yq->nonfinite : nullptr;
+    p.yq_bits = yq ? yq->f.elem_bits : 0;
+    p.yq_block = yq ? yq->f.block : 0;
+    p.yq_rows2 = yq && yq->f.block_rows == 2 ? 1 : 0;
+    const mx::RecParams rp{reinterpret_cast<const unsigned long long *>(ws + l.flag), tag, sa, sw};
+    const int64_t tiles = (int64_t)p.tiles_m * p.tiles_n;
+    if (tiles > INT32_MAX / 2) return MX_ERR_SHAPE;
+    const int pairs = tiles < d.sm_count / 2 ? (int)tiles : d.sm_count / 2;
+    ProfScope prof(KIND_GEMM_TC, st);
+    if (et.any()) MX_CUDA(launch_dep(mx::gemm_rec_kernel<true>, dim3(2 * pairs), dim3(Cfg::THREADS), Cfg::SMEM_BYTES, st, tm, p, rp));
+    else MX_CUDA(launch_dep(mx::gemm_rec_kernel<false>, dim3(2 * pairs), dim3(Cfg::THREADS), Cfg::SMEM_BYTES, st, tm, p, rp));
+    MX_CUDA(cudaGetLastError());
+    return MX_OK;
+}
+
+// A layer on records: activations quantized and weights re-laid in one launch, then the product.
+mx_status_t run_rec_linear(const mx_linear_args_t &a, const float *bias, float *y, int64_t ldy, const QuantizedOut *yq,
+                           uint8_t *ws, DeviceInfo &d, cudaStream_t st, const EpiTail &et)
+{
+    const RecLayout l = rec_layout(a.M, a.N, a.K);
+    const uint64_t tag = next_rec_tag();
+    mx::RecPrepJob job;
+    job.x = a.x; job.M = a.M; job.K = a.K; job.ldx = a.ldx;
+    job.wa = a.fa.elem_bits; job.block = a.fa.block; job.a_rows2 = a.fa.block_rows == 2 ? 1 : 0;
+    job.a = rec_out(l, ws, false, tag);
+    job.pw = rec_packed(a.w_mant, a.w_exp, a.fw, a.N, a.K);
+    job.w = rec_out(l, ws, true, tag);
+    const bool f32 = a.dt == MX_F32, nib = a.fw.elem_bits <= 4;
+    constexpr int PT = 128;                              // as in tc_prepare
+    const int per_sm = (256 / PT) * (f32 ? (nib ? resident_ctas(mx::rec_prep_kernel<float, true>)
+                                                : resident_ctas(mx::rec_prep_kernel<float, false>))
+                                         : (nib ? resident_ctas(mx::rec_prep_kernel<__nv_bfloat16, true>)
+                                                : resident_ctas(mx::rec_prep_kernel<__nv_bfloat16, false>)));
+    const int64_t items = (int64_t)l.panels_a * 16 * l.kblocks + (int64_t)l.panels_w * 16 * ((l.kblocks + 1) / 2);
+    const dim3 grid((unsigned)grid_for(items, PT / 32, d.sm_count, per_sm));
+    {
+        ProfScope prof(KIND_PREP, st);
+        if (f32 && nib) MX_CUDA(launch_dep(mx::rec_prep_kernel<float, true>, grid, dim3(PT), 0, st, job));
+        else if (f32) MX_CUDA(launch_dep(mx::rec_prep_kernel<float, false>, grid, dim3(PT), 0, st, job));
+        else if (nib) MX_CUDA(launch_dep(mx::rec_prep_kernel<__nv_bfloat16, true>, grid, dim3(PT), 0, st, job));
+        else MX_CUDA(launch_dep(mx::rec_prep_kernel<__nv_bfloat16, false>, grid, dim3(PT), 0, st, job));
+        MX_CUDA(cudaGetLastError());
+    }
+    return launch_rec(l, ws, tag, a.M, a.N, a.K, bias, y, ldy, yq, d, st, et);
+}
+
+// A product of two packed operands on records.
+mx_status_t run_rec_gemm(const void *a_mant, const uint8_t *a_exp, const mx_format_t &fa, const void *w_mant,
+                         const uint8_t *w_exp, const mx_format_t &fw, int64_t M, int64_t N, int64_t K, const float *bias,
+                         float *y, int64_t ldy, const QuantizedOut *yq, uint8_t *ws, DeviceInfo &d, cudaStream_t st,
+                         const EpiTail &et)
+{
+    const RecLayout l = rec_layout(M, N, K);
+    const uint64_t tag = next_rec_tag();
+    mx::RecPairJob j;
+    j.pa = rec_packed(a_mant, a_exp, fa, M, K);
+    j.pw = rec_packed(w_mant, w_exp, fw, N, K);
+    j.a = rec_out(l, ws, false, tag);
+    j.w = rec_out(l, ws, true, tag);
+    const bool na = fa.elem_bits <= 4, nw = fw.elem_bits <= 4;
+    const int per_sm = resident_ctas(mx::rec_pair_kernel<true, true>);
+    const int64_t items = (int64_t)(l.panels_a + l.panels_w) * 16 * ((l.kblocks + 1) / 2);
+    const dim3 grid((unsigned)grid_for(items, 8, d.sm_count, per_sm));
+    {
+        ProfScope prof(KIND_DEQUANTIZE, st);
+        if (na && nw) MX_CUDA(launch_dep(mx::rec_pair_kernel<true, true>, grid, dim3(256), 0, st, j));
+        else if (na) MX_CUDA(launch_dep(mx::rec_pair_kernel<true, false>, grid, dim3(256), 0, st, j));
+        else if (nw) MX_CUDA(launch_dep(mx::rec_pair_kernel<false, true>, grid, dim3(256), 0, st, j));
+        else MX_CUDA(launch_dep(mx::rec_pair_kernel<false, false>, grid, dim3(256), 0, st, j));
+        MX_CUDA(cudaGetLastError());
+    }
+    return launch_rec(l, ws, tag, M, N, K, bias, y, ldy, yq, d, st, et);
 }
 
 bool wide_tile(int64_t M, int64_t N, const DeviceInfo &d)
@@ -1133,6 +1353,15 @@ mx_status_t mx_gemm_ex(const void *a_mant, const uint8_t *a_exp, mx_format_t fa,
         one.w_mant = w_mant; one.w_exp = w_exp; one.fw = fw; one.N = N; one.bias = bias; one.y = y; one.ldy = ldy;
         const bool can_stream = stream_layer_ok(one) && (reinterpret_cast<uintptr_t>(w_exp) & 3u) == 0 &&
                                 workspace && workspace_bytes >= stream_table_bytes(1);
+        if (algo == MX_ALGO_AUTO && !can_stream && rec_fits(fa, fw, M, N, K)) {
+            if (!workspace || workspace_bytes < tc_workspace(M, N, K)) return MX_ERR_WORKSPACE;
+            if ((reinterpret_cast<uintptr_t>(workspace) & 255u) != 0) return MX_ERR_ALIGN;
+            DeviceInfo *dr = nullptr;
+            s = device_info(&dr);
+            if (s != MX_OK) return s;
+            return run_rec_gemm(a_mant, a_exp, fa, w_mant, w_exp, fw, M, N, K, bias, y, ldy, nullptr,
+                                static_cast<uint8_t *>(workspace), *dr, static_cast<cudaStream_t>(stream), EpiTail());
+        }
         if (algo == MX_ALGO_AUTO) algo = can_stream ? MX_ALGO_STREAM : MX_ALGO_TCGEN05;
         if (algo == MX_ALGO_STREAM) return grouped_impl(&one, 1, &a_exp, workspace, workspace_bytes, stream);
     }
@@ -1209,6 +1438,7 @@ mx_status_t mx_linear_ex(const void *x, mx_dtype_t dt, int64_t M, int64_t K, int
     one.w_mant = w_mant; one.w_exp = w_exp; one.fw = fw; one.N = N; one.bias = bias; one.y = y; one.ldy = ldy;
     if (fw.packing && algo != MX_ALGO_AUTO && algo != MX_ALGO_TCGEN05 && algo != MX_ALGO_TCGEN05_BLOCKWISE)
         return MX_ERR_FORMAT;
+    const bool any_algo = algo == MX_ALGO_AUTO;
     if (algo == MX_ALGO_AUTO)
         algo = (stream_layer_ok(one) && (reinterpret_cast<uintptr_t>(w_exp) & 3u) == 0) ? MX_ALGO_STREAM
                                                                                      : MX_ALGO_TCGEN05;
@@ -1248,6 +1478,7 @@ mx_status_t mx_linear_ex(const void *x, mx_dtype_t dt, int64_t M, int64_t K, int
     const bool fused = algo == MX_ALGO_TCGEN05_FUSED && (K % 32) == 0 && fw.block_rows == 1;
     if (fused && !fused_ok(K, w_exp)) return MX_ERR_ALIGN;
     if (workspace_bytes < (fused ? fused_workspace(M, K) : tc_workspace(M, N, K))) return MX_ERR_WORKSPACE;
+    if (any_algo && rec_fits(fa, fw, M, N, K)) return run_rec_linear(one, bias, y, ldy, nullptr, ws, *d, st, EpiTail());
     __nv_bfloat16 *a_hat = reinterpret_cast<__nv_bfloat16 *>(ws);
     // the activations' mantissas and exponents go straight to the MMA operand form (exact bf16)
     mx::QuantOut out{nullptr, nullptr, a_hat, K, nullptr};
@@ -1312,14 +1543,17 @@ static mx_status_t gemm_tc_impl(const void *a_mant, const uint8_t *a_exp, mx_for
     __nv_bfloat16 *a_hat = static_cast<__nv_bfloat16 *>(workspace);
     __nv_bfloat16 *w_hat = reinterpret_cast<__nv_bfloat16 *>(static_cast<uint8_t *>(workspace) +
                                                              round256((size_t)M * K * 2));
-    s = launch_dequant_pair(a_mant, a_exp, fa, M, w_mant, w_exp, fw, N, K, a_hat, w_hat, *d, st);
-    if (s != MX_OK) return s;
-    if (y) return run_tc(a_hat, w_hat, M, N, K, bias, y, ldy, *d, st, nullptr, TcBatch(), et);
     QuantizedOut yq;
     yq.mant = static_cast<uint8_t *>(y_mant);
     yq.exps = y_exp;
     yq.nonfinite = nonfinite_count;
     yq.f = fy;
+    if (rec_fits(fa, fw, M, N, K))
+        return run_rec_gemm(a_mant, a_exp, fa, w_mant, w_exp, fw, M, N, K, bias, y, y ? ldy : N, y ? nullptr : &yq,
+                            static_cast<uint8_t *>(workspace), *d, st, et);
+    s = launch_dequant_pair(a_mant, a_exp, fa, M, w_mant, w_exp, fw, N, K, a_hat, w_hat, *d, st);
+    if (s != MX_OK) return s;
+    if (y) return run_tc(a_hat, w_hat, M, N, K, bias, y, ldy, *d, st, nullptr, TcBatch(), et);
     return run_tc(a_hat, w_hat, M, N, K, bias, nullptr, N, *d, st, &yq, TcBatch(), et);
 }
 
@@ -1387,6 +1621,13 @@ static mx_status_t linear_tc_impl(const void *x, mx_dtype_t dt, int64_t M, int64
     mx_linear_args_t one;
     one.x = x; one.dt = dt; one.M = M; one.K = K; one.ldx = ldx; one.fa = fa;
     one.w_mant = w_mant; one.w_exp = w_exp; one.fw = fw; one.N = N; one.bias = bias; one.y = y; one.ldy = y ? ldy : N;
+    QuantizedOut yq;
+    yq.mant = static_cast<uint8_t *>(y_mant);
+    yq.exps = y_exp;
+    yq.nonfinite = nonfinite_count;
+    yq.f = fy;
+    if (!with_ln && rec_fits(fa, fw, M, N, K))
+        return run_rec_linear(one, bias, y, y ? ldy : N, y ? nullptr : &yq, ws, *d, st, et);
     if (with_ln) {
         s = tc_prepare_ln(one, *ln, a_hat, w_hat, *d, st);
     } else {
@@ -1394,11 +1635,6 @@ static mx_status_t linear_tc_impl(const void *x, mx_dtype_t dt, int64_t M, int64
     }
     if (s != MX_OK) return s;
     if (y) return run_tc(a_hat, w_hat, M, N, K, bias, y, ldy, *d, st, nullptr, TcBatch(), et);
-    QuantizedOut yq;
-    yq.mant = static_cast<uint8_t *>(y_mant);
-    yq.exps = y_exp;
-    yq.nonfinite = nonfinite_count;
-    yq.f = fy;
     return run_tc(a_hat, w_hat, M, N, K, bias, nullptr, N, *d, st, &yq, TcBatch(), et);
 }
 
