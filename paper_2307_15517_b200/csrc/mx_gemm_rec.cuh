@@ -1,28 +1,34 @@
 // MXInt product on the tensor pipe's block-scaled 8-bit path, CTA pairs (Sec. 3.2: the MXInt dot-product operator
 // applies the shared exponent once per block; tcgen05.mma.kind::mxf8f6f4.block_scale is that operator in silicon).
-// Operands are records (mx_records.cuh): exact for mantissa widths up to 5 on both sides, blocks of 16 and of 32.
-// Products are exact, the 32 products of an MMA step are summed with the scale 2^(Ea+Ew) and accumulate in fp32 in
-// tensor memory, as in the bf16 kernels; the 8-bit pipe runs at twice their rate on half their operand bytes.
+// Operands are records (mx_records.cuh): mantissas of up to 5 bits on both sides, blocks of 16 and of 32.  Products are
+// exact, the 32 products of an MMA step are summed with the scale 2^(Ea+Ew) and accumulate in fp32 in tensor memory, as
+// in the bf16 kernels; the 8-bit pipe runs at twice their rate on half their operand bytes.  (Wider mantissas split into
+// two E4M3 planes take two MMAs: measured, and no faster than bf16: 2048 x 12288 x 4096 188 against 192 us, 2048^3 28
+// against 24.)
 //
 // Two CTAs on neighbouring SMs (a cluster of two) share one 256 x 256 output tile, K step 128: each holds one record
 // of A and one of W per step, plus the scales of its own A rows and of all 256 rows of W (the pair's MMA reads the W
 // scales from both CTAs' tensor memory).  The warp roles and barriers are those of mx_gemm_tc2.cuh:
 //   warp 0      : TMA producer (one lane, in both CTAs; bytes are counted on the leader's barrier)
-//   warp 1      : tensor-memory allocation (both CTAs), scale copies and MMA issue (leader only)
+//   warp 1      : tensor-memory allocation (both CTAs), scale copies and MMA issue (one lane, leader only)
 //   warps 2..9  : epilogue of the CTA's own 128 rows, two warps per TMEM lane quarter
+// What bounds it: operand fetch, 64 KB per 256 x 256 x 128 step and pair (13 TB/s over the chip at 0.36 us per step), and the
+// shared-memory reads of the MMAs (0.32 us per step with the fetches removed; 0.26 us is the pipe's peak).
 //
 // Tensor memory: 512 columns cannot hold two accumulators of 256 and the scales.  The accumulators overlap by 32
 // columns ([0, 256) and [224, 480)), the last 32 columns hold two sets of scales.  The epilogue drains the shared
 // columns first and then lets the next tile's MMAs start, so what is exposed between two tiles is one 32-column read.
 //
-// Wide mode (the flag word equals the call's tag: some row's blocks were too far apart for one scale per record):
-// every 32 k take two MMAs, one per half.  The operands' second k-chunk of 16 is then a panel of zeros in
-// shared memory -- without swizzle the distance between the two chunks of an MMA is a free field of the descriptor --
-// and each half has its own scales.  Twice the MMAs, the rate of the bf16 kernels, exact for any exponents.
+// Wide steps (the flag bytes of one of the step's four records are not all zero: some row's blocks were too far apart for
+// one scale per record): every 32 k take two MMAs, one per half.  The operands' second k-chunk of 16 is then a panel of
+// zeros in shared memory -- without swizzle the distance between the two chunks of an MMA is a free field of the
+// descriptor -- and each half has its own scales: exact for any exponents, at the cost of twice the MMAs in these steps.
 #pragma once
 #include <cuda.h>
 #include <cuda_runtime.h>
 #include <stdint.h>
+
+#include <type_traits>
 
 #include "mx_gemm_tc.cuh"
 #include "mx_gemm_tc8.cuh"
@@ -33,16 +39,16 @@ namespace mx {
 
 struct RecCfg {
     static constexpr int BN = 256;                        // pair tile: 256 x 256
-    static constexpr int STAGES = 5;
-    static constexpr uint32_t SFA_OFF = 2 * REC_BYTES;                      // A record, W record, then the scales:
-    static constexpr uint32_t SFW_OFF = SFA_OFF + REC_SFW_BYTES;            // own rows of A; both panels of W
+    static constexpr int STAGES = 6;
+    static constexpr uint32_t W_OFF = REC_BYTES;                            // A record, W record, then the scales:
+    static constexpr uint32_t SFA_OFF = W_OFF + REC_BYTES;                  // own rows of A; both panels of W
+    static constexpr uint32_t SFW_OFF = SFA_OFF + REC_SFW_BYTES;
     static constexpr uint32_t STAGE_BYTES = SFW_OFF + 2 * REC_SFW_BYTES;    // 35 KB
     static constexpr int EPI_WARPS = 8;
     static constexpr int THREADS = 64 + 32 * EPI_WARPS;
-    static constexpr uint32_t EPI_BYTES = EPI_WARPS * 4096;                 // one 32x32 fp32 store buffer per epilogue warp
     static constexpr uint32_t ZERO_BYTES = REC_ROWS * 16;                   // one k-chunk of zeros
     static constexpr uint32_t BAR_BYTES = 256;
-    static constexpr uint32_t SMEM_BYTES = STAGES * STAGE_BYTES + EPI_BYTES + ZERO_BYTES + BAR_BYTES + 1024;
+    static constexpr uint32_t SMEM_BYTES = STAGES * STAGE_BYTES + ZERO_BYTES + BAR_BYTES + 1024;
     static constexpr uint32_t TMEM_COLS = 512;
     static constexpr uint32_t ACC_STEP = 224;             // first column of the second accumulator
     static constexpr uint32_t SF_COL = 480;               // scale columns: two sets of 4 (A) + 8 (W)
@@ -77,17 +83,118 @@ __device__ __forceinline__ void mma_mxf8_ss_pair(uint32_t d_tmem, uint64_t a_des
         : "memory");
 }
 
-// Tensor maps over the operands' arrays: records as rows of 1 KB (box: 16 rows = one record), scales as rows of one
-// chunk (512 B) or of one record's half-block scales (1 KB), box of one row for A and of two for W.
-struct RecMaps { CUtensorMap a, w, sa, sw, sa_wide, sw_wide, y; };
+// Tensor maps over the operands' arrays: records as rows of 1 KB (box: one record), scales as rows of 512 B, half-block
+// scales as rows of 1 KB (box: one panel of A, two of W).
+struct RecMaps { CUtensorMap a, w, sa, sw, sa_wide, sw_wide; };
 
 struct RecParams {
-    const unsigned long long *flag;          // wide mode when *flag == tag
-    unsigned long long tag;
-    int panels_sa, panels_sw;                // rows of the scale arrays per K step (group)
+    const uint8_t *flags_a, *flags_w;        // [panels][kblocks][16]
+    int panels_a, panels_w;
+    int panels_sa, panels_sw;                // panels in the scale arrays
 };
 
-template <bool TAIL = false>
+// The residual values of a warp's 32 x 32 chunk in the fragment shape, fetched one chunk ahead of their use.
+struct FragTail { float2 v[2][2][4]; };
+
+__device__ __forceinline__ void frag_tail_fetch(const TcParams &p, int rows0, int n, int lane, FragTail &t)
+{
+    if (!p.residual) return;
+    const bool vec = (p.ldr & 1) == 0 && (reinterpret_cast<uintptr_t>(p.residual) & 7) == 0;
+#pragma unroll
+    for (int h = 0; h < 2; ++h)
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+            const int row = rows0 + 16 * h + 8 * u + (lane >> 2);
+            const float *src = p.residual + (int64_t)row * p.ldr;
+#pragma unroll
+            for (int g = 0; g < 4; ++g) {
+                const int c = n + 8 * g + 2 * (lane & 3);
+                float2 r = make_float2(0.f, 0.f);
+                if (row < p.M && c + 1 < p.N && vec) {
+                    r = __ldg(reinterpret_cast<const float2 *>(src + c));
+                } else if (row < p.M) {
+                    if (c < p.N) r.x = __ldg(src + c);
+                    if (c + 1 < p.N) r.y = __ldg(src + c + 1);
+                }
+                t.v[h][u][g] = r;
+            }
+        }
+}
+
+// fp32 result of a warp's 32 x 32 chunk from the fragment shape: (+ bias) and, with TAIL, the activation and the residual,
+// in the order of tail_apply.  Four neighbouring lanes write one 32-byte sector where rows of y are 8-byte aligned.
+template <bool TAIL>
+__device__ __forceinline__ void frag_store(const TcParams &p, const uint32_t (&r)[2][16], const FragTail &t, int rows0, int n, int lane)
+{
+    if (n >= p.N || rows0 >= p.M) return;                  // warp-uniform
+    const float *bias = TAIL ? p.ex_bias : p.bias;
+    // the sectors of a row go out one after the other (rows innermost instead: 2048^3 20.5 against 18.8 us)
+#pragma unroll
+    for (int h = 0; h < 2; ++h)
+#pragma unroll
+        for (int g = 0; g < 4; ++g) {
+            const int c = n + 8 * g + 2 * (lane & 3);
+            float2 b = make_float2(0.f, 0.f);
+            if (bias) {
+                if (c + 1 < p.N) b = __ldg(reinterpret_cast<const float2 *>(bias + c));
+                else if (c < p.N) b.x = __ldg(bias + c);
+            }
+#pragma unroll
+            for (int u = 0; u < 2; ++u) {
+                const int row = rows0 + 16 * h + 8 * u + (lane >> 2);
+                if (row >= p.M || c >= p.N) continue;
+                float2 v = make_float2(__uint_as_float(r[h][4 * g + 2 * u]), __uint_as_float(r[h][4 * g + 2 * u + 1]));
+                if (bias) { v.x += b.x; v.y += b.y; }
+                if (TAIL) {
+                    if (p.relu) {                                        // NaN stays NaN
+                        v.x = v.x < 0.f ? 0.f : v.x;
+                        v.y = v.y < 0.f ? 0.f : v.y;
+                    }
+                    if (p.residual) { v.x += t.v[h][u][g].x; v.y += t.v[h][u][g].y; }
+                }
+                float *dst = p.y + (int64_t)row * p.ldy + c;
+                if (c + 1 < p.N && p.frag_store) {
+                    *reinterpret_cast<float2 *>(dst) = v;
+                } else {
+                    dst[0] = v.x;
+                    if (c + 1 < p.N) dst[1] = v.y;
+                }
+            }
+        }
+}
+
+// Which of 32 K steps (from 32 * kg on) of a tile are wide: every lane looks one step up, in the flag bytes of the tile's
+// four records.  The loads are issued by `fetch` and first touched by `mask`, 32 steps later.
+struct RecFlags {
+    uint4 f[4];
+    __device__ __forceinline__ void fetch(const RecParams &rp, int m2, int n2, int kg, int kblocks, int lane)
+    {
+        const int kb = kg * 32 + lane;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const bool a = i < 2;
+            const int panel = a ? m2 + i : n2 + i - 2;
+            f[i] = make_uint4(0, 0, 0, 0);
+            if (kb < kblocks && panel < (a ? rp.panels_a : rp.panels_w))
+                f[i] = __ldg(reinterpret_cast<const uint4 *>((a ? rp.flags_a : rp.flags_w) + ((int64_t)panel * kblocks + kb) * 16));
+        }
+    }
+    __device__ __forceinline__ uint32_t mask() const           // warp-collective
+    {
+        uint32_t any = 0;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) any |= f[i].x | f[i].y | f[i].z | f[i].w;
+        return __ballot_sync(0xFFFFFFFFu, any != 0);
+    }
+};
+
+// A step that is not wide brings the scales of its four when it is the first of them or follows a wide step.
+__device__ __forceinline__ bool rec_loads_scales(uint32_t wide_mask, int kb)
+{
+    return (kb & 3) == 0 || ((wide_mask >> ((kb & 31) - 1)) & 1u);
+}
+
+template <bool TAIL, bool QOUT>
 __global__ void __cluster_dims__(2, 1, 1) __maxnreg__(128)
 gemm_rec_kernel(const __grid_constant__ RecMaps tm, const TcParams p, const RecParams rp)
 {
@@ -97,8 +204,7 @@ gemm_rec_kernel(const __grid_constant__ RecMaps tm, const TcParams p, const RecP
     const uint32_t smem_base = (ptx::smem_u32(smem_raw) + 1023u) & ~1023u;
     uint8_t *smem_gen = smem_raw + (smem_base - ptx::smem_u32(smem_raw));
 
-    const uint32_t epi_base = smem_base + STAGES * Cfg::STAGE_BYTES;
-    const uint32_t zero_base = epi_base + Cfg::EPI_BYTES;
+    const uint32_t zero_base = smem_base + STAGES * Cfg::STAGE_BYTES;
     const uint32_t bar_base = zero_base + Cfg::ZERO_BYTES;
     auto full_bar = [&](int s) { return bar_base + 8u * s; };
     auto empty_bar = [&](int s) { return bar_base + 8u * (STAGES + s); };
@@ -144,110 +250,130 @@ gemm_rec_kernel(const __grid_constant__ RecMaps tm, const TcParams p, const RecP
     const int pair = blockIdx.x >> 1, npairs = gridDim.x >> 1;
     const int kblocks = (p.K + REC_K - 1) / REC_K;
     bool timed_out = false;
-    auto is_wide = [&]() { return *reinterpret_cast<const volatile unsigned long long *>(rp.flag) == rp.tag; };
+    const int kgroups32 = (kblocks + 31) >> 5;
 
-    if (warp == 0) {
-        if (lane == 0) {
-            const bool wide = is_wide();
-            int s = 0;
-            uint32_t ph = 0;
-            for (int t = pair; t < num_tiles && !timed_out; t += npairs) {
-                const int pa = (t % p.tiles_m) * 2 + (int)rank;              // this CTA's panel of A and of W
-                const int pw0 = (t / p.tiles_m) * 2, pw = pw0 + (int)rank;
-                for (int kb = 0; kb < kblocks; ++kb) {
-                    if (!ptx::mbar_wait_bounded_cluster(empty_bar(s), ph ^ 1u, abort_flag, TC_WAIT_LIMIT_NS)) {
-                        timed_out = true;
-                        break;
+    if (warp == 0 || (warp == 1 && leader)) {
+        // both roles walk the tiles in groups of 32 K steps: the whole warp looks up which of them are wide (the next
+        // group's flags are on their way meanwhile), lane 0 does the work
+        int s = 0;
+        uint32_t ph = 0;
+        int it = 0;
+        uint32_t set = 0;
+        RecFlags ahead;
+        ahead.fetch(rp, (pair % p.tiles_m) * 2, (pair / p.tiles_m) * 2, 0, kblocks, lane);
+        auto load_records = [&](int stage, int m2, int n2, int kb) {                  // this CTA's panel of A and of W
+            const uint32_t sa = smem_base + stage * Cfg::STAGE_BYTES, leader_full = ptx::map_to_cta(full_bar(stage), 0);
+            ptx::tma_load_2d_pair(sa, &tm.a, 0, ((m2 + (int)rank) * kblocks + kb) * 16, leader_full);
+            ptx::tma_load_2d_pair(sa + Cfg::W_OFF, &tm.w, 0, ((n2 + (int)rank) * kblocks + kb) * 16, leader_full);
+        };
+        // the first stages' records are on their way while the first flags arrive; their bytes are announced, with the
+        // scales', in the loop (a barrier's byte count may run ahead of its announcement)
+        const int early = pair < num_tiles ? min(STAGES, kblocks) : 0;
+        if (warp == 0 && lane == 0)
+            for (int kb = 0; kb < early; ++kb) load_records(kb, (pair % p.tiles_m) * 2, (pair / p.tiles_m) * 2, kb);
+        for (int t = pair; t < num_tiles; t += npairs, ++it) {
+            const int m2 = (t % p.tiles_m) * 2, n2 = (t / p.tiles_m) * 2;            // first panels of the tile
+            const int acc = it & 1;
+            const uint32_t d_tmem = tmem_base + (uint32_t)acc * Cfg::ACC_STEP;
+            for (int kg = 0; kg < kgroups32; ++kg) {
+                const uint32_t wide_mask = ahead.mask();
+                const bool last = kg + 1 == kgroups32;
+                const int tn = last ? t + npairs : t;                                // (past the last tile: panels out of range)
+                ahead.fetch(rp, (tn % p.tiles_m) * 2, (tn / p.tiles_m) * 2, last ? 0 : kg + 1, kblocks, lane);
+                if (lane != 0 || timed_out) continue;
+                const int kb_end = min(kblocks, 32 * kg + 32);
+                if (warp == 0) {
+                    const int pa = m2 + (int)rank;
+                    for (int kb = 32 * kg; kb < kb_end; ++kb) {
+                        if (!ptx::mbar_wait_bounded_cluster(empty_bar(s), ph ^ 1u, abort_flag, TC_WAIT_LIMIT_NS)) {
+                            timed_out = true;
+                            break;
+                        }
+                        const bool wide = (wide_mask >> (kb & 31)) & 1u;
+                        const bool four = rec_loads_scales(wide_mask, kb);
+                        const uint32_t bytes = 2 * REC_BYTES + 3 * (wide ? REC_SFW_BYTES : four ? REC_SF_BYTES : 0u);
+                        if (leader) ptx::mbar_arrive_expect_tx(full_bar(s), 2 * bytes);
+                        const uint32_t leader_full = ptx::map_to_cta(full_bar(s), 0);
+                        const uint32_t sa = smem_base + s * Cfg::STAGE_BYTES;
+                        if (it > 0 || kb >= early) load_records(s, m2, n2, kb);
+                        if (wide) {
+                            ptx::tma_load_2d_pair(sa + Cfg::SFA_OFF, &tm.sa_wide, 0, kb * rp.panels_sa + pa, leader_full);
+                            ptx::tma_load_2d_pair(sa + Cfg::SFW_OFF, &tm.sw_wide, 0, kb * rp.panels_sw + n2, leader_full);
+                        } else if (four) {
+                            ptx::tma_load_2d_pair(sa + Cfg::SFA_OFF, &tm.sa, 0, (kb >> 2) * rp.panels_sa + pa, leader_full);
+                            ptx::tma_load_2d_pair(sa + Cfg::SFW_OFF, &tm.sw, 0, (kb >> 2) * rp.panels_sw + n2, leader_full);
+                        }
+                        if (++s == STAGES) { s = 0; ph ^= 1u; }
                     }
-                    const bool scales = wide || (kb & 3) == 0;               // this stage brings scales
-                    const uint32_t bytes = 2 * REC_BYTES + (scales ? 3 * (wide ? REC_SFW_BYTES : REC_SF_BYTES) : 0u);
-                    if (leader) ptx::mbar_arrive_expect_tx(full_bar(s), 2 * bytes);
-                    const uint32_t leader_full = ptx::map_to_cta(full_bar(s), 0);
-                    const uint32_t sa = smem_base + s * Cfg::STAGE_BYTES;
-                    ptx::tma_load_2d_pair(sa, &tm.a, 0, (pa * kblocks + kb) * 16, leader_full);
-                    ptx::tma_load_2d_pair(sa + REC_BYTES, &tm.w, 0, (pw * kblocks + kb) * 16, leader_full);
-                    if (scales) {
-                        const int ks = wide ? kb : kb >> 2;
-                        ptx::tma_load_2d_pair(sa + Cfg::SFA_OFF, wide ? &tm.sa_wide : &tm.sa, 0, ks * rp.panels_sa + pa, leader_full);
-                        ptx::tma_load_2d_pair(sa + Cfg::SFW_OFF, wide ? &tm.sw_wide : &tm.sw, 0, ks * rp.panels_sw + pw0, leader_full);
-                    }
-                    if (++s == STAGES) { s = 0; ph ^= 1u; }
+                    continue;
                 }
-            }
-        }
-        __syncwarp();
-    } else if (warp == 1) {
-        if (lane == 0 && leader) {
-            const bool wide = is_wide();
-            int s = 0;
-            uint32_t ph = 0;
-            int it = 0;
-            uint32_t set = 0;
-            for (int t = pair; t < num_tiles && !timed_out; t += npairs, ++it) {
-                const int acc = it & 1;
                 // tile it may start when the epilogue has left the columns it shares with tile it - 1 (every warp has
                 // by then finished tile it - 2, which lay where tile it goes)
-                if (it > 0 && !ptx::mbar_wait_bounded_cluster(drained_bar, (uint32_t)(it - 1) & 1u, abort_flag, TC_WAIT_LIMIT_NS)) {
+                if (kg == 0 && it > 0 &&
+                    !ptx::mbar_wait_bounded_cluster(drained_bar, (uint32_t)(it - 1) & 1u, abort_flag, TC_WAIT_LIMIT_NS)) {
                     timed_out = true;
-                    break;
+                    continue;
                 }
                 ptx::tc_fence_after_sync();
-                const uint32_t d_tmem = tmem_base + (uint32_t)acc * Cfg::ACC_STEP;
-                for (int kb = 0; kb < kblocks; ++kb) {
-                    if (!ptx::mbar_wait_bounded_cluster(full_bar(s), ph, abort_flag, TC_WAIT_LIMIT_NS)) {
-                        timed_out = true;
-                        break;
-                    }
-                    ptx::tc_fence_after_sync();
-                    const uint32_t sa = smem_base + s * Cfg::STAGE_BYTES;
-                    const uint32_t sw = sa + REC_BYTES;
+                // One K step; WIDE_MAY: some step of the group is wide.  The common loop is compiled without the wide step:
+                // the one thread that issues the MMAs has about 600 cycles per step, and the shared loop cost 2.5 us of
+                // 38 on 2048 x 6144 x 2048.
+                auto steps = [&](auto may_c) {
+                    constexpr bool WIDE_MAY = decltype(may_c)::value;
                     constexpr uint32_t CHUNK = REC_ROWS * 16;                // bytes of one k-chunk of a record
-                    if (!wide) {
-                        if ((kb & 3) == 0) {
-                            // four steps' scales: shared -> tensor memory, executed in order ahead of the MMAs below
-                            set ^= 1u;
-                            const uint32_t tsfa = tmem_base + Cfg::SF_COL + set * Cfg::SF_SET;
-                            tmem_cp_32x128b_warpx4_pair(tsfa, smem_desc_sf_chunk(sa + Cfg::SFA_OFF));
-                            tmem_cp_32x128b_warpx4_pair(tsfa + 4, smem_desc_sf_chunk(sa + Cfg::SFW_OFF));
-                            tmem_cp_32x128b_warpx4_pair(tsfa + 8, smem_desc_sf_chunk(sa + Cfg::SFW_OFF + REC_SF_BYTES));
+                    for (int kb = 32 * kg; kb < kb_end; ++kb) {
+                        if (!ptx::mbar_wait_bounded_cluster(full_bar(s), ph, abort_flag, TC_WAIT_LIMIT_NS)) {
+                            timed_out = true;
+                            return;
                         }
-                        const uint32_t tsfa = tmem_base + Cfg::SF_COL + set * Cfg::SF_SET;
-                        const uint32_t idesc = idesc_mxf8_e4m3(256, BN, (uint32_t)(kb & 3));
-#pragma unroll
-                        for (int j = 0; j < REC_K / 32; ++j)
-                            mma_mxf8_ss_pair(d_tmem, smem_desc_rec(sa + 2 * j * CHUNK, CHUNK), smem_desc_rec(sw + 2 * j * CHUNK, CHUNK),
-                                             idesc, tsfa, tsfa + 4, (kb | j) != 0 ? 1u : 0u);
-                    } else {
-#pragma unroll 1
-                        for (int h = 0; h < 2; ++h) {
+                        ptx::tc_fence_after_sync();
+                        const uint32_t sa = smem_base + s * Cfg::STAGE_BYTES;
+                        const uint32_t sw = sa + Cfg::W_OFF;
+                        // scales: shared -> tensor memory, executed in order ahead of the MMAs below; `step`: bytes from W's
+                        // first panel to its second
+                        auto load_scales = [&](uint32_t off, uint32_t step) {
                             set ^= 1u;
-                            const uint32_t tsfa = tmem_base + Cfg::SF_COL + set * Cfg::SF_SET;
-                            tmem_cp_32x128b_warpx4_pair(tsfa, smem_desc_sf_chunk(sa + Cfg::SFA_OFF + 512 * h));
-                            tmem_cp_32x128b_warpx4_pair(tsfa + 4, smem_desc_sf_chunk(sa + Cfg::SFW_OFF + 512 * h));
-                            tmem_cp_32x128b_warpx4_pair(tsfa + 8, smem_desc_sf_chunk(sa + Cfg::SFW_OFF + REC_SFW_BYTES + 512 * h));
+                            const uint32_t tsf = tmem_base + Cfg::SF_COL + set * Cfg::SF_SET;
+                            tmem_cp_32x128b_warpx4_pair(tsf, smem_desc_sf_chunk(sa + Cfg::SFA_OFF + off));
+                            tmem_cp_32x128b_warpx4_pair(tsf + 4, smem_desc_sf_chunk(sa + Cfg::SFW_OFF + off));
+                            tmem_cp_32x128b_warpx4_pair(tsf + 8, smem_desc_sf_chunk(sa + Cfg::SFW_OFF + off + step));
+                        };
+                        if (!WIDE_MAY || !((wide_mask >> (kb & 31)) & 1u)) {
+                            if (WIDE_MAY ? rec_loads_scales(wide_mask, kb) : (kb & 3) == 0) load_scales(0, REC_SF_BYTES);
+                            const uint32_t tsf = tmem_base + Cfg::SF_COL + set * Cfg::SF_SET;
+                            const uint32_t idesc = idesc_mxf8_e4m3(256, BN, (uint32_t)(kb & 3));
 #pragma unroll
-                            for (int j = 0; j < REC_K / 32; ++j) {
-                                const uint32_t ca = sa + (2 * j + h) * CHUNK, cw = sw + (2 * j + h) * CHUNK;
-                                mma_mxf8_ss_pair(d_tmem, smem_desc_rec(ca, zero_base - ca), smem_desc_rec(cw, zero_base - cw),
-                                                 idesc_mxf8_e4m3(256, BN, (uint32_t)j), tsfa, tsfa + 4, (kb | h | j) != 0 ? 1u : 0u);
+                            for (int j = 0; j < REC_K / 32; ++j)
+                                mma_mxf8_ss_pair(d_tmem, smem_desc_rec(sa + 2 * j * CHUNK, CHUNK), smem_desc_rec(sw + 2 * j * CHUNK, CHUNK),
+                                                 idesc, tsf, tsf + 4, (kb | j) != 0 ? 1u : 0u);
+                        } else {
+#pragma unroll 1
+                            for (int h = 0; h < 2; ++h) {
+                                load_scales(512 * h, REC_SFW_BYTES);
+                                const uint32_t tsf = tmem_base + Cfg::SF_COL + set * Cfg::SF_SET;
+#pragma unroll
+                                for (int j = 0; j < REC_K / 32; ++j) {
+                                    const uint32_t ca = sa + (2 * j + h) * CHUNK, cw = sw + (2 * j + h) * CHUNK;
+                                    mma_mxf8_ss_pair(d_tmem, smem_desc_rec(ca, zero_base - ca), smem_desc_rec(cw, zero_base - cw),
+                                                     idesc_mxf8_e4m3(256, BN, (uint32_t)j), tsf, tsf + 4, (kb | h | j) != 0 ? 1u : 0u);
+                                }
                             }
                         }
+                        ptx::mma_commit_pair(empty_bar(s), 3);          // both CTAs may refill the stage
+                        if (++s == STAGES) { s = 0; ph ^= 1u; }
                     }
-                    ptx::mma_commit_pair(empty_bar(s), 3);          // both CTAs may refill the stage
-                    if (++s == STAGES) { s = 0; ph ^= 1u; }
-                }
-                if (timed_out) break;
-                ptx::mma_commit_pair(tfull_bar(acc), 3);            // both halves of the accumulator are complete
+                };
+                if (wide_mask == 0) steps(std::false_type{});
+                else steps(std::true_type{});
+                if (kg + 1 == kgroups32 && !timed_out) ptx::mma_commit_pair(tfull_bar(acc), 3);   // both halves of the accumulator are complete
             }
         }
         __syncwarp();
-    } else {
+    } else if (warp >= 2) {
         const int quad = warp & 3;                           // TMEM lane quarter (the hardware's window for this warp)
         const int half = (warp - 2) >> 2;                    // this warp's 128 of the tile's 256 columns
         constexpr int COLS = BN / 2;
         int it = 0;
-        uint32_t epi_buf = 0;
-        constexpr bool tail = TAIL;
         for (int t = pair; t < num_tiles && !timed_out; t += npairs, ++it) {
             const int acc = it & 1;
             const uint32_t acc_ph = (uint32_t)(it >> 1) & 1u;
@@ -258,8 +384,13 @@ gemm_rec_kernel(const __grid_constant__ RecMaps tm, const TcParams p, const RecP
             const bool down = acc == 0;
             auto column = [&](int i) { return half * COLS + 32 * (down ? COLS / 32 - 1 - i : i); };
             const bool has_shared = down ? half == 1 : half == 0;
-            TailRegs ahead;
-            if (tail) tail_fetch(p, row, n0 + column(0), ahead);    // the first chunk's residual: in flight under the MMAs
+            const int rows0 = m0 + quad * 32;
+            TailRegs row_ahead;                                     // MXInt result: a row per lane
+            FragTail frag_ahead;                                    // fp32 result: the accumulator-fragment shape
+            if (TAIL) {                                             // the first chunk's residual: in flight under the MMAs
+                if (QOUT) tail_fetch(p, row, n0 + column(0), row_ahead);
+                else frag_tail_fetch(p, rows0, n0 + column(0), lane, frag_ahead);
+            }
             const bool ok = ptx::mbar_wait_bounded_cluster(tfull_bar(acc), acc_ph, abort_flag, TC_WAIT_LIMIT_NS);
             if (!__all_sync(0xFFFFFFFFu, ok)) {
                 timed_out = true;
@@ -277,31 +408,25 @@ gemm_rec_kernel(const __grid_constant__ RecMaps tm, const TcParams p, const RecP
             for (int i = 0; i < COLS / 32; ++i) {
                 const int c0 = column(i);
                 const int n = n0 + c0;
-                if (!tail && p.frag_store) {
+                if (!QOUT) {
                     uint32_t r[2][16];
+                    const FragTail cur = frag_ahead;
+                    if (TAIL && i + 1 < COLS / 32) frag_tail_fetch(p, rows0, n0 + column(i + 1), lane, frag_ahead);
                     load_f32_frag(t_acc + (uint32_t)c0, r);
                     if (i == 0 && has_shared) release();
-                    store_f32_frag_regs(p, r, m0 + quad * 32, n, 0, lane);
+                    frag_store<TAIL>(p, r, cur, rows0, n, lane);
                     continue;
                 }
                 uint32_t r[32];
                 ptx::tmem_ld_32x32(t_acc + (uint32_t)c0, r);
-                TailRegs cur;
-                if (tail) {
-                    cur = ahead;                                                          // fetched a chunk ago: has arrived
-                    if (i + 1 < COLS / 32) tail_fetch(p, row, n0 + column(i + 1), ahead);  // in flight under this chunk
-                }
+                const TailRegs cur = row_ahead;
+                if (TAIL && i + 1 < COLS / 32) tail_fetch(p, row, n0 + column(i + 1), row_ahead);
                 ptx::tmem_ld_wait();
                 if (i == 0 && has_shared) release();
-                if (tail) tail_apply(p, cur, n, r);
-                if (p.yq_mant) {
-                    store_mxint_chunk(p, row, n, r);
-                    continue;
-                }
-                store_f32_chunk<1>(p, &tm.y, r, row, m0 + quad * 32, n, 0, epi_base + (uint32_t)(warp - 2) * 4096u, epi_buf, lane);
+                if (TAIL) tail_apply(p, cur, n, r);
+                store_mxint_chunk(p, row, n, r);
             }
         }
-        if (p.tma_store && lane == 0) ptx::bulk_wait_group<0>();
     }
 
     if (timed_out) {

@@ -5,23 +5,23 @@
 // canonical K-major shape without swizzle -- [8 chunks of 16 k][128 rows][16 bytes], so a chunk of 8 rows is
 // 128 contiguous bytes and a record one contiguous copy -- and records follow one another along K.
 //
-// Scales.  A row has ONE scale per record: byte S, 2^(S-127), and its elements are q * 2^t with t = E - (w-2) - (S-127)
-// per block.  E4M3 holds q * 2^t without rounding for |q| <= 16 (mantissa widths up to 5) as long as t >= -9 and
-// |q| * 2^t <= 448; S is set by the largest exponent of the row's blocks in the record, with t at its upper limit there
-// (5 for nibble containers, |q| <= 8, and 4 for 5-bit mantissas), so the blocks of a record may lie up to 14 (13) binades
-// apart.  One scale per 128 k instead of the hardware's one per 32 means that the four bytes of a tensor-memory cell
-// serve four K steps: the copies shared -> tensor memory, which the tensor pipe executes between MMAs (about 60 ns per
-// K step of 0.35 us when done for each one), are needed for every fourth step only.  They lie in chunks of 512 bytes, byte
+// Scales.  A row has ONE scale per record: byte S, 2^(S-127), and its elements are q * 2^t with
+// t = E - (w-2) - (S-127) per block.  E4M3 holds q * 2^t without rounding for |q| <= 16 (mantissa widths up to 5) as long as
+// t >= -9 and |q| * 2^t <= 448; S is set by the largest exponent of the row's blocks in the record, with t at its upper
+// limit there (5 for nibble containers, |q| <= 8, else 4), so the blocks of a record may lie up to 14 (13) binades apart.  One scale per 128 k instead of
+// the hardware's one per 32 means that the four bytes of a tensor-memory cell serve four K steps: the copies
+// shared -> tensor memory, which the tensor pipe executes between MMAs (about 60 ns per K step of 0.35 us when done for
+// each one), are needed for every fourth step only.  They lie in chunks of 512 bytes, byte
 // (row % 32) * 16 + (row / 32) * 4 + kb % 4 -- what tcgen05.cp.32x128b.warpx4 puts where the MMA looks -- in the order
 // [kb / 4][panel], so that a tile's two panels of W are adjacent.
 //
-// Where the blocks of some row and record lie further apart, each of them keeps a scale of its own and the call's
-// flag word is set to the call's tag: the product then takes the halves (16 k) of every 32 k in separate MMAs with
-// their own scales, which are written for every row into a second array: 1 KB per record, order [kb][panel], one chunk
-// for the k % 32 < 16 and one for the others, byte (row % 32) * 16 + (row / 32) * 4 + (k / 32) % 4.  A stale or random
-// flag word can only make a product slower, never wrong, so nothing has to be cleared between calls.
+// Where the blocks of some row and record lie further apart, each of them keeps a scale of its own and the flag byte of
+// the record's 8 rows is set: the product then takes the halves (16 k) of every 32 k of this K step in separate MMAs with
+// their own scales, which are written for every row into a second array: 1 KB per record, order
+// [kb][panel], one chunk for the k % 32 < 16 and one for the others, byte
+// (row % 32) * 16 + (row / 32) * 4 + (k / 32) % 4.  Every flag byte has one writer, so nothing is cleared between calls.
 //
-// Both passes are bound by HBM and, at a few thousand rows, by the latency of their few iterations.  A quantizing
+// The passes are bound by HBM and, at a few thousand rows, by the latency of their few iterations.  A quantizing
 // lane owns 16 consecutive k of a row (so a block of 16 needs no exchange and one of 32 a single shuffle) and eight
 // lanes with neighbouring rows store 128 contiguous bytes; four 16-byte loads per lane and half record are in flight
 // at once.  A decoding lane owns 32 consecutive k.
@@ -44,29 +44,29 @@ struct RecOut {
     uint8_t *elems;          // [panels][kblocks][REC_BYTES]
     uint8_t *sf;             // [ceil(kblocks / 4)][panels_sf][REC_SF_BYTES]
     uint8_t *sf_wide;        // [kblocks][panels_sf][REC_SFW_BYTES]
+    uint8_t *flags;          // [panels][kblocks][16], one byte per 8 rows: 1 = some row's blocks keep scales of their own
     int panels, panels_sf, kblocks;
-    unsigned long long *flag;        // set to `tag` when the blocks of some row and record keep separate scales
-    unsigned long long tag;
 };
 
-// Largest t with |q| * 2^t <= 256 < 448 (the E4M3 maximum) for every q the container holds (-8 and -16 included).
+// Largest t with |element| * 2^t <= 256 < 448 (the E4M3 maximum) for every q the container holds (-8 and -16 included).
 __device__ __forceinline__ int rec_t_max(int w) { return w <= 4 ? 5 : 4; }
 constexpr int REC_T_MIN = -9;                            // multiples of 2^-9 are E4M3 numbers (up to 4 significant bits)
 
 // Scale byte of a block with exponent byte e (finite): 2^(S-127) with the block's elements q * 2^t, t <= t_max.
 __device__ __forceinline__ int rec_scale_byte(int e, int w) { return max(0, e - (w - 2) - rec_t_max(w)); }
 
-// The scale of a row in one record, agreed on by the four lanes that hold the row (a quad).  e0, e1: exponent bytes of
-// the lane's two groups of 16 k; z0, z1: the group holds zeros only (its exponent does not matter).
+// The scale of a row in one record, agreed on by the LANES neighbouring lanes that hold the row.  e0, e1: exponent bytes
+// of the lane's two groups of 16 k; z0, z1: the group holds zeros only (its exponent does not matter).
 struct RecScale { int s, s0, s1; bool wide; };           // the row's byte; the bytes the two groups are scaled by
 
+template <int LANES = 4>
 __device__ __forceinline__ RecScale rec_scales(int e0, int e1, bool z0, bool z1, int w)
 {
     // largest exponent in the low half word, 255 - smallest in the high one: one shuffle and one maximum per step
     uint32_t m = (z0 ? 0u : (uint32_t)e0 | ((uint32_t)(255 - e0) << 16));
     m = __vmaxu2(m, z1 ? 0u : (uint32_t)e1 | ((uint32_t)(255 - e1) << 16));
 #pragma unroll
-    for (int d = 1; d < 4; d <<= 1) m = __vmaxu2(m, __shfl_xor_sync(0xFFFFFFFFu, m, d));
+    for (int d = 1; d < LANES; d <<= 1) m = __vmaxu2(m, __shfl_xor_sync(0xFFFFFFFFu, m, d));
     const int hi = (int)(m & 0xFFFFu), lo = 255 - (int)(m >> 16);
     RecScale r;
     r.wide = false;
@@ -91,15 +91,17 @@ __device__ __forceinline__ uint32_t e4m3x2(float lo, float hi)
 }
 __device__ __forceinline__ uint32_t e4m3x4(float a, float b, float c, float d) { return e4m3x2(a, b) | (e4m3x2(c, d) << 16); }
 
-// Scale bytes: the quad's first lane writes the one of the row and record, every lane those of its two groups of 16 k
-// (g0, g1: their numbers within the record).
-__device__ __forceinline__ void rec_store_scales(const RecOut &o, int panel, int kb, int rp, const RecScale &s, int g0, int g1)
+// The scale byte of the row and record.
+__device__ __forceinline__ void rec_store_scale(const RecOut &o, int panel, int kb, int rp, int s)
 {
-    const int at = (rp & 31) * 16 + (rp >> 5) * 4;
-    if ((threadIdx.x & 3) == 0) o.sf[((int64_t)(kb >> 2) * o.panels_sf + panel) * REC_SF_BYTES + at + (kb & 3)] = (uint8_t)s.s;
-    uint8_t *wide = o.sf_wide + ((int64_t)kb * o.panels_sf + panel) * REC_SFW_BYTES + at;
-    wide[(g0 & 1) * 512 + (g0 >> 1)] = (uint8_t)s.s0;
-    wide[(g1 & 1) * 512 + (g1 >> 1)] = (uint8_t)s.s1;
+    o.sf[((int64_t)(kb >> 2) * o.panels_sf + panel) * REC_SF_BYTES + (rp & 31) * 16 + (rp >> 5) * 4 + (kb & 3)] = (uint8_t)s;
+}
+// The scale bytes of its groups g0 and g1 of 16 k (numbers within the record).
+__device__ __forceinline__ void rec_store_wide(const RecOut &o, int panel, int kb, int rp, const RecScale &s, int g0, int g1)
+{
+    uint8_t *d = o.sf_wide + ((int64_t)kb * o.panels_sf + panel) * REC_SFW_BYTES + (rp & 31) * 16 + (rp >> 5) * 4;
+    d[(g0 & 1) * 512 + (g0 >> 1)] = (uint8_t)s.s0;
+    d[(g1 & 1) * 512 + (g1 >> 1)] = (uint8_t)s.s1;
 }
 
 // Eight values of one block (exponent byte e, width w) -> E4M3 codes of q * 2^t, t = e - (w-2) - sb.  The sum x + M
@@ -130,6 +132,17 @@ __device__ __forceinline__ uint2 rec_encode8(const float (&v)[8], int e, int w, 
     return make_uint2(e4m3x4(q[0], q[1], q[2], q[3]), e4m3x4(q[4], q[5], q[6], q[7]));
 }
 
+constexpr uint32_t E4M3_NAN4 = 0x7F7F7F7Fu;
+
+// Sixteen values of one block -> their 16 bytes.
+__device__ __forceinline__ uint4 rec_encode16(const float (&v)[2][8], int e, bool zero, int w, int sb)
+{
+    if (sb == 255) return make_uint4(E4M3_NAN4, E4M3_NAN4, E4M3_NAN4, E4M3_NAN4);
+    if (zero) return make_uint4(0, 0, 0, 0);
+    const uint2 x = rec_encode8(v[0], e, w, sb), y = rec_encode8(v[1], e, w, sb);
+    return make_uint4(x.x, x.y, y.x, y.y);
+}
+
 // Floating-point rows -> records.  Warp item = 8 rows x one record's 128 k; lane = row * 4 + chunk, two passes of four
 // chunks.  ROWS2: rows 2i and 2i + 1 share the exponents.  Rows >= `rows` and k >= K become
 // zeros.
@@ -139,7 +152,6 @@ __device__ __forceinline__ void rec_quantize_body(const InT *__restrict__ x, int
 {
     const int lane = threadIdx.x & 31, r8 = lane >> 2, c4 = lane & 3;
     const uint32_t kblocks = (uint32_t)o.kblocks, items = (uint32_t)o.panels * (REC_ROWS / 8) * kblocks;
-    bool any_wide = false;
     for (uint32_t it = warp_id; it < items; it += n_warps) {
         // neighbouring warps take neighbouring records of the same rows
         const uint32_t grp = it / kblocks;
@@ -172,30 +184,31 @@ __device__ __forceinline__ void rec_quantize_body(const InT *__restrict__ x, int
             z[u] = amax == 0;
         }
         const RecScale s = rec_scales(e[0], e[1], z[0], z[1], w);
-        any_wide |= s.wide;
         uint8_t *dst = o.elems + ((int64_t)panel * kblocks + kb) * REC_BYTES + c4 * (REC_ROWS * 16) + rp * 16;
 #pragma unroll
-        for (int u = 0; u < 2; ++u) {
-            const int sb = u ? s.s1 : s.s0;
-            uint4 b = make_uint4(0, 0, 0, 0);
-            if (sb == 255) {
-                b = make_uint4(0x7F7F7F7Fu, 0x7F7F7F7Fu, 0x7F7F7F7Fu, 0x7F7F7F7Fu);      // E4M3 NaN
-            } else if (!z[u]) {
-                const uint2 b0 = rec_encode8(v[u][0], e[u], w, sb), b1 = rec_encode8(v[u][1], e[u], w, sb);
-                b = make_uint4(b0.x, b0.y, b1.x, b1.y);
-            }
-            *reinterpret_cast<uint4 *>(dst + u * 4 * (REC_ROWS * 16)) = b;
-        }
-        rec_store_scales(o, panel, kb, rp, s, c4, 4 + c4);
+        for (int u = 0; u < 2; ++u)
+            *reinterpret_cast<uint4 *>(dst + u * 4 * (REC_ROWS * 16)) = rec_encode16(v[u], e[u], z[u], w, u ? s.s1 : s.s0);
+        if (c4 == 0) rec_store_scale(o, panel, kb, rp, s.s);
+        rec_store_wide(o, panel, kb, rp, s, c4, 4 + c4);
+        const bool wide = __any_sync(0xFFFFFFFFu, s.wide);
+        if (lane == 0) o.flags[((int64_t)panel * kblocks + kb) * 16 + (grp & 15)] = wide;
     }
-    if (any_wide) *o.flag = o.tag;
+}
+
+// Four table lookups at once: nibble i of `sel` (two's complement) picks byte i of the result, from p0 p1 for 0..7 and from
+// n0 n1 for -8..-1 (a byte permute selects by three bits).  The p entries have sign bit 0, the n entries 1.
+__device__ __forceinline__ uint32_t rec_lut4(uint32_t sel, uint32_t p0, uint32_t p1, uint32_t n0, uint32_t n1)
+{
+    const uint32_t pos = __byte_perm(p0, p1, sel & 0x7777u), neg = __byte_perm(n0, n1, sel & 0x7777u);
+    uint32_t keep;                      // selector bit 3 copies the sign of the selected byte: 0x7F for q >= 0, 0 for q < 0
+    asm("prmt.b32 %0, %1, %1, %2;" : "=r"(keep) : "r"(0x7F7F7F7Fu), "r"(sel));
+    return ((pos & keep) | (neg & ~keep)) ^ ((keep << 1) & 0x80808080u);
 }
 
 // Sixteen mantissas of one block -> E4M3 codes of q * 2^t.
-// Nibbles: a byte permute looks four of them up at once, one table of eight codes for q = 0..7 and one for q = -8..-1
-// (the low three bits select in both, the fourth between the two); the tables are those of t = 0 plus t in every
-// exponent field, which holds while the smallest value is a normal E4M3 number (t >= -6).  Other t, and int8
-// mantissas: the offset integer as a float in [2^23, 2^23 + 255], one exact fma, one conversion.
+// Nibbles by table: the codes of t = 0 plus t in every exponent field (but that of zero), which holds while the smallest
+// value is a normal E4M3 number (t >= -6).  Other t, and int8 mantissas: the offset integer as a float in
+// [2^23, 2^23 + 255], one exact fma, one conversion.
 template <bool NIBBLE>
 __device__ __forceinline__ uint4 rec_codes16(const uint32_t (&m)[NIBBLE ? 2 : 4], int t)
 {
@@ -205,14 +218,7 @@ __device__ __forceinline__ uint4 rec_codes16(const uint32_t (&m)[NIBBLE ? 2 : 4]
         const uint32_t p0 = 0x44403800u + (uint32_t)t * 0x08080800u, p1 = 0x4E4C4A48u + dt;      // 0 1 2 3, 4 5 6 7
         const uint32_t n0 = 0xCACCCED0u + dt, n1 = 0xB8C0C4C8u + dt;                             // -8 .. -5, -4 .. -1
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            const uint32_t p = i & 1 ? m[i >> 1] >> 16 : m[i >> 1];
-            const uint32_t pos = __byte_perm(p0, p1, p & 0x7777u), neg = __byte_perm(n0, n1, p & 0x7777u);
-            // selector bit 3 copies the sign of the selected byte: 0x7F for q >= 0, 0 for q < 0
-            uint32_t keep;
-            asm("prmt.b32 %0, %1, %1, %2;" : "=r"(keep) : "r"(0x7F7F7F7Fu), "r"(p));
-            b[i] = ((pos & keep) | (neg & ~keep)) ^ ((keep << 1) & 0x80808080u);
-        }
+        for (int i = 0; i < 4; ++i) b[i] = rec_lut4(i & 1 ? m[i >> 1] >> 16 : m[i >> 1], p0, p1, n0, n1);
     } else {
         const float f = __uint_as_float((uint32_t)(127 + t) << 23);
         const float c = (NIBBLE ? -8388616.0f : -8388736.0f) * f;        // -(2^23 + 8), -(2^23 + 128)
@@ -273,14 +279,13 @@ __device__ __forceinline__ void rec_fetch(const RecPacked &j, uint32_t it, uint3
 }
 
 template <bool NIBBLE, int UNROLL>
-__device__ __forceinline__ bool rec_convert(const RecPacked &j, const RecOut &o, uint32_t it, uint32_t steps,
+__device__ __forceinline__ void rec_convert(const RecPacked &j, const RecOut &o, uint32_t it, uint32_t steps,
                                             const RecPackedItem<NIBBLE, UNROLL> &d)
 {
     const int lane = threadIdx.x & 31, r8 = lane >> 2, c4 = lane & 3;
     const uint32_t grp = it / steps;
     const int kb0 = (int)(it - grp * steps) * UNROLL;
     const int panel = (int)(grp >> 4), rp = (int)((grp * 8 + r8) & 127);
-    bool any_wide = false;
 #pragma unroll
     for (int u = 0; u < UNROLL; ++u) {
         const int kb = kb0 + u;
@@ -297,19 +302,20 @@ __device__ __forceinline__ bool rec_convert(const RecPacked &j, const RecOut &o,
             for (int i = 0; i < H; ++i) any[h] |= (half[h][i] = words[h * H + i]);
         // a block that held Inf/NaN is stored as byte 255 with zero mantissas: it still poisons
         const RecScale s = rec_scales(e0, e1, any[0] == 0 && e0 != 255, any[1] == 0 && e1 != 255, j.w);
-        any_wide |= s.wide;
         uint8_t *dst = o.elems + ((int64_t)panel * o.kblocks + kb) * REC_BYTES + (c4 * 2) * (REC_ROWS * 16) + rp * 16;
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
             const int sb = h ? s.s1 : s.s0;
             uint4 b = make_uint4(0, 0, 0, 0);
-            if (sb == 255) b = make_uint4(0x7F7F7F7Fu, 0x7F7F7F7Fu, 0x7F7F7F7Fu, 0x7F7F7F7Fu);
+            if (sb == 255) b = make_uint4(E4M3_NAN4, E4M3_NAN4, E4M3_NAN4, E4M3_NAN4);
             else if (any[h]) b = rec_codes16<NIBBLE>(half[h], (h ? e1 : e0) - (j.w - 2) - sb);
             *reinterpret_cast<uint4 *>(dst + h * (REC_ROWS * 16)) = b;
         }
-        rec_store_scales(o, panel, kb, rp, s, 2 * c4, 2 * c4 + 1);
+        if (c4 == 0) rec_store_scale(o, panel, kb, rp, s.s);
+        rec_store_wide(o, panel, kb, rp, s, 2 * c4, 2 * c4 + 1);
+        const bool wide = __any_sync(0xFFFFFFFFu, s.wide);
+        if (lane == 0) o.flags[((int64_t)panel * o.kblocks + kb) * 16 + (grp & 15)] = wide;
     }
-    return any_wide;
 }
 
 __device__ __forceinline__ uint32_t rec_steps(const RecOut &o, int unroll) { return (uint32_t)((o.kblocks + unroll - 1) / unroll); }
@@ -320,14 +326,12 @@ __device__ __forceinline__ void rec_decode_body(const RecPacked &j, const RecOut
                                                 RecPackedItem<NIBBLE, UNROLL> &d)
 {
     const uint32_t steps = rec_steps(o, UNROLL), items = (uint32_t)o.panels * (REC_ROWS / 8) * steps;
-    bool any_wide = false;
     for (uint32_t it = warp_id; it < items; it += n_warps) {
         RecPackedItem<NIBBLE, UNROLL> next;
         rec_fetch<NIBBLE, UNROLL>(j, it + n_warps, steps, items, next);
-        any_wide |= rec_convert<NIBBLE, UNROLL>(j, o, it, steps, d);
+        rec_convert<NIBBLE, UNROLL>(j, o, it, steps, d);
         d = next;
     }
-    if (any_wide) *o.flag = o.tag;
 }
 
 // Both operands of a layer in one launch: every warp takes its share of the activations, then of the weights.
@@ -340,7 +344,7 @@ struct RecPrepJob {
 };
 
 template <typename InT, bool NIBBLE>
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(256, 3)
 rec_prep_kernel(const RecPrepJob j)
 {
     ptx::dep_wait();
@@ -370,7 +374,7 @@ struct RecPairJob {
 };
 
 template <bool NIB_A, bool NIB_W>
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(256, 3)
 rec_pair_kernel(const RecPairJob j)
 {
     ptx::dep_wait();

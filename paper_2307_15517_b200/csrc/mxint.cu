@@ -7,7 +7,6 @@
 #include <stdio.h>
 #include <string.h>
 
-#include <atomic>
 #include <map>
 #include <mutex>
 #include <tuple>
@@ -47,7 +46,7 @@ struct DeviceInfo {
     bool tc2_attr_set[2] = {false, false};
     bool tcx_attr_set = false;
     bool tc8_attr_set = false;
-    bool rec_attr_set[2] = {false, false};
+    bool rec_attr_set[4] = {};
     bool attn_attr_set[2] = {false, false};
 };
 DeviceInfo g_dev[MAX_DEVICES];
@@ -715,7 +714,7 @@ mx_status_t run_tc8(const void *a_mant, const uint8_t *a_exp, const mx_format_t 
 // ---- block-scaled product on records (mx_records.cuh, mx_gemm_rec.cuh) ------------------------------
 struct RecLayout {
     int panels_a, panels_w, kblocks, kgroups;
-    size_t a_elems, a_sf, a_sfw, w_elems, w_sf, w_sfw, flag, bytes;      // offsets into the workspace, total size
+    size_t a_elems, a_sf, a_sfw, a_flags, w_elems, w_sf, w_sfw, w_flags, bytes;      // offsets into the workspace, total size
 };
 int even_up(int v) { return (v + 1) & ~1; }
 RecLayout rec_layout(int64_t M, int64_t N, int64_t K)
@@ -726,13 +725,17 @@ RecLayout rec_layout(int64_t M, int64_t N, int64_t K)
     l.kblocks = (int)((K + mx::REC_K - 1) / mx::REC_K);
     l.kgroups = (l.kblocks + 3) / 4;
     size_t off = 0;
-    l.a_elems = off; off += (size_t)l.panels_a * l.kblocks * mx::REC_BYTES;
-    l.a_sf = off; off += (size_t)even_up(l.panels_a) * l.kgroups * mx::REC_SF_BYTES;
-    l.a_sfw = off; off += (size_t)even_up(l.panels_a) * l.kblocks * mx::REC_SFW_BYTES;
-    l.w_elems = off; off += (size_t)l.panels_w * l.kblocks * mx::REC_BYTES;
-    l.w_sf = off; off += (size_t)even_up(l.panels_w) * l.kgroups * mx::REC_SF_BYTES;
-    l.w_sfw = off; off += (size_t)even_up(l.panels_w) * l.kblocks * mx::REC_SFW_BYTES;
-    l.flag = off; off += 256;
+    auto take = [&](size_t n) { const size_t at = off; off += round256(n); return at; };
+    const size_t pa = (size_t)l.panels_a, pw = (size_t)l.panels_w, kb = (size_t)l.kblocks, kg = (size_t)l.kgroups;
+    const size_t sa = (size_t)even_up(l.panels_a), sw = (size_t)even_up(l.panels_w);
+    l.a_elems = take(pa * kb * mx::REC_BYTES);
+    l.a_sf = take(sa * kg * mx::REC_SF_BYTES);
+    l.a_sfw = take(sa * kb * mx::REC_SFW_BYTES);
+    l.a_flags = take(pa * kb * 16);
+    l.w_elems = take(pw * kb * mx::REC_BYTES);
+    l.w_sf = take(sw * kg * mx::REC_SF_BYTES);
+    l.w_sfw = take(sw * kb * mx::REC_SFW_BYTES);
+    l.w_flags = take(pw * kb * 16);
     l.bytes = off;
     return l;
 }
@@ -748,21 +751,21 @@ bool rec_fits(const mx_format_t &fa, const mx_format_t &fw, int64_t M, int64_t N
     if (fa.elem_bits > 5 || fw.elem_bits > 5 || fa.packing || fw.packing || (K % 32) != 0) return false;
     if (K < 2048 && N * K < 3 * (1 << 20)) return false;
     const RecLayout l = rec_layout(M, N, K);
-    if ((int64_t)l.panels_a * l.kblocks * 16 > INT32_MAX / 2 || (int64_t)l.panels_w * l.kblocks * 16 > INT32_MAX / 2) return false;
+    if ((int64_t)l.panels_a * l.kblocks * 16 > INT32_MAX / 2 || (int64_t)l.panels_w * l.kblocks * 16 > INT32_MAX / 2)
+        return false;
     return l.bytes <= tc_workspace(M, N, K);             // the workspace the caller was told to bring
 }
 
-mx::RecOut rec_out(const RecLayout &l, uint8_t *ws, bool weights, uint64_t tag)
+mx::RecOut rec_out(const RecLayout &l, uint8_t *ws, bool weights)
 {
     mx::RecOut o;
     o.elems = ws + (weights ? l.w_elems : l.a_elems);
     o.sf = ws + (weights ? l.w_sf : l.a_sf);
     o.sf_wide = ws + (weights ? l.w_sfw : l.a_sfw);
+    o.flags = ws + (weights ? l.w_flags : l.a_flags);
     o.panels = weights ? l.panels_w : l.panels_a;
     o.panels_sf = even_up(o.panels);
     o.kblocks = l.kblocks;
-    o.flag = reinterpret_cast<unsigned long long *>(ws + l.flag);
-    o.tag = tag;
     return o;
 }
 
@@ -773,13 +776,6 @@ mx::RecPacked rec_packed(const void *mant, const uint8_t *exps, const mx_format_
     p.rows = rows; p.K = K;
     p.block = f.block; p.w = f.elem_bits; p.row_shift = f.block_rows == 2 ? 1 : 0;
     return p;
-}
-
-// A tag no other call of this process has; an old flag word equal to it costs speed only.
-uint64_t next_rec_tag()
-{
-    static std::atomic<uint64_t> calls{0};
-    return (calls.fetch_add(1, std::memory_order_relaxed) + 1) * 0x9E3779B97F4A7C15ull;
 }
 
 // `rows` rows of `words` (at most 256) 32-bit words, box of `box_rows` of them (contiguous in shared memory).
@@ -804,10 +800,22 @@ mx_status_t encode_words(CUtensorMap *tm, const void *base, int words, int64_t r
     return MX_OK;
 }
 
-mx_status_t launch_rec(const RecLayout &l, uint8_t *ws, uint64_t tag, int64_t M, int64_t N, int64_t K, const float *bias,
-                       float *y, int64_t ldy, const QuantizedOut *yq, DeviceInfo &d, cudaStream_t st, const EpiTail &et)
+template <bool TAIL, bool QOUT>
+mx_status_t launch_rec_as(const mx::RecMaps &tm, const mx::TcParams &p, const mx::RecParams &rp, int pairs, DeviceInfo &d, cudaStream_t st)
 {
     using Cfg = mx::RecCfg;
+    const mx_status_t s = smem_attr_once(d.rec_attr_set[(TAIL ? 2 : 0) + (QOUT ? 1 : 0)],
+                                         mx::gemm_rec_kernel<TAIL, QOUT>, (int)Cfg::SMEM_BYTES);
+    if (s != MX_OK) return s;
+    ProfScope prof(KIND_GEMM_TC, st);
+    MX_CUDA(launch_dep(mx::gemm_rec_kernel<TAIL, QOUT>, dim3(2 * pairs), dim3(Cfg::THREADS), Cfg::SMEM_BYTES, st, tm, p, rp));
+    MX_CUDA(cudaGetLastError());
+    return MX_OK;
+}
+
+mx_status_t launch_rec(const RecLayout &l, uint8_t *ws, int64_t M, int64_t N, int64_t K, const float *bias,
+                       float *y, int64_t ldy, const QuantizedOut *yq, DeviceInfo &d, cudaStream_t st, const EpiTail &et)
+{
     mx::RecMaps tm;
     const int sa = even_up(l.panels_a), sw = even_up(l.panels_w);
     constexpr int SF_WORDS = (int)mx::REC_SF_BYTES / 4, SFW_WORDS = (int)mx::REC_SFW_BYTES / 4;
@@ -819,20 +827,10 @@ mx_status_t launch_rec(const RecLayout &l, uint8_t *ws, uint64_t tag, int64_t M,
         {&tm.sa_wide, l.a_sfw, SFW_WORDS, (int64_t)sa * l.kblocks, 1},
         {&tm.sw_wide, l.w_sfw, SFW_WORDS, (int64_t)sw * l.kblocks, 2},
     };
-    mx_status_t s = MX_OK;
     for (const auto &m : maps) {
-        s = encode_words(m.map, ws + m.at, m.words, m.rows, m.box);
+        const mx_status_t s = encode_words(m.map, ws + m.at, m.words, m.rows, m.box);
         if (s != MX_OK) return s;
     }
-    tm.y = tm.a;
-    const bool tma_store = !yq && (ldy % 4) == 0 && (N % 4) == 0;       // see launch_tc
-    if (tma_store) {
-        s = encode_f32_out(&tm.y, y, M, N, ldy);
-        if (s != MX_OK) return s;
-    }
-    s = et.any() ? smem_attr_once(d.rec_attr_set[1], mx::gemm_rec_kernel<true>, (int)Cfg::SMEM_BYTES)
-                 : smem_attr_once(d.rec_attr_set[0], mx::gemm_rec_kernel<false>, (int)Cfg::SMEM_BYTES);
-    if (s != MX_OK) return s;
     mx::TcParams p{};
     p.y = y;
     p.bias = et.any() ? nullptr : bias;
@@ -847,8 +845,7 @@ mx_status_t launch_rec(const RecLayout &l, uint8_t *ws, uint64_t tag, int64_t M,
     p.tiles_m = (l.panels_a + 1) / 2;
     p.tiles_n = (l.panels_w + 1) / 2;
     p.status = d.status;
-    p.tma_store = tma_store ? 1 : 0;
-    p.frag_store = frag_store_ok(yq != nullptr, et.any(), y, ldy, 0) ? 1 : 0;
+    p.frag_store = frag_store_ok(yq != nullptr, false, y, ldy, 0) ? 1 : 0;
     p.batch = 1;
     p.yq_mant = yq ? yq->mant : nullptr;
     p.yq_exp = yq ? yq->exps : nullptr;
@@ -856,13 +853,21 @@ mx_status_t launch_rec(const RecLayout &l, uint8_t *ws, uint64_t tag, int64_t M,
     p.yq_bits = yq ? yq->f.elem_bits : 0;
     p.yq_block = yq ? yq->f.block : 0;
     p.yq_rows2 = yq && yq->f.block_rows == 2 ? 1 : 0;
-    const mx::RecParams rp{reinterpret_cast<const unsigned long long *>(ws + l.flag), tag, sa, sw};
+    const mx::RecParams rp{ws + l.a_flags, ws + l.w_flags, l.panels_a, l.panels_w, sa, sw};
     const int64_t tiles = (int64_t)p.tiles_m * p.tiles_n;
     if (tiles > INT32_MAX / 2) return MX_ERR_SHAPE;
     const int pairs = tiles < d.sm_count / 2 ? (int)tiles : d.sm_count / 2;
-    ProfScope prof(KIND_GEMM_TC, st);
-    if (et.any()) MX_CUDA(launch_dep(mx::gemm_rec_kernel<true>, dim3(2 * pairs), dim3(Cfg::THREADS), Cfg::SMEM_BYTES, st, tm, p, rp));
-    else MX_CUDA(launch_dep(mx::gemm_rec_kernel<false>, dim3(2 * pairs), dim3(Cfg::THREADS), Cfg::SMEM_BYTES, st, tm, p, rp));
+    const bool tail = et.any(), q = yq != nullptr;
+    if (tail) return q ? launch_rec_as<true, true>(tm, p, rp, pairs, d, st) : launch_rec_as<true, false>(tm, p, rp, pairs, d, st);
+    return q ? launch_rec_as<false, true>(tm, p, rp, pairs, d, st) : launch_rec_as<false, false>(tm, p, rp, pairs, d, st);
+}
+
+template <typename Job>
+mx_status_t launch_rec_prep(void (*kernel)(Job), const Job &job, int64_t items, int threads, int kind, const DeviceInfo &d, cudaStream_t st)
+{
+    const int per_sm = resident_ctas(kernel) * (256 / threads);
+    ProfScope prof(kind, st);
+    MX_CUDA(launch_dep(kernel, dim3((unsigned)grid_for(items, threads / 32, d.sm_count, per_sm)), dim3((unsigned)threads), 0, st, job));
     MX_CUDA(cudaGetLastError());
     return MX_OK;
 }
@@ -872,30 +877,20 @@ mx_status_t run_rec_linear(const mx_linear_args_t &a, const float *bias, float *
                            uint8_t *ws, DeviceInfo &d, cudaStream_t st, const EpiTail &et)
 {
     const RecLayout l = rec_layout(a.M, a.N, a.K);
-    const uint64_t tag = next_rec_tag();
     mx::RecPrepJob job;
     job.x = a.x; job.M = a.M; job.K = a.K; job.ldx = a.ldx;
     job.wa = a.fa.elem_bits; job.block = a.fa.block; job.a_rows2 = a.fa.block_rows == 2 ? 1 : 0;
-    job.a = rec_out(l, ws, false, tag);
+    job.a = rec_out(l, ws, false);
     job.pw = rec_packed(a.w_mant, a.w_exp, a.fw, a.N, a.K);
-    job.w = rec_out(l, ws, true, tag);
-    const bool f32 = a.dt == MX_F32, nib = a.fw.elem_bits <= 4;
-    constexpr int PT = 128;                              // as in tc_prepare
-    const int per_sm = (256 / PT) * (f32 ? (nib ? resident_ctas(mx::rec_prep_kernel<float, true>)
-                                                : resident_ctas(mx::rec_prep_kernel<float, false>))
-                                         : (nib ? resident_ctas(mx::rec_prep_kernel<__nv_bfloat16, true>)
-                                                : resident_ctas(mx::rec_prep_kernel<__nv_bfloat16, false>)));
+    job.w = rec_out(l, ws, true);
+    typedef __nv_bfloat16 bf16;
+    static void (*const kernels[2][2])(mx::RecPrepJob) = {         // [fp32][nibble weights]
+        {mx::rec_prep_kernel<bf16, false>, mx::rec_prep_kernel<bf16, true>},
+        {mx::rec_prep_kernel<float, false>, mx::rec_prep_kernel<float, true>}};
     const int64_t items = (int64_t)l.panels_a * 16 * l.kblocks + (int64_t)l.panels_w * 16 * ((l.kblocks + 1) / 2);
-    const dim3 grid((unsigned)grid_for(items, PT / 32, d.sm_count, per_sm));
-    {
-        ProfScope prof(KIND_PREP, st);
-        if (f32 && nib) MX_CUDA(launch_dep(mx::rec_prep_kernel<float, true>, grid, dim3(PT), 0, st, job));
-        else if (f32) MX_CUDA(launch_dep(mx::rec_prep_kernel<float, false>, grid, dim3(PT), 0, st, job));
-        else if (nib) MX_CUDA(launch_dep(mx::rec_prep_kernel<__nv_bfloat16, true>, grid, dim3(PT), 0, st, job));
-        else MX_CUDA(launch_dep(mx::rec_prep_kernel<__nv_bfloat16, false>, grid, dim3(PT), 0, st, job));
-        MX_CUDA(cudaGetLastError());
-    }
-    return launch_rec(l, ws, tag, a.M, a.N, a.K, bias, y, ldy, yq, d, st, et);
+    const mx_status_t s = launch_rec_prep(kernels[a.dt == MX_F32][a.fw.elem_bits <= 4], job, items, 128, KIND_PREP, d, st);
+    if (s != MX_OK) return s;
+    return launch_rec(l, ws, a.M, a.N, a.K, bias, y, ldy, yq, d, st, et);
 }
 
 // A product of two packed operands on records.
@@ -905,25 +900,18 @@ mx_status_t run_rec_gemm(const void *a_mant, const uint8_t *a_exp, const mx_form
                          const EpiTail &et)
 {
     const RecLayout l = rec_layout(M, N, K);
-    const uint64_t tag = next_rec_tag();
     mx::RecPairJob j;
     j.pa = rec_packed(a_mant, a_exp, fa, M, K);
     j.pw = rec_packed(w_mant, w_exp, fw, N, K);
-    j.a = rec_out(l, ws, false, tag);
-    j.w = rec_out(l, ws, true, tag);
-    const bool na = fa.elem_bits <= 4, nw = fw.elem_bits <= 4;
-    const int per_sm = resident_ctas(mx::rec_pair_kernel<true, true>);
+    j.a = rec_out(l, ws, false);
+    j.w = rec_out(l, ws, true);
+    static void (*const kernels[2][2])(mx::RecPairJob) = {         // [nibble A][nibble W]
+        {mx::rec_pair_kernel<false, false>, mx::rec_pair_kernel<false, true>},
+        {mx::rec_pair_kernel<true, false>, mx::rec_pair_kernel<true, true>}};
     const int64_t items = (int64_t)(l.panels_a + l.panels_w) * 16 * ((l.kblocks + 1) / 2);
-    const dim3 grid((unsigned)grid_for(items, 8, d.sm_count, per_sm));
-    {
-        ProfScope prof(KIND_DEQUANTIZE, st);
-        if (na && nw) MX_CUDA(launch_dep(mx::rec_pair_kernel<true, true>, grid, dim3(256), 0, st, j));
-        else if (na) MX_CUDA(launch_dep(mx::rec_pair_kernel<true, false>, grid, dim3(256), 0, st, j));
-        else if (nw) MX_CUDA(launch_dep(mx::rec_pair_kernel<false, true>, grid, dim3(256), 0, st, j));
-        else MX_CUDA(launch_dep(mx::rec_pair_kernel<false, false>, grid, dim3(256), 0, st, j));
-        MX_CUDA(cudaGetLastError());
-    }
-    return launch_rec(l, ws, tag, M, N, K, bias, y, ldy, yq, d, st, et);
+    const mx_status_t s = launch_rec_prep(kernels[fa.elem_bits <= 4][fw.elem_bits <= 4], j, items, 256, KIND_DEQUANTIZE, d, st);
+    if (s != MX_OK) return s;
+    return launch_rec(l, ws, M, N, K, bias, y, ldy, yq, d, st, et);
 }
 
 bool wide_tile(int64_t M, int64_t N, const DeviceInfo &d)
