@@ -37,6 +37,17 @@ __device__ __forceinline__ float block_max(float v, float *scratch)
     return t;
 }
 
+// One normalised value.  The roundings are spelled out: left to the compiler, whether the last product and the sum became
+// one fma changed with the number of values per thread, and the LayerNorm kernel and the operand pass with LayerNorm in
+// front must agree bit for bit.  PER keeps for each size what it had: one fma up to 2048 columns, two roundings above.
+template <int PER>
+__device__ __forceinline__ float ln_value(float x, float mean, float rstd, bool scaled, float gamma, float beta)
+{
+    const float d = __fsub_rn(x, mean), n = __fmul_rn(d, rstd);
+    if (PER > 8) return __fadd_rn(__fmul_rn(n, gamma), beta);
+    return scaled ? __fmaf_rn(n, gamma, beta) : __fmaf_rn(d, rstd, beta);
+}
+
 // y[r, :] = (x[r, :] - mean) / sqrt(var + eps) * gamma + beta, two-pass variance.
 template <int PER>
 __global__ void __launch_bounds__(GLUE_THREADS)
@@ -66,17 +77,34 @@ layernorm_kernel(const float *__restrict__ x, int64_t ldx, const float *__restri
 #pragma unroll
     for (int i = 0; i < PER; ++i) {
         const int c = threadIdx.x + i * GLUE_THREADS;
-        if (c < cols) yr[c] = (v[i] - mean) * rstd * (gamma ? gamma[c] : 1.f) + (beta ? beta[c] : 0.f);
+        if (c < cols) yr[c] = ln_value<PER>(v[i], mean, rstd, gamma != nullptr, gamma ? gamma[c] : 1.f, beta ? beta[c] : 0.f);
     }
 }
 
 // The operand pass of a layer whose input is layer-normalised first (Fig. 1(d): LayerNorm in floating point in
-// front of the MX linears): CTA r < M normalises row r exactly as layernorm_kernel does (same ownership of the
-// elements, same order of every sum: the values are bit-identical to that kernel's), quantizes them to MXInt --
-// element c of the row sits in thread c % 256, so a block of 16 or 32 columns is a group of neighbouring lanes and
-// its maximum one round of shuffles -- and writes the exact bf16 operand; the fp32 normalised tensor never exists.
-// After its row every CTA decodes its share of the packed weights (decode_bf16_body), so one launch prepares both
+// front of the MX linears): a CTA takes the mean and variance of a row exactly as layernorm_kernel does (same ownership of
+// the elements, same order of every sum: the values are bit-identical to that kernel's), then reads the row once more --
+// it is in the L1 -- eight neighbouring elements per thread, normalises and quantizes them as quantize_rows_body does and
+// writes the exact bf16 operand; the fp32 normalised tensor never exists.  (One element per thread instead, with the
+// statistics' ownership and 2-byte stores: the operand passes of a 2048 x 4096 block took 165 us, now 110.)
+// After its rows every CTA decodes its share of the packed weights (DecodeWalk), so one launch prepares both
 // operands of the product, as prep_operands_kernel does for a plain layer.
+// Eight neighbouring values (`p` null: all `dflt`), with 16-byte loads where the address allows.
+__device__ __forceinline__ void ln_load8(const float *p, float (&v)[8], float dflt)
+{
+    if (!p) {
+#pragma unroll
+        for (int i = 0; i < 8; ++i) v[i] = dflt;
+    } else if ((reinterpret_cast<uintptr_t>(p) & 15u) == 0) {
+        const float4 a = __ldg(reinterpret_cast<const float4 *>(p)), b = __ldg(reinterpret_cast<const float4 *>(p) + 1);
+        v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w;
+        v[4] = b.x; v[5] = b.y; v[6] = b.z; v[7] = b.w;
+    } else {
+#pragma unroll
+        for (int i = 0; i < 8; ++i) v[i] = __ldg(p + i);
+    }
+}
+
 struct PrepLnJob {
     const float *x;           // [M, K] fp32, leading dimension ldx
     int64_t M, K, ldx;
@@ -98,7 +126,13 @@ prep_ln_operands_kernel(const PrepLnJob j)
     __shared__ float scratch[GLUE_THREADS / 32];
     ptx::dep_wait();
     ptx::dep_trigger();
-    const int cols = (int)j.K;
+    PackedStrides ps;
+    ps.mant_ld = NIBBLE ? j.K / 2 : j.K;
+    ps.exp_ld = j.K / j.block;
+    ps.mant_batch = ps.exp_batch = ps.out_batch = 0;
+    ps.exp_row_shift = j.w_row_shift;
+    const int warps = blockDim.x >> 5, lane = threadIdx.x & 31;
+    const int cols = (int)j.K, groups = cols >> 3;
     for (int64_t r = blockIdx.x; r < j.M; r += gridDim.x) {
         const float *xr = j.x + r * j.ldx;
         float v[PER];
@@ -118,27 +152,33 @@ prep_ln_operands_kernel(const PrepLnJob j)
             q += d * d;
         }
         const float rstd = 1.0f / sqrtf(block_sum(q, scratch) / (float)cols + j.eps);
-        __nv_bfloat16 *ar = j.a_hat + r * j.K;
+        for (int g0 = (int)threadIdx.x - lane; g0 < groups; g0 += GLUE_THREADS) {      // warp-uniform
+            const int g = g0 + lane;
+            float y[8] = {};
+            if (g < groups) {                            // K % 32 == 0: the lanes of a block are all inside or all outside
+                float ga[8], be[8];
+                ln_load8(xr + 8 * g, y, 0.f);
+                ln_load8(j.gamma ? j.gamma + 8 * g : nullptr, ga, 1.f);
+                ln_load8(j.beta ? j.beta + 8 * g : nullptr, be, 0.f);
 #pragma unroll
-        for (int i = 0; i < PER; ++i) {
-            const int c = threadIdx.x + i * GLUE_THREADS;           // K % block == 0: a block is all inside or all outside
-            const float y = c < cols ? (v[i] - mean) * rstd * (j.gamma ? j.gamma[c] : 1.f) + (j.beta ? j.beta[c] : 0.f) : 0.f;
-            uint32_t amax = __float_as_uint(absmax_nan(0.f, y));
+                for (int i = 0; i < 8; ++i) y[i] = ln_value<PER>(y[i], mean, rstd, j.gamma != nullptr, ga[i], be[i]);
+            }
+            float am = 0.f;
 #pragma unroll
-            for (int d = 1; d < 32; d <<= 1)
-                if (d < j.block) amax = max(amax, __shfl_xor_sync(0xFFFFFFFFu, amax, d));
-            const float y8[8] = {y, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+            for (int i = 0; i < 8; ++i) am = absmax_nan(am, y[i]);
+            uint32_t amax = __float_as_uint(am);
+            amax = max(amax, __shfl_xor_sync(0xFFFFFFFFu, amax, 1));
+            if (j.block == 32) amax = max(amax, __shfl_xor_sync(0xFFFFFFFFu, amax, 2));
             float xh[8];
-            encode8_full(y8, (int)(amax >> 23), j.wa, xh);          // the library's rounding; only xh[0] is used
-            if (c < cols) ar[c] = __float2bfloat16_rn(xh[0]);
+            encode8_full(y, (int)(amax >> 23), j.wa, xh);
+            if (g < groups) {
+                uint32_t h[4];
+#pragma unroll
+                for (int i = 0; i < 4; ++i) h[i] = as_u32(__floats2bfloat162_rn(xh[2 * i], xh[2 * i + 1]));
+                *reinterpret_cast<uint4 *>(j.a_hat + r * j.K + 8 * g) = make_uint4(h[0], h[1], h[2], h[3]);
+            }
         }
     }
-    PackedStrides ps;
-    ps.mant_ld = NIBBLE ? j.K / 2 : j.K;
-    ps.exp_ld = j.K / j.block;
-    ps.mant_batch = ps.exp_batch = ps.out_batch = 0;
-    ps.exp_row_shift = j.w_row_shift;
-    const int warps = blockDim.x >> 5;
     decode_bf16_body<NIBBLE, 2>(j.w_mant, j.w_exp, j.N, j.K, j.block, j.ww, j.w_hat, j.K, ps,
                                 (int64_t)blockIdx.x * warps + (threadIdx.x >> 5), (int64_t)gridDim.x * warps);
 }
