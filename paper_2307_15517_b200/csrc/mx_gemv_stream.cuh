@@ -66,6 +66,20 @@ struct StreamParams {
                                  // [2l+1] over the exponent bytes [N, K/32], box 16 x 16 rows
 };
 
+// A call of few layers brings its tables along as launch parameters: no copy in front of the kernel.  (A kernel of its own:
+// one that chooses between the two at run time reads both through generic pointers, 515 -> 529 us on 2.7 GB of weights.)
+constexpr int STREAM_INLINE_LAYERS = 4;
+struct StreamInlineParams : StreamParams {
+    StreamLayer inline_layers[STREAM_INLINE_LAYERS];
+    alignas(64) CUtensorMap inline_maps[2 * STREAM_INLINE_LAYERS];
+    __device__ __forceinline__ const StreamLayer *layer_table() const { return inline_layers; }
+    __device__ __forceinline__ const CUtensorMap *map_table() const { return inline_maps; }
+};
+struct StreamTableParams : StreamParams {
+    __device__ __forceinline__ const StreamLayer *layer_table() const { return layers; }
+    __device__ __forceinline__ const CUtensorMap *map_table() const { return tmaps; }
+};
+
 // Geometry of the two variants.
 //   register variant (BULK = false): 8 warps, each lane prefetches four blocks' words with 32-bit
 //     loads; works for any K % 128 == 0.
@@ -152,9 +166,9 @@ __device__ __forceinline__ f32x2_t fmul2(f32x2_t a, f32x2_t b)
 }
 
 // NT = number of 8-token column tiles (1: T <= 8, 2: T <= 16).
-template <int NT, bool BULK>
+template <int NT, bool BULK, typename Params>
 __global__ void __launch_bounds__(StreamCfg<NT, BULK>::THREADS, 1)
-gemv_stream_kernel(const StreamParams p)
+gemv_stream_kernel(const __grid_constant__ Params p)
 {
     using Cfg = StreamCfg<NT, BULK>;
     constexpr int TP = Cfg::TP, WARPS = Cfg::WARPS, STAGES = Cfg::STAGES, CH = Cfg::CH;
@@ -194,11 +208,13 @@ gemv_stream_kernel(const StreamParams p)
     const int per = (p.total_tiles + gridDim.x - 1) / gridDim.x;
     int tile_lo = blockIdx.x * per;
     const int tile_hi = min(tile_lo + per, p.total_tiles);
+    const StreamLayer *layers = p.layer_table();
+    const CUtensorMap *tmaps = p.map_table();
     int li = 0;
-    while (li + 1 < p.n_layers && p.layers[li + 1].tile_begin <= tile_lo) ++li;
+    while (li + 1 < p.n_layers && layers[li + 1].tile_begin <= tile_lo) ++li;
 
     while (tile_lo < tile_hi) {
-        const StreamLayer L = p.layers[li];
+        const StreamLayer L = layers[li];
         const int l_end = min(tile_hi, L.tile_begin + L.n_tiles);
         const int nb = L.K >> 5;
 
@@ -326,7 +342,7 @@ gemv_stream_kernel(const StreamParams p)
                     uint8_t *my_stage = sStage + warp * STAGES * Cfg::MANT_BYTES;
                     uint8_t *my_exps = sExpStage + warp * STAGES * (16 * CH);
                     const uint32_t my_bar = ptx::smem_u32(sBar) + 8 * warp * STAGES;
-                    const CUtensorMap *tm_m = p.tmaps + 2 * li, *tm_e = tm_m + 1;
+                    const CUtensorMap *tm_m = tmaps + 2 * li, *tm_e = tm_m + 1;
                     const int nblk = b_hi - b_lo;                       // multiple of 16
                     auto issue = [&](int step, int st) {              // step: CH-block chunk index from b_lo
                         // after an expired wait (this warp's or, through the flag, another's) nothing new

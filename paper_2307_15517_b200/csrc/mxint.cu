@@ -10,6 +10,7 @@
 #include <map>
 #include <mutex>
 #include <tuple>
+#include <type_traits>
 #include <vector>
 
 #include "../../include/mxint.h"
@@ -42,7 +43,7 @@ struct DeviceInfo {
     uint32_t *status = nullptr;
     bool tc_attr_set[2][4] = {{false, false, false, false}, {false, false, false, false}};
     bool tc_tail_attr_set[2] = {false, false};
-    bool stream_attr_set[4] = {false, false, false, false};
+    bool stream_attr_set[2][4] = {};
     bool tc2_attr_set[2] = {false, false};
     bool tcx_attr_set = false;
     bool tc8_attr_set = false;
@@ -1019,9 +1020,9 @@ mx_status_t encode_u8_rows(CUtensorMap *out, const void *base, int64_t rows, int
     return MX_OK;
 }
 
+// (the caller holds g_wmap_mu)
 mx_status_t packed_weight_maps(const void *w_mant, const void *w_exp, int64_t N, int64_t K, CUtensorMap *out2)
 {
-    std::lock_guard<std::mutex> lk(g_wmap_mu);
     const auto key = std::make_tuple(w_mant, w_exp, N, K);
     auto it = g_wmap_cache.find(key);
     if (it == g_wmap_cache.end()) {
@@ -1063,16 +1064,50 @@ bool same_activation(const mx_linear_args_t &a, const mx_linear_args_t &b)
            a.fa.block == b.fa.block && a.fa.elem_bits == b.fa.elem_bits && a.fa.block_rows == b.fa.block_rows;
 }
 
-template <int NT, bool BULK>
-mx_status_t launch_stream(const mx::StreamParams &sp, size_t smem, int grid, DeviceInfo &d, cudaStream_t st)
+// owner[i]: the first layer with layer i's activation.  Layers that share one usually follow each other.
+void activation_owners(const mx_linear_args_t *layers, int32_t n, std::vector<int> &owner)
 {
-    const mx_status_t as = smem_attr_once(d.stream_attr_set[(NT - 1) * 2 + (BULK ? 1 : 0)],
-                                          mx::gemv_stream_kernel<NT, BULK>, 227 * 1024);
+    owner.resize((size_t)n);
+    std::multimap<const void *, int> firsts;
+    for (int i = 0; i < n; ++i) {
+        owner[i] = i;
+        if (i > 0 && same_activation(layers[i], layers[owner[i - 1]])) {
+            owner[i] = owner[i - 1];
+            continue;
+        }
+        const auto range = firsts.equal_range(layers[i].x);
+        for (auto it = range.first; it != range.second && owner[i] == i; ++it)
+            if (same_activation(layers[i], layers[it->second])) owner[i] = it->second;
+        if (owner[i] == i) firsts.emplace(layers[i].x, i);
+    }
+}
+
+size_t grouped_workspace(const mx_linear_args_t *layers, int32_t n, const std::vector<int> &owner)
+{
+    size_t total = stream_table_bytes(n);
+    for (int i = 0; i < n; ++i)
+        if (owner[i] == i) total += stream_act_bytes(layers[i]);
+    return total;
+}
+
+template <int NT, bool BULK, typename Params>
+mx_status_t launch_stream_as(const Params &sp, size_t smem, int grid, DeviceInfo &d, cudaStream_t st)
+{
+    constexpr bool INLINE = std::is_same<Params, mx::StreamInlineParams>::value;
+    const mx_status_t as = smem_attr_once(d.stream_attr_set[INLINE ? 1 : 0][(NT - 1) * 2 + (BULK ? 1 : 0)],
+                                          mx::gemv_stream_kernel<NT, BULK, Params>, 227 * 1024);
     if (as != MX_OK) return as;
     ProfScope prof(KIND_GEMM_STREAM, st);
-    MX_CUDA(launch_dep(mx::gemv_stream_kernel<NT, BULK>, dim3(grid), dim3(mx::StreamCfg<NT, BULK>::THREADS), smem, st, sp));
+    MX_CUDA(launch_dep(mx::gemv_stream_kernel<NT, BULK, Params>, dim3(grid), dim3(mx::StreamCfg<NT, BULK>::THREADS), smem, st, sp));
     MX_CUDA(cudaGetLastError());
     return MX_OK;
+}
+
+template <typename Params>
+mx_status_t launch_stream(int nt, bool bulk, const Params &sp, size_t smem, int grid, DeviceInfo &d, cudaStream_t st)
+{
+    if (bulk) return nt == 2 ? launch_stream_as<2, true>(sp, smem, grid, d, st) : launch_stream_as<1, true>(sp, smem, grid, d, st);
+    return nt == 2 ? launch_stream_as<2, false>(sp, smem, grid, d, st) : launch_stream_as<1, false>(sp, smem, grid, d, st);
 }
 
 
@@ -1693,14 +1728,11 @@ mx_status_t mx_linear_fused(const void *x, mx_dtype_t dt, int64_t M, int64_t K, 
 size_t mx_linear_grouped_workspace_bytes(const mx_linear_args_t *layers, int32_t n_layers)
 {
     if (!layers || n_layers <= 0) return 0;
-    size_t total = stream_table_bytes(n_layers);
-    for (int i = 0; i < n_layers; ++i) {
+    for (int i = 0; i < n_layers; ++i)
         if (!format_ok(layers[i].fa) || !format_ok(layers[i].fw)) return 0;
-        bool seen = false;
-        for (int j = 0; j < i && !seen; ++j) seen = same_activation(layers[i], layers[j]);
-        if (!seen) total += stream_act_bytes(layers[i]);
-    }
-    return total;
+    std::vector<int> owner;
+    activation_owners(layers, n_layers, owner);
+    return grouped_workspace(layers, n_layers, owner);
 }
 
 // packed_exps == nullptr: layers[i].x are floating-point activations, quantized here.
@@ -1727,7 +1759,9 @@ static mx_status_t grouped_impl(const mx_linear_args_t *layers, int32_t n_layers
         max_nb = nb > max_nb ? nb : max_nb;
         min_nb = nb < min_nb ? nb : min_nb;
     }
-    const size_t need = packed_exps ? stream_table_bytes(n_layers) : mx_linear_grouped_workspace_bytes(layers, n_layers);
+    std::vector<int> owner;
+    if (!packed_exps) activation_owners(layers, n_layers, owner);
+    const size_t need = packed_exps ? stream_table_bytes(n_layers) : grouped_workspace(layers, n_layers, owner);
     if (!workspace || workspace_bytes < need) return MX_ERR_WORKSPACE;
     if ((reinterpret_cast<uintptr_t>(workspace) & 255u) != 0) return MX_ERR_ALIGN;
     const int nt = max_t > 8 ? 2 : 1;
@@ -1756,17 +1790,23 @@ static mx_status_t grouped_impl(const mx_linear_args_t *layers, int32_t n_layers
     size_t off = stream_table_bytes(n_layers);
     const size_t tmap_off = round256((size_t)n_layers * sizeof(mx::StreamLayer));
     const size_t job_off = tmap_off + round256((size_t)n_layers * 2 * sizeof(CUtensorMap));
+    // one image of the three tables (layers, tensor maps, quantization jobs), laid out as in the workspace; a call of few
+    // layers passes the first two as launch parameters instead
+    const bool in_params = n_layers <= mx::STREAM_INLINE_LAYERS;
+    mx::StreamInlineParams sp;
+    std::vector<uint8_t> image(in_params ? 0 : off);
+    mx::StreamLayer *table = in_params ? sp.inline_layers : reinterpret_cast<mx::StreamLayer *>(image.data());
+    CUtensorMap *tmaps = in_params ? sp.inline_maps : reinterpret_cast<CUtensorMap *>(image.data() + tmap_off);
     std::vector<mx::QuantJob> jobs;
     bool any_dt[2] = {false, false};
     int64_t max_chunks = 0;
-    std::vector<mx::StreamLayer> table((size_t)n_layers);
-    std::vector<CUtensorMap> tmaps(bulk ? (size_t)n_layers * 2 : 0);
     std::vector<uint8_t *> act_ptr((size_t)n_layers, nullptr);
+    std::unique_lock<std::mutex> map_lock(g_wmap_mu, std::defer_lock);
+    if (bulk) map_lock.lock();
     int total_tiles = 0;
     for (int i = 0; i < n_layers; ++i) {
         const mx_linear_args_t &a = layers[i];
-        for (int j = 0; j < i && !act_ptr[i] && !packed_exps; ++j)
-            if (same_activation(a, layers[j])) act_ptr[i] = act_ptr[j];
+        if (!packed_exps) act_ptr[i] = act_ptr[owner[i]];
         if (!act_ptr[i] && !packed_exps) {
             act_ptr[i] = ws + off;
             off += stream_act_bytes(a);
@@ -1813,16 +1853,29 @@ static mx_status_t grouped_impl(const mx_linear_args_t *layers, int32_t n_layers
             if (s != MX_OK) return s;
         }
     }
-    if (bulk)
-        MX_CUDA(cudaMemcpyAsync(ws + tmap_off, tmaps.data(), (size_t)n_layers * 2 * sizeof(CUtensorMap),
-                                cudaMemcpyHostToDevice, st));
-    MX_CUDA(cudaMemcpyAsync(ws, table.data(), (size_t)n_layers * sizeof(mx::StreamLayer),
-                            cudaMemcpyHostToDevice, st));
-    // all distinct activation tensors are quantized by one launch per input type
-    if (!jobs.empty()) {
-        MX_CUDA(cudaMemcpyAsync(ws + job_off, jobs.data(), jobs.size() * sizeof(mx::QuantJob), cudaMemcpyHostToDevice, st));
+    if (bulk) map_lock.unlock();
+    // the activations: one tensor, with its sizes as launch parameters; several, by one launch per input type over a table
+    const size_t n_jobs = jobs.size() > 1 ? jobs.size() : 0;
+    if (!in_params) {
+        if (n_jobs) memcpy(image.data() + job_off, jobs.data(), n_jobs * sizeof(mx::QuantJob));
+        // in pieces of at most 64 KB: those travel with the commands, a larger pageable copy goes through the copy engine and
+        // its staging buffer (192 matrices, 66 KB: the call 531 instead of 522 us)
+        const size_t total = job_off + n_jobs * sizeof(mx::QuantJob), piece = 64 * 1024;
+        for (size_t at = 0; at < total; at += piece)
+            MX_CUDA(cudaMemcpyAsync(ws + at, image.data() + at, total - at < piece ? total - at : piece, cudaMemcpyHostToDevice, st));
+    } else if (n_jobs) {
+        MX_CUDA(cudaMemcpyAsync(ws + job_off, jobs.data(), n_jobs * sizeof(mx::QuantJob), cudaMemcpyHostToDevice, st));
+    }
+    if (jobs.size() == 1) {
+        const mx::QuantJob &q = jobs[0];
+        mx_format_t f{};
+        f.block = q.block; f.elem_bits = q.w; f.exp_bits = 8; f.block_rows = 1;
+        s = quantize_rows_any(q.x, q.dt == 0 ? MX_F32 : MX_BF16, q.rows, q.K, q.ldx, f, q.out, *d, st);
+        if (s != MX_OK) return s;
+    }
+    if (n_jobs) {
         const mx::QuantJob *dj = reinterpret_cast<const mx::QuantJob *>(ws + job_off);
-        const dim3 qgrid((unsigned)grid_for((max_chunks + 1) / 2, 256, d->sm_count, 8), (unsigned)jobs.size());
+        const dim3 qgrid((unsigned)grid_for((max_chunks + 1) / 2, 256, d->sm_count, 8), (unsigned)n_jobs);
         if (any_dt[0]) {
             ProfScope prof(KIND_QUANTIZE, st);
             MX_CUDA(launch_dep(mx::quantize_multi_kernel<float, 0>, dim3(qgrid), dim3(256), 0, st, dj));
@@ -1846,17 +1899,17 @@ static mx_status_t grouped_impl(const mx_linear_args_t *layers, int32_t n_layers
     const int tpr = warps / split;
     const int rounds = (total_tiles + tpr - 1) / tpr;
     const int grid = rounds < max_ctas ? rounds : max_ctas;
-    mx::StreamParams sp;
-    sp.layers = reinterpret_cast<const mx::StreamLayer *>(ws);
+    sp.layers = reinterpret_cast<const mx::StreamLayer *>(ws);          // (unused by a call that brings them along)
     sp.n_layers = n_layers;
     sp.total_tiles = total_tiles;
     sp.split = split;
     sp.max_nb = max_nb;
     sp.status = d->status;
     sp.tmaps = reinterpret_cast<const CUtensorMap *>(ws + tmap_off);
-    if (bulk)
-        return nt == 2 ? launch_stream<2, true>(sp, smem, grid, *d, st) : launch_stream<1, true>(sp, smem, grid, *d, st);
-    return nt == 2 ? launch_stream<2, false>(sp, smem, grid, *d, st) : launch_stream<1, false>(sp, smem, grid, *d, st);
+    if (in_params) return launch_stream(nt, bulk, sp, smem, grid, *d, st);
+    mx::StreamTableParams tp;
+    static_cast<mx::StreamParams &>(tp) = sp;
+    return launch_stream(nt, bulk, tp, smem, grid, *d, st);
 }
 
 mx_status_t mx_linear_grouped(const mx_linear_args_t *layers, int32_t n_layers, void *workspace,
