@@ -64,7 +64,10 @@ typedef enum { MX_F32 = 0, MX_BF16 = 1 } mx_dtype_t;
 /* Which kernel computes the block-scaled product. */
 typedef enum {
     MX_ALGO_AUTO = 0,    /* M <= 16 and a streamable format (see mx_linear_grouped): MX_ALGO_STREAM;
-                            everything else: MX_ALGO_TCGEN05                                       */
+                            everything else on tensor cores: elem_bits <= 5 on both operands and K >= 2048
+                            or N * K >= 3 * 2^20: block-scaled E4M3 operands (exact for both block
+                            sizes, any exponents); otherwise MX_ALGO_TCGEN05, with the K range of
+                            few tiles cut over a cluster and the pieces added in fp32, in order      */
     MX_ALGO_SIMT = 1,    /* CUDA-core kernel: exact integer block sums, blocks added in ascending
                             order in fp32 (bit-reproducible; slow; mx_gemm needs no workspace)      */
     MX_ALGO_TCGEN05 = 2, /* tcgen05/TMEM tensor-core kernel on exactly decoded bf16 operands; a

@@ -1,0 +1,254 @@
+// Tensor-core MXInt product for few output tiles and long reductions (a short prompt against a narrow projection): the K
+// range of every 128 x 128 tile is cut over the CTAs of a cluster.  With a tile per CTA such a call leaves most of the
+// chip idle while a few SMs work through all of K (352 x 2048 x 8192: 48 tiles of 128 K steps on 148 SMs).
+//
+// Operands and arithmetic are those of mx_gemm_tc.cuh (exact bf16, fp32 accumulation in tensor memory).  Every CTA
+// accumulates its K steps, leaves its partial tile in its own shared memory (the stage buffers are free by then), and
+// after a cluster barrier each CTA adds up the partials of every S-th chunk of 32 columns through distributed shared
+// memory, in rank order -- deterministic -- and runs the epilogue on it.  Not persistent: one tile per cluster.
+//   warp 0      : TMA producer (one lane)
+//   warp 1      : tensor-memory allocation, MMA issue (one lane)
+//   warps 2..9  : partial tile to shared memory, then reduction and epilogue
+// Every mbarrier wait is bounded; a CTA whose wait expired still reaches both cluster barriers.
+#pragma once
+#include <cuda.h>
+#include <cuda_runtime.h>
+#include <stdint.h>
+
+#include "mx_gemm_tc.cuh"
+#include "mx_ptx.cuh"
+
+namespace mx {
+
+struct SplitKCfg {
+    static constexpr int BN = 128;
+    static constexpr int STAGES = 6;
+    static constexpr uint32_t A_BYTES = TC_BM * TC_BK * 2;
+    static constexpr uint32_t STAGE_BYTES = A_BYTES + BN * TC_BK * 2;       // 32 KB
+    static constexpr int EPI_WARPS = 8;
+    static constexpr int THREADS = 64 + 32 * EPI_WARPS;
+    static constexpr uint32_t SMEM_BYTES = STAGES * STAGE_BYTES + 256 + 1024;
+    static constexpr uint32_t TMEM_COLS = 128;
+    static constexpr int MAX_SPLIT = 4;
+};
+static_assert(SplitKCfg::STAGES * SplitKCfg::STAGE_BYTES >= TC_BM * SplitKCfg::BN * 4, "the partial tile reuses the stages");
+
+// Offset of the 16-byte group `c4` (of 8) of row `row` in chunk `chunk` of a partial tile; neighbouring rows' groups are
+// swizzled so that a row per lane and four rows per warp both read without bank conflicts.
+__device__ __forceinline__ uint32_t splitk_offset(int chunk, int row, int c4)
+{
+    return (uint32_t)(chunk * (TC_BM * 128) + row * 128 + ((c4 ^ (row & 7)) << 4));
+}
+__device__ __forceinline__ float4 ld_cluster_f32x4(uint32_t cluster_addr)
+{
+    float4 v;
+    asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(cluster_addr) : "memory");
+    return v;
+}
+
+template <bool TAIL>
+__global__ void __maxnreg__(128)
+gemm_splitk_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant__ CUtensorMap tmap_w, const TcParams p, int split)
+{
+    using Cfg = SplitKCfg;
+    constexpr int STAGES = Cfg::STAGES;
+    extern __shared__ uint8_t smem_raw[];
+    const uint32_t smem_base = (ptx::smem_u32(smem_raw) + 1023u) & ~1023u;
+    uint8_t *smem_gen = smem_raw + (smem_base - ptx::smem_u32(smem_raw));
+    const uint32_t bar_base = smem_base + STAGES * Cfg::STAGE_BYTES;
+    auto full_bar = [&](int s) { return bar_base + 8u * s; };
+    auto empty_bar = [&](int s) { return bar_base + 8u * (STAGES + s); };
+    const uint32_t done_bar = bar_base + 8u * (2 * STAGES);
+    uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(smem_gen + STAGES * Cfg::STAGE_BYTES + 8 * (2 * STAGES + 1));
+    volatile uint32_t *abort_flag = tmem_slot + 1;
+
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int rank = (int)ptx::cluster_ctarank(), tile = (int)blockIdx.x / split;
+
+    if (threadIdx.x == 0) {
+        for (int s = 0; s < STAGES; ++s) {
+            ptx::mbar_init(full_bar(s), 1);
+            ptx::mbar_init(empty_bar(s), 1);
+        }
+        ptx::mbar_init(done_bar, 1);
+        *abort_flag = 0;
+        ptx::fence_mbar_init();
+        ptx::prefetch_tensormap(&tmap_a);
+        ptx::prefetch_tensormap(&tmap_w);
+    }
+    if (warp == 1) {
+        ptx::tmem_alloc(ptx::smem_u32(tmem_slot), Cfg::TMEM_COLS);
+        ptx::tmem_relinquish();
+    }
+    ptx::tc_fence_before_sync();
+    __syncthreads();
+    ptx::tc_fence_after_sync();
+    const uint32_t tmem_base = *tmem_slot;
+    ptx::dep_wait();
+    if (threadIdx.x == 0) ptx::dep_trigger();
+
+    const int kblocks = (p.K + TC_BK - 1) / TC_BK;                   // split <= kblocks (host): every CTA has a step
+    const int kb0 = (int)((int64_t)kblocks * rank / split), kb1 = (int)((int64_t)kblocks * (rank + 1) / split);
+    const int m0 = (tile % p.tiles_m) * TC_BM, n0 = (tile / p.tiles_m) * Cfg::BN;
+    bool timed_out = false;
+
+    if (warp == 0) {
+        if (lane == 0) {
+            int s = 0;
+            uint32_t ph = 0;
+            for (int kb = kb0; kb < kb1; ++kb) {
+                if (!ptx::mbar_wait_bounded(empty_bar(s), ph ^ 1u, abort_flag, TC_WAIT_LIMIT_NS)) {
+                    timed_out = true;
+                    break;
+                }
+                ptx::mbar_arrive_expect_tx(full_bar(s), Cfg::STAGE_BYTES);
+                const uint32_t sa = smem_base + s * Cfg::STAGE_BYTES;
+                ptx::tma_load_2d(sa, &tmap_a, kb * TC_BK, m0, full_bar(s));
+                ptx::tma_load_2d(sa + Cfg::A_BYTES, &tmap_w, kb * TC_BK, n0, full_bar(s));
+                if (++s == STAGES) { s = 0; ph ^= 1u; }
+            }
+        }
+        __syncwarp();
+    } else if (warp == 1) {
+        if (lane == 0) {
+            constexpr uint32_t idesc = ptx::idesc_bf16_f32(TC_BM, Cfg::BN);
+            int s = 0;
+            uint32_t ph = 0;
+            for (int kb = kb0; kb < kb1; ++kb) {
+                if (!ptx::mbar_wait_bounded(full_bar(s), ph, abort_flag, TC_WAIT_LIMIT_NS)) {
+                    timed_out = true;
+                    break;
+                }
+                ptx::tc_fence_after_sync();
+                const uint32_t sa = smem_base + s * Cfg::STAGE_BYTES, sw = sa + Cfg::A_BYTES;
+#pragma unroll
+                for (int j = 0; j < TC_BK / 16; ++j)
+                    ptx::mma_bf16_ss(tmem_base, ptx::smem_desc_k_sw128(sa, j * 32), ptx::smem_desc_k_sw128(sw, j * 32), idesc,
+                                     (kb != kb0 || j != 0) ? 1u : 0u);
+                ptx::mma_commit(empty_bar(s));
+                if (++s == STAGES) { s = 0; ph ^= 1u; }
+            }
+            if (!timed_out) ptx::mma_commit(done_bar);
+        }
+        __syncwarp();
+    } else {
+        // the partial tile: tensor memory -> this CTA's shared memory.  All its loads have landed and all its MMAs have
+        // read them when done_bar completes.
+        const int quad = warp & 3, half = (warp - 2) >> 2;
+        const bool ok = ptx::mbar_wait_bounded(done_bar, 0, abort_flag, TC_WAIT_LIMIT_NS);
+        if (__all_sync(0xFFFFFFFFu, ok)) {
+            ptx::tc_fence_after_sync();
+            const int row = quad * 32 + lane;
+#pragma unroll 1
+            for (int c = 2 * half; c < 2 * half + 2; ++c) {
+                uint32_t r[32];
+                ptx::tmem_ld_32x32(tmem_base + ((uint32_t)(quad * 32) << 16) + (uint32_t)(32 * c), r);
+                ptx::tmem_ld_wait();
+#pragma unroll
+                for (int v = 0; v < 8; ++v)
+                    *reinterpret_cast<uint4 *>(smem_gen + splitk_offset(c, row, v)) = make_uint4(r[4 * v], r[4 * v + 1], r[4 * v + 2], r[4 * v + 3]);
+            }
+            ptx::tc_fence_before_sync();
+        } else {
+            timed_out = true;
+        }
+    }
+    if (timed_out) {
+        *abort_flag = 1;
+        atomicOr(p.status, STATUS_TIMEOUT_BIT);
+        const uint64_t t0 = ptx::globaltimer_ns();
+        while (ptx::globaltimer_ns() - t0 < 100000ull) __nanosleep(1000);
+    }
+    __syncwarp();
+    ptx::cluster_sync();                                             // every partial tile is in place
+
+    if (warp >= 2) {
+        const int quad = warp & 3, half = (warp - 2) >> 2;
+        // chunks rank, rank + split, ...: alternately to the two warps of a lane quarter
+        int turn = 0;
+        for (int c = rank; c < Cfg::BN / 32; c += split, ++turn) {
+            if ((turn & 1) != half) continue;
+            const int n = n0 + 32 * c, rows0 = m0 + quad * 32;
+            if (n >= p.N || rows0 >= p.M) continue;                  // warp-uniform
+            if (p.yq_mant) {                                         // a row per lane: a block is a lane's own columns
+                const int row = rows0 + lane;
+                TailRegs t;
+                if (TAIL) tail_fetch(p, row, n, t);
+                uint32_t r[32];
+                float acc[32] = {};
+                for (int s = 0; s < split; ++s) {
+                    const uint32_t base = ptx::map_to_cta(smem_base, (uint32_t)s);
+#pragma unroll
+                    for (int v = 0; v < 8; ++v) {
+                        const float4 x = ld_cluster_f32x4(base + splitk_offset(c, quad * 32 + lane, v));
+                        acc[4 * v] = s ? acc[4 * v] + x.x : x.x;
+                        acc[4 * v + 1] = s ? acc[4 * v + 1] + x.y : x.y;
+                        acc[4 * v + 2] = s ? acc[4 * v + 2] + x.z : x.z;
+                        acc[4 * v + 3] = s ? acc[4 * v + 3] + x.w : x.w;
+                    }
+                }
+#pragma unroll
+                for (int v = 0; v < 32; ++v) r[v] = __float_as_uint(acc[v]);
+                if (TAIL) tail_apply(p, t, n, r);
+                store_mxint_chunk(p, row, n, r);
+                continue;
+            }
+            // fp32: four rows of 128 bytes per warp and step
+            const int c4 = lane & 7, col = n + 4 * c4;
+            const float *bias = TAIL ? p.ex_bias : p.bias;
+            float b[4];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) b[i] = bias && col + i < p.N ? __ldg(bias + col + i) : 0.f;
+            const bool vec = col + 4 <= p.N && (p.ldy & 3) == 0 && (reinterpret_cast<uintptr_t>(p.y) & 15) == 0;
+            const bool rvec = TAIL && p.residual && col + 4 <= p.N && (p.ldr & 3) == 0 && (reinterpret_cast<uintptr_t>(p.residual) & 15) == 0;
+#pragma unroll 4
+            for (int i = 0; i < 8; ++i) {
+                const int lr = quad * 32 + 4 * i + (lane >> 3), row = m0 + lr;
+                float v[4];
+                for (int s = 0; s < split; ++s) {
+                    const float4 x = ld_cluster_f32x4(ptx::map_to_cta(smem_base, (uint32_t)s) + splitk_offset(c, lr, c4));
+                    v[0] = s ? v[0] + x.x : x.x;
+                    v[1] = s ? v[1] + x.y : x.y;
+                    v[2] = s ? v[2] + x.z : x.z;
+                    v[3] = s ? v[3] + x.w : x.w;
+                }
+                if (row >= p.M) continue;
+                float res[4] = {0.f, 0.f, 0.f, 0.f};
+                if (TAIL && p.residual) {
+                    const float *src = p.residual + (int64_t)row * p.ldr + col;
+                    if (rvec) {
+                        const float4 q = __ldg(reinterpret_cast<const float4 *>(src));
+                        res[0] = q.x; res[1] = q.y; res[2] = q.z; res[3] = q.w;
+                    } else {
+#pragma unroll
+                        for (int k = 0; k < 4; ++k)
+                            if (col + k < p.N) res[k] = __ldg(src + k);
+                    }
+                }
+#pragma unroll
+                for (int k = 0; k < 4; ++k) {
+                    if (bias) v[k] += b[k];
+                    if (TAIL && p.relu) v[k] = v[k] < 0.f ? 0.f : v[k];          // NaN stays NaN
+                    if (TAIL && p.residual) v[k] += res[k];
+                }
+                float *dst = p.y + (int64_t)row * p.ldy + col;
+                if (vec) {
+                    *reinterpret_cast<float4 *>(dst) = make_float4(v[0], v[1], v[2], v[3]);
+                } else {
+#pragma unroll
+                    for (int k = 0; k < 4; ++k)
+                        if (col + k < p.N) dst[k] = v[k];
+                }
+            }
+        }
+    }
+    __syncwarp();
+    ptx::tc_fence_before_sync();
+    ptx::cluster_sync();                                             // nobody reads this CTA's partial tile any more
+    if (warp == 1) {
+        ptx::tc_fence_after_sync();
+        ptx::tmem_dealloc(tmem_base, Cfg::TMEM_COLS);
+    }
+}
+
+}  // namespace mx

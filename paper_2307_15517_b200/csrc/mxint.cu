@@ -17,6 +17,7 @@
 #include "mx_alt.cuh"
 #include "mx_attention.cuh"
 #include "mx_gemm_simt.cuh"
+#include "mx_gemm_splitk.cuh"
 #include "mx_gemm_tc.cuh"
 #include "mx_gemm_tc2.cuh"
 #include "mx_gemm_rec.cuh"
@@ -48,6 +49,8 @@ struct DeviceInfo {
     bool tcx_attr_set = false;
     bool tc8_attr_set = false;
     bool rec_attr_set[4] = {};
+    bool splitk_attr_set[2] = {false, false};
+    int splitk_clusters[mx::SplitKCfg::MAX_SPLIT + 1] = {-1, -1, -1, -1, -1};
     bool attn_attr_set[2] = {false, false};
 };
 DeviceInfo g_dev[MAX_DEVICES];
@@ -921,10 +924,112 @@ bool wide_tile(int64_t M, int64_t N, const DeviceInfo &d)
     return tiles256 >= (int64_t)d.sm_count * 3 / 4;
 }
 
-// Pre-decoded bf16 weights (both operands fetched by TMA).
+// Clusters of `split` CTAs of the split-K kernel that are resident at once (a cluster does not cross a GPC: 48 clusters of
+// three do not fit on 148 SMs); looked up once.
+mx_status_t splitk_clusters(DeviceInfo &d, int split, int *out)
+{
+    std::lock_guard<std::mutex> lk(g_init_mu);
+    int &known = d.splitk_clusters[split];
+    if (known < 0) {
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3((unsigned)(split * d.sm_count));
+        cfg.blockDim = dim3(mx::SplitKCfg::THREADS);
+        cfg.dynamicSmemBytes = mx::SplitKCfg::SMEM_BYTES;
+        cudaLaunchAttribute attr[1];
+        attr[0].id = cudaLaunchAttributeClusterDimension;
+        attr[0].val.clusterDim.x = (unsigned)split;
+        attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+        cfg.attrs = attr;
+        cfg.numAttrs = 1;
+        MX_CUDA(cudaFuncSetAttribute(mx::gemm_splitk_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)mx::SplitKCfg::SMEM_BYTES));
+        int n = 0;
+        MX_CUDA(cudaOccupancyMaxActiveClusters(&n, mx::gemm_splitk_kernel<false>, &cfg));
+        known = n;
+    }
+    *out = known;
+    return MX_OK;
+}
+
+// Few tiles, long reduction: into how many pieces K is cut over a cluster (see mx_gemm_splitk.cuh); 0 for the one-CTA
+// kernels.  The most pieces whose clusters all fit at once, where the K steps that a CTA is spared are worth the two
+// cluster barriers and the exchange (about 2.5 us against 0.2 us per step: at least 12 steps spared).  Whole calls, split /
+// not (us): 352 x 2048 x 8192 in two 36.8 / 51.5, 352 x 2048 x 2048 15.8 / 17.3, 64 x 768 x 3072 in four 12.7 / 20.2,
+// 512 x 1024 x 4096 18.4 / 27.5, 200 x 1024 x 1024 10.7 / 11.2; but 352 x 2048 x 1024 in two 13.2 / 12.2 and
+// 128 x 768 x 768 in four 10.9 / 10.2.
+mx_status_t splitk_ways(int64_t M, int64_t N, int64_t K, DeviceInfo &d, int *out)
+{
+    *out = 0;
+    const int64_t tiles = ((M + mx::TC_BM - 1) / mx::TC_BM) * ((N + mx::SplitKCfg::BN - 1) / mx::SplitKCfg::BN);
+    const int64_t kblocks = (K + mx::TC_BK - 1) / mx::TC_BK;
+    for (int s = mx::SplitKCfg::MAX_SPLIT; s > 1 && !*out; --s) {
+        if (tiles * s > d.sm_count || kblocks * (s - 1) < 12 * s) continue;
+        int fit = 0;
+        const mx_status_t st = splitk_clusters(d, s, &fit);
+        if (st != MX_OK) return st;
+        if (tiles <= fit) *out = s;
+    }
+    return MX_OK;
+}
+
+mx_status_t launch_splitk(const __nv_bfloat16 *a_hat, const __nv_bfloat16 *w_hat, int64_t M, int64_t N, int64_t K, int split,
+                          const float *bias, float *y, int64_t ldy, const QuantizedOut *yq, DeviceInfo &d, cudaStream_t st,
+                          const EpiTail &et)
+{
+    using Cfg = mx::SplitKCfg;
+    CUtensorMap tm_a, tm_w;
+    mx_status_t s = encode_bf16_rows(&tm_a, a_hat, M, K, mx::TC_BM);
+    if (s != MX_OK) return s;
+    s = encode_bf16_rows(&tm_w, w_hat, N, K, Cfg::BN);
+    if (s != MX_OK) return s;
+    const bool tail = et.any();
+    s = tail ? smem_attr_once(d.splitk_attr_set[1], mx::gemm_splitk_kernel<true>, (int)Cfg::SMEM_BYTES)
+             : smem_attr_once(d.splitk_attr_set[0], mx::gemm_splitk_kernel<false>, (int)Cfg::SMEM_BYTES);
+    if (s != MX_OK) return s;
+    mx::TcParams p{};
+    p.y = y;
+    p.bias = tail ? nullptr : bias;
+    p.ex_bias = tail ? bias : nullptr;
+    p.relu = et.relu;
+    p.residual = et.residual;
+    p.ldr = et.ldr;
+    p.ldy = ldy;
+    p.M = (int)M;
+    p.N = (int)N;
+    p.K = (int)K;
+    p.tiles_m = (int)((M + mx::TC_BM - 1) / mx::TC_BM);
+    p.tiles_n = (int)((N + Cfg::BN - 1) / Cfg::BN);
+    p.status = d.status;
+    p.batch = 1;
+    p.yq_mant = yq ? yq->mant : nullptr;
+    p.yq_exp = yq ? yq->exps : nullptr;
+    p.yq_nonfinite = yq ? yq->nonfinite : nullptr;
+    p.yq_bits = yq ? yq->f.elem_bits : 0;
+    p.yq_block = yq ? yq->f.block : 0;
+    p.yq_rows2 = yq && yq->f.block_rows == 2 ? 1 : 0;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)(p.tiles_m * p.tiles_n * split));
+    cfg.blockDim = dim3(Cfg::THREADS);
+    cfg.dynamicSmemBytes = Cfg::SMEM_BYTES;
+    cfg.stream = st;
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = (unsigned)split;
+    attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[1].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = g_prof.on ? 1 : 2;                     // see launch_dep
+    ProfScope prof(KIND_GEMM_TC, st);
+    if (tail) MX_CUDA(cudaLaunchKernelEx(&cfg, mx::gemm_splitk_kernel<true>, tm_a, tm_w, p, split));
+    else MX_CUDA(cudaLaunchKernelEx(&cfg, mx::gemm_splitk_kernel<false>, tm_a, tm_w, p, split));
+    MX_CUDA(cudaGetLastError());
+    return MX_OK;
+}
+
+// Pre-decoded bf16 weights (both operands fetched by TMA).  may_split: K may be cut (the sum is then not one chain).
 mx_status_t run_tc(const __nv_bfloat16 *a_hat, const __nv_bfloat16 *w_hat, int64_t M, int64_t N,
                    int64_t K, const float *bias, float *y, int64_t ldy, DeviceInfo &d, cudaStream_t st,
-                   const QuantizedOut *yq = nullptr, const TcBatch &tb = TcBatch(), const EpiTail &et = EpiTail())
+                   const QuantizedOut *yq = nullptr, const TcBatch &tb = TcBatch(), const EpiTail &et = EpiTail(), bool may_split = true)
 {
     const PackedW none;
     // CTA pairs (a third less shared-memory traffic per flop) when there is more than one wave of 256 x 256
@@ -935,6 +1040,12 @@ mx_status_t run_tc(const __nv_bfloat16 *a_hat, const __nv_bfloat16 *w_hat, int64
     const int pairs = d.sm_count / 2;
     if (tb.count == 1 && M > 128 && (pair_tiles > pairs || (K >= 4096 && 4 * pair_tiles >= 3 * pairs)))
         return launch_tc2(a_hat, w_hat, M, N, K, bias, y, ldy, yq, d, st, et);
+    if (may_split && tb.count == 1) {
+        int split = 0;
+        const mx_status_t s = splitk_ways(M, N, K, d, &split);
+        if (s != MX_OK) return s;
+        if (split) return launch_splitk(a_hat, w_hat, M, N, K, split, bias, y, ldy, yq, d, st, et);
+    }
     const int64_t tiles256 = ((M + 127) / 128) * ((N + 255) / 256) * tb.count;
     if (N > 128 && tiles256 >= (int64_t)d.sm_count * 3 / 4)
         return launch_tc<256, mx::W_BF16>(a_hat, w_hat, none, M, N, K, bias, y, ldy, yq, d, st, tb, et);
@@ -1370,6 +1481,7 @@ mx_status_t mx_gemm_ex(const void *a_mant, const uint8_t *a_exp, mx_format_t fa,
     mx_status_t s = check_gemm_args(a_mant, a_exp, fa, w_mant, w_exp, fw, M, N, K, bias, y, ldy);
     if (s != MX_OK) return s;
     if (!a_exp) return MX_ERR_NULL;
+    const bool any_algo = algo == MX_ALGO_AUTO;
     {
         mx_linear_args_t one;
         one.x = a_mant; one.dt = MX_F32; one.M = M; one.K = K; one.ldx = K; one.fa = fa;
@@ -1433,7 +1545,7 @@ mx_status_t mx_gemm_ex(const void *a_mant, const uint8_t *a_exp, mx_format_t fa,
     s = launch_dequant_pair(a_mant, a_exp, fa, M, w_mant, w_exp, fw, N, K, a_hat, w_hat, *d, st);
     if (s != MX_OK) return s;
     if (algo == MX_ALGO_TCGEN05_BLOCKWISE) return launch_tcx(a_hat, w_hat, M, N, K, fa.block, bias, y, ldy, *d, st);
-    return run_tc(a_hat, w_hat, M, N, K, bias, y, ldy, *d, st);
+    return run_tc(a_hat, w_hat, M, N, K, bias, y, ldy, *d, st, nullptr, TcBatch(), EpiTail(), any_algo);
 }
 
 mx_status_t mx_gemm(const void *a_mant, const uint8_t *a_exp, mx_format_t fa, const void *w_mant,
@@ -1518,7 +1630,7 @@ mx_status_t mx_linear_ex(const void *x, mx_dtype_t dt, int64_t M, int64_t K, int
     s = tc_prepare(one, a_hat, w_hat, *d, st);
     if (s != MX_OK) return s;
     if (algo == MX_ALGO_TCGEN05_BLOCKWISE) return launch_tcx(a_hat, w_hat, M, N, K, fa.block, bias, y, ldy, *d, st);
-    return run_tc(a_hat, w_hat, M, N, K, bias, y, ldy, *d, st);
+    return run_tc(a_hat, w_hat, M, N, K, bias, y, ldy, *d, st, nullptr, TcBatch(), EpiTail(), any_algo);
 }
 
 mx_status_t mx_linear(const void *x, mx_dtype_t dt, int64_t M, int64_t K, int64_t ldx, mx_format_t fa,
