@@ -448,4 +448,252 @@ gemv_stream_kernel(const __grid_constant__ Params p)
     if (BULK) __syncthreads();                // no warp leaves while another may still be waiting out its copies
 }
 
+// ---- one or two tokens ---------------------------------------------------------------------------
+// With so few tokens the tensor-core form above is bound by instruction issue: an MMA tile serves eight tokens, and its
+// operand set-up and rescale cost the same for one (about 32 warp instructions per 16 x 32 weights).  Here a lane owns a
+// weight row: 16 bytes are the 32 mantissas of one block, eight dp4a per token give the exact block sum in one register (the
+// same 16 * q bytes, the same 1.5 * 2^23 seed), two fmas apply the scales: about 17 instructions at one token and 5 more for
+// the second.  Blocks ascend within a lane, so the result is bit for bit the same chain.
+// A warp owns 32 rows and a ring of stages of 32 rows x 16 blocks (four 16-row x 128-byte mantissa boxes, two exponent
+// boxes); its loads run on into its next tile and the next layer's while the last ones are consumed.  Tokens are staged once
+// per distinct activation tensor, not per layer.  Needs K % 512 == 0 in all layers and 16-byte aligned exponent arrays.
+// 2.7 GB of weights, kernel only: 513 -> 471 us at one token (5.2 -> 5.7 TB/s); 0.7 GB: 148 -> 133 us at two; but 147 -> 184
+// at three and four, and two MMA row tiles per warp in this frame are slower at any number (eight warps hide less than
+// sixteen: 148 -> 214 us at eight tokens), so more tokens stay on the form above.
+template <int TOK> struct Stream32Cfg {
+    static constexpr int WARPS = 8, THREADS = WARPS * 32, ROWS = 32, CH = 16;
+    static constexpr int MANT_BYTES = ROWS * CH * 16;                   // 8 KB
+    static constexpr int EXP_BYTES = ROWS * CH;
+    static constexpr int STAGE_BYTES = MANT_BYTES + EXP_BYTES;
+    static constexpr int MAX_STAGES = 3;
+    static constexpr size_t RED_BYTES = (size_t)WARPS * TOK * 32 * 4;      // split-K exchange
+    static constexpr size_t smem_bytes(int max_nb, int stages)
+    {
+        return 1024 + (size_t)WARPS * stages * STAGE_BYTES + RED_BYTES + (size_t)WARPS * MAX_STAGES * 8 + 16 +
+               (size_t)max_nb * TOK * (32 + 4);
+    }
+};
+
+// Any of four exponent bytes from 226 on: 1.5 * 2^23 * 2^(E-127) is not finite, the seed is taken off before the scale.
+__device__ __forceinline__ bool stream_near_top(uint32_t v)
+{
+    return ((v & 0x80808080u) & ((v & 0x7F7F7F7Fu) + 0x1E1E1E1Eu)) != 0u;
+}
+// Weight scale 2^(E-127) of byte j: moved into the float's exponent field (byte 0 -> the subnormal 2^-127, byte 255 -> Inf,
+// which turns the block into NaN).
+__device__ __forceinline__ uint32_t stream_scale_bits(uint32_t e4, int j)
+{
+    return max((j == 3 ? e4 >> 1 : e4 << (23 - 8 * j)) & 0x7F800000u, 0x00400000u);
+}
+
+// One stage (16 blocks from `b` on) of 32 rows, a row per lane.
+template <int TOK>
+__device__ __forceinline__ void dp_step(const uint8_t *mant, const uint8_t *exps, const uint4 *sB, const float *sCS, int b, int lane, float (&acc)[TOK])
+{
+    const uint8_t *sm = mant + (lane >> 4) * 2048 + (lane & 15) * 128;
+    const uint4 ex = *reinterpret_cast<const uint4 *>(exps + lane * 16);
+    const uint32_t exw[4] = {ex.x, ex.y, ex.z, ex.w};
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        const bool top = stream_near_top(exw[q]);
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const int c = 4 * q + j;
+            const uint4 w = *reinterpret_cast<const uint4 *>(sm + (c >> 3) * 4096 + (((c & 7) ^ (lane & 7)) << 4));
+            const uint32_t ww[4] = {w.x, w.y, w.z, w.w};
+            const float sw = __uint_as_float(stream_scale_bits(exw[q], j));
+            const float mw = sw * -STREAM_MAGIC;
+#pragma unroll
+            for (int k = 0; k < TOK; ++k) {
+                const uint4 t0 = sB[((b + c) * TOK + k) * 2], t1 = sB[((b + c) * TOK + k) * 2 + 1];
+                const uint32_t tt[8] = {t0.x, t0.y, t0.z, t0.w, t1.x, t1.y, t1.z, t1.w};
+                int d = STREAM_MAGIC_INT, d2 = 0;
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    d = __dp4a((int)((ww[i] << 4) & 0xF0F0F0F0u), (int)tt[2 * i], d);
+                    d2 = __dp4a((int)(ww[i] & 0xF0F0F0F0u), (int)tt[2 * i + 1], d2);
+                }
+                const float f = __int_as_float(d + d2);                   // 1.5 * 2^23 + 16 P
+                float pr;                                                  // P * weight scale, exact
+                if (!top) pr = fmaf(f, sw, mw);
+                else pr = fmaf(0.f, sw, (f - STREAM_MAGIC) * sw);          // (+ 0 * scale: NaN for an Inf scale)
+                acc[k] = fmaf(pr, sCS[(b + c) * TOK + k], acc[k]);         // one rounding per block, ascending blocks
+            }
+        }
+    }
+}
+
+template <int TOK, typename Params>
+__global__ void __launch_bounds__(Stream32Cfg<TOK>::THREADS, 1)
+gemv_stream32_kernel(const __grid_constant__ Params p, int stages)
+{
+    using Cfg = Stream32Cfg<TOK>;
+    constexpr int WARPS = Cfg::WARPS, CH = Cfg::CH, ROWS = Cfg::ROWS;
+    extern __shared__ __align__(16) uint8_t smem[];
+    uint8_t *sMant = smem + ((1024u - (ptx::smem_u32(smem) & 1023u)) & 1023u);      // [WARPS][stages][MANT_BYTES]
+    uint8_t *sExp = sMant + WARPS * stages * Cfg::MANT_BYTES;                         // [WARPS][stages][EXP_BYTES]
+    float *sRed = reinterpret_cast<float *>(sExp + WARPS * stages * Cfg::EXP_BYTES);  // split-K exchange
+    uint8_t *sBar = reinterpret_cast<uint8_t *>(sRed) + Cfg::RED_BYTES;               // [WARPS][MAX_STAGES] mbarriers
+    volatile uint32_t *abort_flag = reinterpret_cast<volatile uint32_t *>(sBar + WARPS * Cfg::MAX_STAGES * 8);
+    uint4 *sB = reinterpret_cast<uint4 *>(sBar + WARPS * Cfg::MAX_STAGES * 8 + 16);   // [nb][TOK][2]: per 8 k the even and the odd ones
+    float *sCS = reinterpret_cast<float *>(sB + (size_t)p.max_nb * TOK * 2);          // [nb][TOK]
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    if (threadIdx.x == 0) {
+        for (int i = 0; i < WARPS * Cfg::MAX_STAGES; ++i) ptx::mbar_init(ptx::smem_u32(sBar) + 8 * i, 1);
+        *abort_flag = 0;
+        ptx::fence_mbar_init();
+    }
+    __syncthreads();
+    ptx::dep_wait();                          // the quantized tokens come from the previous launch
+    if (threadIdx.x == 0) ptx::dep_trigger();
+
+    const StreamLayer *layers = p.layer_table();
+    const CUtensorMap *tmaps = p.map_table();
+    const int S = p.split, TPR = WARPS / S, slot = warp / S, piece = warp % S;
+    const int per = (p.total_tiles + gridDim.x - 1) / gridDim.x;
+    const int tile_first = blockIdx.x * per, tile_hi = min(tile_first + per, p.total_tiles);
+    int li = 0;
+    while (li + 1 < p.n_layers && layers[li + 1].tile_begin <= tile_first) ++li;
+
+    // this warp's loads: a cursor over (layer, tile, step) that runs ahead of the arithmetic, across tiles and layers
+    const uint32_t my_bar = ptx::smem_u32(sBar) + 8 * warp * Cfg::MAX_STAGES;
+    const uint32_t my_mant = ptx::smem_u32(sMant) + warp * stages * Cfg::MANT_BYTES;
+    const uint32_t my_exp = ptx::smem_u32(sExp) + warp * stages * Cfg::EXP_BYTES;
+    int c_li = li, c_base = tile_first, c_step = 0, c_begin = 0, c_end = 0, c_nsteps = 0, c_b0 = 0, c_stage = 0;
+    bool c_live = tile_first < tile_hi;
+    auto cursor_layer = [&]() {               // first layer from c_li on that has a tile for this warp
+        while (c_live) {
+            const StreamLayer &L = layers[c_li];
+            c_begin = L.tile_begin;
+            c_end = min(tile_hi, L.tile_begin + L.n_tiles);
+            if (c_base + slot < c_end) {
+                const int nb = L.K >> 5;
+                c_nsteps = nb / S / CH;
+                c_b0 = nb / S * piece;
+                return;
+            }
+            c_base = c_end;
+            ++c_li;
+            c_live = c_base < tile_hi;
+        }
+    };
+    auto issue = [&]() {                      // lane 0: the cursor's step into stage c_stage, then one step on
+        if (!c_live || *abort_flag != 0) return;
+        const uint32_t bar = my_bar + 8 * c_stage, dst = my_mant + c_stage * Cfg::MANT_BYTES, dx = my_exp + c_stage * Cfg::EXP_BYTES;
+        const CUtensorMap *tm_m = tmaps + 2 * c_li, *tm_e = tm_m + 1;
+        const int r0 = (c_base + slot - c_begin) * ROWS, b = c_b0 + c_step * CH;
+        ptx::mbar_arrive_expect_tx(bar, Cfg::STAGE_BYTES);
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {         // (rows >= N read as zero)
+            ptx::tma_load_2d(dst + h * 2048, tm_m, b * 16, r0 + 16 * h, bar);
+            ptx::tma_load_2d(dst + (2 + h) * 2048, tm_m, b * 16 + 128, r0 + 16 * h, bar);
+        }
+#pragma unroll
+        for (int h = 0; h < 2; ++h) ptx::tma_load_2d(dx + h * 256, tm_e, b, r0 + 16 * h, bar);
+        if (++c_stage == stages) c_stage = 0;
+        if (++c_step == c_nsteps) {
+            c_step = 0;
+            c_base += TPR;
+            cursor_layer();
+        }
+    };
+    if (lane == 0) {
+        cursor_layer();
+        for (int i = 0; i < stages; ++i) issue();
+    }
+    __syncwarp();
+
+    int st = 0;                               // stage and parity of the next step to consume
+    uint32_t parity = 0;
+    bool timed_out = false;
+    const uint8_t *staged = nullptr;          // the activation in shared memory, and the weight width its scales carry
+    int staged_bits = 0;
+    int tile_lo = tile_first;
+    while (tile_lo < tile_hi) {
+        const StreamLayer L = layers[li];
+        const int l_end = min(tile_hi, L.tile_begin + L.n_tiles);
+        const int nb = L.K >> 5;
+        if (L.a_mant != staged || L.w_bits != staged_bits) {      // CTA-uniform
+            staged = L.a_mant;
+            staged_bits = L.w_bits;
+            __syncthreads();                  // the previous layer's tokens are consumed
+            for (int i = threadIdx.x; i < nb * TOK * 4; i += Cfg::THREADS) {
+                const int tq = i & 3, tok = (i >> 2) % TOK, b = (i >> 2) / TOK;
+                uint32_t lo = 0, hi = 0;      // 8 mantissas, k = 32b + 8tq ..
+                if (tok < L.T) {
+                    if (L.a_bits <= 4) {
+                        const uint32_t pk = __ldg(reinterpret_cast<const uint32_t *>(L.a_mant + (int64_t)tok * (L.K >> 1) + b * 16 + tq * 4));
+                        uint32_t by[8];
+#pragma unroll
+                        for (int j = 0; j < 8; ++j) by[j] = (uint32_t)((((int)(pk << (28 - 4 * j))) >> 28) & 0xFF);
+                        lo = by[0] | (by[1] << 8) | (by[2] << 16) | (by[3] << 24);
+                        hi = by[4] | (by[5] << 8) | (by[6] << 16) | (by[7] << 24);
+                    } else {
+                        const uint2 v = __ldg(reinterpret_cast<const uint2 *>(L.a_mant + (int64_t)tok * L.K + b * 32 + tq * 8));
+                        lo = v.x;
+                        hi = v.y;
+                    }
+                }
+                reinterpret_cast<uint2 *>(sB)[i] = make_uint2(__byte_perm(lo, hi, 0x6420), __byte_perm(lo, hi, 0x7531));
+                if (tq == 0) {
+                    const int eb = tok < L.T ? (int)__ldg(L.a_exp + (int64_t)(tok >> L.a_rows2) * nb + b) : 0;
+                    sCS[b * TOK + tok] = f32_scale(eb, L.a_bits) * small_neg_pow2(L.w_bits) * 0.0625f;
+                }
+            }
+            __syncthreads();
+        }
+        const int nsteps = nb / S / CH, b_lo = nb / S * piece;
+        for (int base = tile_lo; base < l_end; base += TPR) {
+            const int tile = base + slot;
+            const bool active = tile < l_end;
+            float acc[TOK];
+#pragma unroll
+            for (int k = 0; k < TOK; ++k) acc[k] = 0.f;
+            for (int step = 0; active && step < nsteps && !timed_out; ++step) {
+                const bool ok = ptx::mbar_wait_bounded(my_bar + 8 * st, parity, abort_flag, STREAM_WAIT_LIMIT_NS);
+                if (!__all_sync(0xFFFFFFFFu, ok)) {
+                    timed_out = true;
+                    *abort_flag = 1;          // the other warps stop issuing as well
+                    break;
+                }
+                const uint8_t *mant = sMant + (warp * stages + st) * Cfg::MANT_BYTES, *exps = sExp + (warp * stages + st) * Cfg::EXP_BYTES;
+                dp_step<TOK>(mant, exps, sB, sCS, b_lo + step * CH, lane, acc);
+                __syncwarp();                 // every lane is done reading the stage
+                if (++st == stages) { st = 0; parity ^= 1u; }
+                if (lane == 0) {
+                    ptx::fence_proxy_async_smem();
+                    issue();
+                }
+            }
+            const int row = (tile - L.tile_begin) * ROWS + lane;
+            if (S > 1) {                      // CTA-uniform
+                __syncthreads();
+#pragma unroll
+                for (int k = 0; k < TOK; ++k) sRed[(warp * TOK + k) * 32 + lane] = acc[k];
+                __syncthreads();
+                if (piece == 0) {
+#pragma unroll
+                    for (int k = 0; k < TOK; ++k)
+                        for (int q = 1; q < S; ++q) acc[k] += sRed[((warp + q) * TOK + k) * 32 + lane];
+                }
+            }
+            if (active && piece == 0 && row < L.N) {
+                const float bias = L.bias ? __ldg(L.bias + row) : 0.f;
+#pragma unroll
+                for (int k = 0; k < TOK; ++k)
+                    if (k < L.T) L.y[(int64_t)k * L.ldy + row] = L.bias ? acc[k] + bias : acc[k];
+            }
+        }
+        // (a warp whose wait expired goes through the remaining rounds without steps: the CTA's barriers stay matched)
+        tile_lo = l_end;
+        ++li;
+    }
+    if (timed_out) atomicOr(p.status, 1u);
+    if (*abort_flag != 0) {                   // copies already in flight get time to land before the shared memory is released
+        const uint64_t t0 = ptx::globaltimer_ns();
+        while (ptx::globaltimer_ns() - t0 < 100000ull) __nanosleep(1000);
+    }
+    __syncthreads();
+}
+
 }  // namespace mx

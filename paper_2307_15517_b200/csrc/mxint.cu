@@ -45,6 +45,7 @@ struct DeviceInfo {
     bool tc_attr_set[2][4] = {{false, false, false, false}, {false, false, false, false}};
     bool tc_tail_attr_set[2] = {false, false};
     bool stream_attr_set[2][4] = {};
+    bool stream32_attr_set[2][2] = {};
     bool tc2_attr_set[2] = {false, false};
     bool tcx_attr_set = false;
     bool tc8_attr_set = false;
@@ -1214,6 +1215,24 @@ mx_status_t launch_stream_as(const Params &sp, size_t smem, int grid, DeviceInfo
     return MX_OK;
 }
 
+template <int TOK, typename Params>
+mx_status_t launch_stream32_as(const Params &sp, int stages, size_t smem, int grid, DeviceInfo &d, cudaStream_t st)
+{
+    constexpr bool INLINE = std::is_same<Params, mx::StreamInlineParams>::value;
+    const mx_status_t as = smem_attr_once(d.stream32_attr_set[INLINE ? 1 : 0][TOK - 1], mx::gemv_stream32_kernel<TOK, Params>, 227 * 1024);
+    if (as != MX_OK) return as;
+    ProfScope prof(KIND_GEMM_STREAM, st);
+    MX_CUDA(launch_dep(mx::gemv_stream32_kernel<TOK, Params>, dim3(grid), dim3(mx::Stream32Cfg<TOK>::THREADS), smem, st, sp, stages));
+    MX_CUDA(cudaGetLastError());
+    return MX_OK;
+}
+
+template <typename Params>
+mx_status_t launch_stream32(int tok, const Params &sp, int stages, size_t smem, int grid, DeviceInfo &d, cudaStream_t st)
+{
+    return tok == 1 ? launch_stream32_as<1>(sp, stages, smem, grid, d, st) : launch_stream32_as<2>(sp, stages, smem, grid, d, st);
+}
+
 template <typename Params>
 mx_status_t launch_stream(int nt, bool bulk, const Params &sp, size_t smem, int grid, DeviceInfo &d, cudaStream_t st)
 {
@@ -1855,7 +1874,7 @@ static mx_status_t grouped_impl(const mx_linear_args_t *layers, int32_t n_layers
 {
     if (!layers) return MX_ERR_NULL;
     if (n_layers <= 0) return MX_ERR_SHAPE;
-    int max_t = 0, max_nb = 0, min_nb = INT32_MAX;
+    int max_t = 0, max_nb = 0;
     for (int i = 0; i < n_layers; ++i) {
         const mx_linear_args_t &a = layers[i];
         mx_status_t s = check_gemm_args(a.x, nullptr, a.fa, a.w_mant, a.w_exp, a.fw, a.M, a.N, a.K, a.bias,
@@ -1869,7 +1888,6 @@ static mx_status_t grouped_impl(const mx_linear_args_t *layers, int32_t n_layers
         max_t = a.M > max_t ? (int)a.M : max_t;
         const int nb = (int)(a.K / 32);
         max_nb = nb > max_nb ? nb : max_nb;
-        min_nb = nb < min_nb ? nb : min_nb;
     }
     std::vector<int> owner;
     if (!packed_exps) activation_owners(layers, n_layers, owner);
@@ -1895,6 +1913,26 @@ static mx_status_t grouped_impl(const mx_linear_args_t *layers, int32_t n_layers
     DeviceInfo *d = nullptr;
     mx_status_t s = device_info(&d);
     if (s != MX_OK) return s;
+    // K is cut over the warps of a CTA only when the row tiles alone cannot fill the GPU; `unit`: blocks that a piece must be
+    // a multiple of, in every layer
+    auto choose_split = [&](int64_t tiles, int64_t warp_slots, int unit) {
+        for (int cand = 8; tiles < warp_slots && cand > 1; cand >>= 1) {
+            bool whole = cand <= 4 || tiles * 4 < warp_slots;
+            for (int i = 0; i < n_layers && whole; ++i) whole = (layers[i].K / 32) % (unit * cand) == 0;
+            if (whole) return cand;
+        }
+        return 1;
+    };
+    // one or two tokens: a weight row per lane (see gemv_stream32_kernel), with as many stages as fit beside the tokens
+    int stages = 0;
+    for (int n = mx::Stream32Cfg<1>::MAX_STAGES; bulk && max_t <= 2 && n >= 2 && !stages; --n) {
+        const size_t need = max_t == 1 ? mx::Stream32Cfg<1>::smem_bytes(max_nb, n) : mx::Stream32Cfg<2>::smem_bytes(max_nb, n);
+        if (need <= 227u * 1024u) {
+            stages = n;
+            smem = need;
+        }
+    }
+    const bool rows32 = stages > 0;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
 
     // quantize every distinct activation tensor once, build the device layer table
@@ -1958,7 +1996,7 @@ static mx_status_t grouped_impl(const mx_linear_args_t *layers, int32_t n_layers
         L.w_rows2 = a.fw.block_rows == 2 ? 1 : 0;
         L.a_rows2 = a.fa.block_rows == 2 ? 1 : 0;
         L.tile_begin = total_tiles;
-        L.n_tiles = (int)((a.N + 15) / 16);
+        L.n_tiles = (int)(rows32 ? (a.N + 31) / 32 : (a.N + 15) / 16);
         total_tiles += L.n_tiles;
         if (bulk) {
             s = packed_weight_maps(a.w_mant, a.w_exp, a.N, a.K, &tmaps[(size_t)i * 2]);
@@ -2001,13 +2039,8 @@ static mx_status_t grouped_impl(const mx_linear_args_t *layers, int32_t n_layers
 
     const int ctas_per_sm = (int)((227u * 1024u) / (smem + 1024)) < 4 ? (int)((227u * 1024u) / (smem + 1024)) : 4;
     const int max_ctas = d->sm_count * (ctas_per_sm < 1 ? 1 : ctas_per_sm);
-    const int warps = bulk ? 16 : 8;
-    int split = 1;                         // cut K over warps only when row tiles alone cannot fill the GPU
-    const int unit = bulk ? 16 : 4;        // blocks per row a warp's K piece must be a multiple of
-    if (total_tiles < max_ctas * warps) {
-        for (int cand = 8; cand > 1 && split == 1; cand >>= 1)
-            if (min_nb % (unit * cand) == 0 && (cand <= 4 || total_tiles * 4 < max_ctas * warps)) split = cand;
-    }
+    const int warps = rows32 ? mx::Stream32Cfg<1>::WARPS : bulk ? 16 : 8;
+    const int split = choose_split(total_tiles, (int64_t)max_ctas * warps, bulk ? 16 : 4);
     const int tpr = warps / split;
     const int rounds = (total_tiles + tpr - 1) / tpr;
     const int grid = rounds < max_ctas ? rounds : max_ctas;
@@ -2018,9 +2051,11 @@ static mx_status_t grouped_impl(const mx_linear_args_t *layers, int32_t n_layers
     sp.max_nb = max_nb;
     sp.status = d->status;
     sp.tmaps = reinterpret_cast<const CUtensorMap *>(ws + tmap_off);
-    if (in_params) return launch_stream(nt, bulk, sp, smem, grid, *d, st);
+    if (in_params)
+        return rows32 ? launch_stream32(max_t, sp, stages, smem, grid, *d, st) : launch_stream(nt, bulk, sp, smem, grid, *d, st);
     mx::StreamTableParams tp;
     static_cast<mx::StreamParams &>(tp) = sp;
+    if (rows32) return launch_stream32(max_t, tp, stages, smem, grid, *d, st);
     return launch_stream(nt, bulk, tp, smem, grid, *d, st);
 }
 

@@ -137,3 +137,42 @@ def test_stream_rejects_what_it_cannot_stage(mxb):
     x17 = torch.zeros(17, 256, device="cuda")
     with pytest.raises(mxb.MxError):                       # more than 16 tokens
         mxb.mx_linear(x17, dev["fa"], dev["w_mant"], dev["w_exp"], dev["fw"], 64, algo=mxb.MX_ALGO_STREAM)
+
+
+@pytest.mark.parametrize("T", (1, 2))
+def test_rows_per_lane_kernel_over_mixed_layers(mxb, T):
+    """One or two tokens, K % 512 == 0: layers of different K, width, activation and ragged N in one launch, with weight
+    exponents near the top of the range and a poisoned block; enough rows that K is not cut, so the bits are the oracle's."""
+    layers, refs = [], []
+    for i in range(10):
+        dev, ref = _layer(mxb, T, 512, 4096, seed=70 + i % 2, wa=8 - 4 * (i % 2), ww=4, with_bias=i == 3)
+        if i % 2 and len(layers) > 1:
+            dev["x"] = layers[1]["x"]                                   # a shared activation tensor
+        layers.append(dev)
+        refs.append(ref)
+    for K, N, wa, ww in ((1024, 1001, 8, 3), (1536, 37, 3, 2), (512, 32, 8, 4)):
+        dev, ref = _layer(mxb, T, K, N, seed=K + N, wa=wa, ww=ww, heavy=True)
+        layers.append(dev)
+        refs.append(ref)
+    refs[-1]["ew"][3, 5], refs[-1]["ew"][9, 2] = 240, 255
+    refs[-1]["qw"][9, 64:96] = 0
+    layers[-1]["w_exp"].copy_(torch.from_numpy(refs[-1]["ew"]))
+    layers[-1]["w_mant"].copy_(torch.from_numpy(orc.pack(refs[-1]["qw"], 4)))
+    mxb.mx_linear_grouped(mxb.make_linear_args(layers))
+    assert mxb.mx_poll_status() == 0
+    for dev, ref in zip(layers, refs):
+        _, y_seq, _ = _oracle(ref)
+        y = dev["y"].cpu().numpy()
+        nan = np.isnan(y_seq)
+        assert np.array_equal(nan, np.isnan(y)) and np.array_equal(y[~nan], y_seq[~nan])
+
+
+@pytest.mark.parametrize("T", (1, 2, 5))
+def test_split_reduction_takes_every_layer_of_a_call_into_account(mxb, T):
+    """K is cut over warps for few rows; the pieces must be whole stages in EVERY layer (4608 / 8 pieces is not)."""
+    layers, refs = zip(*[_layer(mxb, T, K, 96, seed=K, heavy=True) for K in (4096, 4608)])
+    mxb.mx_linear_grouped(mxb.make_linear_args(layers))
+    assert mxb.mx_poll_status() == 0
+    for dev, ref in zip(layers, refs):
+        y_ref, _, S = _oracle(ref)
+        assert (np.abs(dev["y"].cpu().numpy().astype(np.float64) - y_ref) <= TOL * S + 1e-37).all()
