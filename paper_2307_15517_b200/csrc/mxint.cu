@@ -1033,13 +1033,18 @@ mx_status_t run_tc(const __nv_bfloat16 *a_hat, const __nv_bfloat16 *w_hat, int64
                    const QuantizedOut *yq = nullptr, const TcBatch &tb = TcBatch(), const EpiTail &et = EpiTail(), bool may_split = true)
 {
     const PackedW none;
-    // CTA pairs (a third less shared-memory traffic per flop) when there is more than one wave of 256 x 256
-    // tiles (+2 % on 2048 x 6144 x 2048, +14 % on 8192^3), or one nearly full wave of long tiles (K >= 4096:
-    // 2048 x 2048 x 8192 runs in 49.5 instead of 56.5 us); a short single wave starts faster on the one-CTA
-    // kernel (2048^3: 19.7 against 22.4 us).
+    // One wave of the smallest tile that gives one: a wave of 128 x 256 tiles takes 1.1 to 1.2 times as long as one of
+    // 128 x 128, not twice (352 x 8192 x 2048, 192 or 96 tiles: 33.3 against 25.7 us per call; 352 x 6144 x 2048, 144 or 72:
+    // 22.9 against 24.4).  Beyond that CTA pairs (a third less shared-memory traffic per flop: 512 x 11008 x 4096 74.3 against
+    // 83.3 us, +14 % on 8192^3), but a ragged half pair is not worth a second wave (300 x 12288 x 4096: 144 tiles of
+    // 128 x 256 62.1, 96 pair tiles 75.0).  Pairs also for one nearly full wave of long tiles (2048 x 2048 x 8192 product
+    // 49.5 against 56.5 us); a short single wave starts faster on the one-CTA kernel (2048^3 call 23.8 against 24.7).
+    const int64_t panels = (M + 127) / 128;
     const int64_t pair_tiles = ((M + 255) / 256) * ((N + 255) / 256);
+    const int64_t tiles128 = panels * ((N + 127) / 128) * tb.count, tiles256 = panels * ((N + 255) / 256) * tb.count;
     const int pairs = d.sm_count / 2;
-    if (tb.count == 1 && M > 128 && (pair_tiles > pairs || (K >= 4096 && 4 * pair_tiles >= 3 * pairs)))
+    const bool long_wave = K >= 4096 && pair_tiles <= pairs && 4 * pair_tiles >= 3 * pairs && (panels & 1) == 0;
+    if (tb.count == 1 && M > 128 && (tiles256 > d.sm_count || long_wave))
         return launch_tc2(a_hat, w_hat, M, N, K, bias, y, ldy, yq, d, st, et);
     if (may_split && tb.count == 1) {
         int split = 0;
@@ -1047,8 +1052,7 @@ mx_status_t run_tc(const __nv_bfloat16 *a_hat, const __nv_bfloat16 *w_hat, int64
         if (s != MX_OK) return s;
         if (split) return launch_splitk(a_hat, w_hat, M, N, K, split, bias, y, ldy, yq, d, st, et);
     }
-    const int64_t tiles256 = ((M + 127) / 128) * ((N + 255) / 256) * tb.count;
-    if (N > 128 && tiles256 >= (int64_t)d.sm_count * 3 / 4)
+    if (N > 128 && tiles128 > d.sm_count)
         return launch_tc<256, mx::W_BF16>(a_hat, w_hat, none, M, N, K, bias, y, ldy, yq, d, st, tb, et);
     return launch_tc<128, mx::W_BF16>(a_hat, w_hat, none, M, N, K, bias, y, ldy, yq, d, st, tb, et);
 }
