@@ -1948,9 +1948,14 @@ static mx_status_t grouped_impl(const mx_linear_args_t *layers, int32_t n_layers
     // layers passes the first two as launch parameters instead
     const bool in_params = n_layers <= mx::STREAM_INLINE_LAYERS;
     mx::StreamInlineParams sp;
-    std::vector<uint8_t> image(in_params ? 0 : off);
-    mx::StreamLayer *table = in_params ? sp.inline_layers : reinterpret_cast<mx::StreamLayer *>(image.data());
-    CUtensorMap *tmaps = in_params ? sp.inline_maps : reinterpret_cast<CUtensorMap *>(image.data() + tmap_off);
+    // (in units that are aligned as its strictest member is: a vector of bytes starts on 16 bytes only)
+    struct alignas(64) ImageLine { uint8_t bytes[64]; };
+    static_assert(alignof(ImageLine) >= alignof(CUtensorMap) && alignof(ImageLine) >= alignof(mx::StreamLayer) &&
+                  alignof(ImageLine) >= alignof(mx::QuantJob), "the tables are written in place");
+    std::vector<ImageLine> image_lines(in_params ? 0 : off / sizeof(ImageLine));       // off: a multiple of 256
+    uint8_t *image = reinterpret_cast<uint8_t *>(image_lines.data());
+    mx::StreamLayer *table = in_params ? sp.inline_layers : reinterpret_cast<mx::StreamLayer *>(image);
+    CUtensorMap *tmaps = in_params ? sp.inline_maps : reinterpret_cast<CUtensorMap *>(image + tmap_off);
     std::vector<mx::QuantJob> jobs;
     bool any_dt[2] = {false, false};
     int64_t max_chunks = 0;
@@ -2011,12 +2016,12 @@ static mx_status_t grouped_impl(const mx_linear_args_t *layers, int32_t n_layers
     // the activations: one tensor, with its sizes as launch parameters; several, by one launch per input type over a table
     const size_t n_jobs = jobs.size() > 1 ? jobs.size() : 0;
     if (!in_params) {
-        if (n_jobs) memcpy(image.data() + job_off, jobs.data(), n_jobs * sizeof(mx::QuantJob));
+        if (n_jobs) memcpy(image + job_off, jobs.data(), n_jobs * sizeof(mx::QuantJob));
         // in pieces of at most 64 KB: those travel with the commands, a larger pageable copy goes through the copy engine and
         // its staging buffer (192 matrices, 66 KB: the call 531 instead of 522 us)
         const size_t total = job_off + n_jobs * sizeof(mx::QuantJob), piece = 64 * 1024;
         for (size_t at = 0; at < total; at += piece)
-            MX_CUDA(cudaMemcpyAsync(ws + at, image.data() + at, total - at < piece ? total - at : piece, cudaMemcpyHostToDevice, st));
+            MX_CUDA(cudaMemcpyAsync(ws + at, image + at, total - at < piece ? total - at : piece, cudaMemcpyHostToDevice, st));
     } else if (n_jobs) {
         MX_CUDA(cudaMemcpyAsync(ws + job_off, jobs.data(), n_jobs * sizeof(mx::QuantJob), cudaMemcpyHostToDevice, st));
     }
