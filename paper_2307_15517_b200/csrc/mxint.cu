@@ -1956,7 +1956,7 @@ static mx_status_t grouped_impl(const mx_linear_args_t *layers, int32_t n_layers
     uint8_t *image = reinterpret_cast<uint8_t *>(image_lines.data());
     mx::StreamLayer *table = in_params ? sp.inline_layers : reinterpret_cast<mx::StreamLayer *>(image);
     CUtensorMap *tmaps = in_params ? sp.inline_maps : reinterpret_cast<CUtensorMap *>(image + tmap_off);
-    std::vector<mx::QuantJob> jobs;
+    std::vector<mx::QuantJob> jobs, pair_jobs;          // (pair_jobs: pairs of tokens share their exponents)
     bool any_dt[2] = {false, false};
     int64_t max_chunks = 0;
     std::vector<uint8_t *> act_ptr((size_t)n_layers, nullptr);
@@ -1979,9 +1979,7 @@ static mx_status_t grouped_impl(const mx_linear_args_t *layers, int32_t n_layers
             job.dt = a.dt == MX_F32 ? 0 : 1;
             job.out = mx::QuantOut{act_ptr[i], act_ptr[i] + round256(mx_mant_bytes(a.M, a.K, a.fa)), nullptr, 0, nullptr};
             if (a.fa.block_rows == 2) {
-                // pairs of tokens share their exponents: the two-row quantizer, one launch for this tensor
-                s = quantize_rows_any(a.x, a.dt, a.M, a.K, a.ldx, a.fa, job.out, *d, st);
-                if (s != MX_OK) return s;
+                pair_jobs.push_back(job);
             } else {
                 jobs.push_back(job);
                 any_dt[job.dt] = true;
@@ -2012,7 +2010,17 @@ static mx_status_t grouped_impl(const mx_linear_args_t *layers, int32_t n_layers
             if (s != MX_OK) return s;
         }
     }
+    // nothing is launched under the lock: a launch may wait for room in its stream, and other threads' calls with it
     if (bulk) map_lock.unlock();
+    auto quantize_one = [&](const mx::QuantJob &q, int block_rows) {
+        mx_format_t f{};
+        f.block = q.block; f.elem_bits = q.w; f.exp_bits = 8; f.block_rows = block_rows;
+        return quantize_rows_any(q.x, q.dt == 0 ? MX_F32 : MX_BF16, q.rows, q.K, q.ldx, f, q.out, *d, st);
+    };
+    for (const mx::QuantJob &q : pair_jobs) {            // the two-row quantizer, one launch per tensor
+        s = quantize_one(q, 2);
+        if (s != MX_OK) return s;
+    }
     // the activations: one tensor, with its sizes as launch parameters; several, by one launch per input type over a table
     const size_t n_jobs = jobs.size() > 1 ? jobs.size() : 0;
     if (!in_params) {
@@ -2026,10 +2034,7 @@ static mx_status_t grouped_impl(const mx_linear_args_t *layers, int32_t n_layers
         MX_CUDA(cudaMemcpyAsync(ws + job_off, jobs.data(), n_jobs * sizeof(mx::QuantJob), cudaMemcpyHostToDevice, st));
     }
     if (jobs.size() == 1) {
-        const mx::QuantJob &q = jobs[0];
-        mx_format_t f{};
-        f.block = q.block; f.elem_bits = q.w; f.exp_bits = 8; f.block_rows = 1;
-        s = quantize_rows_any(q.x, q.dt == 0 ? MX_F32 : MX_BF16, q.rows, q.K, q.ldx, f, q.out, *d, st);
+        s = quantize_one(jobs[0], 1);
         if (s != MX_OK) return s;
     }
     if (n_jobs) {

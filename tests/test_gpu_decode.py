@@ -176,3 +176,45 @@ def test_split_reduction_takes_every_layer_of_a_call_into_account(mxb, T):
     for dev, ref in zip(layers, refs):
         y_ref, _, S = _oracle(ref)
         assert (np.abs(dev["y"].cpu().numpy().astype(np.float64) - y_ref) <= TOL * S + 1e-37).all()
+
+
+def test_two_row_and_plain_activations_of_one_call_from_two_threads(mxb):
+    """Activations whose tokens pair up are quantized by launches of their own, plain ones by one launch over a table; both
+    kinds and both types in one call of more layers than travel as launch parameters, issued by two threads at once."""
+    import threading
+    T, K, N = 2, 1024, 96
+    layers, refs = [], []
+    for i, (rows, dt) in enumerate(((1, torch.float32), (2, torch.float32), (1, torch.bfloat16), (2, torch.bfloat16), (1, torch.float32),
+                                    (2, torch.float32))):
+        x = synth.student_t_activations(T, K, 80 + i).to(dt)
+        w = synth.gaussian_weights(N, K, 90 + i)
+        qa, ea, _ = orc.quantize_2d(x.float().numpy(), 32, rows, 8)
+        qw, ew, _ = orc.quantize(w.numpy(), 32, 4)
+        refs.append(orc.gemm(qa, orc.expand_exponent_rows(ea, rows), 8, qw, ew, 4, 32))
+        layers.append(dict(x=x.cuda(), fa=mxb.MxFormat(32, 8, block_rows=rows), fw=mxb.MxFormat(32, 4), N=N,
+                           w_mant=torch.from_numpy(orc.pack(qw, 4)).cuda(), w_exp=torch.from_numpy(ew).cuda(),
+                           y=torch.empty(T, N, device="cuda")))
+    mxb.mx_linear_grouped(mxb.make_linear_args(layers))
+    assert mxb.mx_poll_status() == 0
+    for L, (y_ref, _, S) in zip(layers, refs):
+        assert (np.abs(L["y"].cpu().numpy().astype(np.float64) - y_ref) <= TOL * S + 1e-37).all()
+    results = [None, None]
+
+    def work(t):
+        stream = torch.cuda.Stream()
+        mine = [dict(L, y=torch.empty_like(L["y"])) for L in layers]
+        args = mxb.make_linear_args(mine)
+        ws = mxb.alloc_workspace(mxb.mx_linear_grouped_workspace_bytes(args))
+        stream.wait_stream(torch.cuda.default_stream())
+        for _ in range(20):
+            mxb.mx_linear_grouped(args, workspace=ws, stream=stream)
+        stream.synchronize()
+        results[t] = [L["y"] for L in mine]
+
+    threads = [threading.Thread(target=work, args=(t,)) for t in range(2)]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    for ys in results:
+        assert ys is not None and all(torch.equal(a, L["y"]) for a, L in zip(ys, layers))
