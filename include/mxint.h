@@ -64,10 +64,15 @@ typedef enum { MX_F32 = 0, MX_BF16 = 1 } mx_dtype_t;
 /* Which kernel computes the block-scaled product. */
 typedef enum {
     MX_ALGO_AUTO = 0,    /* M <= 16 and a streamable format (see mx_linear_grouped): MX_ALGO_STREAM;
-                            everything else on tensor cores: elem_bits <= 5 on both operands and K >= 2048
-                            or N * K >= 3 * 2^20: block-scaled E4M3 operands (exact for both block
-                            sizes, any exponents); otherwise MX_ALGO_TCGEN05, with the K range of
-                            few tiles cut over a cluster and the pieces added in fp32, in order      */
+                            everything else on tensor cores, on operands that hold every value exactly:
+                            - few 128 x 128 tiles (at most 74) and K of 1024 or more: the bf16 operands of
+                              MX_ALGO_TCGEN05, the K range cut over a cluster of two to four CTAs and the
+                              pieces added in fp32, in order;
+                            - else, elem_bits <= 5 and container storage on both operands, K % 32 == 0,
+                              and K >= 2048 or (M + N) * K >= 2^22: block-scaled E4M3 operands (also in
+                              place of a cut where weights are so many that the smaller operand pays);
+                            - else MX_ALGO_TCGEN05.
+                            The sum is taken in another order on each: see the accuracy note below.  */
     MX_ALGO_SIMT = 1,    /* CUDA-core kernel: exact integer block sums, blocks added in ascending
                             order in fp32 (bit-reproducible; slow; mx_gemm needs no workspace)      */
     MX_ALGO_TCGEN05 = 2, /* tcgen05/TMEM tensor-core kernel on exactly decoded bf16 operands; a

@@ -745,20 +745,15 @@ RecLayout rec_layout(int64_t M, int64_t N, int64_t K)
     return l;
 }
 
-// Calls that take the block-scaled product: mantissas that E4M3 holds, container form on both sides, whole groups of
-// 32 along K, and sizes where it is the faster one.  Whole calls, 4-bit, block 16, against the bf16 path (us): the
-// pair tile costs more to start and drain than one CTA's, which short reductions into narrow results do not earn back
-// (256 x 768 x 768 12.9 against 11.5, 512 x 2048 x 1024 13.4 / 13.1); from K = 2048 on it wins everywhere (24 x 256 x
-// 2048 14.7 / 15.4, 2048^3 22.2 / 24.1, 512 x 6144 x 4096 34.2 / 62.5), and so do weights of 3 M elements, whose operand
-// form is half as large (256 x 6144 x 512 12.2 / 13.8; 64 x 4096 x 512, 2 M, 10.9 / 9.9).
+// Calls that the block-scaled product can take: mantissas that E4M3 holds, container form on both sides, whole groups of 32
+// along K, within the workspace the caller was told to bring.
 bool rec_fits(const mx_format_t &fa, const mx_format_t &fw, int64_t M, int64_t N, int64_t K)
 {
     if (fa.elem_bits > 5 || fw.elem_bits > 5 || fa.packing || fw.packing || (K % 32) != 0) return false;
-    if (K < 2048 && N * K < 3 * (1 << 20)) return false;
     const RecLayout l = rec_layout(M, N, K);
     if ((int64_t)l.panels_a * l.kblocks * 16 > INT32_MAX / 2 || (int64_t)l.panels_w * l.kblocks * 16 > INT32_MAX / 2)
         return false;
-    return l.bytes <= tc_workspace(M, N, K);             // the workspace the caller was told to bring
+    return l.bytes <= tc_workspace(M, N, K);
 }
 
 mx::RecOut rec_out(const RecLayout &l, uint8_t *ws, bool weights)
@@ -968,6 +963,32 @@ mx_status_t splitk_ways(int64_t M, int64_t N, int64_t K, DeviceInfo &d, int *out
         const mx_status_t st = splitk_clusters(d, s, &fit);
         if (st != MX_OK) return st;
         if (tiles <= fit) *out = s;
+    }
+    return MX_OK;
+}
+
+// Whether the block-scaled product is the faster one where it fits.  Measured on 550 shapes (1 to 4096 tokens, N 256 to
+// 16384, K 512 to 16384; 4-bit, block 16, device time of whole calls, us, records / bf16):
+// - Where run_tc would cut K, a pair tile's 0.36 us per 128 of K, one tile after another, stand against the split's 0.2 us
+//   per 64 of a piece and its exchange, and against its operand form, which is twice as large.  The estimate below picks the
+//   faster side but for 4 % at most: 1 x 256 x 16384 55.5 / 27.3, 64 x 768 x 3072 18.1 / 12.9, 352 x 2048 x 8192 40.2 / 37.6,
+//   but 16 x 8192 x 8192 56.2 / 60.0 and 128 x 8192 x 16384 113 / 118.
+// - Otherwise records win from K = 2048 on (352 x 4096 x 4096 29.1 / 33.6, 768 x 2048 x 2048 19.1 / 19.3), and below that
+//   where the operands are large enough to pay for the pair tile's longer start and drain: 4096 x 2048 x 768 20.8 / 22.1,
+//   24 x 8192 x 512 11.7 / 12.5, but 1024 x 4096 x 768 15.9 / 14.7, 512 x 2048 x 1024 13.5 / 12.9.  Around the line the two
+//   differ by up to 12 % either way (128 x 12288 x 768 16.7 / 14.8).
+mx_status_t rec_is_faster(int64_t M, int64_t N, int64_t K, DeviceInfo &d, bool *out)
+{
+    int split = 0;
+    const mx_status_t s = splitk_ways(M, N, K, d, &split);
+    if (s != MX_OK) return s;
+    const int64_t operands = (M + N) * K;
+    if (split) {
+        const int64_t rec_ns = 360 * ((K + mx::REC_K - 1) / mx::REC_K);
+        const int64_t steps = ((K + mx::TC_BK - 1) / mx::TC_BK + split - 1) / split;
+        *out = rec_ns < 200 * steps + 1000 + operands * 17 / 100000;
+    } else {
+        *out = K >= 2048 || operands >= (4 << 20);
     }
     return MX_OK;
 }
@@ -1517,8 +1538,12 @@ mx_status_t mx_gemm_ex(const void *a_mant, const uint8_t *a_exp, mx_format_t fa,
             DeviceInfo *dr = nullptr;
             s = device_info(&dr);
             if (s != MX_OK) return s;
-            return run_rec_gemm(a_mant, a_exp, fa, w_mant, w_exp, fw, M, N, K, bias, y, ldy, nullptr,
-                                static_cast<uint8_t *>(workspace), *dr, static_cast<cudaStream_t>(stream), EpiTail());
+            bool rec = false;
+            s = rec_is_faster(M, N, K, *dr, &rec);
+            if (s != MX_OK) return s;
+            if (rec)
+                return run_rec_gemm(a_mant, a_exp, fa, w_mant, w_exp, fw, M, N, K, bias, y, ldy, nullptr,
+                                    static_cast<uint8_t *>(workspace), *dr, static_cast<cudaStream_t>(stream), EpiTail());
         }
         if (algo == MX_ALGO_AUTO) algo = can_stream ? MX_ALGO_STREAM : MX_ALGO_TCGEN05;
         if (algo == MX_ALGO_STREAM) return grouped_impl(&one, 1, &a_exp, workspace, workspace_bytes, stream);
@@ -1636,7 +1661,12 @@ mx_status_t mx_linear_ex(const void *x, mx_dtype_t dt, int64_t M, int64_t K, int
     const bool fused = algo == MX_ALGO_TCGEN05_FUSED && (K % 32) == 0 && fw.block_rows == 1;
     if (fused && !fused_ok(K, w_exp)) return MX_ERR_ALIGN;
     if (workspace_bytes < (fused ? fused_workspace(M, K) : tc_workspace(M, N, K))) return MX_ERR_WORKSPACE;
-    if (any_algo && rec_fits(fa, fw, M, N, K)) return run_rec_linear(one, bias, y, ldy, nullptr, ws, *d, st, EpiTail());
+    bool rec = false;
+    if (any_algo && rec_fits(fa, fw, M, N, K)) {
+        s = rec_is_faster(M, N, K, *d, &rec);
+        if (s != MX_OK) return s;
+    }
+    if (rec) return run_rec_linear(one, bias, y, ldy, nullptr, ws, *d, st, EpiTail());
     __nv_bfloat16 *a_hat = reinterpret_cast<__nv_bfloat16 *>(ws);
     // the activations' mantissas and exponents go straight to the MMA operand form (exact bf16)
     mx::QuantOut out{nullptr, nullptr, a_hat, K, nullptr};
@@ -1706,7 +1736,12 @@ static mx_status_t gemm_tc_impl(const void *a_mant, const uint8_t *a_exp, mx_for
     yq.exps = y_exp;
     yq.nonfinite = nonfinite_count;
     yq.f = fy;
-    if (rec_fits(fa, fw, M, N, K))
+    bool rec = false;
+    if (rec_fits(fa, fw, M, N, K)) {
+        s = rec_is_faster(M, N, K, *d, &rec);
+        if (s != MX_OK) return s;
+    }
+    if (rec)
         return run_rec_gemm(a_mant, a_exp, fa, w_mant, w_exp, fw, M, N, K, bias, y, y ? ldy : N, y ? nullptr : &yq,
                             static_cast<uint8_t *>(workspace), *d, st, et);
     s = launch_dequant_pair(a_mant, a_exp, fa, M, w_mant, w_exp, fw, N, K, a_hat, w_hat, *d, st);
@@ -1784,7 +1819,12 @@ static mx_status_t linear_tc_impl(const void *x, mx_dtype_t dt, int64_t M, int64
     yq.exps = y_exp;
     yq.nonfinite = nonfinite_count;
     yq.f = fy;
-    if (!with_ln && rec_fits(fa, fw, M, N, K))
+    bool rec = false;
+    if (!with_ln && rec_fits(fa, fw, M, N, K)) {
+        s = rec_is_faster(M, N, K, *d, &rec);
+        if (s != MX_OK) return s;
+    }
+    if (rec)
         return run_rec_linear(one, bias, y, y ? ldy : N, y ? nullptr : &yq, ws, *d, st, et);
     if (with_ln) {
         s = tc_prepare_ln(one, *ln, a_hat, w_hat, *d, st);

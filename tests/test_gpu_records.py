@@ -1,5 +1,6 @@
 """GPU parity of the block-scaled product on records (mantissa widths up to 5 on both sides, blocks of 16 and 32): the
-route of mx_linear / mx_gemm and their fused and MXInt-result forms from K = 2048 or 3 M weights on."""
+route of mx_linear / mx_gemm and their fused and MXInt-result forms where there are too many 128 x 128 tiles to cut K (more
+than 74), from K = 2048 or 4 M operand elements on.  Calls of fewer tiles take the product whose K is cut, here as well."""
 import numpy as np
 import pytest
 import torch
@@ -30,11 +31,15 @@ def _poison_free(mxb):
     assert mxb.mx_poll_status() == 0
 
 
-# one row panel / one and a bit / two CTAs' worth; one record step of K, a remainder of 32, of 64; one and two panels of W;
-# N odd in every unit of the stores; a wide result behind a short reduction
-SHAPES = [(17, 130, 2048, 32, 4, 4, 1, "fp32"), (128, 256, 2080, 16, 5, 5, 1, "bf16"), (129, 258, 2176, 16, 4, 3, 1, "fp32"),
-          (300, 385, 2336, 16, 2, 4, 1, "fp32"), (256, 512, 2080, 32, 5, 2, 2, "fp32"), (386, 514, 2080, 16, 3, 5, 2, "bf16"),
-          (100, 6147, 544, 16, 4, 4, 1, "fp32"), (2100, 2330, 2048, 32, 5, 5, 1, "fp32")]
+# records: one row panel / one and a bit / two CTAs' worth; one record step of K, a remainder of 32, of 64; odd and even
+# numbers of panels of W; N odd in every unit of the stores; a wide result behind a short reduction
+SHAPES = [(17, 8450, 2080, 32, 4, 4, 1, "fp32"), (128, 9602, 2080, 16, 5, 5, 1, "bf16"), (129, 5002, 2176, 16, 4, 3, 1, "fp32"),
+          (300, 3201, 2336, 16, 2, 4, 1, "fp32"), (256, 4864, 2080, 32, 5, 2, 2, "fp32"), (386, 2562, 2080, 16, 3, 5, 2, "bf16"),
+          (100, 8195, 544, 16, 4, 4, 1, "fp32"), (2100, 2330, 2048, 32, 5, 5, 1, "fp32")]
+# narrow mantissas in few tiles: K is cut
+SHAPES += [(17, 130, 2048, 32, 4, 4, 1, "fp32"), (128, 256, 2080, 16, 5, 5, 1, "bf16"), (129, 258, 2176, 16, 4, 3, 1, "fp32"),
+           (300, 385, 2336, 16, 2, 4, 1, "fp32"), (256, 512, 2080, 32, 5, 2, 2, "fp32"), (386, 514, 2080, 16, 3, 5, 2, "bf16"),
+           (100, 6147, 544, 16, 4, 4, 1, "fp32")]
 
 
 @pytest.mark.parametrize("shape", SHAPES)
@@ -61,11 +66,12 @@ def test_layer_and_product_within_tolerance(mxb, shape):
         assert intact()
 
 
+@pytest.mark.parametrize("N", (5000, 300))         # records; K cut
 @pytest.mark.parametrize("B", (16, 32))
-def test_any_exponents_are_exact(mxb, B):
+def test_any_exponents_are_exact(mxb, B, N):
     """Exponent bytes anywhere, -2^(w-1) and zero groups included, on operands whose sums are exact in any order: the
     blocks of a row that meet nonzero weights share one exponent, the others lie up to 60 binades away."""
-    M, N, K, wa, ww = 200, 300, 2080, 4, 5
+    M, K, wa, ww = 200, 2080, 4, 5
     rng = np.random.default_rng(B)
     qa = rng.integers(-8, 8, (M, K)).astype(np.int8)
     qw = rng.integers(-16, 16, (N, K)).astype(np.int8)
@@ -109,10 +115,11 @@ def test_any_exponents_are_exact(mxb, B):
         assert np.array_equal(y[~want], y_ref[~want])
 
 
-def test_general_operands_far_apart(mxb):
+@pytest.mark.parametrize("N", (5000, 260))         # records; K cut
+def test_general_operands_far_apart(mxb, N):
     """Every block with an exponent of its own, +-20 binades: each MMA step cuts its addends (16 products and the
     accumulator) at the ulp of the largest, so K/16 steps stay within K/16 * 17 * 2^-23 of S."""
-    M, N, K, B = 150, 260, 2144, 16
+    M, K, B = 150, 2144, 16
     x = synth.student_t_activations(M, K, 1).numpy() * np.ldexp(1.0, np.random.default_rng(1).integers(-20, 21, (M, K // B))).repeat(B, 1)
     w = synth.gaussian_weights(N, K, 2).numpy() * np.ldexp(1.0, np.random.default_rng(2).integers(-20, 21, (N, K // B))).repeat(B, 1)
     x, w = x.astype(np.float32), w.astype(np.float32)
@@ -124,7 +131,7 @@ def test_general_operands_far_apart(mxb):
     assert (np.abs(y.cpu().numpy().astype(np.float64) - y_ref) <= K / 16 * 17 * 2.0 ** -23 * S).all()
 
 
-@pytest.mark.parametrize("shape", [(150, 288, 2080, 16), (300, 544, 2048, 32)])
+@pytest.mark.parametrize("shape", [(150, 5024, 2080, 16), (300, 4128, 2048, 32), (150, 288, 2080, 16), (300, 544, 2048, 32)])
 def test_fused_tail_and_mxint_result_are_the_plain_result_passed_on(mxb, shape):
     M, N, K, B = shape
     fa, fw = mxb.MxFormat(B, 4), mxb.MxFormat(B, 4)
@@ -144,3 +151,23 @@ def test_fused_tail_and_mxint_result_are_the_plain_result_passed_on(mxb, shape):
             want = mxb.mx_quantize(src, fy)
             assert torch.equal(got[0], want[0]) and torch.equal(got[1], want[1])
     _poison_free(mxb)
+
+
+@pytest.mark.parametrize("shape", [(64, 256, 8192), (200, 512, 4096), (1, 1024, 4096)])
+def test_few_tiles_take_the_cut_reduction_whatever_the_width(mxb, shape):
+    """The same values in 4-bit and in 6-bit containers (exponent byte + 2 for the two more fraction bits).  Few tiles and a
+    long K: both calls must run the product whose K is cut, so their sums are rounded alike, bit for bit; the block exponents
+    are spread so that another order of the sum shows."""
+    M, N, K = shape
+    B = 16
+    rng = np.random.default_rng(K)
+    qa, qw = rng.integers(-7, 8, (M, K)).astype(np.int8), rng.integers(-7, 8, (N, K)).astype(np.int8)
+    ea = rng.integers(121, 134, (M, K // B)).astype(np.uint8)
+    ew = rng.integers(121, 134, (N, K // B)).astype(np.uint8)
+    y = [mxb.mx_gemm(_dev(orc.pack(qa, w)), _dev(ea + np.uint8(w - 4)), mxb.MxFormat(B, w), _dev(orc.pack(qw, w)),
+                     _dev(ew + np.uint8(w - 4)), mxb.MxFormat(B, w), M, N, K) for w in (4, 6)]
+    _poison_free(mxb)
+    assert torch.equal(y[0], y[1])
+    chain = mxb.mx_gemm(_dev(orc.pack(qa, 4)), _dev(ea), mxb.MxFormat(B, 4), _dev(orc.pack(qw, 4)), _dev(ew),
+                        mxb.MxFormat(B, 4), M, N, K, algo=mxb.MX_ALGO_TCGEN05)
+    assert not torch.equal(y[0], chain)
