@@ -9,6 +9,7 @@
 
 #include <map>
 #include <mutex>
+#include <new>
 #include <tuple>
 #include <type_traits>
 #include <vector>
@@ -1905,9 +1906,13 @@ size_t mx_linear_grouped_workspace_bytes(const mx_linear_args_t *layers, int32_t
     if (!layers || n_layers <= 0) return 0;
     for (int i = 0; i < n_layers; ++i)
         if (!format_ok(layers[i].fa) || !format_ok(layers[i].fw)) return 0;
-    std::vector<int> owner;
-    activation_owners(layers, n_layers, owner);
-    return grouped_workspace(layers, n_layers, owner);
+    try {
+        std::vector<int> owner;
+        activation_owners(layers, n_layers, owner);
+        return grouped_workspace(layers, n_layers, owner);
+    } catch (const std::bad_alloc &) {                  // no C++ exception leaves a C function
+        return 0;
+    }
 }
 
 // packed_exps == nullptr: layers[i].x are floating-point activations, quantized here.
@@ -1915,7 +1920,7 @@ size_t mx_linear_grouped_workspace_bytes(const mx_linear_args_t *layers, int32_t
 static mx_status_t grouped_impl(const mx_linear_args_t *layers, int32_t n_layers,
                                 const uint8_t *const *packed_exps, void *workspace, size_t workspace_bytes,
                                 void *stream)
-{
+try {
     if (!layers) return MX_ERR_NULL;
     if (n_layers <= 0) return MX_ERR_SHAPE;
     int max_t = 0, max_nb = 0;
@@ -2111,6 +2116,9 @@ static mx_status_t grouped_impl(const mx_linear_args_t *layers, int32_t n_layers
     static_cast<mx::StreamParams &>(tp) = sp;
     if (rows32) return launch_stream32(max_t, tp, stages, smem, grid, *d, st);
     return launch_stream(nt, bulk, tp, smem, grid, *d, st);
+} catch (const std::bad_alloc &) {                      // (the tables of the call are kept in host memory)
+    snprintf(t_cuda_error, sizeof(t_cuda_error), "grouped call: out of host memory for the tables of %d layers", (int)n_layers);
+    return MX_ERR_CUDA;
 }
 
 mx_status_t mx_linear_grouped(const mx_linear_args_t *layers, int32_t n_layers, void *workspace,

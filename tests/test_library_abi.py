@@ -151,3 +151,39 @@ def test_compute_calls_fail_loudly_without_a_gpu(mxb):
     assert rc in (-6, -8)
     with pytest.raises(ValueError):
         mxb.mx_quantize(torch.zeros(4, 64), F(16, 4))       # host tensors are refused
+
+
+_OUT_OF_MEMORY = """
+import ctypes as C, resource
+from paper_2307_15517_b200 import binding as mxb
+n = 1 << 21
+args = (mxb.MxLinearArgs * n)()
+a = args[0]
+a.x, a.dt, a.M, a.K, a.ldx, a.fa = 4096, 0, 1, 128, 128, mxb.MxFormat(32, 8)
+a.w_mant, a.w_exp, a.fw, a.N, a.y, a.ldy = 4096, 4096, mxb.MxFormat(32, 4), 16, 4096, 16
+done, size = 1, C.sizeof(mxb.MxLinearArgs)
+while done < n:                                         # every entry like the first
+    C.memmove(C.addressof(args) + done * size, args, min(done, n - done) * size)
+    done *= 2
+assert mxb.mx_linear_grouped_workspace_bytes(args) > 0
+with open("/proc/self/statm") as f:
+    now = int(f.read().split()[0]) * resource.getpagesize()
+resource.setrlimit(resource.RLIMIT_AS, (now + (1 << 20), resource.RLIM_INFINITY))
+size = mxb.lib.mx_linear_grouped_workspace_bytes(args, n)
+status = mxb.lib.mx_linear_grouped(args, n, 4096, 1 << 40, None)
+text = mxb.lib.mx_last_cuda_error()
+resource.setrlimit(resource.RLIMIT_AS, (resource.RLIM_INFINITY, resource.RLIM_INFINITY))
+print("result", size, status, text.decode())
+"""
+
+
+def test_grouped_entry_points_report_exhausted_host_memory():
+    """They keep a table per call on the host; without memory for it they must answer with an error, not end the process
+    with a C++ exception that leaves a C function."""
+    import subprocess
+    import sys
+    mx_build.build()
+    r = subprocess.run([sys.executable, "-c", _OUT_OF_MEMORY], cwd=ROOT, capture_output=True, text=True, timeout=300)
+    assert r.returncode == 0, r.stderr[-500:]
+    words = r.stdout.split()
+    assert words[:3] == ["result", "0", "-6"] and "memory" in r.stdout
