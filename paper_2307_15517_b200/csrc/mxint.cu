@@ -2181,7 +2181,8 @@ mx_status_t mx_gemm_batched(const void *a_mant, const uint8_t *a_exp, mx_format_
     tb.a_item = a_item;
     tb.w_item = w_item;
     tb.y_batch = stride_y;
-    return run_tc(a_hat, w_hat, M, N, K, nullptr, y, ldy, *d, st, nullptr, tb);
+    // one chain of K steps per output, however many items the call has
+    return run_tc(a_hat, w_hat, M, N, K, nullptr, y, ldy, *d, st, nullptr, tb, EpiTail(), false);
 }
 
 // ---- fused attention ---------------------------------------------------------------------------

@@ -64,3 +64,23 @@ def test_fused_tail_and_mxint_result_of_a_split_product(mxb, shape):
         want = mxb.mx_quantize(src, fy)
         assert torch.equal(got[0], want[0]) and torch.equal(got[1], want[1])
     assert mxb.mx_poll_status() == 0
+
+
+def test_an_item_does_not_depend_on_the_number_of_items(mxb):
+    """mx_gemm_batched of the first item alone and of both: the same bits, and those of the product that never cuts K, on
+    operands (block exponents 24 binades apart) whose sums show their order."""
+    M, N, K, B = 200, 131, 1120, 16
+    rng = np.random.default_rng(7)
+    dev = lambda a: torch.from_numpy(np.ascontiguousarray(a)).cuda()             # noqa: E731
+    f = mxb.MxFormat(B, 8)
+    qa, qw = rng.integers(-127, 128, (M, 2 * K)).astype(np.int8), rng.integers(-127, 128, (N, 2 * K)).astype(np.int8)
+    ea, ew = (rng.integers(115, 140, (rows, 2 * K // B)).astype(np.uint8) for rows in (M, N))
+    am, wm = dev(orc.pack(qa, 8)), dev(orc.pack(qw, 8))
+    y = [torch.zeros(n * M, N, device="cuda") for n in (1, 2)]
+    for n in (1, 2):
+        mxb.mx_gemm_batched(am, dev(ea), f, 2 * K, K, wm, dev(ew), f, 2 * K, K, M, N, K, n, y[n - 1], N, M * N)
+    assert mxb.mx_poll_status() == 0
+    assert torch.equal(y[0], y[1][:M])
+    first = [dev(a[:, :a.shape[1] // 2]) for a in (orc.pack(qa, 8), ea, orc.pack(qw, 8), ew)]
+    chain = mxb.mx_gemm(first[0], first[1], f, first[2], first[3], f, M, N, K, algo=mxb.MX_ALGO_TCGEN05)
+    assert torch.equal(y[0], chain)
