@@ -171,3 +171,53 @@ def test_few_tiles_take_the_cut_reduction_whatever_the_width(mxb, shape):
     chain = mxb.mx_gemm(_dev(orc.pack(qa, 4)), _dev(ea), mxb.MxFormat(B, 4), _dev(orc.pack(qw, 4)), _dev(ew),
                         mxb.MxFormat(B, 4), M, N, K, algo=mxb.MX_ALGO_TCGEN05)
     assert not torch.equal(y[0], chain)
+
+
+@pytest.mark.parametrize("form", ("gemm", "linear"))
+def test_wide_steps_between_narrow_ones(mxb, form):
+    """Single K steps with scales per half block between steps with one scale per row: right before and after each other, at
+    and around a step that reloads the scales of four (multiples of 4), at both sides of the 32 steps that one look at the
+    flags covers, at the end of a tile; in some panels of A and of W only, with up to three tiles per CTA pair.  Codes of at
+    most 3 with exponents 0 to 3 binades above one unit: every sum is exact in any order (9 * 4480 * 2^6 < 2^24)."""
+    M, N, K, B, w = 1280, 7936, 4480, 16, 4                # 155 tiles of 256 x 256, 35 steps
+    steps = K // 128
+    g = torch.Generator().manual_seed(11)
+    sides = []
+    for rows, zero, wild, where in ((M, 1, 0, {130: (1, 5, 31, 32), 600: (2,), 1000: (5, 7, 8, 33, 34)}),
+                                    (N, 0, 1, {77: (2, 31, 34), 5000: (2, 3, 4, 28, 31, 32), 7900: (33,)})):
+        q = torch.randint(-3, 4, (rows, steps, 8, B), generator=g, dtype=torch.int8)
+        e = torch.randint(0, 4, (rows, steps, 8), generator=g) + 125
+        q[:, :, zero] = 0                                 # what the other side has there does not count
+        for row, kbs in where.items():
+            for kb in kbs:
+                q[row, kb, wild] = 3
+                e[row, kb, wild] = 125 - 40
+        q, e = q.view(rows, K), e.view(rows, K // B)
+        value = q.double() * torch.exp2((e - 127 - (w - 2)).double()).repeat_interleave(B, 1)
+        sides.append((_dev(orc.pack(q.numpy(), w)), e.to(torch.uint8).cuda(), value.cuda()))
+    (am, ae, a), (wm, we, b) = sides
+    f = mxb.MxFormat(B, w)
+    want = (a @ b.t()).float()
+    if form == "gemm":
+        y = mxb.mx_gemm(am, ae, f, wm, we, f, M, N, K)
+    else:
+        y = mxb.mx_linear(a.float(), f, wm, we, f, N)     # every value is on the grid of its block's own exponent
+    _poison_free(mxb)
+    assert torch.equal(y, want)
+
+
+def test_narrow_steps_of_blocks_twelve_binades_apart(mxb):
+    """Block exponents anywhere within the 12 binades that one scale per row and 128 k can span: no step is wide.  The pipe
+    aligns the 32 products of a step and the accumulator to the largest and truncates: bounded here by one unit in the last
+    place of S per step, 8.0e-6; measured 1.9e-6 (2.1e-6 for the bf16 chain)."""
+    M, N, K, B, wa, ww = 150, 5000, 2144, 16, 5, 4
+    rng = np.random.default_rng(3)
+    qa, qw = rng.integers(-15, 16, (M, K)).astype(np.int8), rng.integers(-7, 8, (N, K)).astype(np.int8)
+    ea, ew = (rng.integers(121, 134, (rows, K // B)).astype(np.uint8) for rows in (M, N))
+    fa, fw = mxb.MxFormat(B, wa), mxb.MxFormat(B, ww)
+    args = (_dev(orc.pack(qa, wa)), _dev(ea), fa, _dev(orc.pack(qw, ww)), _dev(ew), fw, M, N, K)
+    y = mxb.mx_gemm(*args)
+    _poison_free(mxb)
+    y_ref, _, S = orc.gemm(qa, ea, wa, qw, ew, ww, B)
+    err = np.abs(y.cpu().numpy().astype(np.float64) - y_ref) / S
+    assert err.max() <= K / 32 * 2.0 ** -23
