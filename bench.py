@@ -729,6 +729,7 @@ def run_ours(args):
                          "peak_kind": "%g x the rate of the vendor's bf16 GEMM (burst), %s: nominal 8-bit : bf16 ratio"
                                       % (REC_RATE_OVER_BF16, peaks_kind),
                          "frac_of_sustained_peak": achieved / peak_sustained,
+                         "frac_of_bf16_burst": achieved / peaks["bf16_tflops"],
                          # the bound the silicon sets at the clock sampled during the timed region
                          "peak_clock_derived": peak_clock, "frac_of_clock_derived_peak": achieved / peak_clock,
                          "clock_derived_note": "%d SMs x %d flop/clk x %.0f MHz (median sampled under load)"
@@ -737,6 +738,7 @@ def run_ours(args):
                          "algorithmic_flops_per_launch": flops_step / 4.0,
                          # the whole call (operand preparation + product) against the same peaks
                          "call": {"achieved": per_gpu, "frac": per_gpu / peak,
+                                  "frac_of_bf16_burst": per_gpu / peaks["bf16_tflops"],
                                   "frac_of_sustained_peak": per_gpu / peak_sustained,
                                   "frac_of_clock_derived_peak": per_gpu / peak_clock,
                                   "traffic_per_step": None if PREP_DRAM_BYTES_PER_LAUNCH is None else

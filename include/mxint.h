@@ -68,9 +68,12 @@ typedef enum {
                             - few 128 x 128 tiles (at most 74) and K of 1024 or more: the bf16 operands of
                               MX_ALGO_TCGEN05, the K range cut over a cluster of two to four CTAs and the
                               pieces added in fp32, in order;
-                            - else, elem_bits <= 5 and container storage on both operands, K % 32 == 0,
+                            - else, elem_bits <= 5 and container storage on both operands (mantissas
+                              within -2^(w-1) .. 2^(w-1)-1, as the format defines them), K % 32 == 0,
                               and K >= 2048 or (M + N) * K >= 2^22: block-scaled E4M3 operands (also in
-                              place of a cut where weights are so many that the smaller operand pays);
+                              place of a cut where weights are so many that the smaller operand pays;
+                              where blocks of a row lie more than 13 binades apart nearly everywhere it
+                              takes 11 to 17 % longer than the bf16 operands);
                             - else MX_ALGO_TCGEN05.
                             The sum is taken in another order on each: see the accuracy note below.  */
     MX_ALGO_SIMT = 1,    /* CUDA-core kernel: exact integer block sums, blocks added in ascending
@@ -104,15 +107,26 @@ typedef enum {
  * across blocks open; S[i,j] = sum_b |block term b|):
  *   MX_ALGO_SIMT, MX_ALGO_STREAM : exact block sums, one fp32 rounding per block, ascending blocks;
  *                                  bit-reproducible.
- *   MX_ALGO_TCGEN05(_FUSED), AUTO for M > 16, the _q / batched / static entry points : the tensor
- *                                  pipe aligns the 16 products of a step and the accumulator to the
- *                                  largest and truncates, so the guaranteed bound is
+ *   MX_ALGO_TCGEN05(_FUSED), AUTO for M > 16, the _q / fused / batched / static entry points : the tensor
+ *                                  pipe aligns the products of a step (16 of bf16 operands; of block-
+ *                                  scaled ones 32, or 16 where the blocks of a row lie more than 13
+ *                                  binades apart within 128 k) and the accumulator to the largest and
+ *                                  truncates, so the guaranteed bound is
  *                                  ceil(K/16) * 17 * 2^-23 * S; it is approached only when block
- *                                  scales inside one row differ by many binades.  On operands whose
+ *                                  scales inside one row differ by many binades.  Where AUTO cuts K,
+ *                                  up to four such sums are added in fp32 with round-to-nearest: at
+ *                                  most 3 * 2^-24 * S more, and a shorter chain in each.  On operands whose
  *                                  block exponents spread over <= 2^6 per row (every LLM-shaped
  *                                  workload measured: N(0, sigma) weights, outlier-channel or
  *                                  Student-t activations, K up to 16384) the error stays below
  *                                  1e-5 * S, typically below 1e-6 * S.
+ *                                  Block exponents anywhere within 12 binades, K = 2144, 5 x 4 bits:
+ *                                  block-scaled 1.9e-6 * S, one bf16 chain 2.1e-6 * S.
+ *   Rounding depends on the route, and AUTO's route on the sizes and widths: the same values may differ in
+ *   the last bits between 4-bit and 6-bit containers, between two token counts, and between mx_layernorm +
+ *   mx_linear and mx_linear_fused with a LayerNorm prologue (which takes no block-scaled operands).  mx_linear,
+ *   mx_linear_q and mx_linear_fused without one (mx_gemm, mx_gemm_q and mx_gemm_fused) of the same sizes share
+ *   their route for M > 16.  A named algorithm, mx_gemm_batched and mx_gemm_static never cut K.
  *   MX_ALGO_TCGEN05_BLOCKWISE    : exact block sums out of the tensor pipe, one fp32 rounding per block,
  *                                  ascending blocks: the result of MX_ALGO_SIMT, bit for bit, whatever
  *                                  the operands (block terms inside the fp32 normal range). */
@@ -279,9 +293,10 @@ typedef struct {
  * matrices from HBM exactly once.  Per output the integer block sums are exact and the blocks are
  * added in fp32, in ascending order whenever there are enough weight rows to fill the GPU without
  * cutting K (always the case for tens of layers).  `layers` is HOST memory (read during the
- * call).  Restrictions: M <= 16, both formats block 32, weights elem_bits <= 4, K % 128 == 0,
- * M*K small enough to stage in shared memory (M = 16: K <= 18432); otherwise MX_ERR_SHAPE /
- * MX_ERR_FORMAT.  mx_linear(_ex) with MX_ALGO_STREAM is the one-layer form of this call.
+ * call).  When host memory for the call's tables cannot be had, the size query answers 0 and the call
+ * MX_ERR_CUDA with a text in mx_last_cuda_error().  Restrictions: M <= 16, both formats block 32,
+ * weights elem_bits <= 4, K % 128 == 0, M*K small enough to stage in shared memory (M = 16:
+ * K <= 18432); otherwise MX_ERR_SHAPE / MX_ERR_FORMAT.  mx_linear(_ex) with MX_ALGO_STREAM is the one-layer form of this call.
  */
 MX_API size_t mx_linear_grouped_workspace_bytes(const mx_linear_args_t *layers, int32_t n_layers);
 MX_API mx_status_t mx_linear_grouped(const mx_linear_args_t *layers, int32_t n_layers,

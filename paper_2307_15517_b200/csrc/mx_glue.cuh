@@ -86,7 +86,7 @@ layernorm_kernel(const float *__restrict__ x, int64_t ldx, const float *__restri
 // the elements, same order of every sum: the values are bit-identical to that kernel's), then reads the row once more --
 // it is in the L1 -- eight neighbouring elements per thread, normalises and quantizes them as quantize_rows_body does and
 // writes the exact bf16 operand; the fp32 normalised tensor never exists.  (One element per thread instead, with the
-// statistics' ownership and 2-byte stores: the operand passes of a 2048 x 4096 block took 165 us, now 110.)
+// statistics' ownership and 2-byte stores: the three quantizing passes of a 2048 x 4096 block took 165 us, now 110.)
 // After its rows every CTA decodes its share of the packed weights (DecodeWalk), so one launch prepares both
 // operands of the product, as prep_operands_kernel does for a plain layer.
 // Eight neighbouring values (`p` null: all `dflt`), with 16-byte loads where the address allows.
