@@ -1764,7 +1764,12 @@ static mx_status_t tc_prepare_ln(const mx_linear_args_t &a, const mx_prologue_t 
     j.w_hat = w_hat; j.w_row_shift = a.fw.block_rows == 2 ? 1 : 0;
     const int per = (int)((a.K + mx::GLUE_THREADS - 1) / mx::GLUE_THREADS);
     const bool nib = a.fw.elem_bits <= 4;
-    const unsigned g = (unsigned)(a.M < (int64_t)d.sm_count * 8 ? a.M : (int64_t)d.sm_count * 8);
+    // a CTA per row, but a resident wave where the weights have that much work: a grid of few rows decodes them on few SMs, and
+    // started beside a product that leaves some SMs free, several of its CTAs share one (64 tokens, hidden 4096, FFN 16384,
+    // 8 x 8 bits, the whole block 640 -> 267 us)
+    const int64_t rows = a.M < (int64_t)d.sm_count * 8 ? a.M : (int64_t)d.sm_count * 8;
+    const int64_t decode = grid_for((a.N * (a.K / 32) + 1) / 2, mx::GLUE_THREADS, d.sm_count, 4);
+    const unsigned g = (unsigned)(rows > decode ? rows : decode);
     ProfScope prof(KIND_PREP, st);
 #define MX_LAUNCH_LN(P)                                                                                                  \
     do {                                                                                                                 \

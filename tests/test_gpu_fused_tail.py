@@ -138,7 +138,8 @@ def test_fused_tail_argument_checks(mxb):
     assert torch.count_nonzero(y).item() == 0
 
 
-@pytest.mark.parametrize("case", [(300, 512, 528, 16, True), (129, 1056, 256, 32, False), (2048, 4096, 1024, 16, True)])
+@pytest.mark.parametrize("case", [(300, 512, 528, 16, True), (129, 1056, 256, 32, False), (2048, 4096, 1024, 16, True),
+                                  (17, 1024, 4096, 16, True)])                 # more CTAs for the weights than rows
 def test_layernorm_in_the_operand_pass_equals_the_separate_kernel(mxb, case):
     """mx_linear_fused with a LayerNorm prologue normalises each row with the arithmetic of mx_layernorm and
     quantizes it straight to the operand: the product must equal mx_layernorm followed by mx_linear bit for bit
