@@ -46,7 +46,27 @@ __device__ __forceinline__ float4 ld_cluster_f32x4(uint32_t cluster_addr)
     return v;
 }
 
-template <bool TAIL>
+// The 16-byte groups `c4` of rows row, row + 4, row + 8 and row + 12 of a chunk, added up over the cluster's partial tiles in
+// rank order.  Four loads are in flight per CTA of the cluster: a load from another SM takes as long as the rest of a step.
+__device__ __forceinline__ void splitk_sum4(uint32_t smem_base, int split, int chunk, int row, int c4, float4 (&v)[4])
+{
+    for (int s = 0; s < split; ++s) {
+        const uint32_t base = ptx::map_to_cta(smem_base, (uint32_t)s);
+        float4 x[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) x[i] = ld_cluster_f32x4(base + splitk_offset(chunk, row + 4 * i, c4));
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            v[i].x = s ? v[i].x + x[i].x : x[i].x;
+            v[i].y = s ? v[i].y + x[i].y : x[i].y;
+            v[i].z = s ? v[i].z + x[i].z : x[i].z;
+            v[i].w = s ? v[i].w + x[i].w : x[i].w;
+        }
+    }
+}
+
+// QOUT: an MXInt result (yq_mant), else fp32.
+template <bool TAIL, bool QOUT>
 __global__ void __maxnreg__(128)
 gemm_splitk_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant__ CUtensorMap tmap_w, const TcParams p, int split)
 {
@@ -170,25 +190,29 @@ gemm_splitk_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_cons
             if ((turn & 1) != half) continue;
             const int n = n0 + 32 * c, rows0 = m0 + quad * 32;
             if (n >= p.N || rows0 >= p.M) continue;                  // warp-uniform
-            if (p.yq_mant) {                                         // a row per lane: a block is a lane's own columns
-                const int row = rows0 + lane;
+            if (QOUT) {
+                // MXInt result: a row per lane, so that a block is a lane's own columns.  The sums are taken in whole lines,
+                // four rows per warp and load, and pass through this CTA's own copy of the chunk, which no other CTA reads:
+                // read a row per lane from the other CTAs, a request is 16 bytes of 32 lines (352 x 1024 x 1024 with an
+                // 8-bit result: the call 19.3 us, now 12.9; 13.3 without a cut).
+                const int row = rows0 + lane, c4 = lane & 7;
                 TailRegs t;
                 if (TAIL) tail_fetch(p, row, n, t);
-                uint32_t r[32];
-                float acc[32] = {};
-                for (int s = 0; s < split; ++s) {
-                    const uint32_t base = ptx::map_to_cta(smem_base, (uint32_t)s);
+#pragma unroll 1
+                for (int h = 0; h < 2; ++h) {
+                    const int lr = quad * 32 + 16 * h + (lane >> 3);
+                    float4 v[4];
+                    splitk_sum4(smem_base, split, c, lr, c4, v);
 #pragma unroll
-                    for (int v = 0; v < 8; ++v) {
-                        const float4 x = ld_cluster_f32x4(base + splitk_offset(c, quad * 32 + lane, v));
-                        acc[4 * v] = s ? acc[4 * v] + x.x : x.x;
-                        acc[4 * v + 1] = s ? acc[4 * v + 1] + x.y : x.y;
-                        acc[4 * v + 2] = s ? acc[4 * v + 2] + x.z : x.z;
-                        acc[4 * v + 3] = s ? acc[4 * v + 3] + x.w : x.w;
-                    }
+                    for (int i = 0; i < 4; ++i) *reinterpret_cast<float4 *>(smem_gen + splitk_offset(c, lr + 4 * i, c4)) = v[i];
                 }
+                __syncwarp();
+                uint32_t r[32];
 #pragma unroll
-                for (int v = 0; v < 32; ++v) r[v] = __float_as_uint(acc[v]);
+                for (int v = 0; v < 8; ++v) {
+                    const uint4 x = *reinterpret_cast<const uint4 *>(smem_gen + splitk_offset(c, quad * 32 + lane, v));
+                    r[4 * v] = x.x; r[4 * v + 1] = x.y; r[4 * v + 2] = x.z; r[4 * v + 3] = x.w;
+                }
                 if (TAIL) tail_apply(p, t, n, r);
                 store_mxint_chunk(p, row, n, r);
                 continue;

@@ -51,7 +51,7 @@ struct DeviceInfo {
     bool tcx_attr_set = false;
     bool tc8_attr_set = false;
     bool rec_attr_set[4] = {};
-    bool splitk_attr_set[2] = {false, false};
+    bool splitk_attr_set[4] = {};
     int splitk_clusters[mx::SplitKCfg::MAX_SPLIT + 1] = {-1, -1, -1, -1, -1};
     bool attn_attr_set[2] = {false, false};
 };
@@ -938,9 +938,9 @@ mx_status_t splitk_clusters(DeviceInfo &d, int split, int *out)
         attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
         cfg.attrs = attr;
         cfg.numAttrs = 1;
-        MX_CUDA(cudaFuncSetAttribute(mx::gemm_splitk_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)mx::SplitKCfg::SMEM_BYTES));
+        MX_CUDA(cudaFuncSetAttribute(mx::gemm_splitk_kernel<false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)mx::SplitKCfg::SMEM_BYTES));
         int n = 0;
-        MX_CUDA(cudaOccupancyMaxActiveClusters(&n, mx::gemm_splitk_kernel<false>, &cfg));
+        MX_CUDA(cudaOccupancyMaxActiveClusters(&n, mx::gemm_splitk_kernel<false, false>, &cfg));
         known = n;
     }
     *out = known;
@@ -1004,9 +1004,12 @@ mx_status_t launch_splitk(const __nv_bfloat16 *a_hat, const __nv_bfloat16 *w_hat
     if (s != MX_OK) return s;
     s = encode_bf16_rows(&tm_w, w_hat, N, K, Cfg::BN);
     if (s != MX_OK) return s;
-    const bool tail = et.any();
-    s = tail ? smem_attr_once(d.splitk_attr_set[1], mx::gemm_splitk_kernel<true>, (int)Cfg::SMEM_BYTES)
-             : smem_attr_once(d.splitk_attr_set[0], mx::gemm_splitk_kernel<false>, (int)Cfg::SMEM_BYTES);
+    const bool tail = et.any(), q = yq != nullptr;
+    typedef void (*Kernel)(CUtensorMap, CUtensorMap, mx::TcParams, int);
+    static const Kernel kernels[4] = {mx::gemm_splitk_kernel<false, false>, mx::gemm_splitk_kernel<false, true>,
+                                      mx::gemm_splitk_kernel<true, false>, mx::gemm_splitk_kernel<true, true>};
+    const int which = (tail ? 2 : 0) + (q ? 1 : 0);
+    s = smem_attr_once(d.splitk_attr_set[which], kernels[which], (int)Cfg::SMEM_BYTES);
     if (s != MX_OK) return s;
     mx::TcParams p{};
     p.y = y;
@@ -1043,8 +1046,7 @@ mx_status_t launch_splitk(const __nv_bfloat16 *a_hat, const __nv_bfloat16 *w_hat
     cfg.attrs = attr;
     cfg.numAttrs = g_prof.on ? 1 : 2;                     // see launch_dep
     ProfScope prof(KIND_GEMM_TC, st);
-    if (tail) MX_CUDA(cudaLaunchKernelEx(&cfg, mx::gemm_splitk_kernel<true>, tm_a, tm_w, p, split));
-    else MX_CUDA(cudaLaunchKernelEx(&cfg, mx::gemm_splitk_kernel<false>, tm_a, tm_w, p, split));
+    MX_CUDA(cudaLaunchKernelEx(&cfg, kernels[which], tm_a, tm_w, p, split));
     MX_CUDA(cudaGetLastError());
     return MX_OK;
 }

@@ -40,7 +40,7 @@ def test_split_product_within_tolerance(mxb, shape):
     assert bool((big[M:] == -77.0).all()) and bool((big[:, N:] == -77.0).all())
 
 
-@pytest.mark.parametrize("shape", [(200, 160, 1120, 32), (130, 1056, 1040, 16)])
+@pytest.mark.parametrize("shape", [(200, 160, 1120, 32), (130, 1056, 1040, 16), (300, 1792, 1552, 16), (250, 3840, 2080, 32)])
 def test_fused_tail_and_mxint_result_of_a_split_product(mxb, shape):
     """Operands whose sums are exact in any order (4-bit mantissas, one exponent per operand; 6-bit containers keep the
     call on this route): every form must equal the oracle's value carried on in fp32."""
