@@ -952,14 +952,17 @@ mx_status_t splitk_clusters(DeviceInfo &d, int split, int *out)
 // cluster barriers and the exchange (about 2.5 us against 0.2 us per step: at least 12 steps spared).  Whole calls, split /
 // not (us): 352 x 2048 x 8192 in two 36.8 / 51.5, 352 x 2048 x 2048 15.8 / 17.3, 64 x 768 x 3072 in four 12.7 / 20.2,
 // 512 x 1024 x 4096 18.4 / 27.5, 200 x 1024 x 1024 10.7 / 11.2; but 352 x 2048 x 1024 in two 13.2 / 12.2 and
-// 128 x 768 x 768 in four 10.9 / 10.2.
+// 128 x 768 x 768 in four 10.9 / 10.2.  More than 64 CTAs take longer to exchange and need 16 steps spared: at 12 and 14 the
+// cut of 17 to 33 tiles in four is 0.5 us slower to 1.2 us slower (42 x 4096 x 1024, 42 x 3872 x 1024), at 18 it is 1 to 2 us
+// faster, of 48 to 72 tiles in two within 0.3 us at 12 and 1 to 2 us faster at 16.
 mx_status_t splitk_ways(int64_t M, int64_t N, int64_t K, DeviceInfo &d, int *out)
 {
     *out = 0;
     const int64_t tiles = ((M + mx::TC_BM - 1) / mx::TC_BM) * ((N + mx::SplitKCfg::BN - 1) / mx::SplitKCfg::BN);
     const int64_t kblocks = (K + mx::TC_BK - 1) / mx::TC_BK;
     for (int s = mx::SplitKCfg::MAX_SPLIT; s > 1 && !*out; --s) {
-        if (tiles * s > d.sm_count || kblocks * (s - 1) < 12 * s) continue;
+        const int64_t spared = tiles * s > 64 ? 16 : 12;
+        if (tiles * s > d.sm_count || kblocks * (s - 1) < spared * s) continue;
         int fit = 0;
         const mx_status_t st = splitk_clusters(d, s, &fit);
         if (st != MX_OK) return st;

@@ -17,8 +17,9 @@ def mxb():
     return binding
 
 
-# tiles 1, 4 (four pieces, K steps that do not divide), 42 (three or two), 60 (two), a K remainder of 32, odd N
-SHAPES = [(17, 100, 1024, 16, 8, 4), (200, 131, 1120, 32, 6, 6), (300, 1790, 1552, 16, 8, 8), (250, 3840, 1568, 32, 8, 6)]
+# tiles 1, 4 (four pieces, K steps that do not divide), 18 (four), 42 (three or two), 60 (two; not cut), a K remainder of 32
+SHAPES = [(17, 100, 1024, 16, 8, 4), (200, 131, 1120, 32, 6, 6), (130, 1056, 1552, 16, 8, 4), (300, 1790, 2064, 16, 8, 8),
+          (250, 3840, 2080, 32, 8, 6), (250, 3840, 1568, 32, 8, 6)]
 
 
 @pytest.mark.parametrize("shape", SHAPES)
@@ -40,7 +41,8 @@ def test_split_product_within_tolerance(mxb, shape):
     assert bool((big[M:] == -77.0).all()) and bool((big[:, N:] == -77.0).all())
 
 
-@pytest.mark.parametrize("shape", [(200, 160, 1120, 32), (130, 1056, 1040, 16), (300, 1792, 1552, 16), (250, 3840, 2080, 32)])
+@pytest.mark.parametrize("shape", [(200, 160, 1120, 32), (130, 1056, 1552, 16), (130, 1056, 1040, 16), (300, 1792, 2064, 16),
+                                   (250, 3840, 2080, 32)])
 def test_fused_tail_and_mxint_result_of_a_split_product(mxb, shape):
     """Operands whose sums are exact in any order (4-bit mantissas, one exponent per operand; 6-bit containers keep the
     call on this route): every form must equal the oracle's value carried on in fp32."""
