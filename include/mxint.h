@@ -64,6 +64,10 @@ typedef enum { MX_F32 = 0, MX_BF16 = 1 } mx_dtype_t;
 /* Which kernel computes the block-scaled product. */
 typedef enum {
     MX_ALGO_AUTO = 0,    /* M <= 16 and a streamable format (see mx_linear_grouped): MX_ALGO_STREAM;
+                            mx_linear(_ex) with M <= 16, or M <= 32 and blocks of 32 or a small layer (N * K <=
+                            2^24, K <= 6144), container formats whose weight rows are whole 16-byte units, one-row
+                            activation blocks: the arithmetic of MX_ALGO_STREAM for any of them, K cut over a
+                            cluster of up to eight CTAs whose sums are added in fp32, in order;
                             everything else on tensor cores, on operands that hold every value exactly:
                             - few 128 x 128 tiles (at most 74) and K of 1024 or more: the bf16 operands of
                               MX_ALGO_TCGEN05, the K range cut over a cluster of two to four CTAs and the

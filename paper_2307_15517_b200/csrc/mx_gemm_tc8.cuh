@@ -28,7 +28,6 @@
 #include <stdint.h>
 
 #include "mx_gemm_tc.cuh"
-#include "mx_gemv_stream.cuh"
 #include "mx_ptx.cuh"
 
 namespace mx {
@@ -201,8 +200,8 @@ gemm_tc8_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constan
                     const uint32_t sa = smem_base + s * Cfg::STAGE_STRIDE;
                     ptx::tma_load_2d(sa, &tmap_a, kb * Cfg::BK, tm * TC_BM, full_bar(s));
                     ptx::tma_load_2d(sa + Cfg::A_BYTES, &tmap_w, kb * Cfg::BK, tn * BN, full_bar(s));
-                    bulk_copy_g2s(sa + Cfg::A_BYTES + Cfg::W_BYTES, sfa + ((int64_t)kb * chunks_a + tm) * 512, 512, full_bar(s));
-                    bulk_copy_g2s(sa + Cfg::A_BYTES + Cfg::W_BYTES + 512, sfw + ((int64_t)kb * chunks_w + tn) * 512, 512, full_bar(s));
+                    ptx::bulk_copy_g2s(sa + Cfg::A_BYTES + Cfg::W_BYTES, sfa + ((int64_t)kb * chunks_a + tm) * 512, 512, full_bar(s));
+                    ptx::bulk_copy_g2s(sa + Cfg::A_BYTES + Cfg::W_BYTES + 512, sfw + ((int64_t)kb * chunks_w + tn) * 512, 512, full_bar(s));
                     if (++s == STAGES) { s = 0; ph ^= 1u; }
                 }
             }

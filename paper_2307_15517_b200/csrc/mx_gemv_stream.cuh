@@ -80,48 +80,18 @@ struct StreamTableParams : StreamParams {
     __device__ __forceinline__ const CUtensorMap *map_table() const { return tmaps; }
 };
 
-// Geometry of the two variants.
-//   register variant (BULK = false): 8 warps, each lane prefetches four blocks' words with 32-bit
-//     loads; works for any K % 128 == 0.
-//   TMA variant (BULK = true): 16 warps; every warp owns a ring of STAGES shared-memory stages.
-//     A stage is 16 rows x 16 blocks: two tiled TMA loads of 16 rows x 128 mantissa bytes each
-//     (issued back to back so that DRAM sees 256 contiguous bytes per row -- 128-byte pieces
-//     alone reach only ~70 % of the HBM rate; 128-byte swizzle so that the 8 rows one fragment
-//     load touches fall into different banks) plus one load of 16 rows x 16 exponent bytes.
-//     Global data never passes through the load/store data pipe.  Needs K % 512 == 0 and
-//     16-byte aligned exponent arrays.
-template <int NT, bool BULK> struct StreamCfg {
-    static constexpr int WARPS = BULK ? 16 : 8;
+// Register variant, for calls whose tokens leave no room for weight stages in shared memory: 8 warps, each lane prefetches four
+// blocks' words with 32-bit loads.
+template <int NT> struct StreamCfg {
+    static constexpr int WARPS = 8;
     static constexpr int THREADS = WARPS * 32;
-    static constexpr int STAGES = 2;
-    static constexpr int CH = BULK ? 16 : 4;                       // blocks of 32 per step and row
-    static constexpr int MANT_BYTES = 16 * CH * 16;                // 4096: two boxes of 16 rows x 128 bytes
-    static constexpr int STAGE_BYTES = MANT_BYTES + 16 * CH;       // + 16 rows x 16 exponent bytes
-    static constexpr uint32_t STAGE_TX = STAGE_BYTES;
     static constexpr int TP = NT * 8;                              // padded token count
     static constexpr size_t tokens_bytes(int max_nb) { return (size_t)max_nb * TP * (32 + 4); }
-    static constexpr size_t red_bytes() { return (size_t)WARPS * NT * 4 * 32 * 4; }
-    static constexpr size_t smem_bytes(int max_nb)
-    {
-        // the split-K exchange buffer aliases the weight stages in the TMA variant
-        return tokens_bytes(max_nb) +
-               (BULK ? 1024 /* stage alignment */ + (size_t)WARPS * STAGES * STAGE_BYTES +
-                           (size_t)WARPS * STAGES * 8 + 16
-                     : red_bytes());
-    }
+    static constexpr size_t smem_bytes(int max_nb) { return tokens_bytes(max_nb) + (size_t)WARPS * NT * 4 * 32 * 4; }
 };
 constexpr uint64_t STREAM_WAIT_LIMIT_NS = 400ull * 1000 * 1000;
 constexpr int STREAM_MAGIC_INT = 0x4B400000;        // bit pattern of 1.5 * 2^23
 constexpr float STREAM_MAGIC = 12582912.0f;
-
-// 1-D bulk copy global -> shared (no tensor map, no multicast); 16-byte aligned, size % 16 == 0.
-__device__ __forceinline__ void bulk_copy_g2s(uint32_t dst_smem, const void *src, uint32_t bytes, uint32_t bar)
-{
-    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
-                 :
-                 : "r"(dst_smem), "l"((uint64_t)src), "r"(bytes), "r"(bar)
-                 : "memory");
-}
 
 __device__ __forceinline__ void mma_s8s8_m16n8k32(int (&d)[4], uint32_t a0, uint32_t a1, uint32_t a2,
                                                   uint32_t a3, uint32_t b0, uint32_t b1, const int (&c)[4])
@@ -166,50 +136,28 @@ __device__ __forceinline__ f32x2_t fmul2(f32x2_t a, f32x2_t b)
 }
 
 // NT = number of 8-token column tiles (1: T <= 8, 2: T <= 16).
-template <int NT, bool BULK, typename Params>
-__global__ void __launch_bounds__(StreamCfg<NT, BULK>::THREADS, 1)
+template <int NT, typename Params>
+__global__ void __launch_bounds__(StreamCfg<NT>::THREADS, 1)
 gemv_stream_kernel(const __grid_constant__ Params p)
 {
-    using Cfg = StreamCfg<NT, BULK>;
-    constexpr int TP = Cfg::TP, WARPS = Cfg::WARPS, STAGES = Cfg::STAGES, CH = Cfg::CH;
+    using Cfg = StreamCfg<NT>;
+    constexpr int TP = Cfg::TP, WARPS = Cfg::WARPS;
     extern __shared__ __align__(16) uint8_t smem[];
     uint2 *sB = reinterpret_cast<uint2 *>(smem);                 // [nb][TP][4]: (even-k word, odd-k word)
     // [nb][TP] token block scales; they also carry the weights' binary point 2^-(ww-2) and the 1/16
     // of the shifted nibbles, so the weight scale below is the plain 2^(Ew-127)
     float *sCS = reinterpret_cast<float *>(smem + (size_t)p.max_nb * TP * 32);
-    // BULK: [WARPS][STAGES][4096] swizzled mantissa stages (1024-byte aligned), then
-    // [WARPS][STAGES][256] exponent stages; the split-K exchange buffer [WARPS][NT][4][32] reuses them
-    uint8_t *sStage = reinterpret_cast<uint8_t *>(sCS + (size_t)p.max_nb * TP);
-    if (BULK) sStage += (1024u - (ptx::smem_u32(sStage) & 1023u)) & 1023u;
-    uint8_t *sExpStage = sStage + WARPS * STAGES * Cfg::MANT_BYTES;
-    float *sRed = reinterpret_cast<float *>(sStage);
-    uint8_t *sBar = sStage + (BULK ? WARPS * STAGES * Cfg::STAGE_BYTES : 0);     // [WARPS][STAGES] mbarriers
-    volatile uint32_t *abort_flag = reinterpret_cast<volatile uint32_t *>(sBar + WARPS * STAGES * 8);
-    uint32_t phase_bits = 0;                  // parity per stage barrier of this warp
-    bool timed_out = false;
-    if (BULK) {
-        if (threadIdx.x == 0) {
-            for (int i = 0; i < WARPS * STAGES; ++i) ptx::mbar_init(ptx::smem_u32(sBar) + 8 * i, 1);
-            *abort_flag = 0;
-            ptx::fence_mbar_init();
-        }
-        __syncthreads();
-    }
+    float *sRed = sCS + (size_t)p.max_nb * TP;                    // split-K exchange [WARPS][NT][4][32]
 
     ptx::dep_wait();                          // the quantized tokens come from the previous launch
     if (threadIdx.x == 0) ptx::dep_trigger();
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int g = lane >> 2, t = lane & 3;
     const int S = p.split, TPR = WARPS / S;                      // row tiles per round of the CTA
-    int swz[8];                               // this lane's byte offset of 16-byte chunk c in a swizzled box
-#pragma unroll
-    for (int c = 0; c < 8; ++c) swz[c] = g * 128 + ((c ^ g) << 4) + t * 4;
-
     const int per = (p.total_tiles + gridDim.x - 1) / gridDim.x;
     int tile_lo = blockIdx.x * per;
     const int tile_hi = min(tile_lo + per, p.total_tiles);
     const StreamLayer *layers = p.layer_table();
-    const CUtensorMap *tmaps = p.map_table();
     int li = 0;
     while (li + 1 < p.n_layers && layers[li + 1].tile_begin <= tile_lo) ++li;
 
@@ -316,86 +264,24 @@ gemv_stream_kernel(const __grid_constant__ Params p)
                     if (__any_sync(0xFFFFFFFFu, near_top(r.ea | r.eb))) compute_g(b, r, std::true_type{});
                     else compute_g(b, r, std::false_type{});
                 };
-                if (!BULK) {
-                    auto fetch = [&](int b, Regs &r) {
+                auto fetch = [&](int b, Regs &r) {
 #pragma unroll
-                        for (int j = 0; j < 4; ++j) {
-                            r.a[j] = __ldcs(reinterpret_cast<const uint32_t *>(mA + (b + j) * 16));
-                            r.b[j] = __ldcs(reinterpret_cast<const uint32_t *>(mB + (b + j) * 16));
-                        }
-                        r.ea = __ldcs(reinterpret_cast<const uint32_t *>(eA + b));
-                        r.eb = __ldcs(reinterpret_cast<const uint32_t *>(eB + b));
-                    };
-                    // two register sets alternate, so the prefetched words are never copied
-                    Regs ra, rb;
-                    fetch(b_lo, ra);
-                    for (int b = b_lo; b < b_hi; b += 8) {
-                        const bool second = b + 4 < b_hi;
-                        if (second) fetch(b + 4, rb);
-                        compute(b, ra);
-                        if (b + 8 < b_hi) fetch(b + 8, ra);
-                        if (second) compute(b + 4, rb);
+                    for (int j = 0; j < 4; ++j) {
+                        r.a[j] = __ldcs(reinterpret_cast<const uint32_t *>(mA + (b + j) * 16));
+                        r.b[j] = __ldcs(reinterpret_cast<const uint32_t *>(mB + (b + j) * 16));
                     }
-                } else {
-                    // one lane fills a stage with three tiled TMA loads: mantissa columns [x, x+128) and
-                    // [x+128, x+256) of the 16 rows, and their 16 exponent bytes
-                    uint8_t *my_stage = sStage + warp * STAGES * Cfg::MANT_BYTES;
-                    uint8_t *my_exps = sExpStage + warp * STAGES * (16 * CH);
-                    const uint32_t my_bar = ptx::smem_u32(sBar) + 8 * warp * STAGES;
-                    const CUtensorMap *tm_m = tmaps + 2 * li, *tm_e = tm_m + 1;
-                    const int nblk = b_hi - b_lo;                       // multiple of 16
-                    auto issue = [&](int step, int st) {              // step: CH-block chunk index from b_lo
-                        // after an expired wait (this warp's or, through the flag, another's) nothing new
-                        // is put in flight: the CTA is about to return
-                        if (lane == 0 && !timed_out && *abort_flag == 0) {
-                            const uint32_t bar = my_bar + 8 * st;
-                            const uint32_t dst = ptx::smem_u32(my_stage + st * Cfg::MANT_BYTES);
-                            const int b = b_lo + step * CH;
-                            ptx::mbar_arrive_expect_tx(bar, Cfg::STAGE_TX);
-                            ptx::tma_load_2d(dst, tm_m, b * 16, r0, bar);                 // rows >= N read as zero
-                            ptx::tma_load_2d(dst + 2048, tm_m, b * 16 + 128, r0, bar);
-                            ptx::tma_load_2d(ptx::smem_u32(my_exps + st * (16 * CH)), tm_e, b, r0, bar);
-                        }
-                    };
-                    const int nsteps = nblk / CH;
-                    ptx::fence_proxy_async_smem();                      // earlier generic reads/writes of the stages
-                    __syncwarp();
-                    for (int i = 0; i < STAGES && i < nsteps; ++i) issue(i, i);
-                    int st = 0;
-                    for (int step = 0; step < nsteps && !timed_out; ++step) {
-                        const bool ok = ptx::mbar_wait_bounded(my_bar + 8 * st, (phase_bits >> st) & 1u, abort_flag,
-                                                               STREAM_WAIT_LIMIT_NS);
-                        if (!__all_sync(0xFFFFFFFFu, ok)) {
-                            timed_out = true;
-                            *abort_flag = 1;                          // the other warps stop issuing as well
-                            break;
-                        }
-                        phase_bits ^= 1u << st;
-                        const uint8_t *sm = my_stage + st * Cfg::MANT_BYTES;
-                        const uint8_t *se = my_exps + st * (16 * CH);
-#pragma unroll
-                        for (int q = 0; q < CH / 4; ++q) {
-                            Regs r;
-#pragma unroll
-                            for (int j = 0; j < 4; ++j) {
-                                // box (c >> 3); inside it the 16-byte chunk c & 7 of row r sits at
-                                // chunk (c & 7) ^ (r & 7); rows g and g + 8 share r & 7
-                                const int c = q * 4 + j;
-                                const int off = (c >> 3) * 2048 + swz[c & 7];
-                                r.a[j] = *reinterpret_cast<const uint32_t *>(sm + off);
-                                r.b[j] = *reinterpret_cast<const uint32_t *>(sm + off + 8 * 128);
-                            }
-                            r.ea = *reinterpret_cast<const uint32_t *>(se + g * 16 + q * 4);
-                            r.eb = *reinterpret_cast<const uint32_t *>(se + (g + 8) * 16 + q * 4);
-                            compute(b_lo + step * CH + q * 4, r);
-                        }
-                        __syncwarp();                                 // every lane is done reading the stage
-                        if (step + STAGES < nsteps) {
-                            ptx::fence_proxy_async_smem();
-                            issue(step + STAGES, st);
-                        }
-                        if (++st == STAGES) st = 0;
-                    }
+                    r.ea = __ldcs(reinterpret_cast<const uint32_t *>(eA + b));
+                    r.eb = __ldcs(reinterpret_cast<const uint32_t *>(eB + b));
+                };
+                // two register sets alternate, so the prefetched words are never copied
+                Regs ra, rb;
+                fetch(b_lo, ra);
+                for (int b = b_lo; b < b_hi; b += 8) {
+                    const bool second = b + 4 < b_hi;
+                    if (second) fetch(b + 4, rb);
+                    compute(b, ra);
+                    if (b + 8 < b_hi) fetch(b + 8, ra);
+                    if (second) compute(b + 4, rb);
                 }
             }
             float acc[NT][4];
@@ -421,7 +307,6 @@ gemv_stream_kernel(const __grid_constant__ Params p)
                             acc[n][j] = v;
                         }
                 }
-                __syncthreads();          // the exchange buffer shares memory with the weight stages
             }
             if (active && s == 0) {
 #pragma unroll
@@ -436,16 +321,7 @@ gemv_stream_kernel(const __grid_constant__ Params p)
         }
         tile_lo = l_end;
         ++li;
-        if (BULK && __syncthreads_or(timed_out ? 1 : 0)) break;     // a bounded wait expired: give up
     }
-    if (BULK && timed_out) {
-        *abort_flag = 1;
-        atomicOr(p.status, 1u);
-        // copies already in flight get time to land before the CTA's shared memory is released
-        const uint64_t t0 = ptx::globaltimer_ns();
-        while (ptx::globaltimer_ns() - t0 < 100000ull) __nanosleep(1000);
-    }
-    if (BULK) __syncthreads();                // no warp leaves while another may still be waiting out its copies
 }
 
 // ---- one or two tokens ---------------------------------------------------------------------------
@@ -525,7 +401,7 @@ __device__ __forceinline__ void dp_step(const uint8_t *mant, const uint8_t *exps
 
 template <int TOK, typename Params>
 __global__ void __launch_bounds__(Stream32Cfg<TOK>::THREADS, 1)
-gemv_stream32_kernel(const __grid_constant__ Params p, int stages)
+gemv_stream32_kernel(const __grid_constant__ Params p, int stages, int early)
 {
     using Cfg = Stream32Cfg<TOK>;
     constexpr int WARPS = Cfg::WARPS, CH = Cfg::CH, ROWS = Cfg::ROWS;
@@ -544,8 +420,9 @@ gemv_stream32_kernel(const __grid_constant__ Params p, int stages)
         ptx::fence_mbar_init();
     }
     __syncthreads();
-    ptx::dep_wait();                          // the quantized tokens come from the previous launch
-    if (threadIdx.x == 0) ptx::dep_trigger();
+    // early: the launch in front is this call's quantizer, which lets this one start only after ITS predecessors are complete
+    // and writes tokens only; weights and tables may be read before it has finished
+    if (!early) ptx::dep_wait();
 
     const StreamLayer *layers = p.layer_table();
     const CUtensorMap *tmaps = p.map_table();
@@ -602,6 +479,8 @@ gemv_stream32_kernel(const __grid_constant__ Params p, int stages)
         for (int i = 0; i < stages; ++i) issue();
     }
     __syncwarp();
+    if (early) ptx::dep_wait();               // the quantized tokens
+    if (threadIdx.x == 0) ptx::dep_trigger();
 
     int st = 0;                               // stage and parity of the next step to consume
     uint32_t parity = 0;

@@ -127,6 +127,14 @@ __device__ __forceinline__ void tma_store_3d(const void *tmap, int32_t x, int32_
                  : "memory");
 }
 
+// 1-D bulk copy global -> shared (no tensor map, no multicast); 16-byte aligned, size % 16 == 0.
+__device__ __forceinline__ void bulk_copy_g2s(uint32_t dst_smem, const void *src, uint32_t bytes, uint32_t bar)
+{
+    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
+                 :
+                 : "r"(dst_smem), "l"((uint64_t)src), "r"(bytes), "r"(bar)
+                 : "memory");
+}
 // 2-D tiled store shared -> global (bulk async group); elements outside the tensor are clipped.
 __device__ __forceinline__ void tma_store_2d(const void *tmap, int32_t x, int32_t y, uint32_t src_smem)
 {
@@ -169,6 +177,12 @@ __device__ __forceinline__ uint32_t cluster_ctarank()
 {
     uint32_t r;
     asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+    return r;
+}
+__device__ __forceinline__ uint32_t cluster_nctarank()
+{
+    uint32_t r;
+    asm volatile("mov.u32 %0, %%cluster_nctarank;" : "=r"(r));
     return r;
 }
 // Every thread of both CTAs: arrive (release) and wait (acquire) on the cluster barrier.

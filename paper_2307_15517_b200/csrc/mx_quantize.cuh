@@ -167,10 +167,11 @@ __device__ __forceinline__ float absmax_nan(float m, float x)
 // two's-complement nibbles (w <= 4, returned in p.x) or two words of int8; xh receives the decoded
 // values.  Same arithmetic as
 // quantize_rows_body below (add-only rounding with the block-scaled magic constant, the
-// multiply-based form for blocks near the top of the range or holding Inf/NaN).
+// multiply-based form for blocks near the top of the range or holding Inf/NaN).  BYTES: two words of int8 for every width.
+template <bool BYTES = false>
 __device__ __forceinline__ uint2 encode8_full(const float (&v)[8], int ebyte, int w, float (&xh)[8])
 {
-    const bool nibble = w <= 4;
+    const bool nibble = !BYTES && w <= 4;
     const int qmax = (1 << (w - 1)) - 1;
     const uint32_t off = nibble ? 8u : 128u;
     const bool bad = ebyte == 255;
@@ -219,6 +220,11 @@ __device__ __forceinline__ uint2 encode8_packed(const float (&v)[8], int ebyte, 
 {
     float unused[8];
     return encode8_full(v, ebyte, w, unused);
+}
+__device__ __forceinline__ uint2 encode8_bytes(const float (&v)[8], int ebyte, int w)
+{
+    float unused[8];
+    return encode8_full<true>(v, ebyte, w, unused);
 }
 
 // rows x K, rows contiguous along K with leading dimension ldx.  BLOCK in {16, 32}.

@@ -24,6 +24,7 @@
 #include "mx_gemm_rec.cuh"
 #include "mx_gemm_tc8.cuh"
 #include "mx_gemm_tcx.cuh"
+#include "mx_gemv_mma.cuh"
 #include "mx_gemv_stream.cuh"
 #include "mx_glue.cuh"
 #include "mx_quantize.cuh"
@@ -45,7 +46,10 @@ struct DeviceInfo {
     uint32_t *status = nullptr;
     bool tc_attr_set[2][4] = {{false, false, false, false}, {false, false, false, false}};
     bool tc_tail_attr_set[2] = {false, false};
-    bool stream_attr_set[2][4] = {};
+    bool stream_attr_set[2][2] = {};
+    bool mma_attr_set[2][2] = {};
+    bool gemv_attr_set[12] = {};
+    int gemv_clusters[12][4][2] = {};          // resident clusters by kernel, log2 of the cluster size, two CTAs per SM
     bool stream32_attr_set[2][2] = {};
     bool tc2_attr_set[2] = {false, false};
     bool tcx_attr_set = false;
@@ -1163,24 +1167,25 @@ mx_status_t encode_u8_rows(CUtensorMap *out, const void *base, int64_t rows, int
     return MX_OK;
 }
 
+// out2[0]: over the packed mantissas (rows of row_bytes); out2[1], when nb is not 0: over the exponent bytes (rows of nb).
 // (the caller holds g_wmap_mu)
-mx_status_t packed_weight_maps(const void *w_mant, const void *w_exp, int64_t N, int64_t K, CUtensorMap *out2)
+mx_status_t packed_weight_maps(const void *w_mant, const void *w_exp, int64_t N, int64_t row_bytes, int64_t nb, CUtensorMap *out2)
 {
-    const auto key = std::make_tuple(w_mant, w_exp, N, K);
+    const auto key = std::make_tuple(w_mant, nb ? w_exp : nullptr, N, row_bytes);
     auto it = g_wmap_cache.find(key);
     if (it == g_wmap_cache.end()) {
         const mx_status_t es = ensure_encoder();
         if (es != MX_OK) return es;
-        WeightMaps wm;
-        mx_status_t s = encode_u8_rows(&wm.mant, w_mant, N, K / 2, 128, CU_TENSOR_MAP_SWIZZLE_128B);
+        WeightMaps wm{};
+        mx_status_t s = encode_u8_rows(&wm.mant, w_mant, N, row_bytes, 128, CU_TENSOR_MAP_SWIZZLE_128B);
         if (s != MX_OK) return s;
-        s = encode_u8_rows(&wm.exps, w_exp, N, K / 32, 16, CU_TENSOR_MAP_SWIZZLE_NONE);
+        if (nb) s = encode_u8_rows(&wm.exps, w_exp, N, nb, 16, CU_TENSOR_MAP_SWIZZLE_NONE);
         if (s != MX_OK) return s;
         if (g_wmap_cache.size() > 4096) g_wmap_cache.clear();
         it = g_wmap_cache.emplace(key, wm).first;
     }
     out2[0] = it->second.mant;
-    out2[1] = it->second.exps;
+    if (nb) out2[1] = it->second.exps;
     return MX_OK;
 }
 
@@ -1233,44 +1238,245 @@ size_t grouped_workspace(const mx_linear_args_t *layers, int32_t n, const std::v
     return total;
 }
 
-template <int NT, bool BULK, typename Params>
+template <int NT, typename Params>
 mx_status_t launch_stream_as(const Params &sp, size_t smem, int grid, DeviceInfo &d, cudaStream_t st)
 {
     constexpr bool INLINE = std::is_same<Params, mx::StreamInlineParams>::value;
-    const mx_status_t as = smem_attr_once(d.stream_attr_set[INLINE ? 1 : 0][(NT - 1) * 2 + (BULK ? 1 : 0)],
-                                          mx::gemv_stream_kernel<NT, BULK, Params>, 227 * 1024);
+    const mx_status_t as = smem_attr_once(d.stream_attr_set[INLINE ? 1 : 0][NT - 1], mx::gemv_stream_kernel<NT, Params>, 227 * 1024);
     if (as != MX_OK) return as;
     ProfScope prof(KIND_GEMM_STREAM, st);
-    MX_CUDA(launch_dep(mx::gemv_stream_kernel<NT, BULK, Params>, dim3(grid), dim3(mx::StreamCfg<NT, BULK>::THREADS), smem, st, sp));
+    MX_CUDA(launch_dep(mx::gemv_stream_kernel<NT, Params>, dim3(grid), dim3(mx::StreamCfg<NT>::THREADS), smem, st, sp));
+    MX_CUDA(cudaGetLastError());
+    return MX_OK;
+}
+
+template <int NT, typename Params>
+mx_status_t launch_mma_as(const Params &sp, int warps, int stages, int early, size_t smem, int grid, DeviceInfo &d, cudaStream_t st)
+{
+    constexpr bool INLINE = std::is_same<Params, mx::StreamInlineParams>::value;
+    const mx_status_t as = smem_attr_once(d.mma_attr_set[INLINE ? 1 : 0][NT - 1], mx::gemv_mma_kernel<NT, Params>, 227 * 1024);
+    if (as != MX_OK) return as;
+    ProfScope prof(KIND_GEMM_STREAM, st);
+    MX_CUDA(launch_dep(mx::gemv_mma_kernel<NT, Params>, dim3(grid), dim3(32 * warps), smem, st, sp, stages, early));
     MX_CUDA(cudaGetLastError());
     return MX_OK;
 }
 
 template <int TOK, typename Params>
-mx_status_t launch_stream32_as(const Params &sp, int stages, size_t smem, int grid, DeviceInfo &d, cudaStream_t st)
+mx_status_t launch_stream32_as(const Params &sp, int stages, int early, size_t smem, int grid, DeviceInfo &d, cudaStream_t st)
 {
     constexpr bool INLINE = std::is_same<Params, mx::StreamInlineParams>::value;
     const mx_status_t as = smem_attr_once(d.stream32_attr_set[INLINE ? 1 : 0][TOK - 1], mx::gemv_stream32_kernel<TOK, Params>, 227 * 1024);
     if (as != MX_OK) return as;
     ProfScope prof(KIND_GEMM_STREAM, st);
-    MX_CUDA(launch_dep(mx::gemv_stream32_kernel<TOK, Params>, dim3(grid), dim3(mx::Stream32Cfg<TOK>::THREADS), smem, st, sp, stages));
+    MX_CUDA(launch_dep(mx::gemv_stream32_kernel<TOK, Params>, dim3(grid), dim3(mx::Stream32Cfg<TOK>::THREADS), smem, st, sp, stages, early));
     MX_CUDA(cudaGetLastError());
     return MX_OK;
 }
 
-template <typename Params>
-mx_status_t launch_stream32(int tok, const Params &sp, int stages, size_t smem, int grid, DeviceInfo &d, cudaStream_t st)
-{
-    return tok == 1 ? launch_stream32_as<1>(sp, stages, smem, grid, d, st) : launch_stream32_as<2>(sp, stages, smem, grid, d, st);
-}
+// How a grouped call runs: one or two tokens a weight row per lane; else 16 rows per warp on the integer MMA, 16 warps or 8,
+// whatever fits beside the tokens; else the register variant, which stages the tokens only.
+struct StreamPlan {
+    enum Kind { ROWS32, MMA, REGS } kind = REGS;
+    int warps = 8, stages = 0, rows = 16, unit = 4;      // unit: blocks of 32 that a piece of a cut K is a multiple of
+    size_t smem = 0;
+};
 
 template <typename Params>
-mx_status_t launch_stream(int nt, bool bulk, const Params &sp, size_t smem, int grid, DeviceInfo &d, cudaStream_t st)
+mx_status_t launch_stream(const StreamPlan &sp, int tok, int early, const Params &p, int grid, DeviceInfo &d, cudaStream_t st)
 {
-    if (bulk) return nt == 2 ? launch_stream_as<2, true>(sp, smem, grid, d, st) : launch_stream_as<1, true>(sp, smem, grid, d, st);
-    return nt == 2 ? launch_stream_as<2, false>(sp, smem, grid, d, st) : launch_stream_as<1, false>(sp, smem, grid, d, st);
+    if (sp.kind == StreamPlan::ROWS32)
+        return tok == 1 ? launch_stream32_as<1>(p, sp.stages, early, sp.smem, grid, d, st)
+                        : launch_stream32_as<2>(p, sp.stages, early, sp.smem, grid, d, st);
+    if (sp.kind == StreamPlan::MMA)
+        return tok > 8 ? launch_mma_as<2>(p, sp.warps, sp.stages, early, sp.smem, grid, d, st)
+                       : launch_mma_as<1>(p, sp.warps, sp.stages, early, sp.smem, grid, d, st);
+    return tok > 8 ? launch_stream_as<2>(p, sp.smem, grid, d, st) : launch_stream_as<1>(p, sp.smem, grid, d, st);
 }
 
+// ---- one layer of few tokens in one launch (gemv_single_kernel) ----------------------------------------
+// Container formats whose weight rows are whole 16-byte units (the TMA boxes), one-row activation blocks.
+bool gemv_layer_ok(const mx_linear_args_t &a)
+{
+    const int64_t row_bytes = a.fw.elem_bits <= 4 ? a.K / 2 : a.K;
+    return a.M >= 1 && a.M <= 32 && format_1d(a.fa) && format_ok(a.fw) && a.fa.block == a.fw.block && (row_bytes % 16) == 0;
+}
+
+struct GemvPlan { int cluster, rounds, stages, max_groups, exp_words; size_t smem; };
+
+template <int NT, bool NIB, int BLOCK>
+mx_status_t launch_gemv_as(int slot, const GemvPlan &g, const CUtensorMap &tm, const mx::GemvArgs &args, DeviceInfo &d, cudaStream_t st)
+{
+    const auto kernel = mx::gemv_single_kernel<NT, NIB, BLOCK>;
+    const mx_status_t s = smem_attr_once(d.gemv_attr_set[slot], kernel, 227 * 1024);
+    if (s != MX_OK) return s;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)((args.row_groups + g.rounds - 1) / g.rounds * g.cluster));
+    cfg.blockDim = dim3(mx::GemvCfg::THREADS);
+    cfg.dynamicSmemBytes = g.smem;
+    cfg.stream = st;
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = (unsigned)g.cluster;
+    attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[1].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = g_prof.on ? 1 : 2;                     // see launch_dep
+    ProfScope prof(KIND_GEMM_STREAM, st);
+    MX_CUDA(cudaLaunchKernelEx(&cfg, kernel, tm, args, g.stages));
+    MX_CUDA(cudaGetLastError());
+    return MX_OK;
+}
+
+template <int NT, bool NIB, int BLOCK>
+mx_status_t gemv_resident_as(int slot, int cluster, size_t smem, DeviceInfo &d, int *out)
+{
+    const auto kernel = mx::gemv_single_kernel<NT, NIB, BLOCK>;
+    const mx_status_t s = smem_attr_once(d.gemv_attr_set[slot], kernel, 227 * 1024);
+    if (s != MX_OK) return s;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)(cluster * d.sm_count));
+    cfg.blockDim = dim3(mx::GemvCfg::THREADS);
+    cfg.dynamicSmemBytes = smem;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = (unsigned)cluster;
+    attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    MX_CUDA(cudaOccupancyMaxActiveClusters(out, kernel, &cfg));
+    return MX_OK;
+}
+
+template <int NT, bool NIB, int BLOCK> size_t gemv_smem(const GemvPlan &g)
+{
+    return mx::GemvCfg::smem_bytes<NT, NIB, BLOCK>(g.max_groups, g.stages, g.rounds, g.cluster);
+}
+typedef mx_status_t (*GemvLaunch)(int, const GemvPlan &, const CUtensorMap &, const mx::GemvArgs &, DeviceInfo &, cudaStream_t);
+struct GemvVariant {
+    size_t (*smem)(const GemvPlan &);
+    GemvLaunch launch;
+    mx_status_t (*resident)(int, int, size_t, DeviceInfo &, int *);
+};
+#define MX_GEMV_ONE(NT, NIB, B) {gemv_smem<NT, NIB, B>, launch_gemv_as<NT, NIB, B>, gemv_resident_as<NT, NIB, B>}
+#define MX_GEMV(NT) MX_GEMV_ONE(NT, false, 16), MX_GEMV_ONE(NT, false, 32), MX_GEMV_ONE(NT, true, 16), MX_GEMV_ONE(NT, true, 32)
+const GemvVariant g_gemv[12] = {MX_GEMV(1), MX_GEMV(2), MX_GEMV(4)};      // nibbles, block 32: bits 1, 0
+#undef MX_GEMV
+#undef MX_GEMV_ONE
+int gemv_slot(const mx_linear_args_t &a)
+{
+    const int nt = a.M <= 8 ? 0 : a.M <= 16 ? 1 : 2;
+    return 4 * nt + (a.fw.elem_bits <= 4 ? 2 : 0) + (a.fw.block == 32 ? 1 : 0);
+}
+
+// Clusters of `cluster` CTAs that are resident at once; asked once per kernel, cluster size and number of CTAs that fit an SM.
+mx_status_t gemv_resident(int slot, int cluster, bool two, DeviceInfo &d, int64_t *out)
+{
+    int log2c = 0;
+    while ((1 << log2c) < cluster) ++log2c;
+    int known;
+    {
+        std::lock_guard<std::mutex> lk(g_init_mu);
+        known = d.gemv_clusters[slot][log2c][two];
+    }
+    if (known == 0) {
+        // (asked with the most shared memory of the class)
+        const mx_status_t s = g_gemv[slot].resident(slot, cluster, two ? 112u * 1024u : 227u * 1024u, d, &known);
+        if (s != MX_OK) return s;
+        std::lock_guard<std::mutex> lk(g_init_mu);
+        d.gemv_clusters[slot][log2c][two] = known;
+    }
+    *out = known;
+    return MX_OK;
+}
+
+// The cut of K depends on N and K alone, so a token's bits do not depend on how many others share the call.  Where the row
+// groups alone fill the chip twice over K is not cut (one chain of ascending blocks); else it is cut as often as a cluster
+// allows while the slices are whole steps or the CTAs fit at once (a step fetches 256 bytes of a row whatever its slice needs:
+// 512 x 16384, 8 bits, in eight slices of 64 bytes 35 us).  A CTA then quantizes the smallest slice of the tokens and the most
+// weight bytes are in flight.  Row groups beyond what is resident go to the same clusters, so that a staged slice is used again.
+bool gemv_plan(const mx_linear_args_t &a, DeviceInfo &d, GemvPlan *out)
+{
+    if (!gemv_layer_ok(a)) return false;
+    const bool nib = a.fw.elem_bits <= 4;
+    const int64_t row_bytes = nib ? a.K / 2 : a.K, ng = (row_bytes + 63) / 64, groups = (a.N + mx::GemvCfg::ROWS - 1) / mx::GemvCfg::ROWS;
+    if (ng > INT32_MAX / 64 || groups > INT32_MAX / 64) return false;
+    const int slot = gemv_slot(a);
+    GemvPlan g;
+    g.cluster = 1;
+    if (groups < 2 * d.sm_count)
+        for (int c = 2; c <= mx::GemvCfg::MAX_CLUSTER && c <= ng && (groups * c <= 2 * d.sm_count || ng / c >= 4); c *= 2) g.cluster = c;
+    g.max_groups = 0;
+    const int gb = (nib ? 128 : 64) / a.fw.block;
+    bool words = ((a.K / a.fw.block) % 4) == 0 && (reinterpret_cast<uintptr_t>(a.w_exp) & 3u) == 0;
+    for (int r = 0; r < g.cluster; ++r) {
+        const int lo = (int)(ng * r / g.cluster), hi = (int)(ng * (r + 1) / g.cluster);
+        g.max_groups = hi - lo > g.max_groups ? hi - lo : g.max_groups;
+        words = words && (lo * gb) % 4 == 0;
+    }
+    g.exp_words = words ? 1 : 0;
+    // Two CTAs per SM where that leaves a stage, else one (32 x 8192 x 2048 at one CTA per SM: the clusters do not all fit, two
+    // waves, 34 instead of 25 us).  Row groups beyond what is resident at once go to the same clusters, where a staged slice is
+    // used again; the partial tiles of those rounds come before a third and second stage (5 x 4096 x 11008 with three stages and
+    // three waves 19.5, two stages and three rounds 11.9).
+    constexpr size_t HALF = 112u * 1024u, FULL = 227u * 1024u;
+    const int steps = (g.max_groups + 3) / 4;
+    for (const size_t cap : {HALF, FULL}) {
+        g.stages = 1;
+        g.rounds = 1;
+        g.smem = g_gemv[slot].smem(g);
+        if (g.smem > cap) continue;
+        int64_t resident = 0;
+        const mx_status_t s = gemv_resident(slot, g.cluster, cap == HALF, d, &resident);
+        if (s != MX_OK || resident < 1) return false;
+        const int64_t rounds = (groups + resident - 1) / resident;
+        const int want = (int)(rounds < 8 ? rounds : 8);
+        for (int st = 3; st >= 1; --st) {
+            g.stages = st < steps * want ? st : steps * want;
+            g.rounds = want;
+            g.smem = g_gemv[slot].smem(g);
+            for (; g.smem > cap && st == 1 && g.rounds > 1; g.smem = g_gemv[slot].smem(g)) --g.rounds;
+            if (g.smem <= cap) break;
+        }
+        *out = g;
+        return true;
+    }
+    return false;
+}
+
+// Up to 16 tokens always (operand pass and tensor-core product / this, us: 1 x 4096 x 4096 in blocks of 16 21.5 / 6.8,
+// 16 x 16384 x 16384 in 8 bits 238 / 85, 1 x 768 x 768 9.8 / 4.4).  Up to 32 the arithmetic counts, two rescales per 32 k and
+// token in blocks of 16: 32 x 4096 x 4096 20.2 / 17.3, 1024 x 1024 10.8 / 7.2, 640 x 5120 15.6 / 13.7, but 4096 x 11008
+// 36.1 / 42.1 (three rounds of row groups) and 24 tokens of 8192 x 2048 in 8 bits 24.6 / 25.9; in blocks of 32 4096 x 11008
+// 42.9 / 24.5, 8192 x 2048 24.3 / 19.8, 11008 x 4096 40.9 / 30.5.
+bool gemv_is_faster(const mx_linear_args_t &a)
+{
+    return a.M <= 16 || (a.M <= 32 && (a.fw.block == 32 || (a.N * a.K <= (1 << 24) && a.K <= 6144)));
+}
+
+mx_status_t launch_gemv(const mx_linear_args_t &a, const GemvPlan &g, DeviceInfo &d, cudaStream_t st)
+{
+    CUtensorMap tm;
+    const bool nib = a.fw.elem_bits <= 4;
+    {
+        std::lock_guard<std::mutex> lk(g_wmap_mu);
+        const mx_status_t s = packed_weight_maps(a.w_mant, a.w_exp, a.N, nib ? a.K / 2 : a.K, 0, &tm);
+        if (s != MX_OK) return s;
+    }
+    mx::GemvArgs p;
+    p.x = a.x; p.ldx = a.ldx; p.w_exp = a.w_exp; p.bias = a.bias; p.y = a.y; p.ldy = a.ldy;
+    p.T = (int)a.M; p.N = (int)a.N; p.K = (int)a.K;
+    p.a_bits = a.fa.elem_bits; p.w_bits = a.fw.elem_bits; p.w_rows2 = a.fw.block_rows == 2 ? 1 : 0;
+    p.rounds = g.rounds;
+    p.row_groups = (int)((a.N + mx::GemvCfg::ROWS - 1) / mx::GemvCfg::ROWS);
+    p.exp_words = g.exp_words;
+    p.max_groups = g.max_groups;
+    p.status = d.status;
+    p.bf16 = a.dt == MX_BF16 ? 1 : 0;
+    const int slot = gemv_slot(a);
+    return g_gemv[slot].launch(slot, g, tm, p, d, st);
+}
 
 // Both operands of one layer in the tensor-core form: activations quantized straight to exact
 // bf16, packed weights decoded to bf16.  One launch when K % 32 == 0, else two.
@@ -1667,6 +1873,8 @@ mx_status_t mx_linear_ex(const void *x, mx_dtype_t dt, int64_t M, int64_t K, int
     const bool fused = algo == MX_ALGO_TCGEN05_FUSED && (K % 32) == 0 && fw.block_rows == 1;
     if (fused && !fused_ok(K, w_exp)) return MX_ERR_ALIGN;
     if (workspace_bytes < (fused ? fused_workspace(M, K) : tc_workspace(M, N, K))) return MX_ERR_WORKSPACE;
+    GemvPlan gemv;
+    if (any_algo && gemv_is_faster(one) && gemv_plan(one, *d, &gemv)) return launch_gemv(one, gemv, *d, st);
     bool rec = false;
     if (any_algo && rec_fits(fa, fw, M, N, K)) {
         s = rec_is_faster(M, N, K, *d, &rec);
@@ -1954,26 +2162,14 @@ try {
     if (!workspace || workspace_bytes < need) return MX_ERR_WORKSPACE;
     if ((reinterpret_cast<uintptr_t>(workspace) & 255u) != 0) return MX_ERR_ALIGN;
     const int nt = max_t > 8 ? 2 : 1;
-    // weights staged by bulk copies need 16-byte aligned exponent chunks: K % 512 == 0 everywhere
-    bool bulk = true;
-    for (int i = 0; i < n_layers; ++i)
-        bulk = bulk && (layers[i].K % 512) == 0 && (reinterpret_cast<uintptr_t>(layers[i].w_exp) & 15u) == 0 &&
-               layers[i].fw.block_rows == 1;
-    auto smem_of = [&](bool b) {
-        return nt == 2 ? (b ? mx::StreamCfg<2, true>::smem_bytes(max_nb) : mx::StreamCfg<2, false>::smem_bytes(max_nb))
-                       : (b ? mx::StreamCfg<1, true>::smem_bytes(max_nb) : mx::StreamCfg<1, false>::smem_bytes(max_nb));
-    };
-    size_t smem = smem_of(bulk);
-    if (bulk && smem > 227u * 1024u) {
-        bulk = false;
-        smem = smem_of(false);
-    }
-    if (smem > 227u * 1024u) return MX_ERR_SHAPE;                  // tokens x K too large to stage
+    constexpr size_t SMEM = 227u * 1024u;
+    StreamPlan plan;
+    plan.smem = nt == 2 ? mx::StreamCfg<2>::smem_bytes(max_nb) : mx::StreamCfg<1>::smem_bytes(max_nb);
+    if (plan.smem > SMEM) return MX_ERR_SHAPE;                     // tokens x K too large to stage
     DeviceInfo *d = nullptr;
     mx_status_t s = device_info(&d);
     if (s != MX_OK) return s;
-    // K is cut over the warps of a CTA only when the row tiles alone cannot fill the GPU; `unit`: blocks that a piece must be
-    // a multiple of, in every layer
+    // K is cut over the warps of a CTA only when the row tiles alone cannot fill the GPU; the pieces are whole units in every layer
     auto choose_split = [&](int64_t tiles, int64_t warp_slots, int unit) {
         for (int cand = 8; tiles < warp_slots && cand > 1; cand >>= 1) {
             bool whole = cand <= 4 || tiles * 4 < warp_slots;
@@ -1982,16 +2178,34 @@ try {
         }
         return 1;
     };
-    // one or two tokens: a weight row per lane (see gemv_stream32_kernel), with as many stages as fit beside the tokens
-    int stages = 0;
-    for (int n = mx::Stream32Cfg<1>::MAX_STAGES; bulk && max_t <= 2 && n >= 2 && !stages; --n) {
-        const size_t need = max_t == 1 ? mx::Stream32Cfg<1>::smem_bytes(max_nb, n) : mx::Stream32Cfg<2>::smem_bytes(max_nb, n);
-        if (need <= 227u * 1024u) {
-            stages = n;
-            smem = need;
-        }
+    // exponent boxes of one row per weight row, at 16-byte offsets (gemv_stream32_kernel)
+    bool boxes = max_t <= 2;
+    for (int i = 0; i < n_layers; ++i)
+        boxes = boxes && (layers[i].K % 512) == 0 && (reinterpret_cast<uintptr_t>(layers[i].w_exp) & 15u) == 0 &&
+                layers[i].fw.block_rows == 1;
+    // one layer: one launch -- but for one token of a large one and two of one with very many rows, where the row-per-lane
+    // kernel's loads run ahead over more rows (K x N, one token: 4096 x 11008 8.9 against 10.2 us, 8192 x 16384 15.6 / 19.0,
+    // 4096 x 32000 14.6 / 20.0, but 4096 x 4096 5.5 / 5.7 and on the host one launch less; two: 4096 x 32000 18.6 / 22.0,
+    // 8192 x 16384 20.8 / 21.4, 4096 x 11008 11.0 / 10.3, 8192 x 8192 14.6 / 11.9)
+    if (n_layers == 1 && !packed_exps) {
+        GemvPlan g;
+        const int64_t n = layers[0].N, weights = n * layers[0].K;
+        const bool rows = boxes && (max_t == 1 ? weights >= (1 << 25) : n >= 24576 && weights >= (1 << 26));
+        if (!rows && gemv_plan(layers[0], *d, &g)) return launch_gemv(layers[0], g, *d, static_cast<cudaStream_t>(stream));
     }
-    const bool rows32 = stages > 0;
+    auto take = [&](StreamPlan::Kind kind, int warps, int stages, int rows, int unit, size_t smem) {
+        if (plan.kind != StreamPlan::REGS || smem > SMEM) return;
+        plan.kind = kind; plan.warps = warps; plan.stages = stages; plan.rows = rows; plan.unit = unit; plan.smem = smem;
+    };
+    for (int n = mx::Stream32Cfg<1>::MAX_STAGES; boxes && n >= 2; --n)       // with as many stages as fit beside the tokens
+        take(StreamPlan::ROWS32, mx::Stream32Cfg<1>::WARPS, n, 32, 16,
+             max_t == 1 ? mx::Stream32Cfg<1>::smem_bytes(max_nb, n) : mx::Stream32Cfg<2>::smem_bytes(max_nb, n));
+    auto mma_smem = [&](int warps, int stages) {                             // (8: any cut)
+        return nt == 2 ? mx::MmaStreamCfg::smem_bytes<2>(max_nb / 4, warps, stages, 8) : mx::MmaStreamCfg::smem_bytes<1>(max_nb / 4, warps, stages, 8);
+    };
+    for (int warps = 16; warps >= 8; warps -= 8)
+        for (int n = mx::MmaStreamCfg::MAX_STAGES; n >= 2; --n) take(StreamPlan::MMA, warps, n, 16, 16, mma_smem(warps, n));
+    const bool tma = plan.kind != StreamPlan::REGS;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
 
     // quantize every distinct activation tensor once, build the device layer table
@@ -2016,7 +2230,7 @@ try {
     int64_t max_chunks = 0;
     std::vector<uint8_t *> act_ptr((size_t)n_layers, nullptr);
     std::unique_lock<std::mutex> map_lock(g_wmap_mu, std::defer_lock);
-    if (bulk) map_lock.lock();
+    if (tma) map_lock.lock();
     int total_tiles = 0;
     for (int i = 0; i < n_layers; ++i) {
         const mx_linear_args_t &a = layers[i];
@@ -2058,15 +2272,15 @@ try {
         L.w_rows2 = a.fw.block_rows == 2 ? 1 : 0;
         L.a_rows2 = a.fa.block_rows == 2 ? 1 : 0;
         L.tile_begin = total_tiles;
-        L.n_tiles = (int)(rows32 ? (a.N + 31) / 32 : (a.N + 15) / 16);
+        L.n_tiles = (int)((a.N + plan.rows - 1) / plan.rows);
         total_tiles += L.n_tiles;
-        if (bulk) {
-            s = packed_weight_maps(a.w_mant, a.w_exp, a.N, a.K, &tmaps[(size_t)i * 2]);
+        if (tma) {
+            s = packed_weight_maps(a.w_mant, a.w_exp, a.N, a.K / 2, plan.kind == StreamPlan::ROWS32 ? a.K / 32 : 0, &tmaps[(size_t)i * 2]);
             if (s != MX_OK) return s;
         }
     }
     // nothing is launched under the lock: a launch may wait for room in its stream, and other threads' calls with it
-    if (bulk) map_lock.unlock();
+    if (tma) map_lock.unlock();
     auto quantize_one = [&](const mx::QuantJob &q, int block_rows) {
         mx_format_t f{};
         f.block = q.block; f.elem_bits = q.w; f.exp_bits = 8; f.block_rows = block_rows;
@@ -2106,13 +2320,15 @@ try {
         MX_CUDA(cudaGetLastError());
     }
 
-    const int ctas_per_sm = (int)((227u * 1024u) / (smem + 1024)) < 4 ? (int)((227u * 1024u) / (smem + 1024)) : 4;
-    const int max_ctas = d->sm_count * (ctas_per_sm < 1 ? 1 : ctas_per_sm);
-    const int warps = rows32 ? mx::Stream32Cfg<1>::WARPS : bulk ? 16 : 8;
-    const int split = choose_split(total_tiles, (int64_t)max_ctas * warps, bulk ? 16 : 4);
-    const int tpr = warps / split;
+    const int fit = (int)(SMEM / (plan.smem + 1024));
+    const int ctas_per_sm = plan.kind == StreamPlan::MMA || fit < 1 ? 1 : fit < 4 ? fit : 4;
+    const int max_ctas = d->sm_count * ctas_per_sm;
+    int split = choose_split(total_tiles, (int64_t)max_ctas * plan.warps, plan.unit);
+    if (split == 1 && plan.kind == StreamPlan::MMA) split = choose_split(total_tiles, (int64_t)max_ctas * plan.warps, 4);
+    const int tpr = plan.warps / split;
     const int rounds = (total_tiles + tpr - 1) / tpr;
     const int grid = rounds < max_ctas ? rounds : max_ctas;
+    const int early = packed_exps ? 0 : 1;      // the launch in front is the quantizer above: weights may be fetched meanwhile
     sp.layers = reinterpret_cast<const mx::StreamLayer *>(ws);          // (unused by a call that brings them along)
     sp.n_layers = n_layers;
     sp.total_tiles = total_tiles;
@@ -2120,12 +2336,10 @@ try {
     sp.max_nb = max_nb;
     sp.status = d->status;
     sp.tmaps = reinterpret_cast<const CUtensorMap *>(ws + tmap_off);
-    if (in_params)
-        return rows32 ? launch_stream32(max_t, sp, stages, smem, grid, *d, st) : launch_stream(nt, bulk, sp, smem, grid, *d, st);
+    if (in_params) return launch_stream(plan, max_t, early, sp, grid, *d, st);
     mx::StreamTableParams tp;
     static_cast<mx::StreamParams &>(tp) = sp;
-    if (rows32) return launch_stream32(max_t, tp, stages, smem, grid, *d, st);
-    return launch_stream(nt, bulk, tp, smem, grid, *d, st);
+    return launch_stream(plan, max_t, early, tp, grid, *d, st);
 } catch (const std::bad_alloc &) {                      // (the tables of the call are kept in host memory)
     snprintf(t_cuda_error, sizeof(t_cuda_error), "grouped call: out of host memory for the tables of %d layers", (int)n_layers);
     return MX_ERR_CUDA;
