@@ -23,6 +23,7 @@
 #include "mx_gemm_tc2.cuh"
 #include "mx_gemm_rec.cuh"
 #include "mx_gemm_tc8.cuh"
+#include "mx_gemm_tcw.cuh"
 #include "mx_gemm_tcx.cuh"
 #include "mx_gemv_mma.cuh"
 #include "mx_gemv_stream.cuh"
@@ -52,6 +53,7 @@ struct DeviceInfo {
     int gemv_clusters[12][4][2] = {};          // resident clusters by kernel, log2 of the cluster size, two CTAs per SM
     bool stream32_attr_set[2][2] = {};
     bool tc2_attr_set[2] = {false, false};
+    bool tcw_attr_set[4] = {};
     bool tcx_attr_set = false;
     bool tc8_attr_set = false;
     bool rec_attr_set[4] = {};
@@ -588,6 +590,56 @@ mx_status_t launch_tc2(const __nv_bfloat16 *a_hat, const __nv_bfloat16 *w_hat, i
     return MX_OK;
 }
 
+// CTA pairs with 256 x width tiles (mx_gemm_tcw.cuh).
+mx_status_t launch_tcw(const __nv_bfloat16 *a_hat, const __nv_bfloat16 *w_hat, int64_t M, int64_t N, int64_t K, int width,
+                       const float *bias, float *y, int64_t ldy, const QuantizedOut *yq, DeviceInfo &d, cudaStream_t st,
+                       const EpiTail &et)
+{
+    using Cfg = mx::TcwCfg;
+    CUtensorMap tm_a, tm_w;
+    mx_status_t s = encode_bf16_rows(&tm_a, a_hat, M, K, mx::TC_BM);
+    if (s != MX_OK) return s;
+    s = encode_bf16_rows(&tm_w, w_hat, N, K, width / 4);
+    if (s != MX_OK) return s;
+    const bool tail = et.any(), q = yq != nullptr;
+    typedef void (*Kernel)(CUtensorMap, CUtensorMap, mx::TcParams, int, int);
+    static const Kernel kernels[4] = {mx::gemm_tcw_kernel<false, false>, mx::gemm_tcw_kernel<false, true>,
+                                      mx::gemm_tcw_kernel<true, false>, mx::gemm_tcw_kernel<true, true>};
+    const int which = (tail ? 2 : 0) + (q ? 1 : 0);
+    s = smem_attr_once(d.tcw_attr_set[which], kernels[which], 227 * 1024);
+    if (s != MX_OK) return s;
+    int stages = Cfg::MAX_STAGES;
+    while (Cfg::smem_bytes(width, stages) > 227u * 1024u) --stages;
+    mx::TcParams p{};
+    p.y = y;
+    p.bias = tail ? nullptr : bias;
+    p.ex_bias = tail ? bias : nullptr;
+    p.relu = et.relu;
+    p.residual = et.residual;
+    p.ldr = et.ldr;
+    p.ldy = ldy;
+    p.M = (int)M;
+    p.N = (int)N;
+    p.K = (int)K;
+    p.tiles_m = (int)((M + 255) / 256);
+    p.tiles_n = (int)((N + width - 1) / width);
+    p.status = d.status;
+    p.frag_store = frag_store_ok(q, false, y, ldy, 0) ? 1 : 0;
+    p.batch = 1;
+    p.yq_mant = yq ? yq->mant : nullptr;
+    p.yq_exp = yq ? yq->exps : nullptr;
+    p.yq_nonfinite = yq ? yq->nonfinite : nullptr;
+    p.yq_bits = yq ? yq->f.elem_bits : 0;
+    p.yq_block = yq ? yq->f.block : 0;
+    p.yq_rows2 = yq && yq->f.block_rows == 2 ? 1 : 0;
+    const int tiles = p.tiles_m * p.tiles_n;
+    const int pairs = tiles < d.sm_count / 2 ? tiles : d.sm_count / 2;
+    ProfScope prof(KIND_GEMM_TC, st);
+    MX_CUDA(launch_dep(kernels[which], dim3(2 * pairs), dim3(Cfg::THREADS), Cfg::smem_bytes(width, stages), st, tm_a, tm_w, p, width, stages));
+    MX_CUDA(cudaGetLastError());
+    return MX_OK;
+}
+
 // The block-wise kernel (one tensor-memory accumulator per block, blocks added in fp32 registers):
 // 128 x 128 tiles, fp32 result, one product per launch.
 mx_status_t launch_tcx(const __nv_bfloat16 *a_hat, const __nv_bfloat16 *w_hat, int64_t M, int64_t N, int64_t K,
@@ -1058,6 +1110,30 @@ mx_status_t launch_splitk(const __nv_bfloat16 *a_hat, const __nv_bfloat16 *w_hat
     return MX_OK;
 }
 
+// Width of the pair tiles where one wider than 256 columns fills the chip's pairs in so many fewer rounds that it is the faster
+// one, else 0.  A round of 256 x 256 tiles takes about 5.8 ns per k, its epilogue under the next round's MMAs; a wide one takes
+// 0.9 of that per column -- no less than for 384 columns, whose A operand alone keeps the loads busy -- and its epilogue is
+// exposed.  Products, 256 / wide (us): 512 x 11008 x 4096 61.1 / 45.0 (320: 70 tiles on 74 pairs for 86 in two rounds),
+// 2048 x 4096 x 16384 177 / 165 (480: 72 for 128), 4096 x 4096 x 11008 259 / 227, 384 x 16384 x 8192 102 / 89, 768 x 8192 x 2048
+// 33.2 / 29.6; even or worse, and left alone: 2048 x 4096 x 4096 54.4 / 54.7, 2048 x 12288 x 4096 141 / 145,
+// 4096 x 11008 x 4096 228 / 258 (five exposed epilogues of 38 MB).
+int wide_pair_tile(int64_t M, int64_t N, int64_t K, const DeviceInfo &d)
+{
+    const int64_t rows = (M + 255) / 256, pairs = d.sm_count / 2;
+    auto rounds = [&](int64_t w) { return (rows * ((N + w - 1) / w) + pairs - 1) / pairs; };
+    const int64_t tile_ns = K * 29 / 5;
+    int64_t best = (6000 + rounds(256) * tile_ns) * 93 / 100;
+    int width = 0;
+    for (int w = 288; w <= mx::TcwCfg::MAX_W; w += 32) {
+        const int64_t ns = 2000 + rounds(w) * (tile_ns * (w > 384 ? w : 384) * 9 / 2560 + w * 75 / 4);
+        if (ns < best) {
+            best = ns;
+            width = w;
+        }
+    }
+    return width;
+}
+
 // Pre-decoded bf16 weights (both operands fetched by TMA).  may_split: K may be cut (the sum is then not one chain).
 mx_status_t run_tc(const __nv_bfloat16 *a_hat, const __nv_bfloat16 *w_hat, int64_t M, int64_t N,
                    int64_t K, const float *bias, float *y, int64_t ldy, DeviceInfo &d, cudaStream_t st,
@@ -1075,8 +1151,11 @@ mx_status_t run_tc(const __nv_bfloat16 *a_hat, const __nv_bfloat16 *w_hat, int64
     const int64_t tiles128 = panels * ((N + 127) / 128) * tb.count, tiles256 = panels * ((N + 255) / 256) * tb.count;
     const int pairs = d.sm_count / 2;
     const bool long_wave = K >= 4096 && pair_tiles <= pairs && 4 * pair_tiles >= 3 * pairs && (panels & 1) == 0;
-    if (tb.count == 1 && M > 128 && (tiles256 > d.sm_count || long_wave))
+    if (tb.count == 1 && M > 128 && (tiles256 > d.sm_count || long_wave)) {
+        const int width = wide_pair_tile(M, N, K, d);
+        if (width) return launch_tcw(a_hat, w_hat, M, N, K, width, bias, y, ldy, yq, d, st, et);
         return launch_tc2(a_hat, w_hat, M, N, K, bias, y, ldy, yq, d, st, et);
+    }
     if (may_split && tb.count == 1) {
         int split = 0;
         const mx_status_t s = splitk_ways(M, N, K, d, &split);
