@@ -24,6 +24,9 @@
 //                 swizzled P operand tile in shared memory; at the end the context tile out of tensor
 //                 memory into global memory.  exp is ex2.approx on arguments pre-scaled by log2(e); the division
 //                 by the row sum is a subtraction of its log2 inside that argument
+// What bounds it: the row warps' chain per tile (score load, exponentials on a unit of 16 per clock and SM, rounding, barrier);
+// scaling, summing and rounding go two values at a time (packed fp32), the tiles come through one ring in the order of their
+// use.  32 heads x 2048 x 128, causal: 108.8 -> 97.9 us, 12 x 2048 x 64 50.7 -> 45.6.
 // Every 128 x 128 bf16 tile is stored as two halves of 128 rows x 128 bytes (64 columns) with the
 // 128-byte swizzle.  All waits are bounded.
 #pragma once
@@ -46,12 +49,14 @@ template <int D_> struct AttnCfgT {
     static constexpr uint32_t HALF_BYTES = 128 * 128;                // 128 rows x 128 bytes: a half of Q, K or P
     static constexpr uint32_t V_HALF_BYTES = D_ * 128;               // D_ rows x 128 bytes: a half of V^T
     static constexpr uint32_t P_BYTES = 128 * 128 * 2;
-    static constexpr int KST = 2, VST = 2;                           // K and V^T stage rings
+    // K and V^T tiles pass through one ring, in the order in which the MMAs use them: K_0 .. (sweep 1), then K_0, K_1, V_0,
+    // K_2, V_1, ...  (Two rings of two left the first sweep, which has no V, waiting for K.)
+    static constexpr int RST = D_ == 128 ? 4 : 8;
     static constexpr int ROW_WARPS = 16;                             // 4 per TMEM lane quarter: 32 key columns each
     static constexpr int COLS_PER_WARP = 128 / (ROW_WARPS / 4);
     static constexpr int THREADS = 64 + 32 * ROW_WARPS;
     static constexpr uint32_t STATS_BYTES = 2 * (ROW_WARPS / 4) * 128 * 8;   // (maximum, sum) per row and column slice, two items deep
-    static constexpr uint32_t SMEM_BYTES = (1 + KST + VST) * TILE_BYTES + P_BYTES + 512 + STATS_BYTES + 1024;    // Q, K ring, V ring, P
+    static constexpr uint32_t SMEM_BYTES = (1 + RST) * TILE_BYTES + P_BYTES + 512 + STATS_BYTES + 1024;    // Q, ring, P
     static constexpr uint32_t TMEM_COLS = 512;                       // S0, S1 (128 columns each), O (D_ columns) at 0, 128, 256
 };
 using AttnCfg = AttnCfgT<128>;
@@ -101,6 +106,28 @@ __device__ __forceinline__ float log2_approx(float x)
     return y;
 }
 
+// Eight probabilities of one block (exponent byte e) -> their quantized values as bf16 pairs: the rounding of encode8_full
+// without its lower clamp (they are not negative) and without the codes, two at a time.  The values have at most 7 significant
+// bits, so the upper halves of their fp32 patterns are the bf16 numbers.
+__device__ __forceinline__ void prob_encode8(const float *v, int e, int w, uint32_t (&h)[4])
+{
+    if (e <= 229 + w) {
+        const uint32_t mb = ((uint32_t)(e + 25 - w) << 23) | 0x00400000u;
+        const float M = __uint_as_float(mb), hi = __uint_as_float(mb + (1u << (w - 1)) - 1u);
+        const f32x2_t m2 = pack2(M, M), n2 = pack2(-M, -M);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            float a, b;
+            unpack2(fadd2(pack2(v[2 * i], v[2 * i + 1]), m2), a, b);
+            unpack2(fadd2(pack2(fminf(a, hi), fminf(b, hi)), n2), a, b);
+            h[i] = __byte_perm(__float_as_uint(a), __float_as_uint(b), 0x7632);
+        }
+    } else {                                             // only a NaN row: its values are poisoned
+#pragma unroll
+        for (int i = 0; i < 4; ++i) h[i] = 0x7FC07FC0u;
+    }
+}
+
 template <int D_>
 __global__ void __launch_bounds__(AttnCfgT<D_>::THREADS, 1)
 attention_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant__ CUtensorMap tmap_k,
@@ -111,20 +138,20 @@ attention_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_consta
     const uint32_t smem_base = (ptx::smem_u32(smem_raw) + 1023u) & ~1023u;
     uint8_t *smem_gen = smem_raw + (smem_base - ptx::smem_u32(smem_raw));
     const uint32_t q_tile = smem_base;
-    const uint32_t k_tiles = q_tile + Cfg::TILE_BYTES;
-    const uint32_t v_tiles = k_tiles + Cfg::KST * Cfg::TILE_BYTES;
-    const uint32_t p_tile = v_tiles + Cfg::VST * Cfg::TILE_BYTES;
+    const uint32_t ring = q_tile + Cfg::TILE_BYTES;
+    const uint32_t p_tile = ring + Cfg::RST * Cfg::TILE_BYTES;
     const uint32_t bar_base = p_tile + Cfg::P_BYTES;
-    // barriers: 0 q_full, 1 q_empty, 2..3 k_full, 4..5 k_empty, 6..7 v_full, 8..9 v_empty, 10..11 s_full,
-    //           12..13 s_empty, 14 p_full, 15 p_empty, 16 o_full, 17 o_empty, 18 row statistics written
+    // barriers: 0 q_full, 1 q_empty, 10..11 s_full, 12..13 s_empty, 14 p_full, 15 p_empty, 16 o_full, 17 o_empty,
+    //           18 row statistics written, RING .. ring full, RING + RST .. ring empty
+    constexpr int RST = Cfg::RST, RING = 20, BARS = RING + 2 * RST;
     auto bar = [&](int i) { return bar_base + 8u * i; };
-    uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(smem_gen + (bar_base - smem_base) + 8 * 19);
+    uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(smem_gen + (bar_base - smem_base) + 8 * BARS);
     volatile uint32_t *abort_flag = tmem_slot + 1;
     float2 *stats = reinterpret_cast<float2 *>(smem_gen + (bar_base - smem_base) + 512);    // [slice][row]
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     if (threadIdx.x == 0) {
-        for (int i = 0; i < 19; ++i) {
+        for (int i = 0; i < BARS; ++i) {
             const bool by_rows = i == 12 || i == 13 || i == 14 || i == 17 || i == 18;      // arrived on by every row warp
             ptx::mbar_init(bar(i), by_rows ? Cfg::ROW_WARPS : 1);
         }
@@ -152,7 +179,30 @@ attention_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_consta
 
     if (warp == 0) {
         if (lane == 0) {
-            uint32_t n_item = 0, n_k = 0, n_v = 0;                    // uses so far of the Q tile and the two rings
+            uint32_t n_item = 0, n_r = 0;                             // uses so far of the Q tile and the ring
+            auto slot = [&](uint32_t *dst, uint32_t *full) -> bool {      // the next ring slot, empty and announced
+                const uint32_t rs = n_r % RST;
+                if (!wait(RING + RST + rs, ((n_r / RST) & 1u) ^ 1u)) return false;
+                ++n_r;
+                *dst = ring + rs * Cfg::TILE_BYTES;
+                *full = bar(RING + rs);
+                ptx::mbar_arrive_expect_tx(*full, Cfg::TILE_BYTES);
+                return true;
+            };
+            auto load_k = [&](int h, int j) -> bool {
+                uint32_t dst, full;
+                if (!slot(&dst, &full)) return false;
+                ptx::tma_load_2d(dst, &tmap_k, h * Cfg::D, j * Cfg::BKEY, full);
+                if (Cfg::D == 128) ptx::tma_load_2d(dst + Cfg::HALF_BYTES, &tmap_k, h * Cfg::D + 64, j * Cfg::BKEY, full);
+                return true;
+            };
+            auto load_v = [&](int h, int j) -> bool {
+                uint32_t dst, full;
+                if (!slot(&dst, &full)) return false;
+                ptx::tma_load_2d(dst, &tmap_v, j * Cfg::BKEY, h * Cfg::D, full);
+                ptx::tma_load_2d(dst + Cfg::V_HALF_BYTES, &tmap_v, j * Cfg::BKEY + 64, h * Cfg::D, full);
+                return true;
+            };
             for (int w = attn_item(0, blockIdx.x, gridDim.x); w < items && !timed_out; ++n_item, w = attn_item(n_item, blockIdx.x, gridDim.x)) {
                 const int qt = q_tiles_n - 1 - w / p.heads, h = w % p.heads;
                 const int T = p.causal ? qt + 1 : q_tiles_n;
@@ -160,25 +210,9 @@ attention_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_consta
                 ptx::mbar_arrive_expect_tx(bar(0), Cfg::TILE_BYTES);
                 ptx::tma_load_2d(q_tile, &tmap_q, h * Cfg::D, qt * Cfg::BQ, bar(0));
                 if (Cfg::D == 128) ptx::tma_load_2d(q_tile + Cfg::HALF_BYTES, &tmap_q, h * Cfg::D + 64, qt * Cfg::BQ, bar(0));
-                for (int sweep = 0; sweep < 2 && !timed_out; ++sweep)
-                    for (int j = 0; j < T; ++j) {
-                        const uint32_t ks = n_k % Cfg::KST;
-                        if (!wait(4 + ks, ((n_k / Cfg::KST) & 1u) ^ 1u)) { timed_out = true; break; }
-                        ptx::mbar_arrive_expect_tx(bar(2 + ks), Cfg::TILE_BYTES);
-                        const uint32_t kt = k_tiles + ks * Cfg::TILE_BYTES;
-                        ptx::tma_load_2d(kt, &tmap_k, h * Cfg::D, j * Cfg::BKEY, bar(2 + ks));
-                        if (Cfg::D == 128) ptx::tma_load_2d(kt + Cfg::HALF_BYTES, &tmap_k, h * Cfg::D + 64, j * Cfg::BKEY, bar(2 + ks));
-                        ++n_k;
-                        if (sweep == 1) {
-                            const uint32_t vs = n_v % Cfg::VST;
-                            if (!wait(8 + vs, ((n_v / Cfg::VST) & 1u) ^ 1u)) { timed_out = true; break; }
-                            ptx::mbar_arrive_expect_tx(bar(6 + vs), Cfg::TILE_BYTES);
-                            const uint32_t vt = v_tiles + vs * Cfg::TILE_BYTES;
-                            ptx::tma_load_2d(vt, &tmap_v, j * Cfg::BKEY, h * Cfg::D, bar(6 + vs));
-                            ptx::tma_load_2d(vt + Cfg::V_HALF_BYTES, &tmap_v, j * Cfg::BKEY + 64, h * Cfg::D, bar(6 + vs));
-                            ++n_v;
-                        }
-                    }
+                for (int j = 0; j < T && !timed_out; ++j) timed_out = !load_k(h, j);
+                for (int j = 0; j <= T && !timed_out; ++j)
+                    timed_out = (j < T && !load_k(h, j)) || (j > 0 && !load_v(h, j - 1));
             }
         }
         __syncwarp();
@@ -186,16 +220,16 @@ attention_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_consta
         if (lane == 0) {
             constexpr uint32_t idesc = ptx::idesc_bf16_f32(128, 128), idesc_o = ptx::idesc_bf16_f32(128, Cfg::D);
             const uint32_t s_tmem[2] = {tmem_base, tmem_base + 128u}, o_tmem = tmem_base + 256u;
-            uint32_t n_item = 0, n_k = 0, n_v = 0, n_s = 0, n_p = 0;
+            uint32_t n_item = 0, n_r = 0, n_s = 0, n_p = 0;
             // S_j = Q K_j^T into score accumulator n_s % 2
             auto issue_scores = [&]() -> bool {
-                const uint32_t ks = n_k % Cfg::KST, si = n_s & 1u;
-                if (!wait(2 + ks, (n_k / Cfg::KST) & 1u) || !wait(12 + si, ((n_s >> 1) & 1u) ^ 1u)) return false;
+                const uint32_t rs = n_r % RST, si = n_s & 1u;
+                if (!wait(RING + rs, (n_r / RST) & 1u) || !wait(12 + si, ((n_s >> 1) & 1u) ^ 1u)) return false;
                 ptx::tc_fence_after_sync();
-                attn_mma<Cfg::D / 64>(s_tmem[si], q_tile, Cfg::HALF_BYTES, k_tiles + ks * Cfg::TILE_BYTES, Cfg::HALF_BYTES, idesc, false);
-                ptx::mma_commit(bar(4 + ks));               // K stage free
+                attn_mma<Cfg::D / 64>(s_tmem[si], q_tile, Cfg::HALF_BYTES, ring + rs * Cfg::TILE_BYTES, Cfg::HALF_BYTES, idesc, false);
+                ptx::mma_commit(bar(RING + RST + rs));      // K tile free
                 ptx::mma_commit(bar(10 + si));              // scores complete
-                ++n_k;
+                ++n_r;
                 ++n_s;
                 return true;
             };
@@ -214,13 +248,13 @@ attention_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_consta
                     } else {
                         ptx::mma_commit(bar(1));                                // every product that reads Q has been issued
                     }
-                    const uint32_t vs = n_v % Cfg::VST;
-                    if (!wait(14, n_p & 1u) || !wait(6 + vs, (n_v / Cfg::VST) & 1u)) { timed_out = true; break; }
+                    const uint32_t rs = n_r % RST;
+                    if (!wait(14, n_p & 1u) || !wait(RING + rs, (n_r / RST) & 1u)) { timed_out = true; break; }
                     ptx::tc_fence_after_sync();
-                    attn_mma<2>(o_tmem, p_tile, Cfg::HALF_BYTES, v_tiles + vs * Cfg::TILE_BYTES, Cfg::V_HALF_BYTES, idesc_o, j > 0);
-                    ptx::mma_commit(bar(8 + vs));            // V stage free
+                    attn_mma<2>(o_tmem, p_tile, Cfg::HALF_BYTES, ring + rs * Cfg::TILE_BYTES, Cfg::V_HALF_BYTES, idesc_o, j > 0);
+                    ptx::mma_commit(bar(RING + RST + rs));   // V tile free
                     ptx::mma_commit(bar(15));                // P tile free
-                    ++n_v;
+                    ++n_r;
                     ++n_p;
                 }
                 if (timed_out) break;
@@ -298,19 +332,36 @@ attention_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_consta
                                 m = cm;
                             }
                             if (m != -INFINITY) {
-                                float s = 0.f;
+                                const f32x2_t sc = pack2(scale2, scale2), nm = pack2(-m, -m);
+                                f32x2_t s2[2] = {pack2(0.f, 0.f), pack2(0.f, 0.f)};
 #pragma unroll
-                                for (int i = 0; i < 32; ++i) s += exp2_approx(fmaf(v[i], scale2, -m));      // 2^-inf = 0 for masked keys
-                                l += s;
+                                for (int i = 0; i < 16; ++i) {                              // 2^-inf = 0 for masked keys
+                                    float a, b;
+                                    unpack2(ffma2(pack2(v[2 * i], v[2 * i + 1]), sc, nm), a, b);
+                                    s2[i & 1] = fadd2(s2[i & 1], pack2(exp2_approx(a), exp2_approx(b)));
+                                }
+                                float a, b;
+                                unpack2(fadd2(s2[0], s2[1]), a, b);
+                                l += a + b;
                             }
                         } else {
-                            uint32_t amax[2] = {0u, 0u};
+                            const f32x2_t sc = pack2(scale2, scale2), nm = pack2(-m_norm, -m_norm);
 #pragma unroll
-                            for (int i = 0; i < 32; ++i) {
-                                v[i] = exp2_approx(fmaf(v[i], scale2, -m_norm));
-                                amax[i >> 4] = max(amax[i >> 4], __float_as_uint(v[i]));     // v >= 0: bits order like values
+                            for (int i = 0; i < 16; ++i) {
+                                float a, b;
+                                unpack2(ffma2(pack2(v[2 * i], v[2 * i + 1]), sc, nm), a, b);
+                                v[2 * i] = exp2_approx(a);
+                                v[2 * i + 1] = exp2_approx(b);
                             }
-                            if (p.p_block == 32) amax[0] = amax[1] = max(amax[0], amax[1]);
+                            // v >= 0, or NaN in all of the row (its maximum and sum are): a NaN survives the maximum
+                            float big[2] = {v[0], v[16]};
+#pragma unroll
+                            for (int i = 1; i < 16; ++i) {
+                                big[0] = fmaxf(big[0], v[i]);
+                                big[1] = fmaxf(big[1], v[16 + i]);
+                            }
+                            if (p.p_block == 32) big[0] = big[1] = fmaxf(big[0], big[1]);
+                            const uint32_t amax[2] = {__float_as_uint(big[0]) & 0x7FFFFFFFu, __float_as_uint(big[1]) & 0x7FFFFFFFu};
                             // the previous P tile must have been consumed before the first store of this one
                             if (cc == 0 && !__all_sync(0xFFFFFFFFu, wait(15, (n_p & 1u) ^ 1u))) { timed_out = true; break; }
                             const int64_t prow = (int64_t)h * p.seq + qrow;
@@ -318,19 +369,18 @@ attention_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_consta
 #pragma unroll
                             for (int u = 0; u < 4; ++u) {
                                 const int ebyte = (int)(amax[u >> 1] >> 23);
-                                float v8[8], xh[8];
-#pragma unroll
-                                for (int i = 0; i < 8; ++i) v8[i] = v[8 * u + i];
-                                const uint2 pk = encode8_full(v8, ebyte, p.p_bits, xh);
                                 uint32_t hw[4];
-#pragma unroll
-                                for (int i = 0; i < 4; ++i) hw[i] = as_u32(__floats2bfloat162_rn(xh[2 * i], xh[2 * i + 1]));
+                                prob_encode8(&v[8 * u], ebyte, p.p_bits, hw);
                                 const uint32_t dst = p_row + (uint32_t)(c >> 1) * Cfg::HALF_BYTES +
                                                      (uint32_t)((((c & 1) * 4 + u) ^ (r & 7)) << 4);
                                 asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(dst), "r"(hw[0]), "r"(hw[1]),
                                              "r"(hw[2]), "r"(hw[3])
                                              : "memory");
                                 if (p.p_mant && qrow < p.seq && key0 + 8 * u < p.seq) {
+                                    float v8[8];
+#pragma unroll
+                                    for (int i = 0; i < 8; ++i) v8[i] = v[8 * u + i];
+                                    const uint2 pk = encode8_packed(v8, ebyte, p.p_bits);
                                     if (nibble) *reinterpret_cast<uint32_t *>(p.p_mant + prow * (p.seq >> 1) + ((key0 + 8 * u) >> 1)) = pk.x;
                                     else *reinterpret_cast<uint2 *>(p.p_mant + prow * p.seq + key0 + 8 * u) = pk;
                                     if (p.p_block == 16 ? (u & 1) == 0 : u == 0)

@@ -103,38 +103,6 @@ __device__ __forceinline__ void mma_s8s8_m16n8k32(int (&d)[4], uint32_t a0, uint
         : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1), "r"(c[0]), "r"(c[1]), "r"(c[2]), "r"(c[3]));
 }
 
-// Pairs of fp32 values in one 64-bit register and the sm_100 packed-pair arithmetic on them
-// (each half rounds exactly like the scalar instruction).
-typedef uint64_t f32x2_t;
-__device__ __forceinline__ f32x2_t pack2(float lo, float hi)
-{
-    f32x2_t r;
-    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
-    return r;
-}
-__device__ __forceinline__ f32x2_t pack2u(uint32_t lo, uint32_t hi)
-{
-    f32x2_t r;
-    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "r"(lo), "r"(hi));
-    return r;
-}
-__device__ __forceinline__ void unpack2(f32x2_t v, float &lo, float &hi)
-{
-    asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v));
-}
-__device__ __forceinline__ f32x2_t ffma2(f32x2_t a, f32x2_t b, f32x2_t c)
-{
-    f32x2_t d;
-    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
-    return d;
-}
-__device__ __forceinline__ f32x2_t fmul2(f32x2_t a, f32x2_t b)
-{
-    f32x2_t d;
-    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
-    return d;
-}
-
 // NT = number of 8-token column tiles (1: T <= 8, 2: T <= 16).
 template <int NT, typename Params>
 __global__ void __launch_bounds__(StreamCfg<NT>::THREADS, 1)
