@@ -167,8 +167,77 @@ __device__ __forceinline__ void tail_apply(const TcParams &p, const TailRegs &t,
 // row `row`, i.e. one block of 32 or two blocks of 16 along N; no exchange between lanes is needed.
 // Adds the bias, derives the exponent byte(s), rounds like the quantizer and stores 16 or 32
 // mantissa bytes and one or two exponent bytes.
+// Chunks inside the matrix with one-row blocks whose exponents leave the rounding constant finite in every lane (all but the
+// last columns, the top of the range and non-finite blocks): no predicates per element, whole sectors.
+template <int BLOCK>
+__device__ __forceinline__ bool store_mxint_whole(const TcParams &p, int row, int n, const float (&x)[32])
+{
+    float big[2] = {0.f, 0.f};
+#pragma unroll
+    for (int v = 0; v < 16; ++v) {
+        big[0] = absmax_nan(big[0], x[v]);
+        big[1] = absmax_nan(big[1], x[16 + v]);
+    }
+    if (BLOCK == 32) big[0] = big[1] = absmax_nan(big[0], big[1]);
+    const int e0 = (int)(__float_as_uint(big[0]) >> 23), e1 = (int)(__float_as_uint(big[1]) >> 23), w = p.yq_bits;
+    if (!__all_sync(0xFFFFFFFFu, max(e0, e1) <= 229 + w)) return false;
+    uint32_t c[8];                           // the codes as bytes: x + M has q in the low bits of its pattern (see encode8_full)
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        const uint32_t mb = ((uint32_t)((h ? e1 : e0) + 25 - w) << 23) | 0x00400000u, qmax = (1u << (w - 1)) - 1u;
+        const float M = __uint_as_float(mb), lo = __uint_as_float(mb - qmax), hi = __uint_as_float(mb + qmax);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            uint32_t f[4];
+#pragma unroll
+            for (int j = 0; j < 4; ++j) f[j] = __float_as_uint(fminf(fmaxf(x[16 * h + 4 * i + j] + M, lo), hi));
+            c[4 * h + i] = __byte_perm(__byte_perm(f[0], f[1], 0x0040), __byte_perm(f[2], f[3], 0x0040), 0x5410);
+        }
+    }
+    if (row >= p.M) return true;
+    if (w <= 4) {
+        uint32_t q[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {        // bytes k, k + 1 of a pair become one
+            const uint32_t a = __byte_perm(c[2 * i], c[2 * i + 1], 0x6420), b = __byte_perm(c[2 * i], c[2 * i + 1], 0x7531);
+            q[i] = (a & 0x0F0F0F0Fu) | ((b << 4) & 0xF0F0F0F0u);
+        }
+        uint8_t *dst = p.yq_mant + (int64_t)row * (p.N >> 1) + (n >> 1);
+        if ((p.N & 31) == 0) {
+            *reinterpret_cast<uint4 *>(dst) = make_uint4(q[0], q[1], q[2], q[3]);
+        } else {
+            reinterpret_cast<uint2 *>(dst)[0] = make_uint2(q[0], q[1]);
+            reinterpret_cast<uint2 *>(dst)[1] = make_uint2(q[2], q[3]);
+        }
+    } else {
+        uint8_t *dst = p.yq_mant + (int64_t)row * p.N + n;
+        const uint32_t a[4] = {c[0], c[1], c[2], c[3]}, b[4] = {c[4], c[5], c[6], c[7]};
+        if ((p.N & 31) == 0 && (reinterpret_cast<uintptr_t>(p.yq_mant) & 31u) == 0) {
+            store32(dst, a, b);
+        } else {
+            reinterpret_cast<uint4 *>(dst)[0] = make_uint4(a[0], a[1], a[2], a[3]);
+            reinterpret_cast<uint4 *>(dst)[1] = make_uint4(b[0], b[1], b[2], b[3]);
+        }
+    }
+    uint8_t *de = p.yq_exp + (int64_t)row * (p.N / BLOCK) + n / BLOCK;
+    de[0] = (uint8_t)e0;
+    if (BLOCK == 16) de[1] = (uint8_t)e1;
+    return true;
+}
+
 __device__ __forceinline__ void store_mxint_chunk(const TcParams &p, int row, int n, uint32_t (&r)[32])
 {
+    if (n + 32 <= p.N && !p.yq_rows2) {                    // warp-uniform
+        float x[32];
+#pragma unroll
+        for (int v = 0; v < 8; ++v) {
+            float4 b = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (p.bias) b = __ldg(reinterpret_cast<const float4 *>(p.bias + n) + v);
+            x[4 * v] = __uint_as_float(r[4 * v]) + b.x; x[4 * v + 1] = __uint_as_float(r[4 * v + 1]) + b.y;
+            x[4 * v + 2] = __uint_as_float(r[4 * v + 2]) + b.z; x[4 * v + 3] = __uint_as_float(r[4 * v + 3]) + b.w;
+        }
+        if (p.yq_block == 16 ? store_mxint_whole<16>(p, row, n, x) : store_mxint_whole<32>(p, row, n, x)) return;
+    }
     // every lane of the warp runs the shuffle below; lanes outside the matrix contribute zeros
     const bool live = row < p.M && n < p.N;
     const int64_t nb_row = p.N / p.yq_block;
