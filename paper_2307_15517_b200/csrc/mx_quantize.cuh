@@ -129,6 +129,14 @@ struct QuantOut {
                           // 0,4,1,5,2,6,3,7 (the operand order of the W_NIBBLE_PERM product kernel)
 };
 
+// A pass of two lists deals the second one on from where the first ends: number of warp `wid` of `nw` in the second list after
+// `items` of the first (the warps that had one item less come first).
+__device__ __forceinline__ uint32_t after_items(uint32_t wid, uint32_t nw, uint32_t items)
+{
+    const uint32_t rem = items % nw;
+    return wid >= rem ? wid - rem : wid + nw - rem;
+}
+
 template <typename InT> struct Load8;
 template <> struct Load8<float> {
     static __device__ __forceinline__ void run(const float *p, float (&v)[8])
@@ -642,12 +650,13 @@ attention_operands_kernel(const AttnOperandsJob j)
     const int warps = blockDim.x >> 5;
     const int64_t wid = (int64_t)blockIdx.x * warps + (threadIdx.x >> 5), nw = (int64_t)gridDim.x * warps;
     const QuantOut oq{nullptr, nullptr, j.q_hat, j.hid, nullptr, 0}, ok{nullptr, nullptr, j.k_hat, j.hid, nullptr, 0};
+    const int64_t wk = after_items((uint32_t)wid, (uint32_t)nw, (uint32_t)(j.seq * ((j.hid + 255) >> 8)));
     if (j.block_qk == 16) {
         quantize_rows_body<InT, 16, 2>(static_cast<const InT *>(j.q), j.seq, j.hid, j.ldq, j.w_qk, oq, wid, nw);
-        quantize_rows_body<InT, 16, 2>(static_cast<const InT *>(j.k), j.seq, j.hid, j.ldk, j.w_qk, ok, wid, nw);
+        quantize_rows_body<InT, 16, 2>(static_cast<const InT *>(j.k), j.seq, j.hid, j.ldk, j.w_qk, ok, wk, nw);
     } else {
         quantize_rows_body<InT, 32, 2>(static_cast<const InT *>(j.q), j.seq, j.hid, j.ldq, j.w_qk, oq, wid, nw);
-        quantize_rows_body<InT, 32, 2>(static_cast<const InT *>(j.k), j.seq, j.hid, j.ldk, j.w_qk, ok, wid, nw);
+        quantize_rows_body<InT, 32, 2>(static_cast<const InT *>(j.k), j.seq, j.hid, j.ldk, j.w_qk, ok, wk, nw);
     }
     const QuantOut ov{nullptr, nullptr, j.v_hat, j.seq, nullptr, 0};
     quantize_transposed_body<InT>(tile, static_cast<const InT *>(j.v), j.hid, j.seq, j.ldv, j.block_v, j.w_v, ov,
@@ -891,6 +900,8 @@ decode_bf16_kernel(const uint8_t *__restrict__ mant, const uint8_t *__restrict__
 
 // Both packed operands of a product -> their bf16 operand forms in one launch: every warp takes its share of the
 // rows of A, then of W (the product that follows needs both; two launches would each pay their own ramp and tail).
+// Bound by HBM and L2 writes.  Three CTAs per SM in one wave: with 112 registers (int8 items two at a time) two fitted and the
+// grid, sized for the nibble kernel, made one and a half waves (2048 x 16384 in 8 bits and 4096 x 16384 in 4: 63.8 -> 43.8 us).
 struct DecodePairJob {
     const uint8_t *a_mant, *a_exp, *w_mant, *w_exp;
     int64_t M, N, K;
@@ -899,7 +910,7 @@ struct DecodePairJob {
 };
 
 template <bool NIB_A, bool NIB_W>
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(256, 3)
 decode_pair_kernel(const DecodePairJob j)
 {
     ptx::dep_wait();
@@ -913,8 +924,14 @@ decode_pair_kernel(const DecodePairJob j)
     pw.mant_ld = NIB_W ? j.K / 2 : j.K;
     pa.exp_row_shift = j.a_row_shift;
     pw.exp_row_shift = j.w_row_shift;
-    decode_bf16_body<NIB_A, 2>(j.a_mant, j.a_exp, j.M, j.K, j.block, j.wa, j.a_hat, j.K, pa, wid, nw);
-    decode_bf16_body<NIB_W, 2>(j.w_mant, j.w_exp, j.N, j.K, j.block, j.ww, j.w_hat, j.K, pw, wid, nw);
+    // the weights' items are dealt on from where the first operand's end; their first ones are on their way meanwhile
+    const int64_t ww = after_items((uint32_t)wid, (uint32_t)nw, (uint32_t)(j.M * (((j.K >> 5) + 31) >> 5)));
+    constexpr int UA = NIB_A ? 2 : 1, UW = NIB_W ? 2 : 1;           // 64 bytes per lane in flight on either side
+    DecodeWalk<NIB_W, UW> walk(j.w_mant, j.w_exp, j.N, j.K, j.block, j.ww, j.w_hat, j.K, pw, ww, nw);
+    typename DecodeWalk<NIB_W, UW>::Item first;
+    walk.fetch(first);
+    decode_bf16_body<NIB_A, UA>(j.a_mant, j.a_exp, j.M, j.K, j.block, j.wa, j.a_hat, j.K, pa, wid, nw);
+    walk.run(first);
 }
 
 // ---- dense storage: w bits per element (Eq. 1 counts m + 1 bits per value) ---------------------
@@ -1056,7 +1073,9 @@ prep_operands_kernel(const PrepJob j)
     ps.mant_batch = ps.exp_batch = ps.out_batch = 0;
     ps.exp_row_shift = j.w_row_shift;
     // the first weights are on their way while the activations are quantized
-    DecodeWalk<NIBBLE, 2> walk(j.w_mant, j.w_exp, j.N, j.K, j.block, j.ww, j.w_hat, j.K, ps, wid, nw);
+    // (their items are dealt on from where the activations' end)
+    const int64_t ww = after_items((uint32_t)wid, (uint32_t)nw, (uint32_t)((j.a_rows2 ? j.M >> 1 : j.M) * ((j.K + 255) >> 8)));
+    DecodeWalk<NIBBLE, 2> walk(j.w_mant, j.w_exp, j.N, j.K, j.block, j.ww, j.w_hat, j.K, ps, ww, nw);
     typename DecodeWalk<NIBBLE, 2>::Item first;
     walk.fetch(first);
     QuantOut out{nullptr, nullptr, j.a_hat, j.K, nullptr};

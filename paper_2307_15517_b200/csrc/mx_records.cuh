@@ -96,10 +96,15 @@ __device__ __forceinline__ void rec_store_scale(const RecOut &o, int panel, int 
 {
     o.sf[((int64_t)(kb >> 2) * o.panels_sf + panel) * REC_SF_BYTES + (rp & 31) * 16 + (rp >> 5) * 4 + (kb & 3)] = (uint8_t)s;
 }
-// The scale bytes of its groups g0 and g1 of 16 k (numbers within the record).
-__device__ __forceinline__ void rec_store_wide(const RecOut &o, int panel, int kb, int rp, const RecScale &s, int g0, int g1)
+// The scale bytes of its groups g0 and g1 of 16 k (numbers within the record).  Where none of the warp's rows is wide all
+// eight bytes of a row are its one scale: two lanes write them as words (c4 = number of the lane among its row's four).
+__device__ __forceinline__ void rec_store_wide(const RecOut &o, int panel, int kb, int rp, const RecScale &s, bool wide, int c4, int g0, int g1)
 {
     uint8_t *d = o.sf_wide + ((int64_t)kb * o.panels_sf + panel) * REC_SFW_BYTES + (rp & 31) * 16 + (rp >> 5) * 4;
+    if (!wide) {
+        if (c4 < 2) *reinterpret_cast<uint32_t *>(d + 512 * c4) = (uint32_t)s.s * 0x01010101u;
+        return;
+    }
     d[(g0 & 1) * 512 + (g0 >> 1)] = (uint8_t)s.s0;
     d[(g1 & 1) * 512 + (g1 >> 1)] = (uint8_t)s.s1;
 }
@@ -189,8 +194,8 @@ __device__ __forceinline__ void rec_quantize_body(const InT *__restrict__ x, int
         for (int u = 0; u < 2; ++u)
             *reinterpret_cast<uint4 *>(dst + u * 4 * (REC_ROWS * 16)) = rec_encode16(v[u], e[u], z[u], w, u ? s.s1 : s.s0);
         if (c4 == 0) rec_store_scale(o, panel, kb, rp, s.s);
-        rec_store_wide(o, panel, kb, rp, s, c4, 4 + c4);
         const bool wide = __any_sync(0xFFFFFFFFu, s.wide);
+        rec_store_wide(o, panel, kb, rp, s, wide, c4, c4, 4 + c4);
         if (lane == 0) o.flags[((int64_t)panel * kblocks + kb) * 16 + (grp & 15)] = wide;
     }
 }
@@ -312,8 +317,8 @@ __device__ __forceinline__ void rec_convert(const RecPacked &j, const RecOut &o,
             *reinterpret_cast<uint4 *>(dst + h * (REC_ROWS * 16)) = b;
         }
         if (c4 == 0) rec_store_scale(o, panel, kb, rp, s.s);
-        rec_store_wide(o, panel, kb, rp, s, 2 * c4, 2 * c4 + 1);
         const bool wide = __any_sync(0xFFFFFFFFu, s.wide);
+        rec_store_wide(o, panel, kb, rp, s, wide, c4, 2 * c4, 2 * c4 + 1);
         if (lane == 0) o.flags[((int64_t)panel * o.kblocks + kb) * 16 + (grp & 15)] = wide;
     }
 }
@@ -351,11 +356,13 @@ rec_prep_kernel(const RecPrepJob j)
     ptx::dep_trigger();
     const uint32_t warps = blockDim.x >> 5;
     const uint32_t wid = blockIdx.x * warps + (threadIdx.x >> 5), nw = gridDim.x * warps;
+    // the weights' items are dealt on from where the activations' end, so that no warp has more than one item above the mean
+    const uint32_t ww = after_items(wid, nw, (uint32_t)j.a.panels * (REC_ROWS / 8) * (uint32_t)j.a.kblocks);
     // the first weights are on their way while the activations are quantized
     constexpr int UNROLL = 2;
     RecPackedItem<NIBBLE, UNROLL> d;
     const uint32_t steps = rec_steps(j.w, UNROLL);
-    rec_fetch<NIBBLE, UNROLL>(j.pw, wid, steps, (uint32_t)j.w.panels * (REC_ROWS / 8) * steps, d);
+    rec_fetch<NIBBLE, UNROLL>(j.pw, ww, steps, (uint32_t)j.w.panels * (REC_ROWS / 8) * steps, d);
     const InT *x = static_cast<const InT *>(j.x);
     if (j.block == 16) {
         if (j.a_rows2) rec_quantize_body<InT, 16, true>(x, j.M, j.K, j.ldx, j.wa, j.a, wid, nw);
@@ -364,7 +371,7 @@ rec_prep_kernel(const RecPrepJob j)
         if (j.a_rows2) rec_quantize_body<InT, 32, true>(x, j.M, j.K, j.ldx, j.wa, j.a, wid, nw);
         else rec_quantize_body<InT, 32, false>(x, j.M, j.K, j.ldx, j.wa, j.a, wid, nw);
     }
-    rec_decode_body<NIBBLE, UNROLL>(j.pw, j.w, wid, nw, d);
+    rec_decode_body<NIBBLE, UNROLL>(j.pw, j.w, ww, nw, d);
 }
 
 // The same for two packed operands.
@@ -384,11 +391,12 @@ rec_pair_kernel(const RecPairJob j)
     constexpr int UNROLL = 2;
     RecPackedItem<NIB_A, UNROLL> da;
     RecPackedItem<NIB_W, UNROLL> dw;
-    const uint32_t steps = rec_steps(j.a, UNROLL);
-    rec_fetch<NIB_A, UNROLL>(j.pa, wid, steps, (uint32_t)j.a.panels * (REC_ROWS / 8) * steps, da);
-    rec_fetch<NIB_W, UNROLL>(j.pw, wid, steps, (uint32_t)j.w.panels * (REC_ROWS / 8) * steps, dw);
+    const uint32_t steps = rec_steps(j.a, UNROLL), items_a = (uint32_t)j.a.panels * (REC_ROWS / 8) * steps;
+    const uint32_t ww = after_items(wid, nw, items_a);
+    rec_fetch<NIB_A, UNROLL>(j.pa, wid, steps, items_a, da);
+    rec_fetch<NIB_W, UNROLL>(j.pw, ww, steps, (uint32_t)j.w.panels * (REC_ROWS / 8) * steps, dw);
     rec_decode_body<NIB_A, UNROLL>(j.pa, j.a, wid, nw, da);
-    rec_decode_body<NIB_W, UNROLL>(j.pw, j.w, wid, nw, dw);
+    rec_decode_body<NIB_W, UNROLL>(j.pw, j.w, ww, nw, dw);
 }
 
 }  // namespace mx

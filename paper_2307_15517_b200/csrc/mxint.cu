@@ -323,12 +323,11 @@ mx_status_t launch_dequant_pair(const void *a_mant, const uint8_t *a_exp, const 
     const bool na = fa.elem_bits <= 4, nw = fw.elem_bits <= 4;
     const int64_t items = (M + N) * (K / 32);
     ProfScope prof(KIND_DEQUANTIZE, st);
-    const int per_sm = resident_ctas(mx::decode_pair_kernel<true, true>);
-    const dim3 grid((unsigned)grid_for((items + 1) / 2, 256, d.sm_count, per_sm));
-    if (na && nw) MX_CUDA(launch_dep(mx::decode_pair_kernel<true, true>, dim3(grid), dim3(256), 0, st, j));
-    else if (na) MX_CUDA(launch_dep(mx::decode_pair_kernel<true, false>, dim3(grid), dim3(256), 0, st, j));
-    else if (nw) MX_CUDA(launch_dep(mx::decode_pair_kernel<false, true>, dim3(grid), dim3(256), 0, st, j));
-    else MX_CUDA(launch_dep(mx::decode_pair_kernel<false, false>, dim3(grid), dim3(256), 0, st, j));
+    static void (*const kernels[2][2])(mx::DecodePairJob) = {{mx::decode_pair_kernel<false, false>, mx::decode_pair_kernel<false, true>},
+                                                              {mx::decode_pair_kernel<true, false>, mx::decode_pair_kernel<true, true>}};
+    const auto kernel = kernels[na][nw];
+    const dim3 grid((unsigned)grid_for((items + 1) / 2, 256, d.sm_count, resident_ctas(kernel)));
+    MX_CUDA(launch_dep(kernel, dim3(grid), dim3(256), 0, st, j));
     MX_CUDA(cudaGetLastError());
     return MX_OK;
 }
