@@ -1,4 +1,5 @@
-"""Thin ctypes binding of ``libmxint.so`` -- argument marshalling only.
+"""Thin binding of ``libmxint.so`` -- argument marshalling only: ctypes, and for the plain case of the most frequent calls the
+native module ``_calls`` (the same entry points; it answers None where a call is not its plain case).
 
 Every function has the name of the C entry point it calls (see ``include/mxint.h``) and takes
 torch CUDA tensors for device memory; torch is used for allocation and streams, never for
@@ -167,6 +168,10 @@ def _load() -> C.CDLL:
 
 lib = _load()
 
+from . import _calls                                              # noqa: E402  (linked against the library loaded above)
+
+_calls.set_format_type(MxFormat)
+
 
 def _check(status: int, where: str):
     if status != 0:
@@ -252,6 +257,9 @@ def mx_quantize(x: torch.Tensor, f: MxFormat, mant_out: Optional[torch.Tensor] =
                 nonfinite_count: Optional[torch.Tensor] = None,
                 stream=None) -> Tuple[torch.Tensor, torch.Tensor]:
     """x: [rows, K] fp32/bf16 CUDA tensor (any strides).  Returns (mant uint8, exps uint8)."""
+    done = _calls.quantize(x, f, mant_out, exp_out, nonfinite_count, stream)
+    if done is not None:
+        return done if done.__class__ is tuple else _check(done, "mx_quantize")
     _need_cuda(x, mant_out, exp_out, nonfinite_count)
     assert x.dim() == 2
     rows, K = x.shape
@@ -296,6 +304,10 @@ def mx_cast(mant: torch.Tensor, exps: torch.Tensor, K: int, f_in: MxFormat, f_ou
 
 def mx_dequantize(mant: torch.Tensor, exps: torch.Tensor, K: int, f: MxFormat,
                   dtype=torch.float32, out: Optional[torch.Tensor] = None, stream=None) -> torch.Tensor:
+    if dtype is torch.float32 or dtype is torch.bfloat16:
+        done = _calls.dequantize(mant, exps, K, f, dtype is torch.bfloat16, out, stream)
+        if done is not None:
+            return done if done.__class__ is not int else _check(done, "mx_dequantize")
     _need_cuda(mant, exps, out)
     rows = mant.shape[0]
     if out is None:
@@ -324,6 +336,9 @@ def mx_gemm(a_mant, a_exp, fa: MxFormat, w_mant, w_exp, fw: MxFormat, M: int, N:
 def mx_linear(x: torch.Tensor, fa: MxFormat, w_mant, w_exp, fw: MxFormat, N: int,
               bias: Optional[torch.Tensor] = None, y: Optional[torch.Tensor] = None,
               workspace: Optional[torch.Tensor] = None, algo: int = MX_ALGO_AUTO, stream=None):
+    done = _calls.linear(x, fa, w_mant, w_exp, fw, N, bias, y, workspace, algo, stream)
+    if done is not None:
+        return done if done.__class__ is not int else _check(done, "mx_linear")
     _need_cuda(x, w_mant, w_exp, bias, y, workspace)
     M, K = x.shape
     assert x.stride(1) == 1
@@ -393,6 +408,9 @@ def mx_linear_fused(x: torch.Tensor, fa: MxFormat, w_mant, w_exp, fw: MxFormat, 
     """mx_linear with bias, ReLU and a residual applied in the epilogue.  ``fy`` None: returns the fp32
     result; else returns (y_mant, y_exp), the result quantized to ``fy`` along N.
     ``layernorm`` = (gamma, beta, eps): the rows of x are layer-normalised in front of the quantizer."""
+    done = _calls.linear_fused(x, fa, w_mant, w_exp, fw, N, bias, bool(relu), residual, fy, y, y_mant, y_exp, layernorm, workspace, stream)
+    if done is not None:
+        return done if done.__class__ is not int else _check(done, "mx_linear_fused")
     _need_cuda(x, w_mant, w_exp, bias, residual, y, y_mant, y_exp, workspace)
     pro = None
     if layernorm is not None:
@@ -423,6 +441,9 @@ def mx_gemm_fused(a_mant, a_exp, fa: MxFormat, w_mant, w_exp, fw: MxFormat, M: i
                   residual: Optional[torch.Tensor] = None, fy: Optional[MxFormat] = None, y=None,
                   y_mant=None, y_exp=None, workspace: Optional[torch.Tensor] = None, stream=None):
     """mx_gemm with bias, ReLU and a residual applied in the epilogue; result as for ``mx_linear_fused``."""
+    done = _calls.gemm_fused(a_mant, a_exp, fa, w_mant, w_exp, fw, M, N, K, bias, bool(relu), residual, fy, y, y_mant, y_exp, workspace, stream)
+    if done is not None:
+        return done if done.__class__ is not int else _check(done, "mx_gemm_fused")
     _need_cuda(a_mant, a_exp, w_mant, w_exp, bias, residual, y, y_mant, y_exp, workspace)
     assert residual is None or (residual.stride(1) == 1 and residual.dtype == torch.float32)
     if fy is None:
@@ -511,6 +532,9 @@ def mx_attention_fp(q: torch.Tensor, k: torch.Tensor, v: torch.Tensor, fqk: MxFo
                     ctx: Optional[torch.Tensor] = None, workspace: Optional[torch.Tensor] = None, stream=None):
     """mx_attention on floating-point q, k, v ([seq, heads*head_dim], row-major views allowed): the three
     operands are quantized on the fly (q, k along the head dimension, v along the tokens)."""
+    done = _calls.attention_fp(q, k, v, fqk, fv, heads, head_dim, scale, fp, bool(causal), ctx, workspace, stream)
+    if done is not None:
+        return done if done.__class__ is not int else _check(done, "mx_attention_fp")
     _need_cuda(q, k, v, ctx, workspace)
     seq = q.shape[0]
     assert q.dtype == k.dtype == v.dtype and q.stride(1) == k.stride(1) == v.stride(1) == 1

@@ -1,27 +1,31 @@
-"""Builds ``libmxint.so`` in-tree with nvcc for sm_100a (cross-compiles without a GPU)."""
+"""Builds ``libmxint.so`` in-tree with nvcc for sm_100a (cross-compiles without a GPU), and ``_calls.so``, the native half of
+the binding, with the host compiler against it and torch."""
 from __future__ import annotations
 
 import os
 import subprocess
 import sys
+import sysconfig
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libmxint.so")
 SOURCES = ["mxint.cu"]
+CALLS = os.path.join(HERE, "_calls.so")
 
 
 def _newest_source_mtime() -> float:
     newest = 0.0
     for root in (CSRC, os.path.join(os.path.dirname(HERE), "include")):
         for name in os.listdir(root):
-            if name.endswith((".cu", ".cuh", ".h")):
+            if name.endswith((".cu", ".cuh", ".h", ".cpp")):
                 newest = max(newest, os.path.getmtime(os.path.join(root, name)))
     return newest
 
 
 def build(force: bool = False, verbose: bool = False) -> str:
-    if not force and os.path.exists(LIB) and os.path.getmtime(LIB) >= _newest_source_mtime():
+    newest = _newest_source_mtime()
+    if not force and all(os.path.exists(f) and os.path.getmtime(f) >= newest for f in (LIB, CALLS)):
         return LIB
     nvcc = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")
     tmp = LIB + ".tmp.%d" % os.getpid()
@@ -33,7 +37,23 @@ def build(force: bool = False, verbose: bool = False) -> str:
     cmd += [os.path.join(CSRC, s) for s in SOURCES]
     subprocess.check_call(cmd)
     os.replace(tmp, LIB)
+    _build_calls()
     return LIB
+
+
+def _build_calls() -> None:
+    import torch
+    root = os.path.dirname(torch.__file__)
+    cuda = os.path.dirname(os.path.dirname(os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")))
+    include = [os.path.join(root, "include"), os.path.join(root, "include", "torch", "csrc", "api", "include"),
+               sysconfig.get_paths()["include"], os.path.join(cuda, "include")]
+    tmp = CALLS + ".tmp.%d" % os.getpid()
+    cmd = [os.environ.get("CXX", "g++"), "-std=c++17", "-O2", "-shared", "-fPIC", "-fvisibility=hidden",
+           "-D_GLIBCXX_USE_CXX11_ABI=%d" % int(torch._C._GLIBCXX_USE_CXX11_ABI)] + ["-I" + d for d in include]
+    cmd += ["-o", tmp, os.path.join(CSRC, "calls.cpp"), "-L" + os.path.join(root, "lib"), "-lc10", "-lc10_cuda", "-ltorch_cpu",
+            "-ltorch_python", "-L" + HERE, "-l:libmxint.so", "-Wl,-rpath,$ORIGIN"]
+    subprocess.check_call(cmd)
+    os.replace(tmp, CALLS)
 
 
 if __name__ == "__main__":
