@@ -65,6 +65,122 @@ __device__ __forceinline__ void splitk_sum4(uint32_t smem_base, int split, int c
     }
 }
 
+// An MXInt result of the 32 rows of lane quarter `quad` (from m0 on) of a chunk (32 columns from n on): the cluster's partials
+// added up, a row per lane, so that a block is a lane's own columns.  The sums are taken in whole lines, four rows per warp and
+// load, and pass through this CTA's own copy of the chunk, which no other CTA reads: read a row per lane from the other CTAs, a
+// request is 16 bytes of 32 lines (352 x 1024 x 1024 with an 8-bit result: the call 19.3 us, now 12.9; 13.3 without a cut).
+// Warp-collective, as the next one.
+template <bool TAIL>
+__device__ __forceinline__ void splitk_chunk_q(const TcParams &p, uint8_t *smem_gen, uint32_t smem_base, int split, int c, int m0, int n,
+                                               int quad, int lane)
+{
+    const int rows0 = m0 + quad * 32;
+    if (n >= p.N || rows0 >= p.M) return;                            // warp-uniform
+    const int row = rows0 + lane, c4 = lane & 7;
+    TailRegs t;
+    if (TAIL) tail_fetch(p, row, n, t);
+#pragma unroll 1
+    for (int h = 0; h < 2; ++h) {
+        const int lr = quad * 32 + 16 * h + (lane >> 3);
+        float4 v[4];
+        splitk_sum4(smem_base, split, c, lr, c4, v);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) *reinterpret_cast<float4 *>(smem_gen + splitk_offset(c, lr + 4 * i, c4)) = v[i];
+    }
+    __syncwarp();
+    uint32_t r[32];
+#pragma unroll
+    for (int v = 0; v < 8; ++v) {
+        const uint4 x = *reinterpret_cast<const uint4 *>(smem_gen + splitk_offset(c, quad * 32 + lane, v));
+        r[4 * v] = x.x; r[4 * v + 1] = x.y; r[4 * v + 2] = x.z; r[4 * v + 3] = x.w;
+    }
+    if (TAIL) tail_apply(p, t, n, r);
+    store_mxint_chunk(p, row, n, r);
+}
+
+// fp32: rows m0 + r4 .. + 4 G - 1 of a chunk, 128 bytes each, all 8 loads of the at most 8 / G partials in flight.
+template <bool TAIL, int G>
+__device__ __forceinline__ void splitk_rows4(const TcParams &p, uint32_t smem_base, int split, int c, int m0, int n, int r4, int lane)
+{
+    const int c4 = lane & 7, col = n + 4 * c4, lr = r4 + (lane >> 3);
+    if (n >= p.N || m0 + r4 >= p.M) return;                          // warp-uniform
+    const float *bias = TAIL ? p.ex_bias : p.bias;
+    float4 x[G][8 / G];
+#pragma unroll
+    for (int g = 0; g < G; ++g)
+#pragma unroll
+        for (int s = 0; s < 8 / G; ++s)
+            if (s < split) x[g][s] = ld_cluster_f32x4(ptx::map_to_cta(smem_base, (uint32_t)s) + splitk_offset(c, lr + 4 * g, c4));
+    const bool vec = col + 4 <= p.N && (p.ldy & 3) == 0 && (reinterpret_cast<uintptr_t>(p.y) & 15) == 0;
+    const bool rvec = TAIL && p.residual && col + 4 <= p.N && (p.ldr & 3) == 0 && (reinterpret_cast<uintptr_t>(p.residual) & 15) == 0;
+    float b[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) b[k] = bias && col + k < p.N ? __ldg(bias + col + k) : 0.f;
+#pragma unroll
+    for (int g = 0; g < G; ++g) {
+        const int row = m0 + lr + 4 * g;
+        float v[4] = {x[g][0].x, x[g][0].y, x[g][0].z, x[g][0].w};
+#pragma unroll
+        for (int s = 1; s < 8 / G; ++s) {
+            if (s < split) { v[0] += x[g][s].x; v[1] += x[g][s].y; v[2] += x[g][s].z; v[3] += x[g][s].w; }
+        }
+        if (row >= p.M) continue;
+        float res[4] = {0.f, 0.f, 0.f, 0.f};
+        if (TAIL && p.residual) {
+            const float *src = p.residual + (int64_t)row * p.ldr + col;
+            if (rvec) {
+                const float4 q = __ldg(reinterpret_cast<const float4 *>(src));
+                res[0] = q.x; res[1] = q.y; res[2] = q.z; res[3] = q.w;
+            } else {
+#pragma unroll
+                for (int k = 0; k < 4; ++k)
+                    if (col + k < p.N) res[k] = __ldg(src + k);
+            }
+        }
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            if (bias) v[k] += b[k];
+            if (TAIL && p.relu) v[k] = v[k] < 0.f ? 0.f : v[k];      // NaN stays NaN
+            if (TAIL && p.residual) v[k] += res[k];
+        }
+        float *dst = p.y + (int64_t)row * p.ldy + col;
+        if (vec) {
+            *reinterpret_cast<float4 *>(dst) = make_float4(v[0], v[1], v[2], v[3]);
+        } else {
+#pragma unroll
+            for (int k = 0; k < 4; ++k)
+                if (col + k < p.N) dst[k] = v[k];
+        }
+    }
+}
+
+// The cluster's partial tiles (`chunks` of 32 columns; chunk c is columns 32 (c % row_chunks) from n0 on, rows of panel
+// c / row_chunks) added up and written: in units -- MXInt result: the 32 rows of a lane quarter of a chunk; fp32: 4 G of its
+// rows -- dealt to all `warps` of all CTAs of the cluster.  A unit's loads from the other SMs take about a microsecond, however
+// few they are, so what counts is a warp's number of units: whole chunks dealt to the CTAs (chunk c to CTA c % split, eight
+// units one after the other there) left calls of 33..256 rows at 13.4-14.4 us (K x N = 2048 x 2048), 24.4-26.7 (8192 x 2048) and
+// 20.2-21.4 (4096 x 4096, up to 128 rows); now 11.7-12.9, 22.5-25.1 and 18.4-19.6.
+template <bool TAIL, bool QOUT, int G>
+__device__ __forceinline__ void splitk_units(const TcParams &p, uint8_t *smem_gen, uint32_t smem_base, int split, int chunks, int row_chunks,
+                                             int m0, int n0, int first, int warps, int lane)
+{
+    const int per = QOUT ? 4 : 32 / G;
+    for (int u = first; u < chunks * per; u += split * warps) {
+        const int c = u / per, at = u % per, panel = c / row_chunks, m = m0 + TC_BM * panel, n = n0 + 32 * (c - panel * row_chunks);
+        if (QOUT) splitk_chunk_q<TAIL>(p, smem_gen, smem_base, split, c, m, n, at, lane);
+        else splitk_rows4<TAIL, G>(p, smem_base, split, c, m, n, 4 * G * at, lane);
+    }
+}
+template <bool TAIL, bool QOUT>
+__device__ __forceinline__ void splitk_reduce(const TcParams &p, uint8_t *smem_gen, uint32_t smem_base, int split, int rank, int chunks,
+                                              int row_chunks, int m0, int n0, int warp, int warps, int lane)
+{
+    const int first = rank + split * warp;
+    if (QOUT || split > 4) splitk_units<TAIL, QOUT, 1>(p, smem_gen, smem_base, split, chunks, row_chunks, m0, n0, first, warps, lane);
+    else if (split > 2) splitk_units<TAIL, false, 2>(p, smem_gen, smem_base, split, chunks, row_chunks, m0, n0, first, warps, lane);
+    else splitk_units<TAIL, false, 4>(p, smem_gen, smem_base, split, chunks, row_chunks, m0, n0, first, warps, lane);
+}
+
 // QOUT: an MXInt result (yq_mant), else fp32.
 template <bool TAIL, bool QOUT>
 __global__ void __maxnreg__(128)
@@ -182,90 +298,8 @@ gemm_splitk_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_cons
     __syncwarp();
     ptx::cluster_sync();                                             // every partial tile is in place
 
-    if (warp >= 2) {
-        const int quad = warp & 3, half = (warp - 2) >> 2;
-        // chunks rank, rank + split, ...: alternately to the two warps of a lane quarter
-        int turn = 0;
-        for (int c = rank; c < Cfg::BN / 32; c += split, ++turn) {
-            if ((turn & 1) != half) continue;
-            const int n = n0 + 32 * c, rows0 = m0 + quad * 32;
-            if (n >= p.N || rows0 >= p.M) continue;                  // warp-uniform
-            if (QOUT) {
-                // MXInt result: a row per lane, so that a block is a lane's own columns.  The sums are taken in whole lines,
-                // four rows per warp and load, and pass through this CTA's own copy of the chunk, which no other CTA reads:
-                // read a row per lane from the other CTAs, a request is 16 bytes of 32 lines (352 x 1024 x 1024 with an
-                // 8-bit result: the call 19.3 us, now 12.9; 13.3 without a cut).
-                const int row = rows0 + lane, c4 = lane & 7;
-                TailRegs t;
-                if (TAIL) tail_fetch(p, row, n, t);
-#pragma unroll 1
-                for (int h = 0; h < 2; ++h) {
-                    const int lr = quad * 32 + 16 * h + (lane >> 3);
-                    float4 v[4];
-                    splitk_sum4(smem_base, split, c, lr, c4, v);
-#pragma unroll
-                    for (int i = 0; i < 4; ++i) *reinterpret_cast<float4 *>(smem_gen + splitk_offset(c, lr + 4 * i, c4)) = v[i];
-                }
-                __syncwarp();
-                uint32_t r[32];
-#pragma unroll
-                for (int v = 0; v < 8; ++v) {
-                    const uint4 x = *reinterpret_cast<const uint4 *>(smem_gen + splitk_offset(c, quad * 32 + lane, v));
-                    r[4 * v] = x.x; r[4 * v + 1] = x.y; r[4 * v + 2] = x.z; r[4 * v + 3] = x.w;
-                }
-                if (TAIL) tail_apply(p, t, n, r);
-                store_mxint_chunk(p, row, n, r);
-                continue;
-            }
-            // fp32: four rows of 128 bytes per warp and step
-            const int c4 = lane & 7, col = n + 4 * c4;
-            const float *bias = TAIL ? p.ex_bias : p.bias;
-            float b[4];
-#pragma unroll
-            for (int i = 0; i < 4; ++i) b[i] = bias && col + i < p.N ? __ldg(bias + col + i) : 0.f;
-            const bool vec = col + 4 <= p.N && (p.ldy & 3) == 0 && (reinterpret_cast<uintptr_t>(p.y) & 15) == 0;
-            const bool rvec = TAIL && p.residual && col + 4 <= p.N && (p.ldr & 3) == 0 && (reinterpret_cast<uintptr_t>(p.residual) & 15) == 0;
-#pragma unroll 4
-            for (int i = 0; i < 8; ++i) {
-                const int lr = quad * 32 + 4 * i + (lane >> 3), row = m0 + lr;
-                float v[4];
-                for (int s = 0; s < split; ++s) {
-                    const float4 x = ld_cluster_f32x4(ptx::map_to_cta(smem_base, (uint32_t)s) + splitk_offset(c, lr, c4));
-                    v[0] = s ? v[0] + x.x : x.x;
-                    v[1] = s ? v[1] + x.y : x.y;
-                    v[2] = s ? v[2] + x.z : x.z;
-                    v[3] = s ? v[3] + x.w : x.w;
-                }
-                if (row >= p.M) continue;
-                float res[4] = {0.f, 0.f, 0.f, 0.f};
-                if (TAIL && p.residual) {
-                    const float *src = p.residual + (int64_t)row * p.ldr + col;
-                    if (rvec) {
-                        const float4 q = __ldg(reinterpret_cast<const float4 *>(src));
-                        res[0] = q.x; res[1] = q.y; res[2] = q.z; res[3] = q.w;
-                    } else {
-#pragma unroll
-                        for (int k = 0; k < 4; ++k)
-                            if (col + k < p.N) res[k] = __ldg(src + k);
-                    }
-                }
-#pragma unroll
-                for (int k = 0; k < 4; ++k) {
-                    if (bias) v[k] += b[k];
-                    if (TAIL && p.relu) v[k] = v[k] < 0.f ? 0.f : v[k];          // NaN stays NaN
-                    if (TAIL && p.residual) v[k] += res[k];
-                }
-                float *dst = p.y + (int64_t)row * p.ldy + col;
-                if (vec) {
-                    *reinterpret_cast<float4 *>(dst) = make_float4(v[0], v[1], v[2], v[3]);
-                } else {
-#pragma unroll
-                    for (int k = 0; k < 4; ++k)
-                        if (col + k < p.N) dst[k] = v[k];
-                }
-            }
-        }
-    }
+    if (warp >= 2)
+        splitk_reduce<TAIL, QOUT>(p, smem_gen, smem_base, split, rank, Cfg::BN / 32, Cfg::BN / 32, m0, n0, warp - 2, Cfg::EPI_WARPS, lane);
     __syncwarp();
     ptx::tc_fence_before_sync();
     ptx::cluster_sync();                                             // nobody reads this CTA's partial tile any more

@@ -1005,7 +1005,7 @@ mx_status_t splitk_clusters(DeviceInfo &d, int split, int *out)
 // Few tiles, long reduction: into how many pieces K is cut over a cluster (see mx_gemm_splitk.cuh); 0 for the one-CTA
 // kernels.  The most pieces whose clusters all fit at once, where the K steps that a CTA is spared are worth the two
 // cluster barriers and the exchange (about 2.5 us against 0.2 us per step: at least 12 steps spared).  Whole calls, split /
-// not (us): 352 x 2048 x 8192 in two 36.8 / 51.5, 352 x 2048 x 2048 15.8 / 17.3, 64 x 768 x 3072 in four 12.7 / 20.2,
+// not (us): 352 x 2048 x 8192 in two 34.4 / 51.5, 352 x 2048 x 2048 14.7 / 17.3, 64 x 768 x 3072 in four 12.7 / 20.2,
 // 512 x 1024 x 4096 18.4 / 27.5, 200 x 1024 x 1024 10.7 / 11.2; but 352 x 2048 x 1024 in two 13.2 / 12.2 and
 // 128 x 768 x 768 in four 10.9 / 10.2.  More than 64 CTAs take longer to exchange and need 16 steps spared: at 12 and 14 the
 // cut of 17 to 33 tiles in four is 0.5 us slower to 1.2 us slower (42 x 4096 x 1024, 42 x 3872 x 1024), at 18 it is 1 to 2 us
