@@ -69,6 +69,10 @@ typedef enum {
                             activation blocks: the arithmetic of MX_ALGO_STREAM for any of them, K cut over a
                             cluster of up to eight CTAs whose sums are added in fp32, in order;
                             everything else on tensor cores, on operands that hold every value exactly:
+                            - M <= 384, weights in container form with rows of whole 16-byte units, and
+                              large enough (N * K > 2^21, more from 129 rows on): the bf16 values of
+                              MX_ALGO_TCGEN05, the weights decoded inside the product, the K range cut
+                              over a cluster of up to eight CTAs and the pieces added in fp32, in order;
                             - few 128 x 128 tiles (at most 74) and K of 1024 or more: the bf16 operands of
                               MX_ALGO_TCGEN05, the K range cut over a cluster of two to four CTAs and the
                               pieces added in fp32, in order;
@@ -118,8 +122,8 @@ typedef enum {
  *                                  truncates, so the guaranteed bound is
  *                                  ceil(K/16) * 17 * 2^-23 * S; it is approached only when block
  *                                  scales inside one row differ by many binades.  Where AUTO cuts K,
- *                                  up to four such sums are added in fp32 with round-to-nearest: at
- *                                  most 3 * 2^-24 * S more, and a shorter chain in each.  On operands whose
+ *                                  up to eight such sums are added in fp32 with round-to-nearest: at
+ *                                  most 7 * 2^-24 * S more, and a shorter chain in each.  On operands whose
  *                                  block exponents spread over <= 2^6 per row (every LLM-shaped
  *                                  workload measured: N(0, sigma) weights, outlier-channel or
  *                                  Student-t activations, K up to 16384) the error stays below
@@ -130,7 +134,7 @@ typedef enum {
  *   the last bits between 4-bit and 6-bit containers, between two token counts, and between mx_layernorm +
  *   mx_linear and mx_linear_fused with a LayerNorm prologue (which takes no block-scaled operands).  mx_linear,
  *   mx_linear_q and mx_linear_fused without one (mx_gemm, mx_gemm_q and mx_gemm_fused) of the same sizes share
- *   their route for M > 16.  A named algorithm, mx_gemm_batched and mx_gemm_static never cut K.
+ *   their route for M > 32.  A named algorithm, mx_gemm_batched and mx_gemm_static never cut K.
  *   MX_ALGO_TCGEN05_BLOCKWISE    : exact block sums out of the tensor pipe, one fp32 rounding per block,
  *                                  ascending blocks: the result of MX_ALGO_SIMT, bit for bit, whatever
  *                                  the operands (block terms inside the fp32 normal range). */
@@ -162,8 +166,7 @@ typedef struct {
  * for either operand with MX_ALGO_AUTO, MX_ALGO_TCGEN05(_BLOCKWISE) and MX_ALGO_SIMT, as the result
  * format fy of the _q forms (rows of Y pair up: exponent array [M/2, N/fy.block]), by
  * mx_gemm_batched (items must start on even rows) and by MX_ALGO_STREAM / mx_linear_grouped for
- * either operand (an even number of tokens when the activations pair up; weights in this form are
- * read with plain loads instead of staged boxes); the in-kernel decode (MX_ALGO_TCGEN05_FUSED), the
+ * either operand (an even number of tokens when the activations pair up); the in-kernel decode (MX_ALGO_TCGEN05_FUSED), the
  * fused attention and the static entry point take one-row blocks only (MX_ERR_FORMAT). */
 
 /* ---- size helpers (host only, no CUDA call) ------------------------------------------- */

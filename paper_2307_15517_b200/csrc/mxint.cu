@@ -17,6 +17,7 @@
 #include "../../include/mxint.h"
 #include "mx_alt.cuh"
 #include "mx_attention.cuh"
+#include "mx_gemm_dec.cuh"
 #include "mx_gemm_simt.cuh"
 #include "mx_gemm_splitk.cuh"
 #include "mx_gemm_tc.cuh"
@@ -60,6 +61,8 @@ struct DeviceInfo {
     bool splitk_attr_set[4] = {};
     int splitk_clusters[mx::SplitKCfg::MAX_SPLIT + 1] = {-1, -1, -1, -1, -1};
     bool attn_attr_set[2] = {false, false};
+    bool dec_attr_set[12] = {};
+    int dec_clusters[12][mx::DecCfg::MAX_SPLIT + 1] = {};      // resident clusters by kernel and cluster size
 };
 DeviceInfo g_dev[MAX_DEVICES];
 std::mutex g_init_mu;        // guards every lazily initialised field above and below (calls may come from several host threads)
@@ -1556,6 +1559,138 @@ mx_status_t launch_gemv(const mx_linear_args_t &a, const GemvPlan &g, DeviceInfo
     return g_gemv[slot].launch(slot, g, tm, p, d, st);
 }
 
+// ---- up to 384 rows: weights decoded inside the product (gemm_dec_kernel) --------------------------------
+typedef void (*DecKernel)(CUtensorMap, CUtensorMap, mx::TcParams, mx::DecParams);
+const DecKernel g_dec[12] = {                             // panels - 1, nibbles, MXInt result: 4 * , 2 * , 1 *
+    mx::gemm_dec_kernel<1, false, false>, mx::gemm_dec_kernel<1, false, true>, mx::gemm_dec_kernel<1, true, false>, mx::gemm_dec_kernel<1, true, true>,
+    mx::gemm_dec_kernel<2, false, false>, mx::gemm_dec_kernel<2, false, true>, mx::gemm_dec_kernel<2, true, false>, mx::gemm_dec_kernel<2, true, true>,
+    mx::gemm_dec_kernel<3, false, false>, mx::gemm_dec_kernel<3, false, true>, mx::gemm_dec_kernel<3, true, false>, mx::gemm_dec_kernel<3, true, true>};
+
+struct DecPlan { int which, panels, split, exp_words; };
+
+mx_status_t dec_config(cudaLaunchConfig_t &cfg, cudaLaunchAttribute *attr, int panels, int grid, int split, cudaStream_t st)
+{
+    cfg.gridDim = dim3((unsigned)grid);
+    cfg.blockDim = dim3(mx::DecCfg::THREADS);
+    cfg.dynamicSmemBytes = mx::DecCfg::smem_bytes(panels);
+    cfg.stream = st;
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = (unsigned)split;
+    attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return MX_OK;
+}
+
+bool dec_is_faster(int64_t M, int64_t N, int64_t K, int split, bool rec, int sm_count);
+
+// Whether the product runs there, and into how many pieces K is cut: the most whose clusters all fit at once, of at least four
+// K steps each.
+mx_status_t dec_plan(int64_t M, int64_t N, int64_t K, const mx_format_t &fa, const mx_format_t &fw, const uint8_t *w_exp, bool quantized,
+                     DeviceInfo &d, DecPlan *out, bool *use)
+{
+    *use = false;
+    const bool nib = fw.elem_bits <= 4;
+    const int64_t row_bytes = nib ? K / 2 : K, panels = (M + mx::TC_BM - 1) / mx::TC_BM, tiles = (N + mx::DecCfg::BN - 1) / mx::DecCfg::BN;
+    if (!format_ok(fw) || panels > mx::DecCfg::MAX_P || (row_bytes % 16) != 0 || tiles > INT32_MAX / 16) return MX_OK;
+    out->panels = (int)panels;
+    out->which = 4 * ((int)panels - 1) + (nib ? 2 : 0) + (quantized ? 1 : 0);
+    out->exp_words = ((K / fw.block) % 4) == 0 && (reinterpret_cast<uintptr_t>(w_exp) & 3u) == 0 ? 1 : 0;
+    out->split = 1;
+    const mx_status_t as = smem_attr_once(d.dec_attr_set[out->which], g_dec[out->which], 227 * 1024);
+    if (as != MX_OK) return as;
+    const int64_t kblocks = (K + mx::TC_BK - 1) / mx::TC_BK;
+    for (int s = mx::DecCfg::MAX_SPLIT; s > 1 && out->split == 1; --s) {
+        if (tiles * s > d.sm_count || kblocks < 4 * s) continue;
+        std::lock_guard<std::mutex> lk(g_init_mu);
+        int &known = d.dec_clusters[out->which][s];
+        if (known == 0) {
+            cudaLaunchConfig_t cfg = {};
+            cudaLaunchAttribute attr[2];
+            dec_config(cfg, attr, (int)panels, s * d.sm_count, s, nullptr);
+            MX_CUDA(cudaOccupancyMaxActiveClusters(&known, g_dec[out->which], &cfg));
+        }
+        if (tiles <= known) out->split = s;
+    }
+    bool rec = false;
+    if (rec_fits(fa, fw, M, N, K)) {
+        const mx_status_t rs = rec_is_faster(M, N, K, d, &rec);
+        if (rs != MX_OK) return rs;
+    }
+    *use = dec_is_faster(M, N, K, out->split, rec, d.sm_count);
+    return MX_OK;
+}
+
+mx_status_t launch_dec(const DecPlan &g, const __nv_bfloat16 *a_hat, const void *w_mant, const uint8_t *w_exp, const mx_format_t &fw, int64_t M,
+                       int64_t N, int64_t K, const float *bias, float *y, int64_t ldy, const QuantizedOut *yq, DeviceInfo &d, cudaStream_t st,
+                       const EpiTail &et)
+{
+    CUtensorMap tm_a, tm_r;
+    mx_status_t s = encode_bf16_rows(&tm_a, a_hat, M, K, mx::TC_BM);
+    if (s != MX_OK) return s;
+    s = encode_u8_sw128(&tm_r, w_mant, N, fw.elem_bits <= 4 ? K / 2 : K, mx::DecCfg::BN);
+    if (s != MX_OK) return s;
+    mx::TcParams p{};
+    p.y = y;
+    p.ex_bias = bias;
+    p.relu = et.relu;
+    p.residual = et.residual;
+    p.ldr = et.ldr;
+    p.ldy = ldy;
+    p.M = (int)M;
+    p.N = (int)N;
+    p.K = (int)K;
+    p.tiles_m = 1;
+    p.tiles_n = (int)((N + mx::DecCfg::BN - 1) / mx::DecCfg::BN);
+    p.status = d.status;
+    p.batch = 1;
+    p.yq_mant = yq ? yq->mant : nullptr;
+    p.yq_exp = yq ? yq->exps : nullptr;
+    p.yq_nonfinite = yq ? yq->nonfinite : nullptr;
+    p.yq_bits = yq ? yq->f.elem_bits : 0;
+    p.yq_block = yq ? yq->f.block : 0;
+    p.yq_rows2 = yq && yq->f.block_rows == 2 ? 1 : 0;
+    const mx::DecParams dp{w_exp, fw.elem_bits, fw.block_rows == 2 ? 1 : 0, fw.block, g.split, 1, g.exp_words};
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute attr[2];
+    dec_config(cfg, attr, g.panels, p.tiles_n * g.split, g.split, st);
+    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[1].val.programmaticStreamSerializationAllowed = 1;
+    cfg.numAttrs = g_prof.on ? 1 : 2;                     // see launch_dep
+    ProfScope prof(KIND_GEMM_TC, st);
+    MX_CUDA(cudaLaunchKernelEx(&cfg, g_dec[g.which], tm_a, tm_r, p, dp));
+    MX_CUDA(cudaGetLastError());
+    return MX_OK;
+}
+
+// Whether to run it, against a pass over the weights and then a product (`rec`: of block-scaled records, where
+// that one would run, else of bf16).  Whole calls in a graph, us, without -> with it; 8-bit activations, 4-bit weights, blocks
+// of 16 (records: 4 bits), B200:
+//   rows    K x N         without -> with     records        rows    K x N         without -> with     records
+//   128     768 x 768      10.4 -> 10.0    10.4 -> 10.0      160     6144 x 2048    20.9 ->  19.7    20.8 -> 19.8
+//   33      1024 x 1024     8.6 ->  9.2     8.6 ->  9.2      256     2048 x 6144    21.0 ->  20.3    20.2 -> 20.2
+//   128     1024 x 2048    10.3 -> 10.4                      256     4096 x 4096    24.5 ->  21.3    24.6 -> 21.3
+//   128     1024 x 4096    12.3 -> 10.8    13.2 -> 10.7      256     11008 x 4096   54.1 ->  41.2    53.8 -> 41.2
+//   128     2048 x 6144    17.4 -> 16.2    20.2 -> 16.3      256     4096 x 16384   63.6 ->  52.6    49.2 -> 52.8
+//   128     8192 x 2048    24.2 -> 19.3    24.1 -> 19.2      256     2560 x 10240   31.9 ->  37.4    28.6 -> 37.4
+//   128     4096 x 4096    19.6 -> 16.7    19.6 -> 16.7      384     4096 x 3072    23.9 ->  25.1    23.6 -> 24.8
+//   128     11008 x 4096   41.5 -> 30.9    41.5 -> 30.9      384     4096 x 4096    32.2 ->  27.0    28.5 -> 26.9
+//   128     4096 x 11008   44.9 -> 39.7    37.4 -> 39.6      384     11008 x 4096   76.0 ->  51.1    61.5 -> 50.8
+//   128     8192 x 28672  191.9 -> 135.2  169.0 -> 136.1     384     4096 x 11008   56.2 ->  64.6    54.1 -> 64.4
+//   256     2048 x 2048    12.7 -> 14.7    12.7 -> 14.7      384     8192 x 8192    90.8 ->  65.4    63.6 -> 64.2
+// Up to 128 rows it is the faster one where the weights are large, and where K is too short for the other product to be cut
+// (768 .. 1023; at 512, 100 rows 9.3 -> 10.1).  With more rows a CTA's steps cost more of what decoding them once saves, so there the weights have to be larger; a last
+// wave that leaves three SMs in ten idle (4096 x 11008, 2560 x 10240) costs more than it gives, as do, against records, a K that
+// is not cut.
+bool dec_is_faster(int64_t M, int64_t N, int64_t K, int split, bool rec, int sm_count)
+{
+    const int64_t size = N * K, ctas = (N + mx::DecCfg::BN - 1) / mx::DecCfg::BN * split, waves = (ctas + sm_count - 1) / sm_count;
+    const bool full = 10 * ctas >= 7 * waves * sm_count;
+    if (M <= 128) return (size > (1 << 21) && (full || !rec)) || (K >= 768 && K < 1024 && N >= 768);
+    if (M <= 256) return size >= 3 << 22 && N >= 2560 && full && (split >= 2 || !rec);
+    return size >= 1 << 24 && K >= 4096 && full && (split >= 3 || !rec);
+}
+
 // Both operands of one layer in the tensor-core form: activations quantized straight to exact
 // bf16, packed weights decoded to bf16.  One launch when K % 32 == 0, else two.
 mx_status_t tc_prepare(const mx_linear_args_t &a, __nv_bfloat16 *a_hat, __nv_bfloat16 *w_hat, DeviceInfo &d,
@@ -1822,6 +1957,24 @@ mx_status_t mx_gemm_ex(const void *a_mant, const uint8_t *a_exp, mx_format_t fa,
         one.w_mant = w_mant; one.w_exp = w_exp; one.fw = fw; one.N = N; one.bias = bias; one.y = y; one.ldy = ldy;
         const bool can_stream = stream_layer_ok(one) && (reinterpret_cast<uintptr_t>(w_exp) & 3u) == 0 &&
                                 workspace && workspace_bytes >= stream_table_bytes(1);
+        if (algo == MX_ALGO_AUTO && !can_stream) {
+            DeviceInfo *dd = nullptr;
+            s = device_info(&dd);
+            if (s != MX_OK) return s;
+            bool dec = false;
+            DecPlan plan;
+            s = dec_plan(M, N, K, fa, fw, w_exp, false, *dd, &plan, &dec);
+            if (s != MX_OK) return s;
+            if (dec) {
+                if (!workspace || workspace_bytes < tc_workspace(M, N, K)) return MX_ERR_WORKSPACE;
+                if ((reinterpret_cast<uintptr_t>(workspace) & 255u) != 0) return MX_ERR_ALIGN;
+                __nv_bfloat16 *a_dec = static_cast<__nv_bfloat16 *>(workspace);
+                cudaStream_t sd = static_cast<cudaStream_t>(stream);
+                s = launch_dequant_bf16(a_mant, a_exp, M, K, fa, a_dec, K, *dd, sd);
+                if (s != MX_OK) return s;
+                return launch_dec(plan, a_dec, w_mant, w_exp, fw, M, N, K, bias, y, ldy, nullptr, *dd, sd, EpiTail());
+            }
+        }
         if (algo == MX_ALGO_AUTO && !can_stream && rec_fits(fa, fw, M, N, K)) {
             if (!workspace || workspace_bytes < tc_workspace(M, N, K)) return MX_ERR_WORKSPACE;
             if ((reinterpret_cast<uintptr_t>(workspace) & 255u) != 0) return MX_ERR_ALIGN;
@@ -1953,15 +2106,26 @@ mx_status_t mx_linear_ex(const void *x, mx_dtype_t dt, int64_t M, int64_t K, int
     if (workspace_bytes < (fused ? fused_workspace(M, K) : tc_workspace(M, N, K))) return MX_ERR_WORKSPACE;
     GemvPlan gemv;
     if (any_algo && gemv_is_faster(one) && gemv_plan(one, *d, &gemv)) return launch_gemv(one, gemv, *d, st);
+    __nv_bfloat16 *a_hat = reinterpret_cast<__nv_bfloat16 *>(ws);
+    // the activations' mantissas and exponents go straight to the MMA operand form (exact bf16)
+    mx::QuantOut out{nullptr, nullptr, a_hat, K, nullptr};
+    bool dec = false;
+    DecPlan plan;
+    if (any_algo) {
+        s = dec_plan(M, N, K, fa, fw, w_exp, false, *d, &plan, &dec);
+        if (s != MX_OK) return s;
+    }
+    if (dec) {
+        s = quantize_rows_any(x, dt, M, K, ldx, fa, out, *d, st);
+        if (s != MX_OK) return s;
+        return launch_dec(plan, a_hat, w_mant, w_exp, fw, M, N, K, bias, y, ldy, nullptr, *d, st, EpiTail());
+    }
     bool rec = false;
     if (any_algo && rec_fits(fa, fw, M, N, K)) {
         s = rec_is_faster(M, N, K, *d, &rec);
         if (s != MX_OK) return s;
     }
     if (rec) return run_rec_linear(one, bias, y, ldy, nullptr, ws, *d, st, EpiTail());
-    __nv_bfloat16 *a_hat = reinterpret_cast<__nv_bfloat16 *>(ws);
-    // the activations' mantissas and exponents go straight to the MMA operand form (exact bf16)
-    mx::QuantOut out{nullptr, nullptr, a_hat, K, nullptr};
     if (fused) {
         // 4-bit weights and whole K steps: the lean in-kernel decode, which wants both operands in
         // its own K order inside every group of 8
@@ -2028,6 +2192,15 @@ static mx_status_t gemm_tc_impl(const void *a_mant, const uint8_t *a_exp, mx_for
     yq.exps = y_exp;
     yq.nonfinite = nonfinite_count;
     yq.f = fy;
+    bool dec = false;
+    DecPlan plan;
+    s = dec_plan(M, N, K, fa, fw, w_exp, !y, *d, &plan, &dec);
+    if (s != MX_OK) return s;
+    if (dec) {
+        s = launch_dequant_bf16(a_mant, a_exp, M, K, fa, a_hat, K, *d, st);
+        if (s != MX_OK) return s;
+        return launch_dec(plan, a_hat, w_mant, w_exp, fw, M, N, K, bias, y, y ? ldy : N, y ? nullptr : &yq, *d, st, et);
+    }
     bool rec = false;
     if (rec_fits(fa, fw, M, N, K)) {
         s = rec_is_faster(M, N, K, *d, &rec);
@@ -2116,6 +2289,21 @@ static mx_status_t linear_tc_impl(const void *x, mx_dtype_t dt, int64_t M, int64
     yq.exps = y_exp;
     yq.nonfinite = nonfinite_count;
     yq.f = fy;
+    bool dec = false;
+    DecPlan plan;
+    s = dec_plan(M, N, K, fa, fw, w_exp, !y, *d, &plan, &dec);
+    if (s != MX_OK) return s;
+    if (dec) {
+        if (with_ln) {
+            mx_linear_args_t rows = one;
+            rows.N = 0;                                   // the activations alone
+            s = tc_prepare_ln(rows, *ln, a_hat, w_hat, *d, st);
+        } else {
+            s = quantize_rows_any(x, dt, M, K, ldx, fa, mx::QuantOut{nullptr, nullptr, a_hat, K, nullptr}, *d, st);
+        }
+        if (s != MX_OK) return s;
+        return launch_dec(plan, a_hat, w_mant, w_exp, fw, M, N, K, bias, y, y ? ldy : N, y ? nullptr : &yq, *d, st, et);
+    }
     bool rec = false;
     if (!with_ln && rec_fits(fa, fw, M, N, K)) {
         s = rec_is_faster(M, N, K, *d, &rec);

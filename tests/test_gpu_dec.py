@@ -1,0 +1,86 @@
+"""Up to 384 rows with the packed weights decoded inside the product (gemm_dec_kernel), at the edges of its panels (128 rows),
+tiles (128 columns), pieces of K (pairs of 64) and stages, for every storage form of the weights: against the same product
+behind a pass over the weights.  Both add exact products up in fp32, in orders of their own: at most K/16 rounded additions
+of partial sums on either side, each within 2^-24 of the absolute sum S, for K <= 16384 2^-13 S at the very most; 1e-5 S as
+elsewhere.  The fused tail and the MXInt result come from the same sums."""
+import pytest
+import torch
+
+from paper_2307_15517_b200 import binding as mxb
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("M,K,N,block,wa,ww,rows2", [
+    (17, 4096, 4112, 16, 8, 4, 1),         # one panel, K in four pieces
+    (33, 784, 3002, 16, 8, 8, 1),          # K % 64 == 16, exponent rows of 49 bytes, a ragged last tile; bytes
+    (128, 8224, 2050, 32, 7, 4, 2),        # odd K steps in eight pieces, weights in two-row blocks
+    (64, 96, 32000, 32, 6, 3, 1),          # two K steps, K not cut
+    (100, 2080, 2001, 16, 8, 2, 1),        # odd row length: stores of single values
+    (40, 4096, 2000, 16, 4, 4, 1),         # operands that could be records
+    (129, 3104, 4100, 16, 8, 4, 1),        # two panels
+    (256, 4096, 4096, 32, 8, 8, 1),
+    (256, 1040, 16200, 16, 8, 6, 1),       # K not cut
+    (257, 4112, 4090, 16, 8, 8, 2),        # three panels
+    (384, 8192, 4096, 16, 8, 4, 1),
+    (384, 4192, 4200, 32, 4, 4, 1),
+])
+def test_weights_decoded_in_the_product(M, K, N, block, wa, ww, rows2):
+    g = torch.Generator(device="cuda")
+    g.manual_seed(M + K + N)
+    fa, fw = mxb.MxFormat(block, wa), mxb.MxFormat(block, ww, block_rows=rows2)
+    ld = -(-K // 8) * 8
+    x = torch.randn(M, ld, generator=g, device="cuda")[:, :K]
+    w = torch.randn(N, K, generator=g, device="cuda") * 0.02 * torch.exp2(torch.randint(-9, 9, (N, 1), generator=g, device="cuda").float())
+    wm, we = mxb.mx_quantize(w, fw)
+    bias = torch.randn(N, generator=g, device="cuda")
+
+    def absolute(m, e, f):
+        return mxb.mx_dequantize(m, e, K, f).abs()
+
+    am, ae = mxb.mx_quantize(x, fa)
+    S = absolute(am, ae, fa).double() @ absolute(wm, we, fw).double().t() + bias.abs().double()
+    y = torch.full((M, N + 4), -7.0, device="cuda")
+    mxb.mx_linear(x, fa, wm, we, fw, N, bias=bias, y=y[:, :N])
+    want = mxb.mx_linear(x, fa, wm, we, fw, N, bias=bias, algo=mxb.MX_ALGO_TCGEN05)
+    assert mxb.mx_poll_status() == 0
+    assert (y[:, N:] == -7.0).all()
+    y = y[:, :N].contiguous()
+    assert ((y - want).abs().double() <= 1e-5 * S).all(), float(((y - want).abs().double() / S).max())
+    assert torch.equal(mxb.mx_gemm(am, ae, fa, wm, we, fw, M, N, K, bias=bias), y)
+    res = torch.randn(M, N, generator=g, device="cuda")
+    z = torch.relu(y) + res
+    assert torch.equal(mxb.mx_linear_fused(x, fa, wm, we, fw, N, bias=bias, relu=True, residual=res), z)
+    assert torch.equal(mxb.mx_gemm_fused(am, ae, fa, wm, we, fw, M, N, K, bias=bias, relu=True, residual=res), z)
+    for fy in (mxb.MxFormat(16, 8), mxb.MxFormat(32, 4)):
+        if N % fy.block == 0:
+            for r, call in ((y, lambda: mxb.mx_linear_q(x, fa, wm, we, fw, N, fy, bias=bias)),
+                            (z, lambda: mxb.mx_linear_fused(x, fa, wm, we, fw, N, bias=bias, relu=True, residual=res, fy=fy))):
+                ym, ye = call()
+                qm, qe = mxb.mx_quantize(r, fy)
+                assert torch.equal(ym, qm) and torch.equal(ye, qe)
+    assert mxb.mx_poll_status() == 0
+
+
+@pytest.mark.parametrize("block,ww", [(32, 4), (16, 8)])
+def test_exponent_rows_at_any_address_and_a_normalised_input(block, ww):
+    M, K, N = 70, 4096, 2048
+    g = torch.Generator(device="cuda")
+    g.manual_seed(ww)
+    fa, fw = mxb.MxFormat(block, 8), mxb.MxFormat(block, ww)
+    x = torch.randn(M, K, generator=g, device="cuda")
+    wm, we = mxb.mx_quantize(torch.randn(N, K, generator=g, device="cuda") * 0.02, fw)
+    y = mxb.mx_linear(x, fa, wm, we, fw, N)
+    buf = torch.empty(we.numel() + 1, dtype=torch.uint8, device="cuda")
+    buf[1:] = we.flatten()
+    shifted = buf[1:].view(we.shape)
+    assert shifted.data_ptr() % 4 == 1
+    assert torch.equal(mxb.mx_linear(x, fa, wm, shifted, fw, N), y)
+    gamma, beta = torch.randn(K, generator=g, device="cuda"), torch.randn(K, generator=g, device="cuda")
+    a = mxb.mx_linear_fused(x, fa, wm, we, fw, N, layernorm=(gamma, beta, 1e-5))
+    n = torch.nn.functional.layer_norm(x.double(), (K,), gamma.double(), beta.double(), 1e-5).float()
+    # a normalised value that lands on the other side of a rounding step moves by a step of its block, at most
+    # 2^-6 of the block's largest value: the outputs' error is that of quantizing, the same for both
+    b = mxb.mx_linear(n, fa, wm, we, fw, N, algo=mxb.MX_ALGO_TCGEN05)
+    assert (a - b).norm() <= 2e-3 * b.norm()
+    assert mxb.mx_poll_status() == 0
