@@ -16,7 +16,7 @@
 // Bound by an SM's intake and, up to about eight steps per CTA, by the chain from the first fetch to the last reduced value:
 // 128 x 4096 x 4096 16.7 us as a whole call (19.6 behind a pass over the weights), 128 x 4096 (N) x 11008 30.9 (41.5),
 // 128 x 28672 x 8192 135 (192), 256 x 5120 x 13824 58 (98).  Tried and slower: two K steps per proxy fence and group with four
-// stages of A in place of seven (0.1 to 0.5 us), four groups with fewer stages, plain loads in the decode groups.
+// stages of A in place of seven (0.1 to 0.5 us).
 #pragma once
 #include <cuda.h>
 #include <cuda_runtime.h>

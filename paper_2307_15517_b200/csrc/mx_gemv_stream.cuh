@@ -7,11 +7,9 @@
 // scale per block, blocks added in ascending order in fp32 -- bit-identical to the CUDA-core
 // kernel when a row's blocks are not split over warps.
 //
-//  * weights  : packed 4-bit mantissas [N, K/2] + exponent bytes [N, K/32] (block 32).  TMA
-//               variant: every warp owns a two-stage ring of shared-memory stages, each filled by
-//               three tiled TMA loads (16 rows x 256 mantissa bytes as two 128-byte swizzled boxes,
-//               16 rows x 16 exponent bytes).  Register variant: coalesced 32-bit loads, four blocks
-//               and their four exponent bytes per step, two register sets alternating.
+//  * weights  : packed 4-bit mantissas [N, K/2] + exponent bytes [N, K/32] (block 32), by coalesced
+//               32-bit loads, four blocks and their four exponent bytes per step, two register sets
+//               alternating (any address and K; mx_gemv_mma.cuh fetches by TMA where it can).
 //  * tokens   : already quantized (int8 or nibble container); each CTA stages them once per
 //               layer into shared memory in the operand order of the integer MMA below, together
 //               with their float block scales.
@@ -61,7 +59,7 @@ struct StreamParams {
     int split;                   // 1, 2, 4 or 8
     int max_nb;                  // largest K/32 over the layers (sizes the shared-memory arrays)
     uint32_t *status;            // device status word (bit 0: a bounded wait expired)
-    const CUtensorMap *tmaps;    // BULK: two maps per layer (device memory): [2l] over the packed
+    const CUtensorMap *tmaps;    // kernels that load by TMA: two maps per layer (device memory): [2l] over the packed
                                  // mantissas [N, K/2] bytes, box 128 x 16 rows, 128-byte swizzle;
                                  // [2l+1] over the exponent bytes [N, K/32], box 16 x 16 rows
 };
