@@ -101,3 +101,21 @@ def test_attention_on_floating_point_operands_equals_quantize_then_attention(mxb
     want = mxb.mx_attention(qm, qe, km, ke, fa, vm, ve, fa, seq, H, d, scale, fp, causal=True)
     assert mxb.mx_poll_status() == 0
     assert torch.equal(got, want)
+
+
+@pytest.mark.parametrize("d", [128, 64])
+def test_a_row_sum_is_one_chain_of_ascending_keys(mxb, d):
+    """Key 0 has weight 1, the 31 others 2^-24.5 each, less than half a step of the sum: added one after the other they leave it
+    at 1 and key 0 with the probability 1 (exponent byte 127); in any two or more partial sums they add up to some steps, the
+    probability is below 1 and its MXInt8 code the largest of the binade below, 127/128."""
+    H, seq = 2, 32
+    q = torch.zeros(seq, H * d, device="cuda")
+    q[:, ::d] = 1.0
+    k = torch.zeros(seq, H * d, device="cuda")
+    k[1:, ::d] = -17.0                                          # 17 * log2(e) = 24.53
+    v = torch.zeros(seq, H * d, device="cuda")
+    v[0] = 1.0
+    f = mxb.MxFormat(16, 8)
+    ctx = mxb.mx_attention_fp(q, k, v, f, f, H, d, 1.0, f, causal=False)
+    assert mxb.mx_poll_status() == 0
+    assert (ctx == 1.0).all()
