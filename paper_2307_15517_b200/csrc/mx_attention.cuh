@@ -122,7 +122,7 @@ __device__ __forceinline__ void prob_encode8(const float *v, int e, int w, uint3
             unpack2(fadd2(pack2(fminf(a, hi), fminf(b, hi)), n2), a, b);
             h[i] = __byte_perm(__float_as_uint(a), __float_as_uint(b), 0x7632);
         }
-    } else {                                             // only a NaN row: its values are poisoned
+    } else {                                             // only a block with a NaN: its values are poisoned
 #pragma unroll
         for (int i = 0; i < 4; ++i) h[i] = 0x7FC07FC0u;
     }
@@ -354,14 +354,15 @@ attention_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_consta
                                 v[2 * i] = exp2_approx(a);
                                 v[2 * i + 1] = exp2_approx(b);
                             }
-                            // v >= 0, or NaN in all of the row (its maximum and sum are): a NaN survives the maximum
-                            float big[2] = {v[0], v[16]};
+                            // NaN wins: the maximum and the sum of sweep 1 pass over a slice whose unmasked keys are all NaN,
+                            // so the rest of the row may well be finite
+                            float big[2] = {fabsf(v[0]), fabsf(v[16])};
 #pragma unroll
                             for (int i = 1; i < 16; ++i) {
-                                big[0] = fmaxf(big[0], v[i]);
-                                big[1] = fmaxf(big[1], v[16 + i]);
+                                big[0] = absmax_nan(big[0], v[i]);
+                                big[1] = absmax_nan(big[1], v[16 + i]);
                             }
-                            if (p.p_block == 32) big[0] = big[1] = fmaxf(big[0], big[1]);
+                            if (p.p_block == 32) big[0] = big[1] = absmax_nan(big[0], big[1]);
                             const uint32_t amax[2] = {__float_as_uint(big[0]) & 0x7FFFFFFFu, __float_as_uint(big[1]) & 0x7FFFFFFFu};
                             // the previous P tile must have been consumed before the first store of this one
                             if (cc == 0 && !__all_sync(0xFFFFFFFFu, wait(15, (n_p & 1u) ^ 1u))) { timed_out = true; break; }

@@ -119,3 +119,39 @@ def test_a_row_sum_is_one_chain_of_ascending_keys(mxb, d):
     ctx = mxb.mx_attention_fp(q, k, v, f, f, H, d, 1.0, f, causal=False)
     assert mxb.mx_poll_status() == 0
     assert (ctx == 1.0).all()
+
+
+# (first, length) of the run of non-finite keys: a key alone at either side of a 32-column chunk of the score tile, runs that
+# start there, one that fills a chunk, one across two tiles
+@pytest.mark.parametrize("d", [128, 64])
+@pytest.mark.parametrize("block", [16, 32])
+@pytest.mark.parametrize("causal", [True, False])
+@pytest.mark.parametrize("first,length", [(0, 1), (31, 1), (32, 1), (33, 1), (32, 9), (64, 32), (120, 32)])
+def test_a_non_finite_key_poisons_every_row_that_sees_it(mxb, d, block, causal, first, length):
+    """A block with a NaN or an infinity makes the outputs it touches NaN: the rows of that head whose unmasked keys include it,
+    and no others; the block of the probabilities that holds the key carries exponent byte 255.  As the unfused sequence."""
+    H, seq = 2, 160
+    hid = H * d
+    q, k, v = (synth.student_t_activations(seq, hid, 50 + i).cuda() for i in range(3))
+    k[first:first + length, d + 5] = float("nan") if length % 2 else float("inf")       # of the second head
+    fa, fp = mxb.MxFormat(block, 8), mxb.MxFormat(block, 8)
+    qm, qe = mxb.mx_quantize(q, fa)
+    km, ke = mxb.mx_quantize(k, fa)
+    vm, ve = mxb.mx_quantize(v.t(), fa)
+    scale = 1.0 / math.sqrt(d)
+    ctx, pm, pe = mxb.mx_attention(qm, qe, km, ke, fa, vm, ve, fa, seq, H, d, scale, fp, causal=causal, return_p=True)
+    assert mxb.mx_poll_status() == 0
+    sees = torch.arange(seq, device="cuda") >= first if causal else torch.ones(seq, dtype=torch.bool, device="cuda")
+    want = torch.zeros(seq, hid, dtype=torch.bool, device="cuda")
+    want[:, d:] = sees[:, None]
+    assert torch.equal(torch.isnan(ctx), want)
+    assert (pe[seq:, first // block][sees] == 255).all()
+    assert torch.equal(torch.isnan(mxb.mx_attention_fp(q, k, v, fa, fa, H, d, scale, fp, causal=causal)), want)
+    # the unfused sequence of the second head
+    s = mxb.mx_gemm(qm.view(seq, H, -1)[:, 1].contiguous(), qe.view(seq, H, -1)[:, 1].contiguous(), fa, km.view(seq, H, -1)[:, 1].contiguous(),
+                    ke.view(seq, H, -1)[:, 1].contiguous(), fa, seq, seq, d)
+    if causal:
+        s = s.masked_fill(torch.ones(seq, seq, dtype=torch.bool, device="cuda").triu(1), -math.inf)
+    sm, se = mxb.mx_quantize(torch.softmax(s * scale, dim=1), fp)
+    y = mxb.mx_gemm(sm, se, fp, vm[d:], ve[d:], fa, seq, d, seq)
+    assert torch.equal(torch.isnan(y), want[:, d:])
