@@ -36,7 +36,22 @@ const at::Tensor *tensor(PyObject *o, int *dev, bool needed)
     if (d != *dev) throw Fallback();
     return &t;
 }
+// Throws for a tensor without storage (the wrappers of vmap and grad, whose Python type is torch.Tensor as well).
+void *ptr(const at::Tensor &t) { return t.data_ptr(); }
 void *ptr(const at::Tensor *t) { return t ? t->data_ptr() : nullptr; }
+const uint8_t *bytes_of(const at::Tensor &t) { return static_cast<const uint8_t *>(t.data_ptr()); }
+const float *floats_of(const at::Tensor *t) { return static_cast<const float *>(ptr(t)); }
+
+// A call of the library without the interpreter's lock.  Its arguments are evaluated by the caller, before: what throws there
+// still holds the lock.
+template <typename F, typename... A> mx_status_t unlocked(F call, A... args)
+{
+    mx_status_t s;
+    Py_BEGIN_ALLOW_THREADS
+    s = call(args...);
+    Py_END_ALLOW_THREADS
+    return s;
+}
 
 mx_format_t format(PyObject *o)
 {
@@ -121,11 +136,8 @@ PyObject *quantize(PyObject *, PyObject *const *a, Py_ssize_t n)
         const int64_t rows = x.size(0), K = x.size(1);
         at::Tensor m = mant ? *mant : bytes(rows, f.elem_bits <= 4 ? K / 2 : K, dev);
         at::Tensor e = exps ? *exps : bytes(rows / f.block_rows, K / f.block, dev);
-        mx_status_t s;
-        Py_BEGIN_ALLOW_THREADS
-        s = mx_quantize(x.data_ptr(), dt, rows, K, x.stride(0), x.stride(1), f, m.data_ptr(), static_cast<uint8_t *>(e.data_ptr()),
-                        static_cast<uint32_t *>(ptr(count)), st);
-        Py_END_ALLOW_THREADS
+        const mx_status_t s = unlocked(mx_quantize, ptr(x), dt, rows, K, x.stride(0), x.stride(1), f, ptr(m),
+                                       static_cast<uint8_t *>(ptr(e)), static_cast<uint32_t *>(ptr(count)), st);
         if (s != MX_OK) return PyLong_FromLong(s);
         PyObject *out = PyTuple_New(2);
         if (!out) return nullptr;
@@ -155,10 +167,7 @@ PyObject *dequantize(PyObject *, PyObject *const *a, Py_ssize_t n)
                                : at::empty({rows, K}, at::TensorOptions().dtype(a[4] == Py_True ? at::kBFloat16 : at::kFloat)
                                                           .device(at::kCUDA, (c10::DeviceIndex)dev));
         const mx_dtype_t dt = value_type(out);
-        mx_status_t s;
-        Py_BEGIN_ALLOW_THREADS
-        s = mx_dequantize(mant.data_ptr(), static_cast<const uint8_t *>(exps.data_ptr()), rows, K, f, out.data_ptr(), dt, out.stride(0), st);
-        Py_END_ALLOW_THREADS
+        const mx_status_t s = unlocked(mx_dequantize, ptr(mant), bytes_of(exps), rows, K, f, ptr(out), dt, out.stride(0), st);
         if (s != MX_OK) return PyLong_FromLong(s);
         return given ? Py_NewRef(a[5]) : THPVariable_Wrap(std::move(out));
     });
@@ -183,12 +192,8 @@ PyObject *linear(PyObject *, PyObject *const *a, Py_ssize_t n)
         const int64_t M = x.size(0), K = x.size(1);
         at::Tensor y = given ? *given : floats(M, N, dev);
         const at::Tensor ws = scratch(work, work ? 0 : mx_workspace_bytes_ex(M, N, K, fa, fw, algo), dev);
-        mx_status_t s;
-        Py_BEGIN_ALLOW_THREADS
-        s = mx_linear_ex(x.data_ptr(), dt, M, K, x.stride(0), fa, wm.data_ptr(), static_cast<const uint8_t *>(we.data_ptr()), fw, N,
-                         static_cast<const float *>(ptr(bias)), static_cast<float *>(y.data_ptr()), y.stride(0), ws.data_ptr(),
-                         (size_t)ws.numel(), algo, st);
-        Py_END_ALLOW_THREADS
+        const mx_status_t s = unlocked(mx_linear_ex, ptr(x), dt, M, K, x.stride(0), fa, ptr(wm), bytes_of(we), fw, N,
+                                       floats_of(bias), static_cast<float *>(ptr(y)), y.stride(0), ptr(ws), (size_t)ws.numel(), algo, st);
         if (s != MX_OK) return PyLong_FromLong(s);
         return given ? Py_NewRef(a[7]) : THPVariable_Wrap(std::move(y));
     });
@@ -269,12 +274,9 @@ PyObject *linear_fused(PyObject *, PyObject *const *a, Py_ssize_t n)
         const mx_epilogue_t ep = epilogue(bias, a[7], residual);
         FusedResult r(a[9], y, ym, ye, M, N, dev);
         const at::Tensor ws = scratch(work, work ? 0 : mx_workspace_bytes_ex(M, N, K, fa, fw, MX_ALGO_TCGEN05), dev);
-        mx_status_t s;
-        Py_BEGIN_ALLOW_THREADS
-        s = mx_linear_fused(x.data_ptr(), dt, M, K, x.stride(0), fa, pro.layernorm ? &pro : nullptr, wm.data_ptr(),
-                            static_cast<const uint8_t *>(we.data_ptr()), fw, N, &ep, r.y_ptr(), r.ldy(N), r.fy, r.mant_ptr(), r.exp_ptr(),
-                            ws.data_ptr(), (size_t)ws.numel(), st);
-        Py_END_ALLOW_THREADS
+        const mx_status_t s = unlocked(mx_linear_fused, ptr(x), dt, M, K, x.stride(0), fa, pro.layernorm ? &pro : nullptr,
+                                       ptr(wm), bytes_of(we), fw, N, &ep, r.y_ptr(), r.ldy(N), r.fy, r.mant_ptr(), r.exp_ptr(), ptr(ws),
+                                       (size_t)ws.numel(), st);
         return s != MX_OK ? PyLong_FromLong(s) : r.wrap(a[10], a[11], a[12]);
     });
 }
@@ -298,12 +300,8 @@ PyObject *gemm_fused(PyObject *, PyObject *const *a, Py_ssize_t n)
         const mx_epilogue_t ep = epilogue(bias, a[10], residual);
         FusedResult r(a[12], y, ym, ye, M, N, dev);
         const at::Tensor ws = scratch(work, work ? 0 : mx_workspace_bytes_ex(M, N, K, fa, fw, MX_ALGO_TCGEN05), dev);
-        mx_status_t s;
-        Py_BEGIN_ALLOW_THREADS
-        s = mx_gemm_fused(am.data_ptr(), static_cast<const uint8_t *>(ae.data_ptr()), fa, wm.data_ptr(),
-                          static_cast<const uint8_t *>(we.data_ptr()), fw, M, N, K, &ep, r.y_ptr(), r.ldy(N), r.fy, r.mant_ptr(), r.exp_ptr(),
-                          ws.data_ptr(), (size_t)ws.numel(), st);
-        Py_END_ALLOW_THREADS
+        const mx_status_t s = unlocked(mx_gemm_fused, ptr(am), bytes_of(ae), fa, ptr(wm), bytes_of(we), fw, M, N, K, &ep,
+                                       r.y_ptr(), r.ldy(N), r.fy, r.mant_ptr(), r.exp_ptr(), ptr(ws), (size_t)ws.numel(), st);
         return s != MX_OK ? PyLong_FromLong(s) : r.wrap(a[13], a[14], a[15]);
     });
 }
@@ -328,12 +326,9 @@ PyObject *attention_fp(PyObject *, PyObject *const *a, Py_ssize_t n)
         const int64_t seq = q.size(0);
         at::Tensor ctx = given ? *given : floats(seq, heads * head_dim, dev);
         const at::Tensor ws = scratch(work, work ? 0 : mx_attention_workspace_bytes(seq, heads, head_dim), dev);
-        mx_status_t s;
-        Py_BEGIN_ALLOW_THREADS
-        s = mx_attention_fp(q.data_ptr(), k.data_ptr(), v.data_ptr(), dt, q.stride(0), k.stride(0), v.stride(0), fqk, fv, seq, heads,
-                            head_dim, scale, a[9] == Py_True ? 1 : 0, fp, static_cast<float *>(ctx.data_ptr()), ctx.stride(0),
-                            ws.data_ptr(), (size_t)ws.numel(), st);
-        Py_END_ALLOW_THREADS
+        const mx_status_t s = unlocked(mx_attention_fp, ptr(q), ptr(k), ptr(v), dt, q.stride(0), k.stride(0), v.stride(0), fqk,
+                                       fv, seq, heads, head_dim, scale, a[9] == Py_True ? 1 : 0, fp, static_cast<float *>(ptr(ctx)),
+                                       ctx.stride(0), ptr(ws), (size_t)ws.numel(), st);
         if (s != MX_OK) return PyLong_FromLong(s);
         return given ? Py_NewRef(a[10]) : THPVariable_Wrap(std::move(ctx));
     });

@@ -61,3 +61,43 @@ def test_errors_are_those_of_the_ctypes_route():
                 bad(**more)
             texts.append(str(e.value))
         assert texts[0] == texts[1]
+
+
+@pytest.mark.parametrize("transform", ("vmap", "grad", "functionalize"))
+def test_tensors_without_storage_are_refused_as_by_the_ctypes_route(transform):
+    """The wrappers that vmap, grad and functionalize pass in have the Python type torch.Tensor and no storage: their pointer
+    cannot be taken, in no argument of no call."""
+    f, fy = mxb.MxFormat(16, 8), mxb.MxFormat(32, 4)
+    x, q = torch.randn(32, 64, device="cuda"), torch.randn(32, 3 * 64, device="cuda")
+    (wm, we), (am, ae) = mxb.mx_quantize(torch.randn(32, 64, device="cuda"), f), mxb.mx_quantize(x, f)
+    y, ctx = torch.empty(32, 32, device="cuda"), torch.empty(32, 64, device="cuda")
+    ws = mxb.alloc_workspace(1 << 20)
+
+    def under(call, t):                                                   # `call` with a wrapper of t
+        if transform == "vmap":
+            return torch.func.vmap(call, randomness="different")(t[None])
+        if transform == "grad":
+            return torch.func.grad(lambda v: call(v).sum())(t)
+        return torch.func.functionalize(call)(t)
+
+    calls = [(x, lambda t, **m: mxb.mx_quantize(t, f, **m)[0]),
+             (wm, lambda t, **m: mxb.mx_dequantize(t, we, 64, f, **m)),
+             (x, lambda t, **m: mxb.mx_linear(t, f, wm, we, f, 32, workspace=ws, **m)),
+             (y, lambda t, **m: mxb.mx_linear(x, f, wm, we, f, 32, y=t, workspace=ws, **m)),
+             (x, lambda t, **m: mxb.mx_linear_fused(t, f, wm, we, f, 32, fy=fy, workspace=ws, **m)[0]),
+             (y, lambda t, **m: mxb.mx_linear_fused(x, f, wm, we, f, 32, residual=t, workspace=ws, **m)),
+             (am, lambda t, **m: mxb.mx_gemm_fused(t, ae, f, wm, we, f, 32, 32, 64, workspace=ws, **m)),
+             (q, lambda t, **m: mxb.mx_attention_fp(t[:, :64], t[:, 64:128], t[:, 128:], f, f, 1, 64, 0.125, f, workspace=ws, **m)),
+             (ctx, lambda t, **m: mxb.mx_attention_fp(q[:, :64], q[:, 64:128], q[:, 128:], f, f, 1, 64, 0.125, f, ctx=t, workspace=ws, **m))]
+    for t, call in calls:
+        if transform == "grad" and not t.is_floating_point():
+            continue
+        texts = []
+        for more in ({}, dict(stream=torch.cuda.current_stream())):
+            with pytest.raises(RuntimeError) as e:
+                under(lambda v: call(v, **more), t)
+            texts.append(str(e.value).splitlines()[0])
+        assert texts[0] == texts[1]
+    # the interpreter goes on, with its lock
+    assert torch.equal(mxb.mx_quantize(x, f)[0], am)
+    assert mxb.mx_poll_status() == 0
