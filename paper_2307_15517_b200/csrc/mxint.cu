@@ -1376,11 +1376,26 @@ mx_status_t launch_stream(const StreamPlan &sp, int tok, int early, const Params
 }
 
 // ---- one layer of few tokens in one launch (gemv_single_kernel) ----------------------------------------
-// Container formats whose weight rows are whole 16-byte units (the TMA boxes), one-row activation blocks.
+// Whether the result is written over the activations (y = x in place, say).  Rows of one pitch: by their columns, so that two
+// column ranges of one tensor are apart; else by the ranges of addresses, gaps between the rows included.
+bool result_over_activations(const mx_linear_args_t &a)
+{
+    const int64_t size = a.dt == MX_F32 ? 4 : 2, px = a.ldx * size, py = a.ldy * 4, nx = a.K * size, ny = a.N * 4;
+    const uintptr_t x0 = reinterpret_cast<uintptr_t>(a.x), y0 = reinterpret_cast<uintptr_t>(a.y);
+    if (y0 >= x0 + (uintptr_t)((a.M - 1) * px + nx) || x0 >= y0 + (uintptr_t)((a.M - 1) * py + ny)) return false;
+    if (px != py || a.M == 1) return true;
+    const int64_t d = (int64_t)((y0 > x0 ? y0 - x0 : x0 - y0) % (uintptr_t)px), at = y0 > x0 || d == 0 ? d : px - d;
+    return at < nx || at + ny > px;
+}
+
+// Container formats whose weight rows are whole 16-byte units (the TMA boxes), one-row activation blocks.  Its CTAs read the
+// activations while others already write results, so those must not share memory; the routes with a pass over the activations
+// in front allow it.
 bool gemv_layer_ok(const mx_linear_args_t &a)
 {
     const int64_t row_bytes = a.fw.elem_bits <= 4 ? a.K / 2 : a.K;
-    return a.M >= 1 && a.M <= 32 && format_1d(a.fa) && format_ok(a.fw) && a.fa.block == a.fw.block && (row_bytes % 16) == 0;
+    return a.M >= 1 && a.M <= 32 && format_1d(a.fa) && format_ok(a.fw) && a.fa.block == a.fw.block && (row_bytes % 16) == 0 &&
+           !result_over_activations(a);
 }
 
 struct GemvPlan { int cluster, rounds, stages, max_groups, exp_words; size_t smem; };

@@ -113,3 +113,23 @@ def test_a_tokens_bits_do_not_depend_on_the_others():
     whole = _run(x, qw, ew, None, 16, K, N, block, 8, 8, 1)
     for t0, t1 in ((0, 1), (3, 8), (7, 16)):
         assert np.array_equal(_run(x[t0:t1].contiguous(), qw, ew, None, t1 - t0, K, N, block, 8, 8, 1), whole[t0:t1])
+
+
+@pytest.mark.parametrize("T,K,N,block,ww", [(1, 768, 768, 16, 4), (4, 4096, 4096, 32, 4), (16, 2048, 2048, 16, 8), (24, 768, 768, 16, 4)])
+def test_the_result_may_take_the_activations_place(T, K, N, block, ww):
+    """y = x, rows of x that y starts later in, and two column ranges of one tensor: the activations are read before any
+    result is written."""
+    x, _, _, qw, ew, _ = _case(T, K, N, block, 8, ww, seed=41)
+    fa, fw = mxb.MxFormat(block, 8), mxb.MxFormat(block, ww)
+    wm, we = torch.from_numpy(orc.pack(qw, ww)).cuda(), torch.from_numpy(ew).cuda()
+    S = x.abs().cuda().double() @ mxb.mx_dequantize(wm, we, K, fw).abs().double().t()
+    want = mxb.mx_linear(x.cuda(), fa, wm, we, fw, N)
+    for pitch, xc, yc in ((K, 0, 0), (2 * K, 0, K // 2), (2 * K, K // 2, 0), (2 * K, 0, K), (2 * K, K, 0)):
+        buf = torch.zeros(T, pitch, device="cuda")
+        xv, yv = buf[:, xc:xc + K], buf[:, yc:yc + N]
+        xv.copy_(x)
+        mxb.mx_linear(xv, fa, wm, we, fw, N, y=yv)
+        assert ((yv - want).abs().double() <= 1e-5 * S).all()
+        if abs(xc - yc) == K:
+            assert torch.equal(yv, want) and torch.equal(xv, x.cuda())
+    assert mxb.mx_poll_status() == 0
