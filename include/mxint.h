@@ -114,7 +114,9 @@ typedef enum {
 /* Accuracy of the product kernels against the exactly summed result (Sec. 3.2 leaves the accumulator
  * across blocks open; S[i,j] = sum_b |block term b|):
  *   MX_ALGO_SIMT, MX_ALGO_STREAM : exact block sums, one fp32 rounding per block, ascending blocks;
- *                                  bit-reproducible.
+ *                                  bit-reproducible.  MX_ALGO_STREAM and mx_linear_grouped cut K into up to
+ *                                  eight pieces, added in order, where the call's rows leave warps idle
+ *                                  and the pieces are whole multiples of 128 elements in every layer.
  *   MX_ALGO_TCGEN05(_FUSED), AUTO for M > 16, the _q / fused / batched / static entry points : the tensor
  *                                  pipe aligns the products of a step (16 of bf16 operands; of block-
  *                                  scaled ones 32, or 16 where the blocks of a row lie more than 13
@@ -134,7 +136,7 @@ typedef enum {
  *   the last bits between 4-bit and 6-bit containers, between two token counts, and between mx_layernorm +
  *   mx_linear and mx_linear_fused with a LayerNorm prologue (which takes no block-scaled operands).  mx_linear,
  *   mx_linear_q and mx_linear_fused without one (mx_gemm, mx_gemm_q and mx_gemm_fused) of the same sizes share
- *   their route for M > 32.  A named algorithm, mx_gemm_batched and mx_gemm_static never cut K.
+ *   their route for M > 32.  No other named algorithm cuts K, nor do mx_gemm_batched and mx_gemm_static.
  *   MX_ALGO_TCGEN05_BLOCKWISE    : exact block sums out of the tensor pipe, one fp32 rounding per block,
  *                                  ascending blocks: the result of MX_ALGO_SIMT, bit for bit, whatever
  *                                  the operands (block terms inside the fp32 normal range). */
@@ -261,8 +263,10 @@ MX_API mx_status_t mx_gemm_ex(const void *a_mant, const uint8_t *a_exp, mx_forma
 /*
  * Y[M,N] = Q_fa(X)[M,K] * W[N,K]^T (+ bias): quantizes the activations x ([M,K] of `dt`,
  * leading dimension ldx elements, ldx % 8 == 0) to format fa on the fly and multiplies them
- * with weights already stored in format fw.  Equivalent to mx_quantize followed by mx_gemm,
- * but the quantized activations go straight to the product kernel's operand layout.
+ * with weights already stored in format fw.  The value of mx_quantize followed by mx_gemm, but the
+ * quantized activations go straight to the product kernel's operand layout; with MX_ALGO_SIMT,
+ * MX_ALGO_STREAM and MX_ALGO_TCGEN05 the same bits, with MX_ALGO_AUTO up to the order of the fp32 sums
+ * (M <= 32; the same bits beyond).  y may overlap x.
  */
 MX_API mx_status_t mx_linear(const void *x, mx_dtype_t dt, int64_t M, int64_t K, int64_t ldx,
                       mx_format_t fa, const void *w_mant, const uint8_t *w_exp, mx_format_t fw,

@@ -1487,11 +1487,12 @@ mx_status_t gemv_resident(int slot, int cluster, bool two, DeviceInfo &d, int64_
     return MX_OK;
 }
 
-// The cut of K depends on N and K alone, so a token's bits do not depend on how many others share the call.  Where the row
-// groups alone fill the chip twice over K is not cut (one chain of ascending blocks); else it is cut as often as a cluster
-// allows while the slices are whole steps or the CTAs fit at once (a step fetches 256 bytes of a row whatever its slice needs:
-// 512 x 16384, 8 bits, in eight slices of 64 bytes 35 us).  A CTA then quantizes the smallest slice of the tokens and the most
-// weight bytes are in flight.  Row groups beyond what is resident go to the same clusters, so that a staged slice is used again.
+// The cut of K depends on N and K alone, so among the calls that come here a token's bits do not depend on how many others share
+// it (one or two tokens of a large layer of 4-bit weights in blocks of 32 go elsewhere: see grouped_impl).  Where the row groups
+// alone fill the chip twice over K is not cut (one chain of ascending blocks); else it is cut as often as a cluster allows while
+// the slices are whole steps or the CTAs fit at once (a step fetches 256 bytes of a row whatever its slice needs: 512 x 16384,
+// 8 bits, in eight slices of 64 bytes 35 us).  A CTA then quantizes the smallest slice of the tokens and the most weight bytes
+// are in flight.  Row groups beyond what is resident go to the same clusters, so that a staged slice is used again.
 bool gemv_plan(const mx_linear_args_t &a, DeviceInfo &d, GemvPlan *out)
 {
     if (!gemv_layer_ok(a)) return false;
@@ -1756,7 +1757,7 @@ mx_status_t tc_prepare(const mx_linear_args_t &a, __nv_bfloat16 *a_hat, __nv_bfl
 extern "C" {
 
 static mx_status_t grouped_impl(const mx_linear_args_t *layers, int32_t n_layers,
-                                const uint8_t *const *packed_exps, void *workspace, size_t workspace_bytes,
+                                const uint8_t *const *packed_exps, bool any_order, void *workspace, size_t workspace_bytes,
                                 void *stream);
 
 size_t mx_mant_bytes(int64_t rows, int64_t K, mx_format_t f)
@@ -2004,7 +2005,7 @@ mx_status_t mx_gemm_ex(const void *a_mant, const uint8_t *a_exp, mx_format_t fa,
                                     static_cast<uint8_t *>(workspace), *dr, static_cast<cudaStream_t>(stream), EpiTail());
         }
         if (algo == MX_ALGO_AUTO) algo = can_stream ? MX_ALGO_STREAM : MX_ALGO_TCGEN05;
-        if (algo == MX_ALGO_STREAM) return grouped_impl(&one, 1, &a_exp, workspace, workspace_bytes, stream);
+        if (algo == MX_ALGO_STREAM) return grouped_impl(&one, 1, &a_exp, false, workspace, workspace_bytes, stream);
     }
     if (algo == MX_ALGO_TCGEN05_MXF8) {
         if (!mxf8_fits(fa, fw, K)) return MX_ERR_FORMAT;
@@ -2083,7 +2084,7 @@ mx_status_t mx_linear_ex(const void *x, mx_dtype_t dt, int64_t M, int64_t K, int
     if (algo == MX_ALGO_AUTO)
         algo = (stream_layer_ok(one) && (reinterpret_cast<uintptr_t>(w_exp) & 3u) == 0) ? MX_ALGO_STREAM
                                                                                      : MX_ALGO_TCGEN05;
-    if (algo == MX_ALGO_STREAM) return mx_linear_grouped(&one, 1, workspace, workspace_bytes, stream);
+    if (algo == MX_ALGO_STREAM) return grouped_impl(&one, 1, nullptr, any_algo, workspace, workspace_bytes, stream);
     if (algo != MX_ALGO_SIMT && algo != MX_ALGO_TCGEN05_FUSED && algo != MX_ALGO_TCGEN05 &&
         algo != MX_ALGO_TCGEN05_BLOCKWISE && algo != MX_ALGO_TCGEN05_MXF8)
         return MX_ERR_FORMAT;
@@ -2416,8 +2417,9 @@ size_t mx_linear_grouped_workspace_bytes(const mx_linear_args_t *layers, int32_t
 
 // packed_exps == nullptr: layers[i].x are floating-point activations, quantized here.
 // packed_exps != nullptr: layers[i].x are mantissas already in format fa, packed_exps[i] their exponents.
+// any_order: the algorithm was left open (MX_ALGO_AUTO), K may be cut over a cluster.
 static mx_status_t grouped_impl(const mx_linear_args_t *layers, int32_t n_layers,
-                                const uint8_t *const *packed_exps, void *workspace, size_t workspace_bytes,
+                                const uint8_t *const *packed_exps, bool any_order, void *workspace, size_t workspace_bytes,
                                 void *stream)
 try {
     if (!layers) return MX_ERR_NULL;
@@ -2464,11 +2466,11 @@ try {
     for (int i = 0; i < n_layers; ++i)
         boxes = boxes && (layers[i].K % 512) == 0 && (reinterpret_cast<uintptr_t>(layers[i].w_exp) & 15u) == 0 &&
                 layers[i].fw.block_rows == 1;
-    // one layer: one launch -- but for one token of a large one and two of one with very many rows, where the row-per-lane
+    // one layer, algorithm open: one launch -- but for one token of a large one and two of one with very many rows, where the row-per-lane
     // kernel's loads run ahead over more rows (K x N, one token: 4096 x 11008 8.9 against 10.2 us, 8192 x 16384 15.6 / 19.0,
     // 4096 x 32000 14.6 / 20.0, but 4096 x 4096 5.5 / 5.7 and on the host one launch less; two: 4096 x 32000 18.6 / 22.0,
     // 8192 x 16384 20.8 / 21.4, 4096 x 11008 11.0 / 10.3, 8192 x 8192 14.6 / 11.9)
-    if (n_layers == 1 && !packed_exps) {
+    if (any_order && n_layers == 1 && !packed_exps) {
         GemvPlan g;
         const int64_t n = layers[0].N, weights = n * layers[0].K;
         const bool rows = boxes && (max_t == 1 ? weights >= (1 << 25) : n >= 24576 && weights >= (1 << 26));
@@ -2629,7 +2631,7 @@ try {
 mx_status_t mx_linear_grouped(const mx_linear_args_t *layers, int32_t n_layers, void *workspace,
                               size_t workspace_bytes, void *stream)
 {
-    return grouped_impl(layers, n_layers, nullptr, workspace, workspace_bytes, stream);
+    return grouped_impl(layers, n_layers, nullptr, false, workspace, workspace_bytes, stream);
 }
 
 // ---- batched product (per-head attention matmuls) ------------------------------------------------

@@ -133,3 +133,40 @@ def test_the_result_may_take_the_activations_place(T, K, N, block, ww):
         if abs(xc - yc) == K:
             assert torch.equal(yv, want) and torch.equal(xv, x.cuda())
     assert mxb.mx_poll_status() == 0
+
+
+def _spread(x, block):
+    """Blocks up to 18 binades apart: their terms round when they are added, so that another order gives other bits."""
+    g = torch.Generator().manual_seed(7)
+    return x * torch.exp2(torch.randint(-9, 10, (x.shape[0], x.shape[1] // block), generator=g).float()).repeat_interleave(block, dim=1)
+
+
+@pytest.mark.parametrize("T", (1, 2, 4, 16))
+def test_named_stream_and_grouped_calls_keep_their_chain(T):
+    """K = 1152 has no whole pieces: one chain of ascending blocks, the CUDA-core kernel's bits, whatever AUTO does with the layer.
+    K = 4096 is cut over the warps of a CTA, the same way whether the tokens come packed or not."""
+    N = 4096
+    for K in (1152, 4096):
+        x, _, _, qw, ew, _ = _case(T, K, N, 32, 8, 4, seed=51)
+        x = _spread(x, 32)
+        fa, fw, xd = mxb.MxFormat(32, 8), mxb.MxFormat(32, 4), x.cuda()
+        wm, we = torch.from_numpy(orc.pack(qw, 4)).cuda(), torch.from_numpy(ew).cuda()
+        y = mxb.mx_linear(xd, fa, wm, we, fw, N, algo=mxb.MX_ALGO_STREAM)
+        if K == 1152:
+            assert torch.equal(y, mxb.mx_linear(xd, fa, wm, we, fw, N, algo=mxb.MX_ALGO_SIMT))
+        am, ae = mxb.mx_quantize(xd, fa)
+        assert torch.equal(y, mxb.mx_gemm(am, ae, fa, wm, we, fw, T, N, K, algo=mxb.MX_ALGO_STREAM))
+        g = torch.empty(T, N, device="cuda")
+        mxb.mx_linear_grouped(mxb.make_linear_args([dict(x=xd, fa=fa, w_mant=wm, w_exp=we, fw=fw, N=N, y=g)]))
+        assert torch.equal(y, g)
+    assert mxb.mx_poll_status() == 0
+
+
+@pytest.mark.parametrize("K,N,least", [(4096, 1500, 1), (8192, 4100, 2)])        # 4100 * 8192 > 2^25: one token goes its own way
+def test_bits_of_a_token_among_others_in_4_bits(K, N, least):
+    x, _, _, qw, ew, _ = _case(16, K, N, 32, 8, 4, seed=33)
+    x = _spread(x, 32)
+    whole = _run(x, qw, ew, None, 16, K, N, 32, 8, 4, 1)
+    for t0, t1 in ((0, 1), (2, 4), (3, 8), (7, 16)):
+        if t1 - t0 >= least:
+            assert np.array_equal(_run(x[t0:t1].contiguous(), qw, ew, None, t1 - t0, K, N, 32, 8, 4, 1), whole[t0:t1])
