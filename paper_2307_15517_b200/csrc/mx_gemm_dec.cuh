@@ -34,7 +34,7 @@ struct DecCfg {
     static constexpr int GROUPS = 3, RAW_STAGES = 3;                    // decode groups, each with a W stage; raw stages
     static constexpr int THREADS = 32 * (4 + 4 * GROUPS);
     static constexpr uint32_t PANEL_BYTES = TC_BM * TC_BK * 2, W_BYTES = BN * TC_BK * 2;
-    static constexpr uint32_t RAW_MANT = BN * 128, RAW_EXP = BN * 16;   // 128 mantissa bytes and at most 16 exponent bytes per row
+    static constexpr uint32_t RAW_MANT = BN * 128, RAW_EXP = BN * 20;   // 128 mantissa bytes and the words of at most 16 exponent bytes per row
     static constexpr int stages(int P) { return P == 1 ? 7 : P == 2 ? 3 : 2; }                   // of A: what fits
     static constexpr uint32_t smem_bytes(int P)
     {
@@ -50,7 +50,7 @@ struct DecParams {
     int w_bits, w_rows2, block;
     int split;
     int early;                // 1: the launch in front is this call's activation pass
-    int exp_words;            // 1: a step's exponent bytes are whole aligned words
+    int exp_words;            // 1: every row's exponent bytes start at a whole word
 };
 
 template <int P, bool NIB, bool QOUT>
@@ -64,6 +64,7 @@ gemm_dec_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constan
     constexpr int SPR = 128 / STEP_BYTES;                                // K steps per raw stage
     const bool b16 = dp.block == 16;
     const int EB = (NIB ? 16 : 8) >> (b16 ? 0 : 1);                      // exponent bytes of a row per raw stage
+    const int EW = (EB >> 2) + (dp.exp_words ? 0 : 1);                   // the aligned words that hold them
     extern __shared__ uint8_t smem_raw[];
     const uint32_t smem_base = (ptx::smem_u32(smem_raw) + 1023u) & ~1023u;
     uint8_t *smem_gen = smem_raw + (smem_base - ptx::smem_u32(smem_raw));
@@ -162,7 +163,7 @@ gemm_dec_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constan
         __syncwarp();
     } else if (warp == 2) {
         // raw stages: 128 rows x 128 mantissa bytes in one tiled load, their exponent bytes in the background
-        const int nb = p.K / dp.block, wpr = EB >> 2, raws = (steps + SPR - 1) / SPR;
+        const int nb = p.K / dp.block, raws = (steps + SPR - 1) / SPR;
         for (int i = 0; i < raws; ++i) {
             const int s = i % RS;
             const bool ok = ptx::mbar_wait_bounded(r_empty(s), ((uint32_t)(i / RS) & 1u) ^ 1u, abort_flag, TC_WAIT_LIMIT_NS);
@@ -177,27 +178,24 @@ gemm_dec_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constan
                 ptx::tma_load_2d(raw_base + s * Cfg::RAW_MANT, &tmap_r, kb * STEP_BYTES, n0, r_full(s));      // outside the matrix: zeros
             }
             uint8_t *dx = smem_gen + (exp_base - smem_base) + s * Cfg::RAW_EXP;
-            for (int wi = lane; wi < Cfg::BN * wpr; wi += 32) {
-                const int r = wi / wpr, b = b0 + (wi - r * wpr) * 4;
-                const uint8_t *src = dp.w_exp + (int64_t)(min(n0 + r, p.N - 1) >> dp.w_rows2) * nb;
-                if (dp.exp_words) {
-                    cp_async4(ptx::smem_u32(dx) + wi * 4, b < nb ? src + b : src, b < nb ? 4 : 0);
-                } else {
-                    uint32_t v = 0;
-#pragma unroll
-                    for (int k = 0; k < 4; ++k)
-                        if (b + k < nb) v |= (uint32_t)__ldg(src + b + k) << (8 * k);
-                    reinterpret_cast<uint32_t *>(dx)[wi] = v;
-                }
+            // whole words from the one that holds the row's first byte on, the row's end cut off (zeros): rows at odd addresses byte
+            // by byte, in plain loads, made this warp the kernel's slowest (128 x 2080 x 11008, M x K x N, 8/4 in blocks of 16: 45.9 us
+            // against 24.7; 33 x 11040 x 11008, 8/8, 393 against 95)
+            for (int wi = lane; wi < Cfg::BN * EW; wi += 32) {
+                const int r = wi / EW;
+                const uint8_t *row = dp.w_exp + (int64_t)(min(n0 + r, p.N - 1) >> dp.w_rows2) * nb;
+                const uint32_t skip = (uint32_t)reinterpret_cast<uintptr_t>(row) & 3u;         // (b0 is a multiple of 4)
+                const int at = b0 + (wi - r * EW) * 4 - (int)skip, valid = min(nb - at, 4);
+                cp_async4(ptx::smem_u32(dx) + wi * 4, row + (valid > 0 ? at : -(int)skip), max(valid, 0));
             }
-            if (dp.exp_words) cp_async_arrive(r_full(s));
-            else ptx::mbar_arrive(r_full(s));
+            cp_async_arrive(r_full(s));
         }
     } else if (warp >= 4) {
         // group g fills W stage g with the K steps g, g + 3, ...: a lane a row, both halves of the step.  Eight rows per phase of
         // a 16-byte access, chunks swizzled by the row: no bank conflicts
         const int g = (warp - 4) >> 2, r = 32 * (warp & 3) + lane;
-        const uint8_t *mrow = smem_gen + (raw_base - smem_base) + r * 128, *erow = smem_gen + (exp_base - smem_base) + r * EB;
+        const uint8_t *mrow = smem_gen + (raw_base - smem_base) + r * 128, *erow = smem_gen + (exp_base - smem_base) + r * (4 * EW) +
+                             ((uint32_t)reinterpret_cast<uintptr_t>(dp.w_exp + (int64_t)(min(n0 + r, p.N - 1) >> dp.w_rows2) * (p.K / dp.block)) & 3u);
         uint8_t *dst = smem_gen + (w_base - smem_base) + g * Cfg::W_BYTES + (r >> 3) * 1024 + (r & 7) * 128;
         for (int i = g; i < steps; i += GROUPS) {
             const int j = i % SPR, rs = i / SPR % RS;
@@ -216,7 +214,10 @@ gemm_dec_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constan
                     m[q] = *reinterpret_cast<const uint4 *>(mrow + rs * Cfg::RAW_MANT + ((c ^ (r & 7)) << 4));
                 }
                 const uint8_t *ex = erow + rs * Cfg::RAW_EXP;
-                const uint32_t e = b16 ? (uint32_t)*reinterpret_cast<const uint16_t *>(ex + 4 * j + 2 * h) : (uint32_t)ex[2 * j + h];
+                uint32_t e;
+                if (!b16) e = ex[2 * j + h];
+                else if (dp.exp_words) e = *reinterpret_cast<const uint16_t *>(ex + 4 * j + 2 * h);
+                else e = ex[4 * j + 2 * h] | (uint32_t)ex[4 * j + 2 * h + 1] << 8;
                 uint32_t o[4][4];
                 decode32<NIB>(m, e, b16, dp.w_bits, o);
 #pragma unroll
