@@ -1679,32 +1679,45 @@ mx_status_t launch_dec(const DecPlan &g, const __nv_bfloat16 *a_hat, const void 
     return MX_OK;
 }
 
-// Whether to run it, against a pass over the weights and then a product (`rec`: of block-scaled records, where
-// that one would run, else of bf16).  Whole calls in a graph, us, without -> with it; 8-bit activations, 4-bit weights, blocks
-// of 16 (records: 4 bits), B200:
+// Whether to run it, against a pass over the weights and then a product (`rec`: of block-scaled records, where that one would
+// run, else of bf16).  Whole calls in a graph, us, without -> with it; 8-bit activations, 4-bit weights, blocks of 16 (records:
+// 4 bits), B200:
 //   rows    K x N         without -> with     records        rows    K x N         without -> with     records
-//   128     768 x 768      10.4 -> 10.0    10.4 -> 10.0      160     6144 x 2048    20.9 ->  19.7    20.8 -> 19.8
-//   33      1024 x 1024     8.6 ->  9.2     8.6 ->  9.2      256     2048 x 6144    21.0 ->  20.3    20.2 -> 20.2
-//   128     1024 x 2048    10.3 -> 10.4                      256     4096 x 4096    24.5 ->  21.3    24.6 -> 21.3
-//   128     1024 x 4096    12.3 -> 10.8    13.2 -> 10.7      256     11008 x 4096   54.1 ->  41.2    53.8 -> 41.2
-//   128     2048 x 6144    17.4 -> 16.2    20.2 -> 16.3      256     4096 x 16384   63.6 ->  52.6    49.2 -> 52.8
-//   128     8192 x 2048    24.2 -> 19.3    24.1 -> 19.2      256     2560 x 10240   31.9 ->  37.4    28.6 -> 37.4
-//   128     4096 x 4096    19.6 -> 16.7    19.6 -> 16.7      384     4096 x 3072    23.9 ->  25.1    23.6 -> 24.8
-//   128     11008 x 4096   41.5 -> 30.9    41.5 -> 30.9      384     4096 x 4096    32.2 ->  27.0    28.5 -> 26.9
-//   128     4096 x 11008   44.9 -> 39.7    37.4 -> 39.6      384     11008 x 4096   76.0 ->  51.1    61.5 -> 50.8
-//   128     8192 x 28672  191.9 -> 135.2  169.0 -> 136.1     384     4096 x 11008   56.2 ->  64.6    54.1 -> 64.4
-//   256     2048 x 2048    12.7 -> 14.7    12.7 -> 14.7      384     8192 x 8192    90.8 ->  65.4    63.6 -> 64.2
-// Up to 128 rows it is the faster one where the weights are large, and where K is too short for the other product to be cut
-// (768 .. 1023; at 512, 100 rows 9.3 -> 10.1).  With more rows a CTA's steps cost more of what decoding them once saves, so there the weights have to be larger; a last
-// wave that leaves three SMs in ten idle (4096 x 11008, 2560 x 10240) costs more than it gives, as do, against records, a K that
-// is not cut.
+//   128     1024 x 4096    12.5 -> 10.7    13.1 -> 10.6      128     4096 x 22528   84.2 ->  76.6    73.9 -> 76.8
+//   128     2048 x 6144    17.4 -> 16.6    20.1 -> 16.4      128     2048 x 28672   52.0 ->  46.7    45.9 -> 46.5
+//   128     8192 x 2048    24.0 -> 19.5    24.0 -> 19.7      128     4096 x 32000  111.5 ->  77.8    94.2 -> 77.8
+//   128     4096 x 4096    19.5 -> 16.8    19.3 -> 16.8      256     2048 x 2560    13.7 ->  14.9    13.7 -> 14.9
+//   128     1024 x 9600    15.0 -> 16.4    16.2 -> 16.4      256     4096 x 4096    24.2 ->  21.9    24.0 -> 21.9
+//   64      1024 x 9600    14.5 -> 15.6    15.4 -> 15.6      256     11008 x 4096   54.1 ->  40.1    54.1 -> 39.9
+//   128     256 x 9600     13.1 -> 10.4    13.1 -> 10.4      256     1024 x 16384   19.3 ->  21.9    19.0 -> 21.9
+//   128     4096 x 9600    41.2 -> 39.7    35.4 -> 39.7      256     3072 x 14336   48.3 ->  42.2    34.8 -> 42.2
+//   128     1024 x 16384   17.2 -> 16.8    18.2 -> 16.8      256     4096 x 16384   63.9 ->  52.8    49.2 -> 52.8
+//   128     4096 x 16384   59.2 -> 39.9    47.3 -> 40.1      384     4096 x 3072    23.4 ->  24.8    23.2 -> 25.0
+//   128     1024 x 19072   20.5 -> 30.7    23.1 -> 30.5      384     4096 x 4096    31.3 ->  26.2    27.4 -> 26.4
+//   128     4096 x 19072   75.6 -> 76.0    65.9 -> 76.0      384     4096 x 6144    35.6 ->  37.7    31.3 -> 37.3
+//   128     1024 x 28672   24.4 -> 31.5    27.2 -> 31.3      384     6144 x 6144    52.2 ->  50.6    43.4 -> 50.2
+//   128     1344 x 28672   36.7 -> 36.3    35.0 -> 36.3      384     8192 x 8192    90.5 ->  63.1    63.1 -> 63.5
+// Up to 128 rows: while its CTAs make one wave that leaves at most three SMs in ten idle, wherever the weights are large.  A
+// second wave repeats ramp and exchange, which the other product overlaps with its loads: from K = 1344 on where it is full, from
+// 4096 on where not.  A single wave that is not full and not cut is worth it against bf16 only, for very short K or long.
+// Below 2 M weights the other product is not cut under 16 K steps of 64; this one, cut in three pieces from 12 steps on, is the
+// faster one then (without / with, 8/4: 64 x 768 x 256 9.6 / 8.9, 64 x 896 x 1024 10.4 / 10.2, 96 x 960 x 512 10.6 / 10.3; in two
+// pieces 64 x 704 x 512 9.5 / 10.5; against a cut one 64 x 992 x 512 8.6 / 9.4), beyond 96 rows while a piece has four steps
+// (128 x 768: N = 256 9.5 / 9.7, 512 9.9 / 9.8, 2048 10.2 / 9.9; 128 x 896 x 512 10.7 / 10.8).
+// With more rows a CTA's steps cost more of what decoding them once saves, so there the weights have to be larger, or K long.
 bool dec_is_faster(int64_t M, int64_t N, int64_t K, int split, bool rec, int sm_count)
 {
     const int64_t size = N * K, ctas = (N + mx::DecCfg::BN - 1) / mx::DecCfg::BN * split, waves = (ctas + sm_count - 1) / sm_count;
     const bool full = 10 * ctas >= 7 * waves * sm_count;
-    if (M <= 128) return (size > (1 << 21) && (full || !rec)) || (K >= 768 && K < 1024 && N >= 768);
-    if (M <= 256) return size >= 3 << 22 && N >= 2560 && full && (split >= 2 || !rec);
-    return size >= 1 << 24 && K >= 4096 && full && (split >= 3 || !rec);
+    if (M <= 128) {
+        const int64_t steps = (K + mx::TC_BK - 1) / mx::TC_BK;
+        if (size <= (1 << 21)) return steps >= 12 && steps < 16 && (M <= 96 || (steps == 12 && N >= 512));
+        if (full) return waves == 1 || K >= 1280;
+        if (rec) return false;
+        return split >= 2 || (waves == 1 ? K < 512 || K >= 3072 : K >= 4096);
+    }
+    if (M <= 256) return size >= 3 << 22 && N >= 2560 && full && (split >= 2 || (!rec && K >= 3072));
+    return size >= 1 << 24 && K >= (split == 3 ? 6144 : 4096) && full && (split >= 4 || !rec);
 }
 
 // Both operands of one layer in the tensor-core form: activations quantized straight to exact

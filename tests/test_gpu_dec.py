@@ -24,6 +24,11 @@ pytestmark = pytest.mark.gpu
     (257, 4112, 4090, 16, 8, 8, 2),        # three panels
     (384, 8192, 4096, 16, 8, 4, 1),
     (384, 4192, 4200, 32, 4, 4, 1),
+    (64, 160, 14400, 32, 6, 3, 1),         # three K steps, K not cut, one wave
+    (100, 1344, 28416, 16, 8, 4, 1),       # two waves
+    (96, 720, 130, 16, 8, 8, 1),           # few weights: twelve K steps in three pieces
+    (33, 960, 300, 32, 8, 4, 1),           # ... fifteen
+    (256, 3088, 16200, 16, 8, 6, 1),       # two panels, K not cut
 ])
 def test_weights_decoded_in_the_product(M, K, N, block, wa, ww, rows2):
     g = torch.Generator(device="cuda")
@@ -84,3 +89,28 @@ def test_exponent_rows_at_any_address_and_a_normalised_input(block, ww):
     b = mxb.mx_linear(n, fa, wm, we, fw, N, algo=mxb.MX_ALGO_TCGEN05)
     assert (a - b).norm() <= 2e-3 * b.norm()
     assert mxb.mx_poll_status() == 0
+
+
+def _launches(call):
+    mxb.mx_profile_begin()
+    call()
+    return {kind: n for kind, (_, n) in mxb.mx_profile_end().items()}
+
+
+@pytest.mark.parametrize("M,K,N,block,wa,ww,decoded", [
+    (64, 704, 512, 16, 8, 4, False), (64, 768, 512, 16, 8, 4, True), (33, 960, 256, 16, 8, 4, True), (33, 992, 256, 16, 8, 4, False),
+    (128, 768, 256, 16, 8, 4, False), (128, 768, 768, 16, 4, 4, True), (128, 896, 768, 16, 8, 4, False),
+    (128, 1024, 9600, 16, 8, 4, False), (64, 1024, 9600, 16, 8, 4, False), (128, 256, 9600, 16, 8, 4, True), (128, 4096, 9600, 16, 8, 4, True),
+    (128, 1024, 18944, 16, 8, 4, True), (128, 1024, 19072, 16, 8, 4, False), (128, 1024, 28672, 16, 8, 4, False),
+    (128, 1344, 28672, 16, 8, 4, True), (128, 4096, 19072, 16, 8, 4, True), (128, 2048, 19072, 16, 8, 4, False),
+    (256, 1024, 16384, 16, 8, 4, False), (256, 3072, 14336, 16, 8, 4, True), (384, 4096, 6144, 16, 8, 4, False),
+    (384, 4096, 4096, 16, 8, 4, True), (100, 2080, 3002, 16, 8, 4, True),
+])
+def test_sizes_at_which_the_weights_are_decoded_in_the_product(M, K, N, block, wa, ww, decoded):
+    """Either side of the lines of the rule, by the launches: with it a pass over the activations alone."""
+    fa, fw = mxb.MxFormat(block, wa), mxb.MxFormat(block, ww)
+    x = torch.randn(M, K, device="cuda")
+    wm, we = mxb.mx_quantize(torch.randn(N, K, device="cuda"), fw)
+    n = _launches(lambda: mxb.mx_linear(x, fa, wm, we, fw, N))
+    assert (n["quantize"] == 1 and n["prep"] == n["dequantize"] == 0) == decoded, n
+    assert n["gemm_tc"] == 1
