@@ -9,10 +9,14 @@ negative status from the library raises ``MxError``.
 from __future__ import annotations
 
 import ctypes as C
+import importlib.util
 import os
+import warnings
 from typing import Optional, Tuple
 
 import torch
+
+from . import build as mx_build
 
 _HERE = os.path.dirname(os.path.abspath(__file__))
 LIB_PATH = os.path.join(_HERE, "libmxint.so")
@@ -168,9 +172,28 @@ def _load() -> C.CDLL:
 
 lib = _load()
 
-from . import _calls                                              # noqa: E402  (linked against the library loaded above)
 
-_calls.set_format_type(MxFormat)
+class _NoCalls:
+    """Stands in for the native half: no call is its plain case."""
+    quantize = dequantize = linear = linear_fused = gemm_fused = attention_fp = staticmethod(lambda *args: None)
+
+
+def _load_calls():
+    """The native half of the binding (linked against the library loaded above), or its stand-in where it was not built for this
+    interpreter and torch: the calls are the same, marshalled by ctypes."""
+    try:
+        spec = importlib.util.spec_from_file_location(__package__ + "._calls", mx_build.calls_path())
+        module = importlib.util.module_from_spec(spec)
+        spec.loader.exec_module(module)
+        module.set_format_type(MxFormat)
+        return module
+    except ImportError as e:
+        warnings.warn("%s; calls are marshalled by ctypes, several microseconds each. "
+                      "`python -m paper_2307_15517_b200.build` builds the native half" % e, RuntimeWarning, stacklevel=2)
+        return _NoCalls
+
+
+_calls = _load_calls()
 
 
 def _check(status: int, where: str):

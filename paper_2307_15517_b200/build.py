@@ -1,5 +1,5 @@
-"""Builds ``libmxint.so`` in-tree with nvcc for sm_100a (cross-compiles without a GPU), and ``_calls.so``, the native half of
-the binding, with the host compiler against it and torch."""
+"""Builds ``libmxint.so`` in-tree with nvcc for sm_100a (cross-compiles without a GPU), and the native half of the binding with
+the host compiler against it, torch and the interpreter, whose versions its name carries (``calls_path``)."""
 from __future__ import annotations
 
 import os
@@ -11,7 +11,12 @@ HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libmxint.so")
 SOURCES = ["mxint.cu"]
-CALLS = os.path.join(HERE, "_calls.so")
+
+
+def calls_path() -> str:
+    """The native half of the binding for THIS interpreter and torch: another pair finds no file of its name and builds its own."""
+    import torch
+    return os.path.join(HERE, "_calls-torch%s%s" % (torch.__version__, sysconfig.get_config_var("EXT_SUFFIX")))
 
 
 def _newest_source_mtime() -> float:
@@ -25,8 +30,20 @@ def _newest_source_mtime() -> float:
 
 def build(force: bool = False, verbose: bool = False) -> str:
     newest = _newest_source_mtime()
-    if not force and all(os.path.exists(f) and os.path.getmtime(f) >= newest for f in (LIB, CALLS)):
+
+    def current(f: str) -> bool:
+        return not force and os.path.exists(f) and os.path.getmtime(f) >= newest
+
+    calls = calls_path()
+    if not current(LIB):
+        _build_library(verbose)
+    elif current(calls):
         return LIB
+    _build_calls(calls)
+    return LIB
+
+
+def _build_library(verbose: bool) -> None:
     nvcc = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")
     tmp = LIB + ".tmp.%d" % os.getpid()
     cmd = [nvcc, "-std=c++17", "-O3", "-lineinfo", "-gencode", "arch=compute_100a,code=sm_100a",
@@ -37,23 +54,21 @@ def build(force: bool = False, verbose: bool = False) -> str:
     cmd += [os.path.join(CSRC, s) for s in SOURCES]
     subprocess.check_call(cmd)
     os.replace(tmp, LIB)
-    _build_calls()
-    return LIB
 
 
-def _build_calls() -> None:
+def _build_calls(path: str) -> None:
     import torch
     root = os.path.dirname(torch.__file__)
     cuda = os.path.dirname(os.path.dirname(os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")))
     include = [os.path.join(root, "include"), os.path.join(root, "include", "torch", "csrc", "api", "include"),
                sysconfig.get_paths()["include"], os.path.join(cuda, "include")]
-    tmp = CALLS + ".tmp.%d" % os.getpid()
+    tmp = path + ".tmp.%d" % os.getpid()
     cmd = [os.environ.get("CXX", "g++"), "-std=c++17", "-O2", "-shared", "-fPIC", "-fvisibility=hidden",
            "-D_GLIBCXX_USE_CXX11_ABI=%d" % int(torch._C._GLIBCXX_USE_CXX11_ABI)] + ["-I" + d for d in include]
     cmd += ["-o", tmp, os.path.join(CSRC, "calls.cpp"), "-L" + os.path.join(root, "lib"), "-lc10", "-lc10_cuda", "-ltorch_cpu",
             "-ltorch_python", "-L" + HERE, "-l:libmxint.so", "-Wl,-rpath,$ORIGIN"]
     subprocess.check_call(cmd)
-    os.replace(tmp, CALLS)
+    os.replace(tmp, path)
 
 
 if __name__ == "__main__":

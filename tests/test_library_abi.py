@@ -187,3 +187,40 @@ def test_grouped_entry_points_report_exhausted_host_memory():
     assert r.returncode == 0, r.stderr[-500:]
     words = r.stdout.split()
     assert words[:3] == ["result", "0", "-6"] and "memory" in r.stdout
+
+
+_WITHOUT_NATIVE_CALLS = r"""
+import os, sys, warnings
+from paper_2307_15517_b200 import build
+path = os.path.join(sys.argv[1], os.path.basename(build.calls_path()))
+if sys.argv[2] == "broken":
+    open(path, "wb").write(b"of another interpreter")
+build.calls_path = lambda: path
+with warnings.catch_warnings(record=True) as w:
+    warnings.simplefilter("always")
+    from paper_2307_15517_b200 import binding as mxb
+import torch
+print("result", len([x for x in w if "ctypes" in str(x.message)]), mxb._calls.quantize(torch.zeros(2, 16), mxb.MxFormat(16, 4), None, None, None, None))
+try:
+    mxb.mx_quantize(torch.zeros(2, 16), mxb.MxFormat(16, 4))
+except ValueError as e:
+    print("error", e)
+"""
+
+
+@pytest.mark.parametrize("state", ("missing", "broken"))
+def test_binding_works_without_its_native_half(tmp_path, state):
+    """One that was built for another interpreter or torch, or not at all: the calls go through ctypes."""
+    import subprocess
+    import sys
+    mx_build.build()
+    r = subprocess.run([sys.executable, "-c", _WITHOUT_NATIVE_CALLS, str(tmp_path), state], cwd=ROOT, capture_output=True, text=True, timeout=300)
+    assert r.returncode == 0, r.stderr[-500:]
+    assert r.stdout.splitlines()[0] == "result 1 None" and "error device tensors required" in r.stdout
+
+
+def test_native_half_is_named_for_interpreter_and_torch(mxb):
+    import sysconfig
+    name = os.path.basename(mx_build.calls_path())
+    assert name.endswith(sysconfig.get_config_var("EXT_SUFFIX")) and torch.__version__ in name
+    assert os.path.exists(mx_build.calls_path()) and mxb._calls.__name__.endswith("._calls")
