@@ -2466,19 +2466,22 @@ try {
     mx_status_t s = device_info(&d);
     if (s != MX_OK) return s;
     // K is cut over the warps of a CTA only when the row tiles alone cannot fill the GPU; the pieces are whole units in every layer
-    auto choose_split = [&](int64_t tiles, int64_t warp_slots, int unit) {
+    auto choose_split = [&](int64_t tiles, int64_t warp_slots, int unit, int least) {      // least: blocks in a piece
         for (int cand = 8; tiles < warp_slots && cand > 1; cand >>= 1) {
-            bool whole = cand <= 4 || tiles * 4 < warp_slots;
-            for (int i = 0; i < n_layers && whole; ++i) whole = (layers[i].K / 32) % (unit * cand) == 0;
-            if (whole) return cand;
+            bool fits = cand <= 4 || tiles * 4 < warp_slots;
+            for (int i = 0; i < n_layers && fits; ++i) fits = (layers[i].K / 32) % (unit * cand) == 0 && layers[i].K / 32 >= least * cand;
+            if (fits) return cand;
         }
         return 1;
     };
-    // exponent boxes of one row per weight row, at 16-byte offsets (gemv_stream32_kernel)
-    bool boxes = max_t <= 2;
-    for (int i = 0; i < n_layers; ++i)
-        boxes = boxes && (layers[i].K % 512) == 0 && (reinterpret_cast<uintptr_t>(layers[i].w_exp) & 15u) == 0 &&
-                layers[i].fw.block_rows == 1;
+    // whole steps of the TMA kernels with exponent bytes of one row per weight row at 16-byte offsets
+    bool whole = true;
+    int64_t sum_weights = 0;
+    for (int i = 0; i < n_layers; ++i) {
+        whole = whole && (layers[i].K % 512) == 0 && (reinterpret_cast<uintptr_t>(layers[i].w_exp) & 15u) == 0 && layers[i].fw.block_rows == 1;
+        sum_weights += layers[i].N * layers[i].K;
+    }
+    const bool boxes = whole && max_t <= 2;              // exponents in boxes as well (gemv_stream32_kernel)
     // one layer, algorithm open: one launch -- but for one token of a large one and two of one with very many rows, where the row-per-lane
     // kernel's loads run ahead over more rows (K x N, one token: 4096 x 11008 8.9 against 10.2 us, 8192 x 16384 15.6 / 19.0,
     // 4096 x 32000 14.6 / 20.0, but 4096 x 4096 5.5 / 5.7 and on the host one launch less; two: 4096 x 32000 18.6 / 22.0,
@@ -2499,7 +2502,12 @@ try {
     auto mma_smem = [&](int warps, int stages) {                             // (8: any cut)
         return nt == 2 ? mx::MmaStreamCfg::smem_bytes<2>(max_nb / 4, warps, stages, 8) : mx::MmaStreamCfg::smem_bytes<1>(max_nb / 4, warps, stages, 8);
     };
-    for (int warps = 16; warps >= 8; warps -= 8)
+    // Few weights in rows of partial steps: the register variant, whose CTAs of eight warps spread the tiles over more of the chip
+    // and start without barriers (registers / MMA, us, B200, K x N: packed tokens, one layer, 4 tokens of 1152 x 3072 7.7 / 9.5,
+    // 2176 x 8192 12.4 / 13.0, 4224 x 4096 21.3 / 20.3, 16 of 640 x 640 6.9 / 10.5, of 1152 x 3072 10.3 / 11.3; twelve layers of
+    // 640 x 640 14.4 / 15.7, four of 1152 x 3072 11.0 / 11.2, twelve 18.5 / 17.6; beyond 8 tokens 15.4 / 16.6, 13.9 / 13.0, 26.8 / 18.5)
+    const bool few = !whole && (max_t <= 8 ? sum_weights < (1 << 23) : sum_weights < (max_nb < 768 / 32 ? 1 << 23 : packed_exps ? 1 << 22 : 0));
+    for (int warps = 16; warps >= 8 && !few; warps -= 8)
         for (int n = mx::MmaStreamCfg::MAX_STAGES; n >= 2; --n) take(StreamPlan::MMA, warps, n, 16, 16, mma_smem(warps, n));
     const bool tma = plan.kind != StreamPlan::REGS;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
@@ -2619,8 +2627,9 @@ try {
     const int fit = (int)(SMEM / (plan.smem + 1024));
     const int ctas_per_sm = plan.kind == StreamPlan::MMA || fit < 1 ? 1 : fit < 4 ? fit : 4;
     const int max_ctas = d->sm_count * ctas_per_sm;
-    int split = choose_split(total_tiles, (int64_t)max_ctas * plan.warps, plan.unit);
-    if (split == 1 && plan.kind == StreamPlan::MMA) split = choose_split(total_tiles, (int64_t)max_ctas * plan.warps, 4);
+    int split = choose_split(total_tiles, (int64_t)max_ctas * plan.warps, plan.unit, plan.unit);
+    // (a piece of less than a step costs a step: four layers of 512 x 4096, 3 tokens, in four pieces 10.0 us, not cut 7.9)
+    if (split == 1 && plan.kind == StreamPlan::MMA) split = choose_split(total_tiles, (int64_t)max_ctas * plan.warps, 4, 16);
     const int tpr = plan.warps / split;
     const int rounds = (total_tiles + tpr - 1) / tpr;
     const int grid = rounds < max_ctas ? rounds : max_ctas;
