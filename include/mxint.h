@@ -305,7 +305,9 @@ typedef struct {
  * added in fp32, in ascending order whenever there are enough weight rows to fill the GPU without
  * cutting K (always the case for tens of layers).  `layers` is HOST memory (read during the
  * call).  When host memory for the call's tables cannot be had, the size query answers 0 and the call
- * MX_ERR_CUDA with a text in mx_last_cuda_error().  Restrictions: M <= 16, both formats block 32,
+ * MX_ERR_CUDA with a text in mx_last_cuda_error(); so does a call under stream capture unless it has at
+ * most four layers with one activation tensor (larger ones copy tables from the call's host memory).
+ * Restrictions: M <= 16, both formats block 32,
  * weights elem_bits <= 4, K % 128 == 0, M*K small enough to stage in shared memory (M = 16:
  * K <= 18432); otherwise MX_ERR_SHAPE / MX_ERR_FORMAT.  mx_linear(_ex) with MX_ALGO_STREAM is the one-layer form of this call.
  */

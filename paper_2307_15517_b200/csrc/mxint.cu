@@ -2590,12 +2590,22 @@ try {
         f.block = q.block; f.elem_bits = q.w; f.exp_bits = 8; f.block_rows = block_rows;
         return quantize_rows_any(q.x, q.dt == 0 ? MX_F32 : MX_BF16, q.rows, q.K, q.ldx, f, q.out, *d, st);
     };
+    // the activations: one tensor, with its sizes as launch parameters; several, by one launch per input type over a table
+    const size_t n_jobs = jobs.size() > 1 ? jobs.size() : 0;
+    if (!in_params || n_jobs) {          // a captured copy would read this call's tables at every replay, long after they are gone
+        cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+        if (cudaStreamIsCapturing(st, &cap) != cudaSuccess) {
+            (void)cudaGetLastError();
+        } else if (cap != cudaStreamCaptureStatusNone) {
+            snprintf(t_cuda_error, sizeof(t_cuda_error), "grouped call: its tables are copied from host memory of the call, which a stream capture cannot hold "
+                     "(capture calls of up to %d layers with one activation tensor)", mx::STREAM_INLINE_LAYERS);
+            return MX_ERR_CUDA;
+        }
+    }
     for (const mx::QuantJob &q : pair_jobs) {            // the two-row quantizer, one launch per tensor
         s = quantize_one(q, 2);
         if (s != MX_OK) return s;
     }
-    // the activations: one tensor, with its sizes as launch parameters; several, by one launch per input type over a table
-    const size_t n_jobs = jobs.size() > 1 ? jobs.size() : 0;
     if (!in_params) {
         if (n_jobs) memcpy(image + job_off, jobs.data(), n_jobs * sizeof(mx::QuantJob));
         // in pieces of at most 64 KB: those travel with the commands, a larger pageable copy goes through the copy engine and

@@ -218,3 +218,39 @@ def test_two_row_and_plain_activations_of_one_call_from_two_threads(mxb):
         t.join()
     for ys in results:
         assert ys is not None and all(torch.equal(a, L["y"]) for a, L in zip(ys, layers))
+
+
+@pytest.mark.parametrize("n_layers,shared", [(4, True), (5, True), (2, False)])
+def test_a_capture_holds_only_calls_that_bring_their_tables_along(mxb, n_layers, shared):
+    """Tables that travel as launch parameters can be replayed; those that are copied from the call's host memory are refused
+    while a stream captures, before anything is launched."""
+    devs = [_layer(mxb, 3, 512, 256, 60 + i)[0] for i in range(n_layers)]
+    for d in devs:
+        if shared:
+            d["x"] = devs[0]["x"]
+    args = mxb.make_linear_args(devs)
+    ws = mxb.alloc_workspace(mxb.mx_linear_grouped_workspace_bytes(args))
+    mxb.mx_linear_grouped(args, workspace=ws)
+    torch.cuda.synchronize()
+    want = [d["y"].clone() for d in devs]
+    for d in devs:
+        d["y"].zero_()
+    graph = torch.cuda.CUDAGraph()
+    touched = torch.zeros(1, device="cuda")
+    torch.cuda.synchronize()
+    with torch.cuda.graph(graph):
+        touched += 1
+        if n_layers <= 4 and shared:
+            mxb.mx_linear_grouped(args, workspace=ws)
+        else:
+            with pytest.raises(mxb.MxError) as e:
+                mxb.mx_linear_grouped(args, workspace=ws)
+            assert e.value.status == -6 and "capture" in str(e.value)
+    graph.replay()
+    torch.cuda.synchronize()
+    assert touched.item() == 1
+    for d, w in zip(devs, want):
+        assert torch.equal(d["y"], w if n_layers <= 4 and shared else torch.zeros_like(w))
+    mxb.mx_linear_grouped(args, workspace=ws)
+    assert all(torch.equal(d["y"], w) for d, w in zip(devs, want))
+    assert mxb.mx_poll_status() == 0
