@@ -348,11 +348,13 @@ bool cached_map(const MapKey &key, CUtensorMap *out)
     *out = it->second;
     return true;
 }
+// (without host memory for the entry the map is encoded again next time: no C++ exception leaves a C function)
 void remember_map(const MapKey &key, const CUtensorMap &tm)
-{
+try {
     std::lock_guard<std::mutex> lk(g_map_mu);
     if (g_map_cache.size() > 8192) g_map_cache.clear();
     g_map_cache[key] = tm;
+} catch (const std::bad_alloc &) {
 }
 
 // The driver's tensor-map encoder, looked up once.
@@ -1262,8 +1264,14 @@ mx_status_t packed_weight_maps(const void *w_mant, const void *w_exp, int64_t N,
         if (s != MX_OK) return s;
         if (nb) s = encode_u8_rows(&wm.exps, w_exp, N, nb, 16, CU_TENSOR_MAP_SWIZZLE_NONE);
         if (s != MX_OK) return s;
-        if (g_wmap_cache.size() > 4096) g_wmap_cache.clear();
-        it = g_wmap_cache.emplace(key, wm).first;
+        out2[0] = wm.mant;
+        if (nb) out2[1] = wm.exps;
+        try {                            // without host memory for the entry they are encoded again next time
+            if (g_wmap_cache.size() > 4096) g_wmap_cache.clear();
+            g_wmap_cache.emplace(key, wm);
+        } catch (const std::bad_alloc &) {
+        }
+        return MX_OK;
     }
     out2[0] = it->second.mant;
     if (nb) out2[1] = it->second.exps;
