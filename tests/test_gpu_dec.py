@@ -114,3 +114,81 @@ def test_sizes_at_which_the_weights_are_decoded_in_the_product(M, K, N, block, w
     n = _launches(lambda: mxb.mx_linear(x, fa, wm, we, fw, N))
     assert (n["quantize"] == 1 and n["prep"] == n["dequantize"] == 0) == decoded, n
     assert n["gemm_tc"] == 1
+
+
+def check_ends_of_the_range(M, K, N, block, ww):
+    """Weight blocks with the exponent bytes 0, 225, 226, 254 and 255, a NaN and an infinity among the activations, against the
+    CUDA-core kernel: the same NaN, the other sums within the tolerance (1e-37: sums below the normal range)."""
+    g = torch.Generator(device="cuda")
+    g.manual_seed(M + ww)
+    fa, fw = mxb.MxFormat(block, 8), mxb.MxFormat(block, ww)
+    x = torch.randn(M, K, generator=g, device="cuda")
+    x[:12] *= 2.0 ** -20
+    x[2, 100], x[7, K - 1] = float("nan"), float("inf")
+    x[-1] *= 2.0 ** -110
+    wm, we = mxb.mx_quantize(torch.randn(N, K, generator=g, device="cuda") * 0.02, fw)
+    per = block // 2 if ww <= 4 else block                # bytes of a block
+    for row, blk, e in ((3, 1, 0), (4, 2, 225), (5, 3, 226), (6, 0, 254), (N - 1, K // block - 1, 255), (130, 4, 255)):
+        we[row, blk] = e
+        if e not in (0, 255):                             # one small mantissa: the row's sums stay below the largest float
+            wm[row, blk * per:(blk + 1) * per] = 0
+            wm[row, blk * per] = 1
+            x[:, blk * block] *= 2.0 ** -30
+    y = mxb.mx_linear(x, fa, wm, we, fw, N)
+    want = mxb.mx_linear(x, fa, wm, we, fw, N, algo=mxb.MX_ALGO_SIMT)
+    assert mxb.mx_poll_status() == 0
+    nan = torch.isnan(want)
+    assert nan[2].all() and nan[7].all() and nan[:, N - 1].all() and nan[:, 130].all() and not nan[0, :130].any()
+    assert torch.equal(torch.isnan(y), nan)
+    a, w = (mxb.mx_dequantize(*mxb.mx_quantize(x, fa), K, fa), mxb.mx_dequantize(wm, we, K, fw))
+    S = a.nan_to_num(0.0).abs().double() @ w.nan_to_num(0.0).abs().double().t()
+    ok = ~nan
+    assert torch.isfinite(want[ok]).all()
+    assert ((y - want).abs().double()[ok] <= 1e-5 * S[ok] + 1e-37).all()
+
+
+@pytest.mark.parametrize("M,K,N,block,ww", [(40, 4096, 2048, 16, 4), (128, 4128, 4096, 16, 8), (200, 4096, 4100, 32, 4), (300, 4112, 4224, 16, 8)])
+def test_exponents_at_the_ends_of_the_range_decoded_in_the_product(M, K, N, block, ww):
+    assert _launches(lambda: mxb.mx_linear(torch.zeros(M, K, device="cuda"), mxb.MxFormat(block, 8), *mxb.mx_quantize(
+        torch.zeros(N, K, device="cuda"), mxb.MxFormat(block, ww)), mxb.MxFormat(block, ww), N))["prep"] == 0
+    check_ends_of_the_range(M, K, N, block, ww)
+
+
+@pytest.mark.parametrize("case", ("decoded", "decoded, exponents at odd addresses", "grouped", "one token"))
+def test_weights_written_by_the_launch_in_front(case):
+    """The kernels that fetch weights while the pass over the activations still runs: weights quantized into the same buffers
+    right before each call, with nothing in between, are the ones that it uses."""
+    M, K, N = {"grouped": (5, 2048, 8192), "one token": (1, 4096, 11008)}.get(case, (128, 4096 + 16 * ("odd" in case), 4096))
+    block = 16 if "decoded" in case else 32
+    g = torch.Generator(device="cuda")
+    g.manual_seed(len(case))
+    fa, fw = mxb.MxFormat(block, 8), mxb.MxFormat(block, 8 if "odd" in case else 4)
+    x = torch.randn(M, K, generator=g, device="cuda")
+    ws = [torch.randn(N, K, generator=g, device="cuda") for _ in range(6)]
+    wm, we = mxb.mx_quantize(ws[0], fw)
+    work = mxb.alloc_workspace(mxb.mx_workspace_bytes(M, N, K, fa, fw))
+
+    def call(m, e, y):
+        if case == "grouped":
+            args = mxb.make_linear_args([dict(x=x, fa=fa, w_mant=m, w_exp=e, fw=fw, N=N, y=y)] * 2)
+            mxb.mx_linear_grouped(args, workspace=grouped)
+        else:
+            mxb.mx_linear(x, fa, m, e, fw, N, y=y, workspace=work)
+
+    if case == "grouped":
+        grouped = mxb.alloc_workspace(mxb.mx_linear_grouped_workspace_bytes(
+            mxb.make_linear_args([dict(x=x, fa=fa, w_mant=wm, w_exp=we, fw=fw, N=N, y=x)] * 2)))
+    want = []
+    for w in ws:
+        m, e = mxb.mx_quantize(w, fw)
+        want.append(torch.empty(M, N, device="cuda"))
+        torch.cuda.synchronize()
+        call(m, e, want[-1])
+        torch.cuda.synchronize()
+    got = [torch.empty(M, N, device="cuda") for _ in range(24)]
+    for i, y in enumerate(got):
+        mxb.mx_quantize(ws[i % 6], fw, wm, we)
+        call(wm, we, y)
+    for i, y in enumerate(got):
+        assert torch.equal(y, want[i % 6]), i
+    assert mxb.mx_poll_status() == 0

@@ -43,3 +43,43 @@ def test_wide_tiles_have_the_bits_of_narrow_calls(M, N, K):
             qm, qe = mxb.mx_quantize(z, fy)
             assert torch.equal(zm, qm) and torch.equal(ze, qe)
     assert mxb.mx_poll_status() == 0
+
+
+def _width(M, N, K, pairs=74):
+    """The host's rule for the width of the pair tiles (0: 256), restated: it decides what the shapes below run."""
+    rows = (M + 255) // 256
+    rounds = lambda w: (rows * ((N + w - 1) // w) + pairs - 1) // pairs      # noqa: E731
+    tile, width = K * 29 // 5, 0
+    best = (6000 + rounds(256) * tile) * 93 // 100
+    for w in range(288, 513, 32):
+        ns = 2000 + rounds(w) * (tile * max(w, 384) * 9 // 2560 + w * 75 // 4)
+        if ns < best:
+            best, width = ns, w
+    return width
+
+
+# more than 384 rows, so that no other kernel takes them; every width that the rule picks, ragged in M, N and K
+@pytest.mark.parametrize("M,N,K,width", [(414, 9686, 1040, 288), (521, 7662, 1040, 320), (528, 7936, 1040, 352), (516, 8680, 2064, 384),
+                                         (524, 9240, 2064, 416), (516, 10184, 4112, 448), (2040, 4080, 16400, 480)])
+def test_every_width_has_the_bits_of_narrow_calls(M, N, K, width):
+    assert torch.cuda.get_device_properties(0).multi_processor_count != 148 or _width(M, N, K) == width
+    g, x, fa, wm, we, fw = _operands(M, N, K, M + N)
+    bias = torch.randn(N, generator=g, device="cuda")
+    y = mxb.mx_linear(x, fa, wm, we, fw, N, bias=bias, algo=mxb.MX_ALGO_TCGEN05)
+    for n in range(0, N, 1024):
+        cols = min(1024, N - n)
+        assert torch.equal(y[:, n:n + cols], mxb.mx_linear(x, fa, wm[n:n + cols], we[n:n + cols], fw, cols, bias=bias[n:n + cols].clone(),
+                                                           algo=mxb.MX_ALGO_TCGEN05))
+    res = torch.randn(M, N, generator=g, device="cuda")
+    assert torch.equal(mxb.mx_linear_fused(x, fa, wm, we, fw, N, bias=bias, relu=True, residual=res), torch.relu(y) + res)
+    if N % 16 == 0:
+        fy = mxb.MxFormat(16, 8)
+        ym, ye = mxb.mx_linear_q(x, fa, wm, we, fw, N, fy, bias=bias)
+        qm, qe = mxb.mx_quantize(y, fy)
+        assert torch.equal(ym, qm) and torch.equal(ye, qe)
+    assert mxb.mx_poll_status() == 0
+
+
+def test_exponents_at_the_ends_of_the_range_on_wide_tiles():
+    from tests.test_gpu_dec import check_ends_of_the_range
+    check_ends_of_the_range(414, 1040, 9686, 16, 4)
