@@ -61,9 +61,13 @@ __device__ __forceinline__ uint64_t globaltimer_ns()
 // ---- programmatic dependent launch ---------------------------------------------------------------
 // A kernel launched with the programmatic-stream-serialization attribute may become resident while
 // its predecessor in the stream still runs.  dep_wait() blocks until every predecessor grid has
-// completed and its memory is visible (a no-op for an ordinary launch): nothing before it may touch
-// global memory that another kernel writes or reads.  dep_trigger() lets the next kernel of the
-// stream be scheduled once every CTA of this grid has called it or exited.
+// completed and its memory is visible (a no-op for an ordinary launch).  dep_trigger() lets the next
+// kernel of the stream be scheduled once every CTA of this grid has called it or exited.
+// Every kernel calls dep_wait() before dep_trigger().  So when a kernel starts, all grids but the one
+// right in front of it are complete: before its dep_wait() it may touch only global memory that this
+// one grid neither writes nor (if it is written here) reads.  Most kernels touch none; three, launched
+// behind a pass of their own call that writes the activations' operand form and nothing else, fetch
+// weights and tables there (gemm_dec_kernel, gemv_mma_kernel, gemv_stream32_kernel: `early`).
 __device__ __forceinline__ void dep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void dep_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 

@@ -190,7 +190,8 @@ int grid_for(int64_t work_items, int threads, int sm_count, int ctas_per_sm)
 
 // Launch that may overlap the tail of the previous kernel in the stream (programmatic dependent
 // launch): the kernel becomes resident early, sets up, and blocks in ptx::dep_wait() until its
-// predecessor has completed.  Only for kernels that call dep_wait() before touching global memory.
+// predecessor has completed.  Only for kernels that keep the rule beside dep_wait(): no global memory
+// before it but what the kernel right in front leaves alone, and dep_wait() before dep_trigger().
 template <typename... KArgs, typename... Args>
 cudaError_t launch_dep(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
                        Args &&...args)
@@ -1118,7 +1119,8 @@ mx_status_t launch_splitk(const __nv_bfloat16 *a_hat, const __nv_bfloat16 *w_hat
 // one, else 0.  A round of 256 x 256 tiles takes about 5.8 ns per k, its epilogue under the next round's MMAs; a wide one takes
 // 0.9 of that per column -- no less than for 384 columns, whose A operand alone keeps the loads busy -- and its epilogue is
 // exposed.  Products, 256 / wide (us): 512 x 11008 x 4096 61.1 / 45.0 (320: 70 tiles on 74 pairs for 86 in two rounds),
-// 2048 x 4096 x 16384 177 / 165 (480: 72 for 128), 4096 x 4096 x 11008 259 / 227, 384 x 16384 x 8192 102 / 89, 768 x 8192 x 2048
+// 2048 x 4096 x 16384 177 / 165 (480: 72 for 128), 4096 x 4096 x 11008 259 / 227, 384 x 16384 x 8192 102 / 89 (by name: AUTO decodes these
+// weights in the product), 768 x 8192 x 2048
 // 33.2 / 29.6; even or worse, and left alone: 2048 x 4096 x 4096 54.4 / 54.7, 2048 x 12288 x 4096 141 / 145,
 // 4096 x 11008 x 4096 228 / 258 (five exposed epilogues of 38 MB).
 int wide_pair_tile(int64_t M, int64_t N, int64_t K, const DeviceInfo &d)
