@@ -69,10 +69,12 @@ typedef enum {
                             activation blocks: the arithmetic of MX_ALGO_STREAM for any of them, K cut over a
                             cluster of up to eight CTAs whose sums are added in fp32, in order;
                             everything else on tensor cores, on operands that hold every value exactly:
-                            - M <= 384, weights in container form with rows of whole 16-byte units, and
-                              large enough (N * K > 2^21, more from 129 rows on): the bf16 values of
-                              MX_ALGO_TCGEN05, the weights decoded inside the product, the K range cut
-                              over a cluster of up to eight CTAs and the pieces added in fp32, in order;
+                            - M <= 384, weights in container form with rows of whole 16-byte units, where
+                              that measures faster (N * K > 2^21, more from 129 rows on, in column tiles
+                              that fill the chip or with long K; few weights for 704 < K <= 960): the
+                              bf16 values of MX_ALGO_TCGEN05, the weights decoded inside the product, the
+                              K range cut over a cluster of up to eight CTAs and the pieces added in fp32,
+                              in order;
                             - few 128 x 128 tiles (at most 74) and K of 1024 or more: the bf16 operands of
                               MX_ALGO_TCGEN05, the K range cut over a cluster of two to four CTAs and the
                               pieces added in fp32, in order;
