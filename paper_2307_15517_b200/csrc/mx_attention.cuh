@@ -73,19 +73,16 @@ struct AttnParams {
     uint32_t *status;
 };
 
-// D[tmem] (+)= A[smem tile] * B[smem tile]^T over K = 64 * HALVES (halves of four steps of 16); a_half / b_half
-// are the byte distances between the halves of the two tiles.
+// D[tmem] (+)= A[smem tile] * B[smem tile]^T over K = 64 * HALVES (halves of four steps of 16); a, b: descriptors of the two
+// tiles, a_half / b_half the distances between their halves in units of 16 bytes.
 template <int HALVES>
-__device__ __forceinline__ void attn_mma(uint32_t d_tmem, uint32_t a_tile, uint32_t a_half, uint32_t b_tile, uint32_t b_half,
-                                         uint32_t idesc, bool accumulate)
+__device__ __forceinline__ void attn_mma(uint32_t d_tmem, uint64_t a, uint32_t a_half, uint64_t b, uint32_t b_half, uint32_t idesc, bool accumulate)
 {
 #pragma unroll
     for (int hh = 0; hh < HALVES; ++hh)
 #pragma unroll
         for (int j = 0; j < 4; ++j)
-            ptx::mma_bf16_ss(d_tmem, ptx::smem_desc_k_sw128(a_tile + hh * a_half, j * 32),
-                             ptx::smem_desc_k_sw128(b_tile + hh * b_half, j * 32), idesc,
-                             (accumulate || hh || j) ? 1u : 0u);
+            ptx::mma_bf16_ss(d_tmem, a + hh * a_half + 2u * j, b + hh * b_half + 2u * j, idesc, (accumulate || hh || j) ? 1u : 0u);
 }
 
 // Item of CTA b in round k of G CTAs: the direction alternates between rounds.
@@ -217,49 +214,56 @@ attention_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_consta
         }
         __syncwarp();
     } else if (warp == 1) {
-        if (lane == 0) {
-            constexpr uint32_t idesc = ptx::idesc_bf16_f32(128, 128), idesc_o = ptx::idesc_bf16_f32(128, Cfg::D);
-            const uint32_t s_tmem[2] = {tmem_base, tmem_base + 128u}, o_tmem = tmem_base + 256u;
-            uint32_t n_item = 0, n_r = 0, n_s = 0, n_p = 0;
-            // S_j = Q K_j^T into score accumulator n_s % 2
-            auto issue_scores = [&]() -> bool {
-                const uint32_t rs = n_r % RST, si = n_s & 1u;
-                if (!wait(RING + rs, (n_r / RST) & 1u) || !wait(12 + si, ((n_s >> 1) & 1u) ^ 1u)) return false;
-                ptx::tc_fence_after_sync();
-                attn_mma<Cfg::D / 64>(s_tmem[si], q_tile, Cfg::HALF_BYTES, ring + rs * Cfg::TILE_BYTES, Cfg::HALF_BYTES, idesc, false);
+        // the whole warp runs the loop, its elected lane issues (see ptx::elect_one)
+        constexpr uint32_t idesc = ptx::idesc_bf16_f32(128, 128), idesc_o = ptx::idesc_bf16_f32(128, Cfg::D);
+        constexpr uint32_t HALF16 = Cfg::HALF_BYTES >> 4, V_HALF16 = Cfg::V_HALF_BYTES >> 4;
+        const uint32_t tm = __shfl_sync(0xFFFFFFFFu, tmem_base, 0), o_tmem = tm + 256u;
+        const uint64_t desc_q = ptx::smem_desc_k_sw128(q_tile, 0), desc_r = ptx::smem_desc_k_sw128(ring, 0), desc_p = ptx::smem_desc_k_sw128(p_tile, 0);
+        uint32_t n_item = 0, n_r = 0, n_s = 0, n_p = 0;
+        auto all = [&](bool ok) -> bool { return __all_sync(0xFFFFFFFFu, ok); };
+        auto ring_desc = [&](uint32_t rs) -> uint64_t { return desc_r + (uint64_t)(rs * (Cfg::TILE_BYTES >> 4)); };
+        // S_j = Q K_j^T into score accumulator n_s % 2
+        auto issue_scores = [&]() -> bool {
+            const uint32_t rs = n_r % RST, si = n_s & 1u;
+            if (!all(wait(RING + rs, (n_r / RST) & 1u) && wait(12 + si, ((n_s >> 1) & 1u) ^ 1u))) return false;
+            ptx::tc_fence_after_sync();
+            if (ptx::elect_one()) {
+                attn_mma<Cfg::D / 64>(tm + si * 128u, desc_q, HALF16, ring_desc(rs), HALF16, idesc, false);
                 ptx::mma_commit(bar(RING + RST + rs));      // K tile free
                 ptx::mma_commit(bar(10 + si));              // scores complete
-                ++n_r;
-                ++n_s;
-                return true;
-            };
-            for (int w = attn_item(0, blockIdx.x, gridDim.x); w < items && !timed_out; ++n_item, w = attn_item(n_item, blockIdx.x, gridDim.x)) {
-                const int qt = q_tiles_n - 1 - w / p.heads;
-                const int T = p.causal ? qt + 1 : q_tiles_n;
-                if (!wait(0, n_item & 1u)) { timed_out = true; break; }
-                for (int j = 0; j < T && !timed_out; ++j)                       // sweep 1: statistics
-                    if (!issue_scores()) timed_out = true;
-                if (timed_out) break;
-                if (!wait(17, (n_item & 1u) ^ 1u)) { timed_out = true; break; }  // previous item's context has been read
-                if (!issue_scores()) { timed_out = true; break; }                // sweep 2: S_0
-                for (int j = 0; j < T; ++j) {
-                    if (j + 1 < T) {
-                        if (!issue_scores()) { timed_out = true; break; }       // S_{j+1} runs under the softmax of S_j
-                    } else {
-                        ptx::mma_commit(bar(1));                                // every product that reads Q has been issued
-                    }
-                    const uint32_t rs = n_r % RST;
-                    if (!wait(14, n_p & 1u) || !wait(RING + rs, (n_r / RST) & 1u)) { timed_out = true; break; }
-                    ptx::tc_fence_after_sync();
-                    attn_mma<2>(o_tmem, p_tile, Cfg::HALF_BYTES, ring + rs * Cfg::TILE_BYTES, Cfg::V_HALF_BYTES, idesc_o, j > 0);
+            }
+            ++n_r;
+            ++n_s;
+            return true;
+        };
+        for (int w = attn_item(0, blockIdx.x, gridDim.x); w < items && !timed_out; ++n_item, w = attn_item(n_item, blockIdx.x, gridDim.x)) {
+            const int qt = q_tiles_n - 1 - w / p.heads;
+            const int T = p.causal ? qt + 1 : q_tiles_n;
+            if (!all(wait(0, n_item & 1u))) { timed_out = true; break; }
+            for (int j = 0; j < T && !timed_out; ++j)                       // sweep 1: statistics
+                if (!issue_scores()) timed_out = true;
+            if (timed_out) break;
+            if (!all(wait(17, (n_item & 1u) ^ 1u))) { timed_out = true; break; }  // previous item's context has been read
+            if (!issue_scores()) { timed_out = true; break; }                // sweep 2: S_0
+            for (int j = 0; j < T; ++j) {
+                if (j + 1 < T) {
+                    if (!issue_scores()) { timed_out = true; break; }       // S_{j+1} runs under the softmax of S_j
+                } else if (ptx::elect_one()) {
+                    ptx::mma_commit(bar(1));                                // every product that reads Q has been issued
+                }
+                const uint32_t rs = n_r % RST;
+                if (!all(wait(14, n_p & 1u) && wait(RING + rs, (n_r / RST) & 1u))) { timed_out = true; break; }
+                ptx::tc_fence_after_sync();
+                if (ptx::elect_one()) {
+                    attn_mma<2>(o_tmem, desc_p, HALF16, ring_desc(rs), V_HALF16, idesc_o, j > 0);
                     ptx::mma_commit(bar(RING + RST + rs));   // V tile free
                     ptx::mma_commit(bar(15));                // P tile free
-                    ++n_r;
-                    ++n_p;
                 }
-                if (timed_out) break;
-                ptx::mma_commit(bar(16));                    // context complete
+                ++n_r;
+                ++n_p;
             }
+            if (timed_out) break;
+            if (ptx::elect_one()) ptx::mma_commit(bar(16));  // context complete
         }
         __syncwarp();
     } else {

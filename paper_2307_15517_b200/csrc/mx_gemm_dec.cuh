@@ -123,43 +123,53 @@ gemm_dec_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constan
     if (threadIdx.x == 0) ptx::dep_trigger();
 
     if (warp == 0) {
-        if (lane == 0) {
-            for (int i = 0; i < steps; ++i) {
-                const int s = i % STAGES;
-                if (!ptx::mbar_wait_bounded(a_empty(s), ((uint32_t)(i / STAGES) & 1u) ^ 1u, abort_flag, TC_WAIT_LIMIT_NS)) {
-                    timed_out = true;
-                    break;
-                }
+        int s = 0;
+        uint32_t ph = 0;
+        for (int i = 0; i < steps; ++i) {
+            if (!__all_sync(0xFFFFFFFFu, ptx::mbar_wait_bounded(a_empty(s), ph ^ 1u, abort_flag, TC_WAIT_LIMIT_NS))) {
+                timed_out = true;
+                break;
+            }
+            if (ptx::elect_one()) {
                 ptx::mbar_arrive_expect_tx(a_full(s), A_BYTES);
 #pragma unroll
                 for (int q = 0; q < P; ++q)
                     ptx::tma_load_2d(smem_base + s * A_BYTES + q * Cfg::PANEL_BYTES, &tmap_a, (kb0 + i) * TC_BK, q * TC_BM, a_full(s));
             }
+            if (++s == STAGES) { s = 0; ph ^= 1u; }
         }
         __syncwarp();
     } else if (warp == 1) {
-        if (lane == 0) {
-            constexpr uint32_t idesc = ptx::idesc_bf16_f32(TC_BM, Cfg::BN);
-            for (int i = 0; i < steps; ++i) {
-                const int s = i % STAGES, g = i % GROUPS;
-                if (!ptx::mbar_wait_bounded(a_full(s), (uint32_t)(i / STAGES) & 1u, abort_flag, TC_WAIT_LIMIT_NS) ||
-                    !ptx::mbar_wait_bounded(w_full(g), (uint32_t)(i / GROUPS) & 1u, abort_flag, TC_WAIT_LIMIT_NS)) {
-                    timed_out = true;
-                    break;
-                }
-                ptx::tc_fence_after_sync();
-                const uint32_t sa = smem_base + s * A_BYTES, sw = w_base + g * Cfg::W_BYTES;
+        constexpr uint32_t idesc = ptx::idesc_bf16_f32(TC_BM, Cfg::BN);
+        const uint32_t tm = __shfl_sync(0xFFFFFFFFu, tmem_base, 0);
+        const uint64_t desc_a = ptx::smem_desc_k_sw128(smem_base, 0), desc_w = ptx::smem_desc_k_sw128(w_base, 0);
+        int s = 0, g = 0;
+        uint32_t ph = 0, gph = 0;
+        bool ready = false;                                              // the next step's operands are there already
+        for (int i = 0; i < steps; ++i) {
+            if (!ready && !__all_sync(0xFFFFFFFFu, ptx::mbar_wait_bounded(a_full(s), ph, abort_flag, TC_WAIT_LIMIT_NS) &&
+                                                   ptx::mbar_wait_bounded(w_full(g), gph, abort_flag, TC_WAIT_LIMIT_NS))) {
+                timed_out = true;
+                break;
+            }
+            ptx::tc_fence_after_sync();
+            const int cur = s, curg = g;
+            if (++s == STAGES) { s = 0; ph ^= 1u; }
+            if (++g == GROUPS) { g = 0; gph ^= 1u; }
+            const bool ahead_a = ptx::mbar_test(a_full(s), ph), ahead_w = ptx::mbar_test(w_full(g), gph);      // answers arrive meanwhile
+            if (ptx::elect_one()) {
+                const uint64_t da = desc_a + (uint64_t)((uint32_t)cur * (A_BYTES >> 4)), dw = desc_w + (uint64_t)((uint32_t)curg * (Cfg::W_BYTES >> 4));
 #pragma unroll
                 for (int q = 0; q < P; ++q)
 #pragma unroll
                     for (int j = 0; j < TC_BK / 16; ++j)
-                        ptx::mma_bf16_ss(tmem_base + 128u * q, ptx::smem_desc_k_sw128(sa + q * Cfg::PANEL_BYTES, j * 32),
-                                         ptx::smem_desc_k_sw128(sw, j * 32), idesc, (i | j) != 0 ? 1u : 0u);
-                ptx::mma_commit(a_empty(s));
-                ptx::mma_commit(w_empty(g));
+                        ptx::mma_bf16_ss(tm + 128u * q, da + (uint32_t)(q * (Cfg::PANEL_BYTES >> 4) + 2 * j), dw + 2u * j, idesc, (i | j) != 0 ? 1u : 0u);
+                ptx::mma_commit(a_empty(cur));
+                ptx::mma_commit(w_empty(curg));
             }
-            if (!timed_out) ptx::mma_commit(done_bar);
+            ready = __all_sync(0xFFFFFFFFu, ahead_a && ahead_w);
         }
+        if (!timed_out && ptx::elect_one()) ptx::mma_commit(done_bar);
         __syncwarp();
     } else if (warp == 2) {
         // raw stages: 128 rows x 128 mantissa bytes in one tiled load, their exponent bytes in the background

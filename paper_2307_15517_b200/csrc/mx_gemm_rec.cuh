@@ -253,8 +253,11 @@ gemm_rec_kernel(const __grid_constant__ RecMaps tm, const TcParams p, const RecP
     const int kgroups32 = (kblocks + 31) >> 5;
 
     if (warp == 0 || (warp == 1 && leader)) {
-        // both roles walk the tiles in groups of 32 K steps: the whole warp looks up which of them are wide (the next
-        // group's flags are on their way meanwhile), lane 0 does the work
+        // both roles walk the tiles in groups of 32 K steps: the warp looks up which of them are wide (the next group's flags
+        // are on their way meanwhile), its elected lane issues
+        const uint32_t tm_base = __shfl_sync(0xFFFFFFFFu, tmem_base, 0);
+        const uint64_t desc_a = smem_desc_rec(smem_base, REC_ROWS * 16), desc_sf = smem_desc_sf_chunk(smem_base);
+        bool ready = false;                                   // the next step's operands are there already
         int s = 0;
         uint32_t ph = 0;
         int it = 0;
@@ -269,39 +272,41 @@ gemm_rec_kernel(const __grid_constant__ RecMaps tm, const TcParams p, const RecP
         // the first stages' records are on their way while the first flags arrive; their bytes are announced, with the
         // scales', in the loop (a barrier's byte count may run ahead of its announcement)
         const int early = pair < num_tiles ? min(STAGES, kblocks) : 0;
-        if (warp == 0 && lane == 0)
+        if (warp == 0 && ptx::elect_one())
             for (int kb = 0; kb < early; ++kb) load_records(kb, (pair % p.tiles_m) * 2, (pair / p.tiles_m) * 2, kb);
         for (int t = pair; t < num_tiles; t += npairs, ++it) {
             const int m2 = (t % p.tiles_m) * 2, n2 = (t / p.tiles_m) * 2;            // first panels of the tile
             const int acc = it & 1;
-            const uint32_t d_tmem = tmem_base + (uint32_t)acc * Cfg::ACC_STEP;
+            const uint32_t d_tmem = tm_base + (uint32_t)acc * Cfg::ACC_STEP;
             for (int kg = 0; kg < kgroups32; ++kg) {
                 const uint32_t wide_mask = ahead.mask();
                 const bool last = kg + 1 == kgroups32;
                 const int tn = last ? t + npairs : t;                                // (past the last tile: panels out of range)
                 ahead.fetch(rp, (tn % p.tiles_m) * 2, (tn / p.tiles_m) * 2, last ? 0 : kg + 1, kblocks, lane);
-                if (lane != 0 || timed_out) continue;
+                if (timed_out) continue;
                 const int kb_end = min(kblocks, 32 * kg + 32);
                 if (warp == 0) {
                     const int pa = m2 + (int)rank;
                     for (int kb = 32 * kg; kb < kb_end; ++kb) {
-                        if (!ptx::mbar_wait_bounded_cluster(empty_bar(s), ph ^ 1u, abort_flag, TC_WAIT_LIMIT_NS)) {
+                        if (!__all_sync(0xFFFFFFFFu, ptx::mbar_wait_bounded_relaxed(empty_bar(s), ph ^ 1u, abort_flag, TC_WAIT_LIMIT_NS))) {
                             timed_out = true;
                             break;
                         }
-                        const bool wide = (wide_mask >> (kb & 31)) & 1u;
-                        const bool four = rec_loads_scales(wide_mask, kb);
-                        const uint32_t bytes = 2 * REC_BYTES + 3 * (wide ? REC_SFW_BYTES : four ? REC_SF_BYTES : 0u);
-                        if (leader) ptx::mbar_arrive_expect_tx(full_bar(s), 2 * bytes);
-                        const uint32_t leader_full = ptx::map_to_cta(full_bar(s), 0);
-                        const uint32_t sa = smem_base + s * Cfg::STAGE_BYTES;
-                        if (it > 0 || kb >= early) load_records(s, m2, n2, kb);
-                        if (wide) {
-                            ptx::tma_load_2d_pair(sa + Cfg::SFA_OFF, &tm.sa_wide, 0, kb * rp.panels_sa + pa, leader_full);
-                            ptx::tma_load_2d_pair(sa + Cfg::SFW_OFF, &tm.sw_wide, 0, kb * rp.panels_sw + n2, leader_full);
-                        } else if (four) {
-                            ptx::tma_load_2d_pair(sa + Cfg::SFA_OFF, &tm.sa, 0, (kb >> 2) * rp.panels_sa + pa, leader_full);
-                            ptx::tma_load_2d_pair(sa + Cfg::SFW_OFF, &tm.sw, 0, (kb >> 2) * rp.panels_sw + n2, leader_full);
+                        if (ptx::elect_one()) {
+                            const bool wide = (wide_mask >> (kb & 31)) & 1u;
+                            const bool four = rec_loads_scales(wide_mask, kb);
+                            const uint32_t bytes = 2 * REC_BYTES + 3 * (wide ? REC_SFW_BYTES : four ? REC_SF_BYTES : 0u);
+                            if (leader) ptx::mbar_arrive_expect_tx(full_bar(s), 2 * bytes);
+                            const uint32_t leader_full = ptx::map_to_cta(full_bar(s), 0);
+                            const uint32_t sa = smem_base + s * Cfg::STAGE_BYTES;
+                            if (it > 0 || kb >= early) load_records(s, m2, n2, kb);
+                            if (wide) {
+                                ptx::tma_load_2d_pair(sa + Cfg::SFA_OFF, &tm.sa_wide, 0, kb * rp.panels_sa + pa, leader_full);
+                                ptx::tma_load_2d_pair(sa + Cfg::SFW_OFF, &tm.sw_wide, 0, kb * rp.panels_sw + n2, leader_full);
+                            } else if (four) {
+                                ptx::tma_load_2d_pair(sa + Cfg::SFA_OFF, &tm.sa, 0, (kb >> 2) * rp.panels_sa + pa, leader_full);
+                                ptx::tma_load_2d_pair(sa + Cfg::SFW_OFF, &tm.sw, 0, (kb >> 2) * rp.panels_sw + n2, leader_full);
+                            }
                         }
                         if (++s == STAGES) { s = 0; ph ^= 1u; }
                     }
@@ -310,62 +315,69 @@ gemm_rec_kernel(const __grid_constant__ RecMaps tm, const TcParams p, const RecP
                 // tile it may start when the epilogue has left the columns it shares with tile it - 1 (every warp has
                 // by then finished tile it - 2, which lay where tile it goes)
                 if (kg == 0 && it > 0 &&
-                    !ptx::mbar_wait_bounded_cluster(drained_bar, (uint32_t)(it - 1) & 1u, abort_flag, TC_WAIT_LIMIT_NS)) {
+                    !__all_sync(0xFFFFFFFFu, ptx::mbar_wait_bounded_relaxed(drained_bar, (uint32_t)(it - 1) & 1u, abort_flag, TC_WAIT_LIMIT_NS))) {
                     timed_out = true;
                     continue;
                 }
                 ptx::tc_fence_after_sync();
-                // One K step; WIDE_MAY: some step of the group is wide.  The common loop is compiled without the wide step:
-                // the one thread that issues the MMAs has about 600 cycles per step, and the shared loop cost 2.5 us of
-                // 38 on 2048 x 6144 x 2048.
+                // One K step; WIDE_MAY: some step of the group is wide.  The common loop is compiled without the wide step: the
+                // issuing lane has about 500 clocks per step.
                 auto steps = [&](auto may_c) {
                     constexpr bool WIDE_MAY = decltype(may_c)::value;
                     constexpr uint32_t CHUNK = REC_ROWS * 16;                // bytes of one k-chunk of a record
                     for (int kb = 32 * kg; kb < kb_end; ++kb) {
-                        if (!ptx::mbar_wait_bounded_cluster(full_bar(s), ph, abort_flag, TC_WAIT_LIMIT_NS)) {
+                        if (!ready && !__all_sync(0xFFFFFFFFu, ptx::mbar_wait_bounded(full_bar(s), ph, abort_flag, TC_WAIT_LIMIT_NS))) {
                             timed_out = true;
                             return;
                         }
                         ptx::tc_fence_after_sync();
-                        const uint32_t sa = smem_base + s * Cfg::STAGE_BYTES;
-                        const uint32_t sw = sa + Cfg::W_OFF;
-                        // scales: shared -> tensor memory, executed in order ahead of the MMAs below; `step`: bytes from W's
-                        // first panel to its second
-                        auto load_scales = [&](uint32_t off, uint32_t step) {
-                            set ^= 1u;
-                            const uint32_t tsf = tmem_base + Cfg::SF_COL + set * Cfg::SF_SET;
-                            tmem_cp_32x128b_warpx4_pair(tsf, smem_desc_sf_chunk(sa + Cfg::SFA_OFF + off));
-                            tmem_cp_32x128b_warpx4_pair(tsf + 4, smem_desc_sf_chunk(sa + Cfg::SFW_OFF + off));
-                            tmem_cp_32x128b_warpx4_pair(tsf + 8, smem_desc_sf_chunk(sa + Cfg::SFW_OFF + off + step));
-                        };
-                        if (!WIDE_MAY || !((wide_mask >> (kb & 31)) & 1u)) {
-                            if (WIDE_MAY ? rec_loads_scales(wide_mask, kb) : (kb & 3) == 0) load_scales(0, REC_SF_BYTES);
-                            const uint32_t tsf = tmem_base + Cfg::SF_COL + set * Cfg::SF_SET;
-                            const uint32_t idesc = idesc_mxf8_e4m3(256, BN, (uint32_t)(kb & 3));
+                        const int cur = s;
+                        if (++s == STAGES) { s = 0; ph ^= 1u; }
+                        const bool there = ptx::mbar_test(full_bar(s), ph);  // its answer arrives while the MMAs are issued
+                        const bool wide = WIDE_MAY && ((wide_mask >> (kb & 31)) & 1u);
+                        const bool scales = wide || (WIDE_MAY ? rec_loads_scales(wide_mask, kb) : (kb & 3) == 0);
+                        const uint32_t first = set ^ 1u;                     // the set that this step's scales go to, if it loads any
+                        if (scales && !wide) set ^= 1u;                      // (a wide step loads twice and ends where it began)
+                        if (ptx::elect_one()) {
+                            const uint32_t off16 = (uint32_t)cur * (Cfg::STAGE_BYTES >> 4);
+                            const uint64_t da = desc_a + off16, dw = da + (Cfg::W_OFF >> 4), dsf = desc_sf + off16;
+                            // scales: shared -> tensor memory, executed in order ahead of the MMAs below; `step`: bytes from W's
+                            // first panel to its second
+                            auto load_scales = [&](uint32_t tsf, uint32_t off, uint32_t step) {
+                                tmem_cp_32x128b_warpx4_pair(tsf, dsf + ((Cfg::SFA_OFF + off) >> 4));
+                                tmem_cp_32x128b_warpx4_pair(tsf + 4, dsf + ((Cfg::SFW_OFF + off) >> 4));
+                                tmem_cp_32x128b_warpx4_pair(tsf + 8, dsf + ((Cfg::SFW_OFF + off + step) >> 4));
+                            };
+                            if (!wide) {
+                                const uint32_t tsf = tm_base + Cfg::SF_COL + set * Cfg::SF_SET;
+                                if (scales) load_scales(tsf, 0, REC_SF_BYTES);
+                                const uint32_t idesc = idesc_mxf8_e4m3(256, BN, (uint32_t)(kb & 3));
 #pragma unroll
-                            for (int j = 0; j < REC_K / 32; ++j)
-                                mma_mxf8_ss_pair(d_tmem, smem_desc_rec(sa + 2 * j * CHUNK, CHUNK), smem_desc_rec(sw + 2 * j * CHUNK, CHUNK),
-                                                 idesc, tsf, tsf + 4, (kb | j) != 0 ? 1u : 0u);
-                        } else {
+                                for (int j = 0; j < REC_K / 32; ++j)
+                                    mma_mxf8_ss_pair(d_tmem, da + (uint32_t)(2 * j * CHUNK >> 4), dw + (uint32_t)(2 * j * CHUNK >> 4), idesc, tsf, tsf + 4,
+                                                     (kb | j) != 0 ? 1u : 0u);
+                            } else {
+                                const uint32_t sa = smem_base + cur * Cfg::STAGE_BYTES, sw = sa + Cfg::W_OFF;
 #pragma unroll 1
-                            for (int h = 0; h < 2; ++h) {
-                                load_scales(512 * h, REC_SFW_BYTES);
-                                const uint32_t tsf = tmem_base + Cfg::SF_COL + set * Cfg::SF_SET;
+                                for (int h = 0; h < 2; ++h) {
+                                    const uint32_t tsf = tm_base + Cfg::SF_COL + (first ^ (uint32_t)h) * Cfg::SF_SET;
+                                    load_scales(tsf, 512 * h, REC_SFW_BYTES);
 #pragma unroll
-                                for (int j = 0; j < REC_K / 32; ++j) {
-                                    const uint32_t ca = sa + (2 * j + h) * CHUNK, cw = sw + (2 * j + h) * CHUNK;
-                                    mma_mxf8_ss_pair(d_tmem, smem_desc_rec(ca, zero_base - ca), smem_desc_rec(cw, zero_base - cw),
-                                                     idesc_mxf8_e4m3(256, BN, (uint32_t)j), tsf, tsf + 4, (kb | h | j) != 0 ? 1u : 0u);
+                                    for (int j = 0; j < REC_K / 32; ++j) {
+                                        const uint32_t ca = sa + (2 * j + h) * CHUNK, cw = sw + (2 * j + h) * CHUNK;
+                                        mma_mxf8_ss_pair(d_tmem, smem_desc_rec(ca, zero_base - ca), smem_desc_rec(cw, zero_base - cw),
+                                                         idesc_mxf8_e4m3(256, BN, (uint32_t)j), tsf, tsf + 4, (kb | h | j) != 0 ? 1u : 0u);
+                                    }
                                 }
                             }
+                            ptx::mma_commit_pair(empty_bar(cur), 3);         // both CTAs may refill the stage
                         }
-                        ptx::mma_commit_pair(empty_bar(s), 3);          // both CTAs may refill the stage
-                        if (++s == STAGES) { s = 0; ph ^= 1u; }
+                        ready = __all_sync(0xFFFFFFFFu, there);
                     }
                 };
                 if (wide_mask == 0) steps(std::false_type{});
                 else steps(std::true_type{});
-                if (kg + 1 == kgroups32 && !timed_out) ptx::mma_commit_pair(tfull_bar(acc), 3);   // both halves of the accumulator are complete
+                if (kg + 1 == kgroups32 && !timed_out && ptx::elect_one()) ptx::mma_commit_pair(tfull_bar(acc), 3);   // both halves of the accumulator are complete
             }
         }
         __syncwarp();
@@ -391,7 +403,7 @@ gemm_rec_kernel(const __grid_constant__ RecMaps tm, const TcParams p, const RecP
                 if (QOUT) tail_fetch(p, row, n0 + column(0), row_ahead);
                 else frag_tail_fetch(p, rows0, n0 + column(0), lane, frag_ahead);
             }
-            const bool ok = ptx::mbar_wait_bounded_cluster(tfull_bar(acc), acc_ph, abort_flag, TC_WAIT_LIMIT_NS);
+            const bool ok = ptx::mbar_wait_bounded_relaxed(tfull_bar(acc), acc_ph, abort_flag, TC_WAIT_LIMIT_NS);
             if (!__all_sync(0xFFFFFFFFu, ok)) {
                 timed_out = true;
                 break;
@@ -400,7 +412,7 @@ gemm_rec_kernel(const __grid_constant__ RecMaps tm, const TcParams p, const RecP
             auto release = [&]() {                                  // warp-collective
                 ptx::tc_fence_before_sync();
                 __syncwarp();
-                if (lane == 0) ptx::mbar_arrive_cluster(ptx::map_to_cta(drained_bar, 0));
+                if (lane == 0) ptx::mbar_arrive_cluster_relaxed(ptx::map_to_cta(drained_bar, 0));
             };
             if (!has_shared) release();
             const uint32_t t_acc = tmem_base + ((uint32_t)(quad * 32) << 16) + (uint32_t)acc * Cfg::ACC_STEP;

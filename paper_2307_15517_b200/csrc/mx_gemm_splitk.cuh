@@ -229,43 +229,47 @@ gemm_splitk_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_cons
     bool timed_out = false;
 
     if (warp == 0) {
-        if (lane == 0) {
-            int s = 0;
-            uint32_t ph = 0;
-            for (int kb = kb0; kb < kb1; ++kb) {
-                if (!ptx::mbar_wait_bounded(empty_bar(s), ph ^ 1u, abort_flag, TC_WAIT_LIMIT_NS)) {
-                    timed_out = true;
-                    break;
-                }
+        int s = 0;
+        uint32_t ph = 0;
+        for (int kb = kb0; kb < kb1; ++kb) {
+            if (!__all_sync(0xFFFFFFFFu, ptx::mbar_wait_bounded(empty_bar(s), ph ^ 1u, abort_flag, TC_WAIT_LIMIT_NS))) {
+                timed_out = true;
+                break;
+            }
+            if (ptx::elect_one()) {
                 ptx::mbar_arrive_expect_tx(full_bar(s), Cfg::STAGE_BYTES);
                 const uint32_t sa = smem_base + s * Cfg::STAGE_BYTES;
                 ptx::tma_load_2d(sa, &tmap_a, kb * TC_BK, m0, full_bar(s));
                 ptx::tma_load_2d(sa + Cfg::A_BYTES, &tmap_w, kb * TC_BK, n0, full_bar(s));
-                if (++s == STAGES) { s = 0; ph ^= 1u; }
             }
+            if (++s == STAGES) { s = 0; ph ^= 1u; }
         }
         __syncwarp();
     } else if (warp == 1) {
-        if (lane == 0) {
-            constexpr uint32_t idesc = ptx::idesc_bf16_f32(TC_BM, Cfg::BN);
-            int s = 0;
-            uint32_t ph = 0;
-            for (int kb = kb0; kb < kb1; ++kb) {
-                if (!ptx::mbar_wait_bounded(full_bar(s), ph, abort_flag, TC_WAIT_LIMIT_NS)) {
-                    timed_out = true;
-                    break;
-                }
-                ptx::tc_fence_after_sync();
-                const uint32_t sa = smem_base + s * Cfg::STAGE_BYTES, sw = sa + Cfg::A_BYTES;
-#pragma unroll
-                for (int j = 0; j < TC_BK / 16; ++j)
-                    ptx::mma_bf16_ss(tmem_base, ptx::smem_desc_k_sw128(sa, j * 32), ptx::smem_desc_k_sw128(sw, j * 32), idesc,
-                                     (kb != kb0 || j != 0) ? 1u : 0u);
-                ptx::mma_commit(empty_bar(s));
-                if (++s == STAGES) { s = 0; ph ^= 1u; }
+        constexpr uint32_t idesc = ptx::idesc_bf16_f32(TC_BM, Cfg::BN);
+        const uint32_t tm = __shfl_sync(0xFFFFFFFFu, tmem_base, 0);
+        const uint64_t desc0 = ptx::smem_desc_k_sw128(smem_base, 0);
+        int s = 0;
+        uint32_t ph = 0;
+        bool ready = false;                                          // the next step's operands are there already
+        for (int kb = kb0; kb < kb1; ++kb) {
+            if (!ready && !__all_sync(0xFFFFFFFFu, ptx::mbar_wait_bounded(full_bar(s), ph, abort_flag, TC_WAIT_LIMIT_NS))) {
+                timed_out = true;
+                break;
             }
-            if (!timed_out) ptx::mma_commit(done_bar);
+            ptx::tc_fence_after_sync();
+            const int cur = s;
+            if (++s == STAGES) { s = 0; ph ^= 1u; }
+            const bool ahead = ptx::mbar_test(full_bar(s), ph);      // its answer arrives while the MMAs are issued
+            if (ptx::elect_one()) {
+                const uint64_t da = desc0 + (uint64_t)((uint32_t)cur * (Cfg::STAGE_BYTES >> 4)), dw = da + (Cfg::A_BYTES >> 4);
+#pragma unroll
+                for (int j = 0; j < TC_BK / 16; ++j) ptx::mma_bf16_ss(tm, da + 2u * j, dw + 2u * j, idesc, (kb != kb0 || j != 0) ? 1u : 0u);
+                ptx::mma_commit(empty_bar(cur));
+            }
+            ready = __all_sync(0xFFFFFFFFu, ahead);
         }
+        if (!timed_out && ptx::elect_one()) ptx::mma_commit(done_bar);
         __syncwarp();
     } else {
         // the partial tile: tensor memory -> this CTA's shared memory.  All its loads have landed and all its MMAs have

@@ -467,17 +467,17 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant
     bool timed_out = false;
 
     if (warp == 0) {
-        if (lane == 0) {
-            int s = 0;
-            uint32_t ph = 0;
-            for (int t = blockIdx.x; t < num_tiles && !timed_out; t += gridDim.x) {
-                const int tb = t / tiles_item, tt = t - tb * tiles_item;
-                const int m0 = (tt % p.tiles_m) * TC_BM, n0 = (tt / p.tiles_m) * BN;
-                for (int kb = 0; kb < kblocks; ++kb) {
-                    if (!ptx::mbar_wait_bounded(empty_bar(s), ph ^ 1u, abort_flag, TC_WAIT_LIMIT_NS)) {
-                        timed_out = true;
-                        break;
-                    }
+        int s = 0;
+        uint32_t ph = 0;
+        for (int t = blockIdx.x; t < num_tiles && !timed_out; t += gridDim.x) {
+            const int tb = t / tiles_item, tt = t - tb * tiles_item;
+            const int m0 = (tt % p.tiles_m) * TC_BM, n0 = (tt / p.tiles_m) * BN;
+            for (int kb = 0; kb < kblocks; ++kb) {
+                if (!__all_sync(0xFFFFFFFFu, ptx::mbar_wait_bounded(empty_bar(s), ph ^ 1u, abort_flag, TC_WAIT_LIMIT_NS))) {
+                    timed_out = true;
+                    break;
+                }
+                if (ptx::elect_one()) {
                     ptx::mbar_arrive_expect_tx(full_bar(s), FUSED ? Cfg::A_BYTES : Cfg::STAGE_BYTES);
                     const uint32_t sa = smem_base + s * Cfg::STAGE_BYTES;
                     if (!FUSED && p.batch > 1) {
@@ -487,46 +487,45 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant
                         ptx::tma_load_2d(sa, &tmap_a, kb * TC_BK, m0, full_bar(s));
                         if (!FUSED) ptx::tma_load_2d(sa + Cfg::A_BYTES, &tmap_w, kb * TC_BK, n0, full_bar(s));
                     }
-                    if (++s == STAGES) { s = 0; ph ^= 1u; }
                 }
+                if (++s == STAGES) { s = 0; ph ^= 1u; }
             }
         }
         __syncwarp();
     } else if (warp == 1) {
-        if (lane == 0) {
-            constexpr uint32_t idesc = ptx::idesc_bf16_f32(TC_BM, BN);
-            int s = 0;
-            uint32_t ph = 0;
-            int it = 0;
-            for (int t = blockIdx.x; t < num_tiles && !timed_out; t += gridDim.x, ++it) {
-                const int acc = it & 1;
-                const uint32_t acc_ph = (uint32_t)(it >> 1) & 1u;
-                if (!ptx::mbar_wait_bounded(tempty_bar(acc), acc_ph ^ 1u, abort_flag, TC_WAIT_LIMIT_NS)) {
-                    timed_out = true;
-                    break;
-                }
-                ptx::tc_fence_after_sync();
-                const uint32_t d_tmem = tmem_base + (uint32_t)(acc * BN);
-                for (int kb = 0; kb < kblocks; ++kb) {
-                    if (!ptx::mbar_wait_bounded(full_bar(s), ph, abort_flag, TC_WAIT_LIMIT_NS)) {
+        constexpr uint32_t idesc = ptx::idesc_bf16_f32(TC_BM, BN);
+        const uint32_t tm = __shfl_sync(0xFFFFFFFFu, tmem_base, 0);
+        const uint64_t desc0 = ptx::smem_desc_k_sw128(smem_base, 0);
+        int s = 0, it = 0;
+        uint32_t ph = 0;
+        bool ready = false;                                  // the next step's operands are there already
+        for (int t = blockIdx.x; t < num_tiles && !timed_out; t += gridDim.x, ++it) {
+            const int acc = it & 1;
+            const uint32_t acc_ph = (uint32_t)(it >> 1) & 1u;
+            bool ok = ptx::mbar_wait_bounded(tempty_bar(acc), acc_ph ^ 1u, abort_flag, TC_WAIT_LIMIT_NS);
+            const uint32_t d_tmem = tm + (uint32_t)(acc * BN);
+            for (int kb = 0; kb < kblocks; ++kb) {
+                if (kb == 0 || !ready) {
+                    ok = ok && (ready || ptx::mbar_wait_bounded(full_bar(s), ph, abort_flag, TC_WAIT_LIMIT_NS));
+                    if (!__all_sync(0xFFFFFFFFu, ok)) {
                         timed_out = true;
                         break;
                     }
-                    ptx::tc_fence_after_sync();
-                    const uint32_t sa = smem_base + s * Cfg::STAGE_BYTES;
-                    const uint32_t sw = sa + Cfg::A_BYTES;
-#pragma unroll
-                    for (int j = 0; j < TC_BK / 16; ++j) {
-                        ptx::mma_bf16_ss(d_tmem, ptx::smem_desc_k_sw128(sa, j * 32),
-                                         ptx::smem_desc_k_sw128(sw, j * 32), idesc,
-                                         (kb | j) != 0 ? 1u : 0u);
-                    }
-                    ptx::mma_commit(empty_bar(s));          // stage free once these MMAs retire
-                    if (++s == STAGES) { s = 0; ph ^= 1u; }
                 }
-                if (timed_out) break;
-                ptx::mma_commit(tfull_bar(acc));            // accumulator complete
+                ptx::tc_fence_after_sync();
+                const int cur = s;
+                if (++s == STAGES) { s = 0; ph ^= 1u; }
+                const bool ahead = ptx::mbar_test(full_bar(s), ph);      // its answer arrives while the MMAs are issued
+                if (ptx::elect_one()) {
+                    const uint64_t da = desc0 + (uint64_t)((uint32_t)cur * (Cfg::STAGE_BYTES >> 4)), dw = da + (Cfg::A_BYTES >> 4);
+#pragma unroll
+                    for (int j = 0; j < TC_BK / 16; ++j) ptx::mma_bf16_ss(d_tmem, da + 2u * j, dw + 2u * j, idesc, (kb | j) != 0 ? 1u : 0u);
+                    ptx::mma_commit(empty_bar(cur));                         // stage free once these MMAs retire
+                }
+                ready = __all_sync(0xFFFFFFFFu, ahead);
             }
+            if (timed_out) break;
+            if (ptx::elect_one()) ptx::mma_commit(tfull_bar(acc));          // accumulator complete
         }
         __syncwarp();
     } else if (WMODE == W_NIBBLE_PERM && warp >= TC_THREADS / 32) {

@@ -102,61 +102,61 @@ gemm_tc2_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constan
     bool timed_out = false;
 
     if (warp == 0) {
-        if (lane == 0) {
-            int s = 0;
-            uint32_t ph = 0;
-            for (int t = pair; t < num_tiles && !timed_out; t += npairs) {
-                const int m0 = (t % p.tiles_m) * 256 + (int)rank * 128;
-                const int n0 = (t / p.tiles_m) * BN + (int)rank * (BN / 2);
-                for (int kb = 0; kb < kblocks; ++kb) {
-                    if (!ptx::mbar_wait_bounded_cluster(empty_bar(s), ph ^ 1u, abort_flag, TC_WAIT_LIMIT_NS)) {
-                        timed_out = true;
-                        break;
-                    }
+        int s = 0;
+        uint32_t ph = 0;
+        for (int t = pair; t < num_tiles && !timed_out; t += npairs) {
+            const int m0 = (t % p.tiles_m) * 256 + (int)rank * 128;
+            const int n0 = (t / p.tiles_m) * BN + (int)rank * (BN / 2);
+            for (int kb = 0; kb < kblocks; ++kb) {
+                if (!__all_sync(0xFFFFFFFFu, ptx::mbar_wait_bounded_relaxed(empty_bar(s), ph ^ 1u, abort_flag, TC_WAIT_LIMIT_NS))) {
+                    timed_out = true;
+                    break;
+                }
+                if (ptx::elect_one()) {
                     if (leader) ptx::mbar_arrive_expect_tx(full_bar(s), 2 * Cfg::STAGE_BYTES);
                     const uint32_t leader_full = ptx::map_to_cta(full_bar(s), 0);
                     const uint32_t sa = smem_base + s * Cfg::STAGE_BYTES;
                     ptx::tma_load_2d_pair(sa, &tmap_a, kb * TC_BK, m0, leader_full);
                     ptx::tma_load_2d_pair(sa + Cfg::A_BYTES, &tmap_w, kb * TC_BK, n0, leader_full);
-                    if (++s == STAGES) { s = 0; ph ^= 1u; }
                 }
+                if (++s == STAGES) { s = 0; ph ^= 1u; }
             }
         }
         __syncwarp();
     } else if (warp == 1) {
-        if (lane == 0 && leader) {
-            constexpr uint32_t idesc = ptx::idesc_bf16_f32(256, BN);
-            int s = 0;
-            uint32_t ph = 0;
-            int it = 0;
-            for (int t = pair; t < num_tiles && !timed_out; t += npairs, ++it) {
-                const int acc = it & 1;
-                const uint32_t acc_ph = (uint32_t)(it >> 1) & 1u;
-                if (!ptx::mbar_wait_bounded_cluster(tempty_bar(acc), acc_ph ^ 1u, abort_flag, TC_WAIT_LIMIT_NS)) {
-                    timed_out = true;
-                    break;
-                }
-                ptx::tc_fence_after_sync();
-                const uint32_t d_tmem = tmem_base + (uint32_t)(acc * BN);
-                for (int kb = 0; kb < kblocks; ++kb) {
-                    if (!ptx::mbar_wait_bounded_cluster(full_bar(s), ph, abort_flag, TC_WAIT_LIMIT_NS)) {
+        constexpr uint32_t idesc = ptx::idesc_bf16_f32(256, BN);
+        const uint32_t tm = __shfl_sync(0xFFFFFFFFu, tmem_base, 0);
+        const uint64_t desc0 = ptx::smem_desc_k_sw128(smem_base, 0);
+        int s = 0, it = 0;
+        uint32_t ph = 0;
+        bool ready = false;                                  // the next step's operands are there already
+        for (int t = leader ? pair : num_tiles; t < num_tiles && !timed_out; t += npairs, ++it) {
+            const int acc = it & 1;
+            const uint32_t acc_ph = (uint32_t)(it >> 1) & 1u;
+            bool ok = ptx::mbar_wait_bounded_relaxed(tempty_bar(acc), acc_ph ^ 1u, abort_flag, TC_WAIT_LIMIT_NS);
+            const uint32_t d_tmem = tm + (uint32_t)(acc * BN);
+            for (int kb = 0; kb < kblocks; ++kb) {
+                if (kb == 0 || !ready) {
+                    ok = ok && (ready || ptx::mbar_wait_bounded(full_bar(s), ph, abort_flag, TC_WAIT_LIMIT_NS));
+                    if (!__all_sync(0xFFFFFFFFu, ok)) {
                         timed_out = true;
                         break;
                     }
-                    ptx::tc_fence_after_sync();
-                    const uint32_t sa = smem_base + s * Cfg::STAGE_BYTES;
-                    const uint32_t sw = sa + Cfg::A_BYTES;
-#pragma unroll
-                    for (int j = 0; j < TC_BK / 16; ++j) {
-                        ptx::mma_bf16_ss_pair(d_tmem, ptx::smem_desc_k_sw128(sa, j * 32),
-                                              ptx::smem_desc_k_sw128(sw, j * 32), idesc, (kb | j) != 0 ? 1u : 0u);
-                    }
-                    ptx::mma_commit_pair(empty_bar(s), 3);          // both CTAs may refill the stage
-                    if (++s == STAGES) { s = 0; ph ^= 1u; }
                 }
-                if (timed_out) break;
-                ptx::mma_commit_pair(tfull_bar(acc), 3);            // both halves of the accumulator are complete
+                ptx::tc_fence_after_sync();
+                const int cur = s;
+                if (++s == STAGES) { s = 0; ph ^= 1u; }
+                const bool ahead = ptx::mbar_test(full_bar(s), ph);      // its answer arrives while the MMAs are issued
+                if (ptx::elect_one()) {
+                    const uint64_t da = desc0 + (uint64_t)((uint32_t)cur * (Cfg::STAGE_BYTES >> 4)), dw = da + (Cfg::A_BYTES >> 4);
+#pragma unroll
+                    for (int j = 0; j < TC_BK / 16; ++j) ptx::mma_bf16_ss_pair(d_tmem, da + 2u * j, dw + 2u * j, idesc, (kb | j) != 0 ? 1u : 0u);
+                    ptx::mma_commit_pair(empty_bar(cur), 3);                         // both CTAs may refill the stage
+                }
+                ready = __all_sync(0xFFFFFFFFu, ahead);
             }
+            if (timed_out) break;
+            if (ptx::elect_one()) ptx::mma_commit_pair(tfull_bar(acc), 3);          // accumulator complete
         }
         __syncwarp();
     } else {
@@ -173,7 +173,7 @@ gemm_tc2_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constan
             const int row = m0 + quad * 32 + lane;
             TailRegs ahead;
             if (tail) tail_fetch(p, row, n0 + col0, ahead);    // the first chunk's residual: in flight under the MMAs
-            const bool ok = ptx::mbar_wait_bounded_cluster(tfull_bar(acc), acc_ph, abort_flag, TC_WAIT_LIMIT_NS);
+            const bool ok = ptx::mbar_wait_bounded_relaxed(tfull_bar(acc), acc_ph, abort_flag, TC_WAIT_LIMIT_NS);
             if (!__all_sync(0xFFFFFFFFu, ok)) {
                 timed_out = true;
                 break;
@@ -204,7 +204,7 @@ gemm_tc2_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constan
             }
             ptx::tc_fence_before_sync();
             __syncwarp();
-            if (lane == 0) ptx::mbar_arrive_cluster(ptx::map_to_cta(tempty_bar(acc), 0));
+            if (lane == 0) ptx::mbar_arrive_cluster_relaxed(ptx::map_to_cta(tempty_bar(acc), 0));
         }
         if (p.tma_store && lane == 0) ptx::bulk_wait_group<0>();
     }

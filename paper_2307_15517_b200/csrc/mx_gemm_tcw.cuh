@@ -81,60 +81,63 @@ gemm_tcw_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constan
     bool timed_out = false;
 
     if (warp == 0) {
-        if (lane == 0) {
-            int s = 0;
-            uint32_t ph = 0;
-            for (int t = pair; t < num_tiles && !timed_out; t += npairs) {
-                const int m0 = (t % p.tiles_m) * 256 + (int)rank * 128;
-                const int n0 = (t / p.tiles_m) * width + (int)rank * (bn / 2);     // this CTA's rows of either half
-                for (int kb = 0; kb < kblocks; ++kb) {
-                    if (!ptx::mbar_wait_bounded_cluster(empty_bar(s), ph ^ 1u, abort_flag, TC_WAIT_LIMIT_NS)) {
-                        timed_out = true;
-                        break;
-                    }
+        int s = 0;
+        uint32_t ph = 0;
+        for (int t = pair; t < num_tiles && !timed_out; t += npairs) {
+            const int m0 = (t % p.tiles_m) * 256 + (int)rank * 128;
+            const int n0 = (t / p.tiles_m) * width + (int)rank * (bn / 2);     // this CTA's rows of either half
+            for (int kb = 0; kb < kblocks; ++kb) {
+                if (!__all_sync(0xFFFFFFFFu, ptx::mbar_wait_bounded_relaxed(empty_bar(s), ph ^ 1u, abort_flag, TC_WAIT_LIMIT_NS))) {
+                    timed_out = true;
+                    break;
+                }
+                if (ptx::elect_one()) {
                     if (leader) ptx::mbar_arrive_expect_tx(full_bar(s), 2 * stage_bytes);
                     const uint32_t leader_full = ptx::map_to_cta(full_bar(s), 0);
                     const uint32_t sa = smem_base + s * stage_bytes, sw = sa + Cfg::A_BYTES;
                     ptx::tma_load_2d_pair(sa, &tmap_a, kb * TC_BK, m0, leader_full);
                     ptx::tma_load_2d_pair(sw, &tmap_w, kb * TC_BK, n0, leader_full);
                     ptx::tma_load_2d_pair(sw + (uint32_t)bn * TC_BK, &tmap_w, kb * TC_BK, n0 + bn, leader_full);
-                    if (++s == stages) { s = 0; ph ^= 1u; }
                 }
+                if (++s == stages) { s = 0; ph ^= 1u; }
             }
         }
         __syncwarp();
     } else if (warp == 1) {
-        if (lane == 0 && leader) {
-            const uint32_t idesc = ptx::idesc_bf16_f32(256, bn);
-            int s = 0;
-            uint32_t ph = 0;
-            int it = 0;
-            for (int t = pair; t < num_tiles && !timed_out; t += npairs, ++it) {
-                if (!ptx::mbar_wait_bounded_cluster(tempty_bar, ((uint32_t)it & 1u) ^ 1u, abort_flag, TC_WAIT_LIMIT_NS)) {
-                    timed_out = true;
-                    break;
-                }
-                ptx::tc_fence_after_sync();
-                for (int kb = 0; kb < kblocks; ++kb) {
-                    if (!ptx::mbar_wait_bounded_cluster(full_bar(s), ph, abort_flag, TC_WAIT_LIMIT_NS)) {
+        const uint32_t idesc = ptx::idesc_bf16_f32(256, bn);
+        const uint32_t tm = __shfl_sync(0xFFFFFFFFu, tmem_base, 0);
+        const uint64_t desc0 = ptx::smem_desc_k_sw128(smem_base, 0);
+        const uint32_t half16 = (uint32_t)bn * TC_BK >> 4;       // a half's rows, in units of 16 bytes
+        int s = 0, it = 0;
+        uint32_t ph = 0;
+        bool ready = false;                                      // the next step's operands are there already
+        for (int t = leader ? pair : num_tiles; t < num_tiles && !timed_out; t += npairs, ++it) {
+            bool ok = ptx::mbar_wait_bounded_relaxed(tempty_bar, ((uint32_t)it & 1u) ^ 1u, abort_flag, TC_WAIT_LIMIT_NS);
+            for (int kb = 0; kb < kblocks; ++kb) {
+                if (kb == 0 || !ready) {
+                    ok = ok && (ready || ptx::mbar_wait_bounded(full_bar(s), ph, abort_flag, TC_WAIT_LIMIT_NS));
+                    if (!__all_sync(0xFFFFFFFFu, ok)) {
                         timed_out = true;
                         break;
                     }
-                    ptx::tc_fence_after_sync();
-                    const uint32_t sa = smem_base + s * stage_bytes, sw = sa + Cfg::A_BYTES;
+                }
+                ptx::tc_fence_after_sync();
+                const int cur = s;
+                if (++s == stages) { s = 0; ph ^= 1u; }
+                const bool ahead = ptx::mbar_test(full_bar(s), ph);      // its answer arrives while the MMAs are issued
+                if (ptx::elect_one()) {
+                    const uint64_t da = desc0 + (uint64_t)((uint32_t)cur * (stage_bytes >> 4)), dw = da + (Cfg::A_BYTES >> 4);
 #pragma unroll
                     for (int h = 0; h < 2; ++h)
 #pragma unroll
                         for (int j = 0; j < TC_BK / 16; ++j)
-                            ptx::mma_bf16_ss_pair(tmem_base + (uint32_t)(h * bn), ptx::smem_desc_k_sw128(sa, j * 32),
-                                                  ptx::smem_desc_k_sw128(sw + (uint32_t)(h * bn) * TC_BK, j * 32), idesc,
-                                                  (kb | j) != 0 ? 1u : 0u);
-                    ptx::mma_commit_pair(empty_bar(s), 3);          // both CTAs may refill the stage
-                    if (++s == stages) { s = 0; ph ^= 1u; }
+                            ptx::mma_bf16_ss_pair(tm + (uint32_t)(h * bn), da + 2u * j, dw + (h ? half16 : 0u) + 2u * j, idesc, (kb | j) != 0 ? 1u : 0u);
+                    ptx::mma_commit_pair(empty_bar(cur), 3);             // both CTAs may refill the stage
                 }
-                if (timed_out) break;
-                ptx::mma_commit_pair(tfull_bar, 3);
+                ready = __all_sync(0xFFFFFFFFu, ahead);
             }
+            if (timed_out) break;
+            if (ptx::elect_one()) ptx::mma_commit_pair(tfull_bar, 3);
         }
         __syncwarp();
     } else {
@@ -150,7 +153,7 @@ gemm_tcw_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constan
                 if (QOUT) tail_fetch(p, row, n0 + 32 * group, row_ahead);
                 else frag_tail_fetch(p, rows0, n0 + 32 * group, lane, frag_ahead);
             }
-            const bool ok = ptx::mbar_wait_bounded_cluster(tfull_bar, (uint32_t)it & 1u, abort_flag, TC_WAIT_LIMIT_NS);
+            const bool ok = ptx::mbar_wait_bounded_relaxed(tfull_bar, (uint32_t)it & 1u, abort_flag, TC_WAIT_LIMIT_NS);
             if (!__all_sync(0xFFFFFFFFu, ok)) {
                 timed_out = true;
                 break;
@@ -178,7 +181,7 @@ gemm_tcw_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constan
             }
             ptx::tc_fence_before_sync();
             __syncwarp();
-            if (lane == 0) ptx::mbar_arrive_cluster(ptx::map_to_cta(tempty_bar, 0));
+            if (lane == 0) ptx::mbar_arrive_cluster_relaxed(ptx::map_to_cta(tempty_bar, 0));
         }
     }
 

@@ -102,6 +102,20 @@ __device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity)
     return ok != 0;
 }
 
+// One look at the phase with `parity`, without waiting.
+__device__ __forceinline__ bool mbar_test(uint32_t bar, uint32_t parity)
+{
+    uint32_t ok;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(ok)
+        : "r"(bar), "r"(parity)
+        : "memory");
+    return ok != 0;
+}
+
 // Bounded wait: polls until the phase with `parity` completes, the CTA-wide abort flag is
 // raised, or `limit_ns` of wall time has passed.  Returns false in the last two cases.
 __device__ __forceinline__ bool mbar_wait_bounded(uint32_t bar, uint32_t parity,
@@ -267,6 +281,34 @@ __device__ __forceinline__ bool mbar_wait_bounded_cluster(uint32_t bar, uint32_t
         }
     }
 }
+// Arrival and bounded wait that order nothing but tensor-memory accesses (with tcgen05.fence on either side) and the completion
+// of asynchronous copies and MMAs: what the pair's pipeline barriers are for.  Release and acquire at cluster scope also order
+// the thread's accesses to global and shared memory, which none of that needs and which costs the thread microseconds.
+__device__ __forceinline__ void mbar_arrive_cluster_relaxed(uint32_t cluster_addr)
+{
+    asm volatile("mbarrier.arrive.relaxed.cluster.shared::cluster.b64 _, [%0];" ::"r"(cluster_addr) : "memory");
+}
+__device__ __forceinline__ bool mbar_wait_bounded_relaxed(uint32_t bar, uint32_t parity, volatile uint32_t *abort_flag, uint64_t limit_ns)
+{
+    uint64_t t0 = 0;
+    for (uint32_t it = 1;; ++it) {
+        uint32_t ok;
+        asm volatile(
+            "{\n\t.reg .pred p;\n\t"
+            "mbarrier.try_wait.parity.relaxed.cluster.shared::cta.b64 p, [%1], %2;\n\t"
+            "selp.u32 %0, 1, 0, p;\n\t}"
+            : "=r"(ok)
+            : "r"(bar), "r"(parity)
+            : "memory");
+        if (ok) return true;
+        if ((it & 0x3FF) == 0) {
+            if (*abort_flag) return false;
+            const uint64_t now = globaltimer_ns();
+            if (t0 == 0) t0 = now;
+            else if (now - t0 > limit_ns) return false;
+        }
+    }
+}
 // 2-D tiled load into this CTA's shared memory whose bytes are counted on a barrier of the pair's
 // leader CTA (`bar_cluster`: a shared::cluster address).  No multicast.
 __device__ __forceinline__ void tma_load_2d_pair(uint32_t dst_smem, const void *tmap, int32_t x, int32_t y,
@@ -313,6 +355,18 @@ __device__ __forceinline__ void mma_commit_pair(uint32_t bar, uint16_t cta_mask)
     asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;" ::"r"(bar),
                  "h"(cta_mask)
                  : "memory");
+}
+
+// One lane of the (whole, converged) warp: the same every time.  The warps that issue TMA loads and MMAs run their loops as a
+// whole and let the elected lane issue: what a loop computes is then uniform and stays in uniform registers, which the issuing
+// instructions take their operands from.  With a loop of one lane (`if (lane == 0)`) four MMAs and two commits took 470 clocks
+// to issue, now 230, and those loops bounded the products: whole calls 384 x 8192 x 8192 63 -> 59 us (8/4 bits), 4096^3 89 -> 79
+// (4/4), 4096 x 11008 x 4096 181 -> 158 (4/2).
+__device__ __forceinline__ bool elect_one()
+{
+    uint32_t p;
+    asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xFFFFFFFF;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(p));
+    return p != 0;
 }
 
 // ---- MMA -------------------------------------------------------------------------------------
