@@ -537,101 +537,83 @@ quantize_strided_kernel(const InT *__restrict__ x, int64_t rows, int64_t K, int6
     }
 }
 
-// Blocks along the slow axis of a row-major tensor (stride_row == 1: x[r, k] = base[k * stride_k + r],
-// e.g. V of attention quantized along the token axis).  A CTA owns 32 rows r and walks k in tiles of
-// 256: every warp reads 128 contiguous bytes per k (coalesced), the tile is transposed through
-// shared memory, then 8 lanes cover the 256 k of one row -- 32 consecutive k each, i.e. two blocks
-// of 16 or one of 32 -- so that they write 128 (nibbles) or 256 contiguous bytes per row.
-// Tile element (r, k) sits at r * 264 + k + k / 32: with this padding both the transposing store
-// and the per-lane reads are (nearly) free of bank conflicts.
-// CTA-wide body (256 threads, every thread must call it): CTA `cta` of `n_ctas` walks the 32 x 256 tiles.
+// Blocks along the slow axis of a row-major tensor (stride_row == 1: x[r, k] = base[k * stride_k + r], e.g. V of attention
+// quantized along the token axis).  Item of a warp: 32 rows x 32 k, a lane a row, whose 32 values it has in flight at once;
+// neighbouring lanes read neighbouring columns, 64 or 128 contiguous bytes per k, and a lane's results are whole sectors (half a
+// sector for nibbles) of its row.  Nothing is exchanged: a block of 16 or 32 is a lane's own registers.
+// Bound by HBM, below some 4 M elements by one round trip to memory.  Through tiles of 32 x 256 in shared memory, a warp's loads
+// came in eight round trips one after another (bf16 to MXInt5 and fp32 to MXInt4, us, tiles / this): 352 x 2048 4.9 / 2.4 and
+// 4.5 / 2.4, 2048 x 2048 8.9 / 6.2 and 8.6 / 7.7, 8192 x 2048 26 / 17 and 31 / 20, 16384 x 8192 217 / 123 and 219 / 132.
+// K % 32 == 0; every lane of the warp may be called with any item.
 template <typename InT>
-__device__ __forceinline__ void quantize_transposed_body(float *tile, const InT *__restrict__ x, int64_t rows, int64_t K,
-                                                         int64_t stride_k, int block, int w, const QuantOut &out,
-                                                         int cta, int n_ctas)
+__device__ __forceinline__ void quantize_columns_body(const InT *__restrict__ x, int64_t rows, int64_t K, int64_t stride_k, int block, int w,
+                                                      const QuantOut &out, int64_t warp_id, int64_t n_warps)
 {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int lane = threadIdx.x & 31;
+    const int64_t row_tiles = (rows + 31) >> 5, items = row_tiles * (K >> 5), nb_row = K / block;
     const bool nibble = w <= 4;
-    const int64_t nb_row = K / block, mant_ld = nibble ? (K >> 1) : K;
-    const int64_t row_tiles = (rows + 31) >> 5, k_tiles = (K + 255) >> 8;
-    for (int64_t tix = cta; tix < row_tiles * k_tiles; tix += n_ctas) {
-        const int64_t r0 = (tix % row_tiles) * 32, k0 = (tix / row_tiles) * 256;
-        __syncthreads();                                    // the previous tile has been consumed
-#pragma unroll 4
-        for (int kk = warp; kk < 256; kk += 8) {
-            const int64_t k = k0 + kk;
-            float v = 0.f;
-            if (k < K && r0 + lane < rows) v = (float)x[k * stride_k + r0 + lane];
-            tile[lane * 264 + kk + (kk >> 5)] = v;
+    for (int64_t it = warp_id; it < items; it += n_warps) {
+        const int64_t kt = it / row_tiles, row = (it - kt * row_tiles) * 32 + lane, k0 = kt * 32;
+        if (row >= rows) continue;
+        const InT *src = x + k0 * stride_k + row;
+        float v[4][8];
+#pragma unroll
+        for (int i = 0; i < 32; ++i) v[i >> 3][i & 7] = (float)src[i * stride_k];
+        uint32_t amax[2];
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            float am = 0.f;
+#pragma unroll
+            for (int i = 0; i < 16; ++i) am = absmax_nan(am, v[2 * h + (i >> 3)][i & 7]);
+            amax[h] = __float_as_uint(am);
         }
-        __syncthreads();
-        const int r = threadIdx.x >> 3, kg = threadIdx.x & 7;       // 32 k starting at k0 + 32 * kg of row r0 + r
-        const int64_t row = r0 + r, kb = k0 + 32 * kg;
-        if (row < rows && kb < K) {                                  // K % block == 0 and 32 % block == 0: whole blocks
-            const float *src = tile + r * 264 + kg * 33;
-            float v[4][8];
-            uint32_t amax[2] = {0u, 0u};
+        if (block == 32) amax[0] = amax[1] = max(amax[0], amax[1]);
+        const int e[2] = {(int)(amax[0] >> 23), (int)(amax[1] >> 23)};                // 255 <=> an Inf or NaN in the block
+        uint2 pk[4];
 #pragma unroll
-            for (int c = 0; c < 4; ++c) {
-                float am = 0.f;
-#pragma unroll
-                for (int i = 0; i < 8; ++i) {
-                    v[c][i] = src[c * 8 + i];
-                    am = absmax_nan(am, v[c][i]);
-                }
-                amax[c >> 1] = max(amax[c >> 1], __float_as_uint(am));
+        for (int c = 0; c < 4; ++c) {
+            float xh[8];
+            pk[c] = encode8_full(v[c], e[c >> 1], w, xh);
+            if (out.xhat) {                                                           // the decoded values, exact in bf16
+                uint4 h;
+                h.x = as_u32(__floats2bfloat162_rn(xh[0], xh[1]));
+                h.y = as_u32(__floats2bfloat162_rn(xh[2], xh[3]));
+                h.z = as_u32(__floats2bfloat162_rn(xh[4], xh[5]));
+                h.w = as_u32(__floats2bfloat162_rn(xh[6], xh[7]));
+                *reinterpret_cast<uint4 *>(out.xhat + row * out.ld_xhat + k0 + 8 * c) = h;
             }
-            if (block == 32) amax[0] = amax[1] = max(amax[0], amax[1]);
-            uint2 pk[4];
-#pragma unroll
-            for (int c = 0; c < 4; ++c) {
-                float xh[8];
-                pk[c] = encode8_full(v[c], (int)(amax[c >> 1] >> 23), w, xh);
-                if (out.xhat) {                                       // the decoded values, exact in bf16
-                    uint4 h;
-                    h.x = as_u32(__floats2bfloat162_rn(xh[0], xh[1]));
-                    h.y = as_u32(__floats2bfloat162_rn(xh[2], xh[3]));
-                    h.z = as_u32(__floats2bfloat162_rn(xh[4], xh[5]));
-                    h.w = as_u32(__floats2bfloat162_rn(xh[6], xh[7]));
-                    *reinterpret_cast<uint4 *>(out.xhat + row * out.ld_xhat + kb + 8 * c) = h;
-                }
-            }
-            if (!out.mant) continue;                                  // operand form only
-            if (nibble)
-                *reinterpret_cast<uint4 *>(out.mant + row * mant_ld + (kb >> 1)) = make_uint4(pk[0].x, pk[1].x, pk[2].x, pk[3].x);
-            else {
-                uint4 *dst = reinterpret_cast<uint4 *>(out.mant + row * mant_ld + kb);
-                dst[0] = make_uint4(pk[0].x, pk[0].y, pk[1].x, pk[1].y);
-                dst[1] = make_uint4(pk[2].x, pk[2].y, pk[3].x, pk[3].y);
-            }
-            const int e0 = (int)(amax[0] >> 23), e1 = (int)(amax[1] >> 23);
-            if (block == 32) {
-                out.exps[row * nb_row + (kb >> 5)] = (uint8_t)e0;
-                if (e0 == 255 && out.nonfinite) atomicAdd(out.nonfinite, 1u);
-            } else {
-                out.exps[row * nb_row + (kb >> 4)] = (uint8_t)e0;
-                out.exps[row * nb_row + (kb >> 4) + 1] = (uint8_t)e1;
-                if (out.nonfinite) {
-                    if (e0 == 255) atomicAdd(out.nonfinite, 1u);
-                    if (e1 == 255) atomicAdd(out.nonfinite, 1u);
-                }
-            }
+        }
+        if (!out.mant) continue;                                                      // operand form only
+        if (nibble) {
+            *reinterpret_cast<uint4 *>(out.mant + row * (K >> 1) + (k0 >> 1)) = make_uint4(pk[0].x, pk[1].x, pk[2].x, pk[3].x);
+        } else {
+            uint4 *dst = reinterpret_cast<uint4 *>(out.mant + row * K + k0);
+            dst[0] = make_uint4(pk[0].x, pk[0].y, pk[1].x, pk[1].y);
+            dst[1] = make_uint4(pk[2].x, pk[2].y, pk[3].x, pk[3].y);
+        }
+        uint8_t *de = out.exps + row * nb_row + k0 / block;
+        de[0] = (uint8_t)e[0];
+        if (block == 16) de[1] = (uint8_t)e[1];
+        if (out.nonfinite) {
+            if (e[0] == 255) atomicAdd(out.nonfinite, 1u);
+            if (block == 16 && e[1] == 255) atomicAdd(out.nonfinite, 1u);
         }
     }
 }
 
+// One item per warp, CTAs of two warps.
 template <typename InT>
-__global__ void __launch_bounds__(256)
-quantize_transposed_kernel(const InT *__restrict__ x, int64_t rows, int64_t K, int64_t stride_k, int block, int w,
-                           QuantOut out)
+__global__ void __launch_bounds__(64)
+quantize_columns_kernel(const InT *__restrict__ x, int64_t rows, int64_t K, int64_t stride_k, int block, int w, const QuantOut out)
 {
-    __shared__ float tile[32 * 264];
-    quantize_transposed_body<InT>(tile, x, rows, K, stride_k, block, w, out, (int)blockIdx.x, (int)gridDim.x);
+    ptx::dep_wait();
+    ptx::dep_trigger();
+    quantize_columns_body<InT>(x, rows, K, stride_k, block, w, out, (int64_t)blockIdx.x * 2 + (threadIdx.x >> 5), (int64_t)gridDim.x * 2);
 }
 
 // The three operands of the fused attention in one launch (256 threads per CTA): every warp takes its share of the
-// rows of q and of k (blocks along the head dimension, written in operand form), then every CTA its share of the
-// tiles of v (blocks along the tokens, written transposed).
+// rows of q and of k (blocks along the head dimension, written in operand form), then of v (blocks along the tokens, written
+// transposed).
 struct AttnOperandsJob {
     const void *q, *k, *v;
     int64_t seq, hid, ldq, ldk, ldv;
@@ -644,13 +626,13 @@ template <typename InT>
 __global__ void __launch_bounds__(256)
 attention_operands_kernel(const AttnOperandsJob j)
 {
-    __shared__ float tile[32 * 264];
     ptx::dep_wait();
     ptx::dep_trigger();
     const int warps = blockDim.x >> 5;
     const int64_t wid = (int64_t)blockIdx.x * warps + (threadIdx.x >> 5), nw = (int64_t)gridDim.x * warps;
     const QuantOut oq{nullptr, nullptr, j.q_hat, j.hid, nullptr, 0}, ok{nullptr, nullptr, j.k_hat, j.hid, nullptr, 0};
-    const int64_t wk = after_items((uint32_t)wid, (uint32_t)nw, (uint32_t)(j.seq * ((j.hid + 255) >> 8)));
+    const uint32_t row_items = (uint32_t)(j.seq * ((j.hid + 255) >> 8));
+    const int64_t wk = after_items((uint32_t)wid, (uint32_t)nw, row_items), wv = after_items((uint32_t)wk, (uint32_t)nw, row_items);
     if (j.block_qk == 16) {
         quantize_rows_body<InT, 16, 2>(static_cast<const InT *>(j.q), j.seq, j.hid, j.ldq, j.w_qk, oq, wid, nw);
         quantize_rows_body<InT, 16, 2>(static_cast<const InT *>(j.k), j.seq, j.hid, j.ldk, j.w_qk, ok, wk, nw);
@@ -659,8 +641,7 @@ attention_operands_kernel(const AttnOperandsJob j)
         quantize_rows_body<InT, 32, 2>(static_cast<const InT *>(j.k), j.seq, j.hid, j.ldk, j.w_qk, ok, wk, nw);
     }
     const QuantOut ov{nullptr, nullptr, j.v_hat, j.seq, nullptr, 0};
-    quantize_transposed_body<InT>(tile, static_cast<const InT *>(j.v), j.hid, j.seq, j.ldv, j.block_v, j.w_v, ov,
-                                  (int)blockIdx.x, (int)gridDim.x);
+    quantize_columns_body<InT>(static_cast<const InT *>(j.v), j.hid, j.seq, j.ldv, j.block_v, j.w_v, ov, wv, nw);
 }
 
 // (mant, exps) -> decoded values, 8 elements per thread.

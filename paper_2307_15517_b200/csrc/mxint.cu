@@ -227,6 +227,16 @@ mx_status_t launch_quantize_rows(const InT *x, int64_t rows, int64_t K, int64_t 
             MX_CUDA(launch_dep(mx::quantize_rows2_kernel<InT, 32>, dim3(grid), dim3(256), 0, st, x, rows, K, ldx, f.elem_bits, out));
         return MX_OK;
     }
+    if (chunks <= (int64_t)d.sm_count * 512) {             // few items: one per warp, in small CTAs on all SMs
+        const unsigned g = (unsigned)((rows * ((K / 8 + 31) / 32) + 1) / 2);
+        ProfScope prof(KIND_QUANTIZE, st);
+        if (f.block == 16)
+            MX_CUDA(launch_dep(mx::quantize_rows_kernel<InT, 16, 1>, dim3(g), dim3(64), 0, st, x, rows, K, ldx, (int)f.elem_bits, out));
+        else
+            MX_CUDA(launch_dep(mx::quantize_rows_kernel<InT, 32, 1>, dim3(g), dim3(64), 0, st, x, rows, K, ldx, (int)f.elem_bits, out));
+        MX_CUDA(cudaGetLastError());
+        return MX_OK;
+    }
     constexpr int UNROLL = 2;
     // at most one resident wave of CTAs: the grid-stride loop does the rest without a ragged second wave
     const int per_sm = f.block == 16 ? resident_ctas(mx::quantize_rows_kernel<InT, 16, UNROLL>)
@@ -237,6 +247,18 @@ mx_status_t launch_quantize_rows(const InT *x, int64_t rows, int64_t K, int64_t 
         MX_CUDA(launch_dep(mx::quantize_rows_kernel<InT, 16, UNROLL>, dim3(grid), dim3(256), 0, st, x, rows, K, ldx, f.elem_bits, out));
     else
         MX_CUDA(launch_dep(mx::quantize_rows_kernel<InT, 32, UNROLL>, dim3(grid), dim3(256), 0, st, x, rows, K, ldx, f.elem_bits, out));
+    MX_CUDA(cudaGetLastError());
+    return MX_OK;
+}
+
+template <typename InT>
+mx_status_t launch_quantize_columns(const InT *x, int64_t rows, int64_t K, int64_t stride_k, const mx_format_t &f, const mx::QuantOut &out,
+                                    const DeviceInfo &d, cudaStream_t st)
+{
+    const int64_t ctas = (((rows + 31) / 32) * (K / 32) + 1) / 2;
+    ProfScope prof(KIND_QUANTIZE, st);
+    MX_CUDA(launch_dep(mx::quantize_columns_kernel<InT>, dim3((unsigned)(ctas < INT32_MAX ? ctas : INT32_MAX)), dim3(64), 0, st, x, rows, K, stride_k,
+                       (int)f.block, (int)f.elem_bits, out));
     MX_CUDA(cudaGetLastError());
     return MX_OK;
 }
@@ -268,10 +290,23 @@ mx_status_t launch_dequant_bf16(const void *mant, const uint8_t *exps, int64_t r
 {
     const int64_t chunks = rows * (K / 8);
     if (chunks == 0 || batch == 0) return MX_OK;
-    ProfScope prof(KIND_DEQUANTIZE, st);
     const uint8_t *m = static_cast<const uint8_t *>(mant);
     const bool wide_ok = (K % 32) == 0 && (ps.mant_ld % 16) == 0 && (ps.mant_batch % 16) == 0;
-    if (wide_ok) {                          // 32 elements per thread, 16-byte loads and stores
+    const bool nib = f.elem_bits <= 4;
+    if (wide_ok && batch == 1 && (K % 1024) != 0 && ld == K && ps.mant_ld == (nib ? K / 2 : K) && ps.exp_ld == K / f.block && !ps.exp_row_shift &&
+        rows > 1 && rows * K / 32 <= INT32_MAX / 2) {
+        // a dense tensor is one long row: warps of rows that are no whole segments would have idle lanes (352 columns: 21 of 32)
+        mx::PackedStrides flat = ps;
+        flat.mant_ld *= rows;
+        flat.exp_ld *= rows;
+        return launch_dequant_bf16(mant, exps, 1, rows * K, f, out, rows * K, flat, 1, d, st);
+    }
+    ProfScope prof(KIND_DEQUANTIZE, st);
+    if (wide_ok && rows * (K / 32) * batch <= (int64_t)d.sm_count * 256) {      // few items: one per warp, in small CTAs on all SMs
+        const dim3 grid((unsigned)(rows * ((K / 32 + 31) / 32) + 1) / 2, (unsigned)batch);
+        if (nib) MX_CUDA(launch_dep(mx::decode_bf16_kernel<true, 1>, dim3(grid), dim3(64), 0, st, m, exps, rows, K, f.block, f.elem_bits, out, ld, ps));
+        else MX_CUDA(launch_dep(mx::decode_bf16_kernel<false, 1>, dim3(grid), dim3(64), 0, st, m, exps, rows, K, f.block, f.elem_bits, out, ld, ps));
+    } else if (wide_ok) {                   // 32 elements per thread, 16-byte loads and stores
         constexpr int UNROLL = 2;
         const int64_t items = rows * (K / 32);
         const int per_sm = f.elem_bits <= 4 ? resident_ctas(mx::decode_bf16_kernel<true, UNROLL>)
@@ -1867,17 +1902,8 @@ mx_status_t mx_quantize(const void *x, mx_dtype_t dt, int64_t rows, int64_t K, i
     if (stride_k == 1) return quantize_rows_any(x, dt, rows, K, stride_row, f, out, *d, st);
     if (stride_row == 1 && (K % 32) == 0 && (reinterpret_cast<uintptr_t>(mant_out) & 15u) == 0) {
         // a transposed view: blocks along the slow axis of a row-major tensor
-        const int64_t tiles = ((rows + 31) / 32) * ((K + 255) / 256);
-        const int tgrid = (int)(tiles < (int64_t)d->sm_count * 4 ? tiles : (int64_t)d->sm_count * 4);
-        ProfScope prof(KIND_QUANTIZE, st);
-        if (dt == MX_F32)
-            mx::quantize_transposed_kernel<float><<<tgrid, 256, 0, st>>>(static_cast<const float *>(x), rows, K, stride_k,
-                                                                         f.block, f.elem_bits, out);
-        else
-            mx::quantize_transposed_kernel<__nv_bfloat16><<<tgrid, 256, 0, st>>>(static_cast<const __nv_bfloat16 *>(x), rows, K,
-                                                                                 stride_k, f.block, f.elem_bits, out);
-        MX_CUDA(cudaGetLastError());
-        return MX_OK;
+        if (dt == MX_F32) return launch_quantize_columns(static_cast<const float *>(x), rows, K, stride_k, f, out, *d, st);
+        return launch_quantize_columns(static_cast<const __nv_bfloat16 *>(x), rows, K, stride_k, f, out, *d, st);
     }
     const int grid = grid_for(rows * (K / f.block), 256, d->sm_count, 8);
     ProfScope prof(KIND_QUANTIZE, st);
@@ -2858,8 +2884,8 @@ mx_status_t mx_attention_fp(const void *q, const void *k, const void *v, mx_dtyp
         j.seq = seq; j.hid = hid; j.ldq = ldq; j.ldk = ldk; j.ldv = ldv;
         j.block_qk = fqk.block; j.w_qk = fqk.elem_bits; j.block_v = fv.block; j.w_v = fv.elem_bits;
         j.q_hat = q_hat; j.k_hat = k_hat; j.v_hat = v_hat;
-        const int64_t row_items = seq * ((hid + 255) / 256), tiles = ((hid + 31) / 32) * ((seq + 255) / 256);
-        const int64_t want = (row_items + 7) / 8 > tiles ? (row_items + 7) / 8 : tiles;      // 8 warps per CTA
+        const int64_t items = 2 * seq * ((hid + 255) / 256) + ((hid + 31) / 32) * (seq / 32);
+        const int64_t want = (items + 7) / 8;                                                // 8 warps per CTA
         const int per_sm = dt == MX_F32 ? resident_ctas(mx::attention_operands_kernel<float>)
                                         : resident_ctas(mx::attention_operands_kernel<__nv_bfloat16>);
         const int64_t cap = (int64_t)d->sm_count * per_sm;
