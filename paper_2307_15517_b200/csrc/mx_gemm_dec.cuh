@@ -207,39 +207,66 @@ gemm_dec_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constan
         const uint8_t *mrow = smem_gen + (raw_base - smem_base) + r * 128, *erow = smem_gen + (exp_base - smem_base) + r * (4 * EW) +
                              ((uint32_t)reinterpret_cast<uintptr_t>(dp.w_exp + (int64_t)(min(n0 + r, p.N - 1) >> dp.w_rows2) * (p.K / dp.block)) & 3u);
         uint8_t *dst = smem_gen + (w_base - smem_base) + g * Cfg::W_BYTES + (r >> 3) * 1024 + (r & 7) * 128;
+        // each barrier is looked at well before its answer is needed: waiting for one that is long complete takes 130 clocks
+        bool there = false;                                              // the raw stage is known to be full
         for (int i = g; i < steps; i += GROUPS) {
             const int j = i % SPR, rs = i / SPR % RS;
-            const bool ok = ptx::mbar_wait_bounded(r_full(rs), (uint32_t)(i / SPR / RS) & 1u, abort_flag, TC_WAIT_LIMIT_NS) &&
-                            ptx::mbar_wait_bounded(w_empty(g), ((uint32_t)(i / GROUPS) & 1u) ^ 1u, abort_flag, TC_WAIT_LIMIT_NS);
-            if (!__all_sync(0xFFFFFFFFu, ok)) {
+            const uint32_t w_ph = ((uint32_t)(i / GROUPS) & 1u) ^ 1u;
+            if (!there && !__all_sync(0xFFFFFFFFu, ptx::mbar_wait_bounded(r_full(rs), (uint32_t)(i / SPR / RS) & 1u, abort_flag, TC_WAIT_LIMIT_NS))) {
                 timed_out = true;
                 break;
             }
-#pragma unroll
-            for (int h = 0; h < 2; ++h) {
-                uint4 m[NIB ? 1 : 2];
+            bool free = ptx::mbar_test(w_empty(g), w_ph);
+            // (the exponents of all 32 rows: one path per warp)
+            const uint32_t e4 = step_exps(erow + rs * Cfg::RAW_EXP, j, b16, dp.exp_words);
+            auto load = [&](int h, uint4 (&m)[NIB ? 1 : 2]) {
 #pragma unroll
                 for (int q = 0; q < (NIB ? 1 : 2); ++q) {
                     const int c = NIB ? 2 * j + h : 4 * j + 2 * h + q;                        // 16-byte chunk of the row's 128 bytes
                     m[q] = *reinterpret_cast<const uint4 *>(mrow + rs * Cfg::RAW_MANT + ((c ^ (r & 7)) << 4));
                 }
-                const uint8_t *ex = erow + rs * Cfg::RAW_EXP;
-                uint32_t e;
-                if (!b16) e = ex[2 * j + h];
-                else if (dp.exp_words) e = *reinterpret_cast<const uint16_t *>(ex + 4 * j + 2 * h);
-                else e = ex[4 * j + 2 * h] | (uint32_t)ex[4 * j + 2 * h + 1] << 8;
-                uint32_t o[4][4];
-                decode32<NIB>(m, e, b16, dp.w_bits, o);
+            };
+            auto store = [&](int h, const uint32_t (&o)[4][4]) {
+                if (h == 0)                                              // the stage is needed only now
+                    free = __all_sync(0xFFFFFFFFu, free) ||
+                           __all_sync(0xFFFFFFFFu, ptx::mbar_wait_bounded(w_empty(g), w_ph, abort_flag, TC_WAIT_LIMIT_NS));
 #pragma unroll
                 for (int q = 0; q < 4; ++q)
                     *reinterpret_cast<uint4 *>(dst + (((h * 4 + q) ^ (r & 7)) << 4)) = make_uint4(o[q][0], o[q][1], o[q][2], o[q][3]);
+            };
+            uint4 m[2][NIB ? 1 : 2];
+            load(0, m[0]);
+            load(1, m[1]);
+            if (__all_sync(0xFFFFFFFFu, exps_plain(e4, dp.w_bits))) {
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    uint32_t o[4][4];
+                    decode32_plain<NIB>(m[h], (e4 >> (16 * h)) & 0xFFu, (e4 >> (16 * h + 8)) & 0xFFu, dp.w_bits, o);
+                    store(h, o);
+                }
+            } else {
+#pragma unroll 1
+                for (int h = 0; h < 2; ++h) {                            // (read again: an array indexed by a loop would live in memory)
+                    uint4 again[NIB ? 1 : 2];
+                    uint32_t o[4][4];
+                    load(h, again);
+                    decode32_perm<NIB>(again, (e4 >> (16 * h)) & 0xFFu, (e4 >> (16 * h + 8)) & 0xFFu, dp.w_bits, o);
+                    store(h, o);
+                }
             }
+            if (!free) {
+                timed_out = true;
+                break;
+            }
+            const int in = i + GROUPS;
+            const bool next = in < steps && ptx::mbar_test(r_full(in / SPR % RS), (uint32_t)(in / SPR / RS) & 1u);
             ptx::fence_proxy_async_smem();                               // the decoded rows -> visible to the MMA
             __syncwarp();
             if (lane == 0) {
                 ptx::mbar_arrive(w_full(g));
                 ptx::mbar_arrive(r_empty(rs));
             }
+            there = __all_sync(0xFFFFFFFFu, next);
         }
         if (dp.early) ptx::dep_wait();                                   // before the results are written
         // the partial tiles: tensor memory -> this CTA's shared memory.  All its loads have landed, the raw stages are consumed

@@ -117,6 +117,7 @@ struct PrepLnJob {
     int ww;
     __nv_bfloat16 *w_hat;     // [N, K]
     int w_row_shift;
+    int perm;                 // 1: a_hat in the K order of the products that decode their weights
 };
 
 template <int PER, bool NIBBLE>
@@ -130,6 +131,7 @@ prep_ln_operands_kernel(const PrepLnJob j)
     ps.mant_ld = NIBBLE ? j.K / 2 : j.K;
     ps.exp_ld = j.K / j.block;
     ps.mant_batch = ps.exp_batch = ps.out_batch = 0;
+    ps.perm = 0;
     ps.exp_row_shift = j.w_row_shift;
     const int warps = blockDim.x >> 5, lane = threadIdx.x & 31;
     const int cols = (int)j.K, groups = cols >> 3;
@@ -175,6 +177,7 @@ prep_ln_operands_kernel(const PrepLnJob j)
                 uint32_t h[4];
 #pragma unroll
                 for (int i = 0; i < 4; ++i) h[i] = as_u32(__floats2bfloat162_rn(xh[2 * i], xh[2 * i + 1]));
+                if (j.perm) perm8(h);
                 *reinterpret_cast<uint4 *>(j.a_hat + r * j.K + 8 * g) = make_uint4(h[0], h[1], h[2], h[3]);
             }
         }

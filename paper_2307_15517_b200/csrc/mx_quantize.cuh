@@ -77,7 +77,7 @@ __device__ __forceinline__ void decode8_nibbles(uint32_t p, __nv_bfloat162 s, __
     uint32_t v[4];
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
-        const uint32_t x = (((p >> (4 * i)) & 0x000F000Fu) ^ 0x00080008u) | 0x43004300u;   // (n_i, n_{i+4})
+        const uint32_t x = ((p >> (4 * i)) & 0x000F000Fu) ^ 0x43084308u;                    // (n_i, n_{i+4})
         v[i] = as_u32(__hfma2(as_bf162(x), s, c));
     }
     out[0] = __byte_perm(v[0], v[1], 0x5410);      // (k0, k1)
@@ -117,6 +117,7 @@ struct PackedStrides {
     int64_t mant_batch, exp_batch;    // bytes between batch items
     int64_t out_batch;                // elements between batch items of the output
     int exp_row_shift;                // 1: two adjacent rows share one row of exponent bytes (two-row blocks)
+    int perm;                         // 1: bf16 output in the K order of the products that decode their weights (see QuantOut)
 };
 
 struct QuantOut {
@@ -126,8 +127,18 @@ struct QuantOut {
     int64_t ld_xhat;
     uint32_t *nonfinite;  // nullable
     int xhat_perm;        // 1: inside every group of 8 consecutive k, xhat holds k in the order
-                          // 0,4,1,5,2,6,3,7 (the operand order of the W_NIBBLE_PERM product kernel)
+                          // 0,4,1,5,2,6,3,7 (the operand order of the product kernels that decode their weights)
 };
+
+// Eight bf16 values, k ascending -> k in the order 0,4,1,5,2,6,3,7.
+__device__ __forceinline__ void perm8(uint32_t (&h)[4])
+{
+    const uint32_t a = __byte_perm(h[0], h[2], 0x5410), b = __byte_perm(h[0], h[2], 0x7632);
+    h[2] = __byte_perm(h[1], h[3], 0x5410);
+    h[3] = __byte_perm(h[1], h[3], 0x7632);
+    h[0] = a;
+    h[1] = b;
+}
 
 // A pass of two lists deals the second one on from where the first ends: number of warp `wid` of `nw` in the second list after
 // `items` of the first (the warps that had one item less come first).
@@ -696,6 +707,7 @@ dequantize_kernel(const uint8_t *__restrict__ mant, const uint8_t *__restrict__ 
                 const __nv_bfloat16 hi = __float2bfloat16_rn(decode_value(q[2 * i + 1], ebyte, w));
                 h[i] = (uint32_t)__bfloat16_as_ushort(lo) | ((uint32_t)__bfloat16_as_ushort(hi) << 16);
             }
+            if (ps.perm) perm8(h);
             *reinterpret_cast<uint4 *>(o) = make_uint4(h[0], h[1], h[2], h[3]);
         }
     }
@@ -751,6 +763,61 @@ __device__ __forceinline__ void decode32(const uint4 (&m)[NIBBLE ? 1 : 2], uint3
             }
         }
     }
+}
+
+// A row's K step of 64 inside a product: two groups of 32 packed values with four exponent bytes, one per 16 k, in `e`.  The
+// order of k in every group of eight is 0,4,1,5,2,6,3,7, the one in which masked nibbles leave a word, and the scales are built
+// for blocks whose exponents keep scale and constant plain bf16 (fp32) numbers: half the integer instructions of decode32, whose
+// work is what bounds those products.
+__device__ __forceinline__ bool exps_plain(uint32_t e, int w)
+{
+    // bytes E - (w-1) in 0 .. 223, i.e. scale fields in 1 .. 224.  A byte that borrows is above 223 itself.
+    const uint32_t t = e - (uint32_t)(w - 1) * 0x01010101u;
+    return (t & (t << 1) & (t << 2) & 0x80808080u) == 0;
+}
+template <bool NIBBLE>
+__device__ __forceinline__ void decode32_plain(const uint4 (&m)[NIBBLE ? 1 : 2], uint32_t e0, uint32_t e1, int w, uint32_t (&o)[4][4])
+{
+    const uint32_t w8[8] = {m[0].x, m[0].y, m[0].z, m[0].w,
+                            m[NIBBLE ? 0 : 1].x, m[NIBBLE ? 0 : 1].y, m[NIBBLE ? 0 : 1].z, m[NIBBLE ? 0 : 1].w};
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+        const uint32_t e = j < 2 ? e0 : e1;
+        if (NIBBLE) {
+            const uint32_t s = e * 0x00800080u - (uint32_t)(w - 2) * 0x00800080u, c = s + 0x83888388u;      // -136 * s
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+                o[j][i] = as_u32(__hfma2(as_bf162(((w8[j] >> (4 * i)) & 0x000F000Fu) ^ 0x43084308u), as_bf162(s), as_bf162(c)));
+        } else {
+            const uint32_t sb = (e - (uint32_t)(w - 2)) << 23;
+            const float s = __uint_as_float(sb), c = __uint_as_float(sb + 0x8B800080u);                     // -(2^23 + 128) * s
+            const uint32_t t0 = w8[2 * j] ^ 0x80808080u, t1 = w8[2 * j + 1] ^ 0x80808080u;
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const float a = fmaf(__uint_as_float(__byte_perm(t0, 0x4B000000u, 0x7540 | i)), s, c);
+                const float b = fmaf(__uint_as_float(__byte_perm(t1, 0x4B000000u, 0x7540 | i)), s, c);
+                o[j][i] = __byte_perm(__float_as_uint(a), __float_as_uint(b), 0x7632);                      // exact in bf16
+            }
+        }
+    }
+}
+// any exponents
+template <bool NIBBLE>
+__device__ __forceinline__ void decode32_perm(const uint4 (&m)[NIBBLE ? 1 : 2], uint32_t e0, uint32_t e1, int w, uint32_t (&o)[4][4])
+{
+    decode32<NIBBLE>(m, e0 | (e1 << 8), true, w, o);
+#pragma unroll
+    for (int j = 0; j < 4; ++j) perm8(o[j]);
+}
+// The four exponent bytes of K step j of a row whose bytes of a raw stage start at `ex`.
+__device__ __forceinline__ uint32_t step_exps(const uint8_t *ex, int j, bool b16, int exp_words)
+{
+    if (b16) {
+        if (exp_words) return *reinterpret_cast<const uint32_t *>(ex + 4 * j);
+        return ex[4 * j] | (uint32_t)ex[4 * j + 1] << 8 | (uint32_t)ex[4 * j + 2] << 16 | (uint32_t)ex[4 * j + 3] << 24;
+    }
+    const uint32_t e = exp_words ? *reinterpret_cast<const uint16_t *>(ex + 2 * j) : ex[2 * j] | (uint32_t)ex[2 * j + 1] << 8;
+    return __byte_perm(e, 0, 0x1100);
 }
 
 // Eight 32-bit words to a 32-byte aligned address, one whole sector per lane.
@@ -826,6 +893,10 @@ template <bool NIBBLE, int UNROLL> struct DecodeWalk {
             if (d.row[u] < 0) continue;
             uint32_t o[4][4];
             decode32<NIBBLE>(d.m[u], d.e[u], b16, w, o);
+            if (ps.perm) {
+#pragma unroll
+                for (int j = 0; j < 4; ++j) perm8(o[j]);
+            }
             __nv_bfloat16 *dst = out + d.row[u] * ld_out + (int64_t)d.kc[u] * 32;
             if (sectors) {
                 store32(dst, o[0], o[1]);
@@ -901,6 +972,7 @@ decode_pair_kernel(const DecodePairJob j)
     PackedStrides pa, pw;
     pa.exp_ld = pw.exp_ld = j.K / j.block;
     pa.mant_batch = pa.exp_batch = pa.out_batch = pw.mant_batch = pw.exp_batch = pw.out_batch = 0;
+    pa.perm = pw.perm = 0;
     pa.mant_ld = NIB_A ? j.K / 2 : j.K;
     pw.mant_ld = NIB_W ? j.K / 2 : j.K;
     pa.exp_row_shift = j.a_row_shift;
@@ -995,7 +1067,7 @@ dense_unpack_kernel(const uint8_t *__restrict__ dense, int64_t rows, int64_t K, 
 template <typename OutT>
 __global__ void __launch_bounds__(256)
 dequantize_dense_kernel(const uint8_t *__restrict__ dense, const uint8_t *__restrict__ exps, int64_t rows, int64_t K,
-                        int block, int w, int exp_row_shift, OutT *__restrict__ out, int64_t ld_out)
+                        int block, int w, int exp_row_shift, OutT *__restrict__ out, int64_t ld_out, int perm)
 {
     ptx::dep_wait();
     ptx::dep_trigger();
@@ -1016,6 +1088,7 @@ dequantize_dense_kernel(const uint8_t *__restrict__ dense, const uint8_t *__rest
             uint32_t h[4];
 #pragma unroll
             for (int i = 0; i < 4; ++i) h[i] = as_u32(__floats2bfloat162_rn(f[2 * i], f[2 * i + 1]));
+            if (perm) perm8(h);
             *reinterpret_cast<uint4 *>(o) = make_uint4(h[0], h[1], h[2], h[3]);
         }
     }
@@ -1052,6 +1125,7 @@ prep_operands_kernel(const PrepJob j)
     ps.mant_ld = NIBBLE ? j.K / 2 : j.K;
     ps.exp_ld = j.K / j.block;
     ps.mant_batch = ps.exp_batch = ps.out_batch = 0;
+    ps.perm = 0;
     ps.exp_row_shift = j.w_row_shift;
     // the first weights are on their way while the activations are quantized
     // (their items are dealt on from where the activations' end)

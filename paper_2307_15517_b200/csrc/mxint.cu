@@ -279,6 +279,7 @@ mx::PackedStrides dense_strides(int64_t K, const mx_format_t &f)
     ps.exp_ld = K / f.block;
     ps.mant_batch = ps.exp_batch = ps.out_batch = 0;
     ps.exp_row_shift = f.block_rows == 2 ? 1 : 0;
+    ps.perm = 0;
     return ps;
 }
 
@@ -326,18 +327,20 @@ mx_status_t launch_dequant_bf16(const void *mant, const uint8_t *exps, int64_t r
 
 mx_status_t launch_dequant_bf16(const void *mant, const uint8_t *exps, int64_t rows, int64_t K,
                                 const mx_format_t &f, __nv_bfloat16 *out, int64_t ld,
-                                const DeviceInfo &d, cudaStream_t st)
+                                const DeviceInfo &d, cudaStream_t st, bool perm = false)
 {
     if (f.packing) {                    // dense storage: w bits per element
         if (rows == 0 || K == 0) return MX_OK;
         ProfScope prof(KIND_DEQUANTIZE, st);
         MX_CUDA(launch_dep(mx::dequantize_dense_kernel<__nv_bfloat16>, dim3(grid_for(rows * (K / 8), 256, d.sm_count, 8)),
                            dim3(256), 0, st, static_cast<const uint8_t *>(mant), exps, rows, K, (int)f.block,
-                           (int)f.elem_bits, f.block_rows == 2 ? 1 : 0, out, ld));
+                           (int)f.elem_bits, f.block_rows == 2 ? 1 : 0, out, ld, perm ? 1 : 0));
         MX_CUDA(cudaGetLastError());
         return MX_OK;
     }
-    return launch_dequant_bf16(mant, exps, rows, K, f, out, ld, dense_strides(K, f), 1, d, st);
+    mx::PackedStrides ps = dense_strides(K, f);
+    ps.perm = perm ? 1 : 0;
+    return launch_dequant_bf16(mant, exps, rows, K, f, out, ld, ps, 1, d, st);
 }
 
 // Both operands of a product, (mant, exps) -> bf16 [rows, K]: one launch when both are in container form with
@@ -1993,7 +1996,7 @@ mx_status_t mx_dequantize(const void *mant, const uint8_t *exps, int64_t rows, i
         ProfScope prof(KIND_DEQUANTIZE, st);
         MX_CUDA(launch_dep(mx::dequantize_dense_kernel<float>, dim3(grid_for(rows * (K / 8), 256, d->sm_count, 8)), dim3(256), 0,
                            st, static_cast<const uint8_t *>(mant), exps, rows, K, (int)f.block, (int)f.elem_bits,
-                           f.block_rows == 2 ? 1 : 0, static_cast<float *>(out), ld_out));
+                           f.block_rows == 2 ? 1 : 0, static_cast<float *>(out), ld_out, 0));
         MX_CUDA(cudaGetLastError());
         return MX_OK;
     }
@@ -2035,7 +2038,7 @@ mx_status_t mx_gemm_ex(const void *a_mant, const uint8_t *a_exp, mx_format_t fa,
                 if ((reinterpret_cast<uintptr_t>(workspace) & 255u) != 0) return MX_ERR_ALIGN;
                 __nv_bfloat16 *a_dec = static_cast<__nv_bfloat16 *>(workspace);
                 cudaStream_t sd = static_cast<cudaStream_t>(stream);
-                s = launch_dequant_bf16(a_mant, a_exp, M, K, fa, a_dec, K, *dd, sd);
+                s = launch_dequant_bf16(a_mant, a_exp, M, K, fa, a_dec, K, *dd, sd, true);
                 if (s != MX_OK) return s;
                 return launch_dec(plan, a_dec, w_mant, w_exp, fw, M, N, K, bias, y, ldy, nullptr, *dd, sd, EpiTail());
             }
@@ -2181,6 +2184,7 @@ mx_status_t mx_linear_ex(const void *x, mx_dtype_t dt, int64_t M, int64_t K, int
         if (s != MX_OK) return s;
     }
     if (dec) {
+        out.xhat_perm = 1;
         s = quantize_rows_any(x, dt, M, K, ldx, fa, out, *d, st);
         if (s != MX_OK) return s;
         return launch_dec(plan, a_hat, w_mant, w_exp, fw, M, N, K, bias, y, ldy, nullptr, *d, st, EpiTail());
@@ -2262,7 +2266,7 @@ static mx_status_t gemm_tc_impl(const void *a_mant, const uint8_t *a_exp, mx_for
     s = dec_plan(M, N, K, fa, fw, w_exp, !y, *d, &plan, &dec);
     if (s != MX_OK) return s;
     if (dec) {
-        s = launch_dequant_bf16(a_mant, a_exp, M, K, fa, a_hat, K, *d, st);
+        s = launch_dequant_bf16(a_mant, a_exp, M, K, fa, a_hat, K, *d, st, true);
         if (s != MX_OK) return s;
         return launch_dec(plan, a_hat, w_mant, w_exp, fw, M, N, K, bias, y, y ? ldy : N, y ? nullptr : &yq, *d, st, et);
     }
@@ -2283,7 +2287,7 @@ static mx_status_t gemm_tc_impl(const void *a_mant, const uint8_t *a_exp, mx_for
 // The same for the layer: activations quantized on the fly.
 // The operand pass with LayerNorm in front of the activation quantizer (see prep_ln_operands_kernel).
 static mx_status_t tc_prepare_ln(const mx_linear_args_t &a, const mx_prologue_t &ln, __nv_bfloat16 *a_hat,
-                                 __nv_bfloat16 *w_hat, DeviceInfo &d, cudaStream_t st)
+                                 __nv_bfloat16 *w_hat, DeviceInfo &d, cudaStream_t st, bool perm = false)
 {
     mx::PrepLnJob j;
     j.x = static_cast<const float *>(a.x); j.M = a.M; j.K = a.K; j.ldx = a.ldx;
@@ -2291,6 +2295,7 @@ static mx_status_t tc_prepare_ln(const mx_linear_args_t &a, const mx_prologue_t 
     j.wa = a.fa.elem_bits; j.block = a.fa.block; j.a_hat = a_hat;
     j.w_mant = static_cast<const uint8_t *>(a.w_mant); j.w_exp = a.w_exp; j.N = a.N; j.ww = a.fw.elem_bits;
     j.w_hat = w_hat; j.w_row_shift = a.fw.block_rows == 2 ? 1 : 0;
+    j.perm = perm ? 1 : 0;
     const int per = (int)((a.K + mx::GLUE_THREADS - 1) / mx::GLUE_THREADS);
     const bool nib = a.fw.elem_bits <= 4;
     // a CTA per row, but a resident wave where the weights have that much work: a grid of few rows decodes them on few SMs, and
@@ -2362,9 +2367,9 @@ static mx_status_t linear_tc_impl(const void *x, mx_dtype_t dt, int64_t M, int64
         if (with_ln) {
             mx_linear_args_t rows = one;
             rows.N = 0;                                   // the activations alone
-            s = tc_prepare_ln(rows, *ln, a_hat, w_hat, *d, st);
+            s = tc_prepare_ln(rows, *ln, a_hat, w_hat, *d, st, true);
         } else {
-            s = quantize_rows_any(x, dt, M, K, ldx, fa, mx::QuantOut{nullptr, nullptr, a_hat, K, nullptr}, *d, st);
+            s = quantize_rows_any(x, dt, M, K, ldx, fa, mx::QuantOut{nullptr, nullptr, a_hat, K, nullptr, 1}, *d, st);
         }
         if (s != MX_OK) return s;
         return launch_dec(plan, a_hat, w_mant, w_exp, fw, M, N, K, bias, y, y ? ldy : N, y ? nullptr : &yq, *d, st, et);
@@ -2740,6 +2745,7 @@ mx_status_t mx_gemm_batched(const void *a_mant, const uint8_t *a_exp, mx_format_
         ps.mant_ld = f.elem_bits <= 4 ? ld / 2 : ld;
         ps.exp_ld = ld / f.block;
         ps.mant_batch = f.elem_bits <= 4 ? bstride / 2 : bstride;
+        ps.perm = 0;
         ps.exp_row_shift = f.block_rows == 2 ? 1 : 0;   // rows 2i, 2i+1 read one row of exponent bytes
         // an item starts (bstride / ld) rows down and (bstride % ld) elements into the row
         ps.exp_batch = ((bstride / ld) >> ps.exp_row_shift) * (ld / f.block) + (bstride % ld) / f.block;
