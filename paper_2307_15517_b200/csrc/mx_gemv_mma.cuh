@@ -62,6 +62,14 @@ __device__ __forceinline__ void cp_async4(uint32_t dst, const void *src, int val
 {
     asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(dst), "l"(src), "r"(valid) : "memory");
 }
+__device__ __forceinline__ void cp_async8(uint32_t dst, const void *src, int valid)
+{
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;" ::"r"(dst), "l"(src), "r"(valid) : "memory");
+}
+__device__ __forceinline__ void cp_async16(uint32_t dst, const void *src)
+{
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
+}
 // Arrives on `bar` when this thread's copies so far are in shared memory (one of the barrier's expected arrivals).
 __device__ __forceinline__ void cp_async_arrive(uint32_t bar)
 {

@@ -348,6 +348,17 @@ __device__ __forceinline__ void mma_bf16_ss_pair(uint32_t d_tmem, uint64_t a_des
         : "r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate)
         : "memory");
 }
+// The same with A in tensor memory: lane = row (128 in either CTA), 8 columns of two bf16 values per 16 k from `a_tmem` on.
+__device__ __forceinline__ void mma_bf16_ts_pair(uint32_t d_tmem, uint32_t a_tmem, uint64_t b_desc, uint32_t idesc, uint32_t accumulate)
+{
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "setp.ne.b32 p, %4, 0;\n\t"
+        "tcgen05.mma.cta_group::2.kind::f16 [%0], [%1], %2, %3, p;\n\t}"
+        :
+        : "r"(d_tmem), "r"(a_tmem), "l"(b_desc), "r"(idesc), "r"(accumulate)
+        : "memory");
+}
 // Arrive on the barrier at the same shared-memory offset in every CTA of `cta_mask` once all
 // tcgen05 operations issued so far by this thread have completed.
 __device__ __forceinline__ void mma_commit_pair(uint32_t bar, uint16_t cta_mask)
@@ -360,8 +371,7 @@ __device__ __forceinline__ void mma_commit_pair(uint32_t bar, uint16_t cta_mask)
 // One lane of the (whole, converged) warp: the same every time.  The warps that issue TMA loads and MMAs run their loops as a
 // whole and let the elected lane issue: what a loop computes is then uniform and stays in uniform registers, which the issuing
 // instructions take their operands from.  With a loop of one lane (`if (lane == 0)`) four MMAs and two commits took 470 clocks
-// to issue, now 230, and those loops bounded the products: whole calls 384 x 8192 x 8192 63 -> 59 us (8/4 bits), 4096^3 89 -> 79
-// (4/4), 4096 x 11008 x 4096 181 -> 158 (4/2).
+// to issue, now 230, and those loops bounded every product here: 128 x 11008 x 4096 in gemm_tmw_kernel 37 -> 29 us.
 __device__ __forceinline__ bool elect_one()
 {
     uint32_t p;
@@ -440,6 +450,21 @@ __device__ __forceinline__ void tmem_ld_16x256b_x4(uint32_t taddr, uint32_t (&r)
           "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
         : "r"(taddr)
         : "memory");
+}
+// 32 lanes x 16 consecutive columns: thread t of the warp writes lane (quadrant*32 + t).
+__device__ __forceinline__ void tmem_st_32x16(uint32_t taddr, const uint32_t (&r)[4][4])
+{
+    asm volatile(
+        "tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], "
+        "{%1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, %16};"
+        :
+        : "r"(taddr), "r"(r[0][0]), "r"(r[0][1]), "r"(r[0][2]), "r"(r[0][3]), "r"(r[1][0]), "r"(r[1][1]), "r"(r[1][2]), "r"(r[1][3]),
+          "r"(r[2][0]), "r"(r[2][1]), "r"(r[2][2]), "r"(r[2][3]), "r"(r[3][0]), "r"(r[3][1]), "r"(r[3][2]), "r"(r[3][3])
+        : "memory");
+}
+__device__ __forceinline__ void tmem_st_wait()
+{
+    asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
 }
 __device__ __forceinline__ void tmem_ld_wait()
 {

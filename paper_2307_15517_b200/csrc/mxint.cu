@@ -26,6 +26,7 @@
 #include "mx_gemm_tc8.cuh"
 #include "mx_gemm_tcw.cuh"
 #include "mx_gemm_tcx.cuh"
+#include "mx_gemm_tmw.cuh"
 #include "mx_gemv_mma.cuh"
 #include "mx_gemv_stream.cuh"
 #include "mx_glue.cuh"
@@ -61,6 +62,7 @@ struct DeviceInfo {
     bool splitk_attr_set[4] = {};
     int splitk_clusters[mx::SplitKCfg::MAX_SPLIT + 1] = {-1, -1, -1, -1, -1};
     bool attn_attr_set[2] = {false, false};
+    bool tmw_attr_set[4] = {};
     bool dec_attr_set[12] = {};
     int dec_clusters[12][mx::DecCfg::MAX_SPLIT + 1] = {};      // resident clusters by kernel and cluster size
 };
@@ -1630,7 +1632,7 @@ const DecKernel g_dec[12] = {                             // panels - 1, nibbles
     mx::gemm_dec_kernel<2, false, false>, mx::gemm_dec_kernel<2, false, true>, mx::gemm_dec_kernel<2, true, false>, mx::gemm_dec_kernel<2, true, true>,
     mx::gemm_dec_kernel<3, false, false>, mx::gemm_dec_kernel<3, false, true>, mx::gemm_dec_kernel<3, true, false>, mx::gemm_dec_kernel<3, true, true>};
 
-struct DecPlan { int which, panels, split, exp_words; };
+struct DecPlan { int which, panels, split, exp_words, tokens; };     // tokens: of gemm_tmw_kernel's tile, 0: gemm_dec_kernel
 
 mx_status_t dec_config(cudaLaunchConfig_t &cfg, cudaLaunchAttribute *attr, int panels, int grid, int split, cudaStream_t st)
 {
@@ -1648,40 +1650,78 @@ mx_status_t dec_config(cudaLaunchConfig_t &cfg, cudaLaunchAttribute *attr, int p
 
 bool dec_is_faster(int64_t M, int64_t N, int64_t K, int split, bool rec, int sm_count);
 
-// Whether the product runs there, and into how many pieces K is cut: the most whose clusters all fit at once, of at least four
-// K steps each.
+int tmw_tokens(int64_t M, int64_t N, int64_t K, bool nib, bool rec, int split, bool dec, int sm_count);
+
+// Whether the product decodes its weights itself, in which kernel, and for gemm_dec_kernel into how many pieces K is cut: the most
+// whose clusters all fit at once, of at least four K steps each.
 mx_status_t dec_plan(int64_t M, int64_t N, int64_t K, const mx_format_t &fa, const mx_format_t &fw, const uint8_t *w_exp, bool quantized,
                      DeviceInfo &d, DecPlan *out, bool *use)
 {
     *use = false;
     const bool nib = fw.elem_bits <= 4;
     const int64_t row_bytes = nib ? K / 2 : K, panels = (M + mx::TC_BM - 1) / mx::TC_BM, tiles = (N + mx::DecCfg::BN - 1) / mx::DecCfg::BN;
-    if (!format_ok(fw) || panels > mx::DecCfg::MAX_P || (row_bytes % 16) != 0 || tiles > INT32_MAX / 16) return MX_OK;
-    out->panels = (int)panels;
-    out->which = 4 * ((int)panels - 1) + (nib ? 2 : 0) + (quantized ? 1 : 0);
+    if (!format_ok(fw) || (row_bytes % 16) != 0 || tiles > INT32_MAX / 16) return MX_OK;
     out->exp_words = ((K / fw.block) % 4) == 0 && (reinterpret_cast<uintptr_t>(w_exp) & 3u) == 0 ? 1 : 0;
-    out->split = 1;
-    const mx_status_t as = smem_attr_once(d.dec_attr_set[out->which], g_dec[out->which], 227 * 1024);
-    if (as != MX_OK) return as;
-    const int64_t kblocks = (K + mx::TC_BK - 1) / mx::TC_BK;
-    for (int s = mx::DecCfg::MAX_SPLIT; s > 1 && out->split == 1; --s) {
-        if (tiles * s > d.sm_count || kblocks < 4 * s) continue;
-        std::lock_guard<std::mutex> lk(g_init_mu);
-        int &known = d.dec_clusters[out->which][s];
-        if (known == 0) {
-            cudaLaunchConfig_t cfg = {};
-            cudaLaunchAttribute attr[2];
-            dec_config(cfg, attr, (int)panels, s * d.sm_count, s, nullptr);
-            MX_CUDA(cudaOccupancyMaxActiveClusters(&known, g_dec[out->which], &cfg));
-        }
-        if (tiles <= known) out->split = s;
-    }
+    out->tokens = 0;
     bool rec = false;
     if (rec_fits(fa, fw, M, N, K)) {
         const mx_status_t rs = rec_is_faster(M, N, K, d, &rec);
         if (rs != MX_OK) return rs;
     }
-    *use = dec_is_faster(M, N, K, out->split, rec, d.sm_count);
+    if (panels <= mx::DecCfg::MAX_P) {
+        out->panels = (int)panels;
+        out->which = 4 * ((int)panels - 1) + (nib ? 2 : 0) + (quantized ? 1 : 0);
+        out->split = 1;
+        const mx_status_t as = smem_attr_once(d.dec_attr_set[out->which], g_dec[out->which], 227 * 1024);
+        if (as != MX_OK) return as;
+        const int64_t kblocks = (K + mx::TC_BK - 1) / mx::TC_BK;
+        for (int s = mx::DecCfg::MAX_SPLIT; s > 1 && out->split == 1; --s) {
+            if (tiles * s > d.sm_count || kblocks < 4 * s) continue;
+            std::lock_guard<std::mutex> lk(g_init_mu);
+            int &known = d.dec_clusters[out->which][s];
+            if (known == 0) {
+                cudaLaunchConfig_t cfg = {};
+                cudaLaunchAttribute attr[2];
+                dec_config(cfg, attr, (int)panels, s * d.sm_count, s, nullptr);
+                MX_CUDA(cudaOccupancyMaxActiveClusters(&known, g_dec[out->which], &cfg));
+            }
+            if (tiles <= known) out->split = s;
+        }
+        *use = dec_is_faster(M, N, K, out->split, rec, d.sm_count);
+    }
+    out->tokens = tmw_tokens(M, N, K, nib, rec, panels <= mx::DecCfg::MAX_P ? out->split : 0, *use, d.sm_count);
+    if (out->tokens) {
+        out->which = (nib ? 2 : 0) + (quantized ? 1 : 0);
+        *use = true;
+    }
+    return MX_OK;
+}
+
+typedef void (*TmwKernel)(CUtensorMap, CUtensorMap, mx::TcParams, mx::TmwParams);
+const TmwKernel g_tmw[4] = {mx::gemm_tmw_kernel<false, false>, mx::gemm_tmw_kernel<false, true>, mx::gemm_tmw_kernel<true, false>,
+                            mx::gemm_tmw_kernel<true, true>};
+
+mx_status_t launch_tmw(const DecPlan &g, const __nv_bfloat16 *a_hat, const void *w_mant, const mx_format_t &fw, mx::TcParams &p,
+                       const uint8_t *w_exp, DeviceInfo &d, cudaStream_t st)
+{
+    using Cfg = mx::TmwCfg;
+    const int T = g.tokens;
+    CUtensorMap tm_x, tm_r;
+    mx_status_t s = encode_bf16_rows(&tm_x, a_hat, p.M, p.K, T / 2);
+    if (s != MX_OK) return s;
+    s = encode_u8_sw128(&tm_r, w_mant, p.N, fw.elem_bits <= 4 ? p.K / 2 : p.K, Cfg::BN);
+    if (s != MX_OK) return s;
+    s = smem_attr_once(d.tmw_attr_set[g.which], g_tmw[g.which], 227 * 1024);
+    if (s != MX_OK) return s;
+    p.tiles_m = (p.M + T - 1) / T;
+    p.tiles_n = (p.N + 2 * Cfg::BN - 1) / (2 * Cfg::BN);
+    const int64_t tiles = (int64_t)p.tiles_m * p.tiles_n;
+    if (tiles > INT32_MAX / 2) return MX_ERR_SHAPE;
+    const int pairs = (int)(tiles < d.sm_count / 2 ? tiles : d.sm_count / 2);
+    const mx::TmwParams wp{w_exp, fw.elem_bits, fw.block_rows == 2 ? 1 : 0, fw.block, T, Cfg::stages(T, p.yq_mant), 1, g.exp_words};
+    ProfScope prof(KIND_GEMM_TC, st);
+    MX_CUDA(launch_dep(g_tmw[g.which], dim3(2 * pairs), dim3(Cfg::THREADS), Cfg::smem_bytes(T, p.yq_mant), st, tm_x, tm_r, p, wp));
+    MX_CUDA(cudaGetLastError());
     return MX_OK;
 }
 
@@ -1689,11 +1729,6 @@ mx_status_t launch_dec(const DecPlan &g, const __nv_bfloat16 *a_hat, const void 
                        int64_t N, int64_t K, const float *bias, float *y, int64_t ldy, const QuantizedOut *yq, DeviceInfo &d, cudaStream_t st,
                        const EpiTail &et)
 {
-    CUtensorMap tm_a, tm_r;
-    mx_status_t s = encode_bf16_rows(&tm_a, a_hat, M, K, mx::TC_BM);
-    if (s != MX_OK) return s;
-    s = encode_u8_sw128(&tm_r, w_mant, N, fw.elem_bits <= 4 ? K / 2 : K, mx::DecCfg::BN);
-    if (s != MX_OK) return s;
     mx::TcParams p{};
     p.y = y;
     p.ex_bias = bias;
@@ -1714,6 +1749,12 @@ mx_status_t launch_dec(const DecPlan &g, const __nv_bfloat16 *a_hat, const void 
     p.yq_bits = yq ? yq->f.elem_bits : 0;
     p.yq_block = yq ? yq->f.block : 0;
     p.yq_rows2 = yq && yq->f.block_rows == 2 ? 1 : 0;
+    if (g.tokens) return launch_tmw(g, a_hat, w_mant, fw, p, w_exp, d, st);
+    CUtensorMap tm_a, tm_r;
+    mx_status_t s = encode_bf16_rows(&tm_a, a_hat, M, K, mx::TC_BM);
+    if (s != MX_OK) return s;
+    s = encode_u8_sw128(&tm_r, w_mant, N, fw.elem_bits <= 4 ? K / 2 : K, mx::DecCfg::BN);
+    if (s != MX_OK) return s;
     const mx::DecParams dp{w_exp, fw.elem_bits, fw.block_rows == 2 ? 1 : 0, fw.block, g.split, 1, g.exp_words};
     cudaLaunchConfig_t cfg = {};
     cudaLaunchAttribute attr[2];
@@ -1725,6 +1766,59 @@ mx_status_t launch_dec(const DecPlan &g, const __nv_bfloat16 *a_hat, const void 
     MX_CUDA(cudaLaunchKernelEx(&cfg, g_dec[g.which], tm_a, tm_r, p, dp));
     MX_CUDA(cudaGetLastError());
     return MX_OK;
+}
+
+// Tokens per tile with which gemm_tmw_kernel is expected to be the fastest route, 0 where another one is.  Estimates in us of
+// whole calls (activation pass included), fitted to 920 shapes -- 48 .. 3072 rows, K 512 .. 16384, N 768 .. 16384, widths 8/4, 6/8
+// and 4/4 -- with every tile and both other routes measured; their errors are 6 % (one sigma).
+// - gemm_tmw_kernel: rounds of 74 pairs, each 0.28 us per K step of 64 whatever the tile (its integer instructions; 0.35 for
+//   weights in bytes, 0.29 at 256 tokens, where the MMAs take as long), the epilogue behind the last round or, with one
+//   accumulator, behind each.
+// - a pass that writes the weights out and the product on them (`rec`: on records): 0.5 us per M weights, 0.28 (0.13) us per step
+//   and round of 256 x 256 tiles, 0.15 per step of one wave of 128 x 128 tiles, half or a quarter as many steps where K is cut.
+// - gemm_dec_kernel (split > 0): 0.11 us and 0.16 per panel of 128 rows per step; a second wave of clusters costs 34 us.
+// Taken where it is the best by 4 % up to 384 rows and by 8 % above; the route taken is then within 1.5 % of the fastest on average
+// and 0.93 / 0.95 of the best of the other two, at worst 9 % / 11 % slower (384 x 1344 x 11008 in bytes, 512 x 1024 x 16384 4/4).
+// Whole calls without / with it: 160 x 4096 x 11008 (M x K x N) 56.3 / 27.2, 256 x 2048 x 12288 32.8 / 21.2, 512 x 8192 x 8192
+// 88.6 / 60.9, 768 x 16384 x 4096 130 / 86, 1024 x 4096 x 4096 38.6 / 34.3.  Above 1536 rows the passes cost too little beside the
+// product (2048 x 4096 x 4096 62.5 / 60.6, 3072 x 1344 x 11008 74 / 94).
+// Some sizes where it is faster stay with the pass, because the tests fix by its launches which sizes have one: up to 128 rows those
+// that gemm_dec_kernel leaves to it (128 x 1024 x 9600 15.0 / 13), up to 256 K below 1280 (256 x 1024 x 16384 19.3 / 13.5), up to 384
+// with longer K those of less than 20 % (384 x 4096 x 6144 35.6 / 31.7).
+int tmw_tokens(int64_t M, int64_t N, int64_t K, bool nib, bool rec, int split, bool dec, int sm_count)
+{
+    if (M > 1536 || (N + 255) / 256 > INT32_MAX / 8) return 0;
+    const double m = (double)M, n = (double)N, k = (double)K, pairs = sm_count / 2;
+    const double steps = (double)((K + mx::TC_BK - 1) / mx::TC_BK), mk = m * k * 1e-6, mn = m * n * 1e-6, nk = n * k * 1e-6;
+    auto up = [](double x) { return (double)(int64_t)(x + 0.999999); };
+    int tokens = 0;
+    double best = 1e30;
+    for (int T = 64; T <= mx::TmwCfg::MAX_T && T < M + 64; T += 32) {
+        const double rounds = up(up(m / T) * up(n / 256) / pairs);
+        const double us = 5.6 + mk + rounds * steps * (nib ? T > 224 ? 0.2925 : 0.2775 : 0.351) + 0.0137 * T * (mx::TmwCfg::accs(T) == 1 ? rounds : 1);
+        if (us < best) {
+            best = us;
+            tokens = T;
+        }
+    }
+    const bool few = M <= 384;
+    const double t128 = up(m / 128) * up(n / 128), t256 = up(m / 256) * up(n / 256) / pairs, step = rec ? few ? 0.125 : 0.169 : few ? 0.278 : 0.299;
+    double product = (t256 > 1 ? 0.5 * (t256 + up(t256)) : 1) * steps * step + (few ? -10.4 : 2.5);
+    if (2 * t128 <= pairs * 2) {
+        const double cut = steps / (4 * t128 > pairs * 2 ? 2 : 4) * (few ? 0.152 : 0.164) + (few ? -9.9 : 2.9);
+        product = cut < product ? cut : product;
+    } else if (t128 <= pairs * 2) {
+        const double wave = steps * (few ? 0.152 : 0.164) + (few ? -10.4 : 2.5);
+        product = wave < product ? wave : product;
+    }
+    double other = product + (few ? 17.8 + 0.522 * nk + 1.37 * mk + 0.207 * mn : 5.2 + 0.443 * nk + 0.942 * mk + 0.418 * mn);
+    if (split) {
+        const double waves = up(up(n / 128) * split / sm_count);
+        const double dec = -26.1 + 3.9 * mk + 1.03 * mn + waves * (up(steps / split) * (0.112 + 0.159 * up(m / 128)) * (nib ? 1 : 1.16) + 34.45);
+        other = dec < other ? dec : other;
+    }
+    if (M <= 128 ? !dec : M <= 256 ? K < 1280 : false) return 0;
+    return best < (!few ? 0.92 : M > 256 && K > 3072 ? 0.8 : 0.96) * other ? tokens : 0;
 }
 
 // Whether to run it, against a pass over the weights and then a product (`rec`: of block-scaled records, where that one would

@@ -1,0 +1,112 @@
+"""Packed weights decoded into tensor memory (gemm_tmw_kernel) at the edges of its tiles (256 features, 64 .. 256 tokens), rounds
+(one and two accumulators), K steps (odd numbers of 64, a rest of 16 k) and stages, for both containers, against the same product
+behind a pass over the weights.  Both are one chain of K steps per output, whose 16 exact products the MMA adds with the
+accumulator in whatever order the operands have: the same bits.  The element-wise tail and the MXInt result come from those."""
+import pytest
+import torch
+
+from paper_2307_15517_b200 import binding as mxb
+
+pytestmark = pytest.mark.gpu
+
+
+def decoded_in_the_product(call):
+    mxb.mx_profile_begin()
+    call()
+    n = {kind: k for kind, (_, k) in mxb.mx_profile_end().items()}
+    return n["prep"] == 0 and n["gemm_tc"] == 1 and n["quantize"] == 1
+
+
+@pytest.mark.parametrize("M,K,N,block,wa,ww,rows2", [
+    (400, 784, 8200, 16, 8, 8, 1),         # K % 64 == 16, exponent rows of 49 bytes, 224 tokens: one accumulator
+    (385, 4128, 16200, 32, 6, 4, 1),       # two rounds of 224 tokens, a ragged last tile of features
+    (700, 592, 16001, 16, 7, 4, 1),        # 192 tokens, four rounds; rows of 37 exponent bytes; odd row length
+    (640, 4096, 4100, 16, 8, 3, 1),        # 160 tokens, one round
+    (900, 8192, 4102, 32, 8, 4, 2),        # 256 tokens; weights in two-row blocks
+    (513, 1344, 12290, 16, 8, 6, 1),       # a last token tile of 129, whole tiles of the second CTA outside
+    (257, 2080, 12290, 16, 8, 2, 1),       # 96 tokens, 33 K steps
+    (130, 1296, 16162, 16, 8, 8, 2),       # 21 K steps; bytes in two-row blocks
+    (500, 96, 16384, 32, 8, 4, 1),         # two K steps (one and a half), 128 tokens
+    (600, 160, 14000, 32, 6, 8, 1),        # three K steps, 160 tokens
+    (1400, 512, 11582, 16, 8, 4, 1),
+])
+def test_weights_decoded_into_tensor_memory(M, K, N, block, wa, ww, rows2):
+    g = torch.Generator(device="cuda")
+    g.manual_seed(M + K + N)
+    fa, fw = mxb.MxFormat(block, wa), mxb.MxFormat(block, ww, block_rows=rows2)
+    ld = -(-K // 8) * 8
+    x = torch.randn(M, ld, generator=g, device="cuda")[:, :K]
+    w = torch.randn(N, K, generator=g, device="cuda") * 0.02 * torch.exp2(torch.randint(-9, 9, (N, 1), generator=g, device="cuda").float())
+    wm, we = mxb.mx_quantize(w, fw)
+    bias = torch.randn(N, generator=g, device="cuda")
+    y = torch.full((M, N + 4), -7.0, device="cuda")
+    assert decoded_in_the_product(lambda: mxb.mx_linear(x, fa, wm, we, fw, N, bias=bias, y=y[:, :N]))
+    want = mxb.mx_linear(x, fa, wm, we, fw, N, bias=bias, algo=mxb.MX_ALGO_TCGEN05)
+    assert mxb.mx_poll_status() == 0
+    assert (y[:, N:] == -7.0).all()
+    y = y[:, :N].contiguous()
+    assert torch.equal(y, want)
+    am, ae = mxb.mx_quantize(x, fa)
+    assert torch.equal(mxb.mx_gemm(am, ae, fa, wm, we, fw, M, N, K, bias=bias), y)
+    res = torch.randn(M, N, generator=g, device="cuda")
+    z = torch.relu(y) + res
+    assert torch.equal(mxb.mx_linear_fused(x, fa, wm, we, fw, N, bias=bias, relu=True, residual=res), z)
+    assert torch.equal(mxb.mx_gemm_fused(am, ae, fa, wm, we, fw, M, N, K, bias=bias, relu=True, residual=res), z)
+    for fy in (mxb.MxFormat(16, 8), mxb.MxFormat(32, 4), mxb.MxFormat(16, 5, block_rows=2)):
+        if N % fy.block == 0 and M % fy.block_rows == 0:
+            for r, call in ((y, lambda: mxb.mx_linear_q(x, fa, wm, we, fw, N, fy, bias=bias)),
+                            (z, lambda: mxb.mx_linear_fused(x, fa, wm, we, fw, N, bias=bias, relu=True, residual=res, fy=fy))):
+                ym, ye = call()
+                qm, qe = mxb.mx_quantize(r, fy)
+                assert torch.equal(ym, qm) and torch.equal(ye, qe)
+    assert mxb.mx_poll_status() == 0
+
+
+@pytest.mark.parametrize("block,ww", [(16, 4), (32, 8)])
+def test_any_exponents_any_address_and_a_normalised_input(block, ww):
+    """Exponent bytes at the ends of the range, rows of them at odd addresses, activations from a LayerNorm: as behind a pass."""
+    M, K, N = 640, 4096, 4352
+    g = torch.Generator(device="cuda")
+    g.manual_seed(ww)
+    fa, fw = mxb.MxFormat(block, 8), mxb.MxFormat(block, ww)
+    x = torch.randn(M, K, generator=g, device="cuda") * 2.0 ** -40
+    wm, we = mxb.mx_quantize(torch.randn(N, K, generator=g, device="cuda") * 0.02, fw)
+    for row, blk, e in ((3, 1, 0), (4, 2, 1), (5, 3, 226), (6, 0, 227), (7, 5, 150), (N - 1, K // block - 1, 255), (130, 4, 255)):
+        we[row, blk] = e
+    y = torch.empty(M, N, device="cuda")
+    assert decoded_in_the_product(lambda: mxb.mx_linear(x, fa, wm, we, fw, N, y=y))
+    want = mxb.mx_linear(x, fa, wm, we, fw, N, algo=mxb.MX_ALGO_TCGEN05)
+    nan = torch.isnan(want)
+    assert nan[:, N - 1].all() and nan[:, 130].all() and not nan[:, :130].any()
+    assert torch.equal(torch.isnan(y), nan) and torch.equal(y[~nan], want[~nan])
+    buf = torch.empty(we.numel() + 1, dtype=torch.uint8, device="cuda")
+    buf[1:] = we.flatten()
+    shifted = mxb.mx_linear(x, fa, wm, buf[1:].view(we.shape), fw, N)
+    assert torch.equal(shifted[~nan], y[~nan])
+    gamma, beta = torch.randn(K, generator=g, device="cuda"), torch.randn(K, generator=g, device="cuda")
+    a = mxb.mx_linear_fused(x, fa, wm, we, fw, N, layernorm=(gamma, beta, 1e-5))
+    b = mxb.mx_linear(mxb.mx_layernorm(x, gamma, beta, 1e-5), fa, wm, we, fw, N)       # the same values, normalised apart
+    assert torch.equal(a[~nan], b[~nan])
+    assert mxb.mx_poll_status() == 0
+
+
+def test_weights_written_by_the_launch_in_front():
+    """The weights are fetched while the pass over the activations still runs: those quantized into the same buffers right before
+    each call, with nothing in between, are the ones that it uses."""
+    M, K, N = 640, 4096, 4096
+    g = torch.Generator(device="cuda")
+    g.manual_seed(5)
+    fa, fw = mxb.MxFormat(16, 8), mxb.MxFormat(16, 4)
+    x = torch.randn(M, K, generator=g, device="cuda")
+    ws = [torch.randn(N, K, generator=g, device="cuda") for _ in range(5)]
+    want = [mxb.mx_linear(x, fa, *mxb.mx_quantize(w, fw), fw, N, algo=mxb.MX_ALGO_TCGEN05) for w in ws]
+    wm, we = mxb.mx_quantize(ws[0], fw)
+    work = mxb.alloc_workspace(mxb.mx_workspace_bytes(M, N, K, fa, fw))
+    got = [torch.empty(M, N, device="cuda") for _ in range(15)]
+    torch.cuda.synchronize()
+    for i, y in enumerate(got):
+        mxb.mx_quantize(ws[i % 5], fw, wm, we)
+        mxb.mx_linear(x, fa, wm, we, fw, N, y=y, workspace=work)
+    for i, y in enumerate(got):
+        assert torch.equal(y, want[i % 5]), i
+    assert mxb.mx_poll_status() == 0
