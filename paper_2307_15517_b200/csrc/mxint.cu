@@ -1180,6 +1180,19 @@ int wide_pair_tile(int64_t M, int64_t N, int64_t K, const DeviceInfo &d)
     return width;
 }
 
+// Width of the pair tiles that fill one round, where the tiles of one CTA would fill one too, else 0.  An SM takes in 58 bytes per
+// clock, and a 128 x 256 tile of one CTA needs 48 KB per K step of 64, half a 256 x W pair tile (128 + W / 2) * 128 bytes: from 160 to
+// 224 columns the pair tiles are the faster ones by 5 to 15 %.  Whole calls (us): 1237 x 2048 x 2048 (M x K x N) 21.2 / 18.2, 1024 x 2048
+// x 3002 23.1 / 20.6, 1536 x 4096 x 2048 37.0 / 33.1, 768 x 4096 x 4096 37.5 / 33.4, 512 x 2048 x 6144 25.3 / 22.3.  Narrower ones are as
+// many as the 128 x 128 tiles and gain nothing (1024 x 2048 x 2048, 128 columns, 16.1 / 16.9), 256 columns neither (24.1 / 24.6).
+int one_round_width(int64_t M, int64_t N, const DeviceInfo &d)
+{
+    const int64_t rows = (M + 255) / 256, cols = d.sm_count / 2 / rows;
+    if (!cols) return 0;
+    const int64_t w = ((N + cols - 1) / cols + 31) / 32 * 32;
+    return w >= 160 && w <= 224 ? (int)w : 0;
+}
+
 // Pre-decoded bf16 weights (both operands fetched by TMA).  may_split: K may be cut (the sum is then not one chain).
 mx_status_t run_tc(const __nv_bfloat16 *a_hat, const __nv_bfloat16 *w_hat, int64_t M, int64_t N,
                    int64_t K, const float *bias, float *y, int64_t ldy, DeviceInfo &d, cudaStream_t st,
@@ -1201,6 +1214,10 @@ mx_status_t run_tc(const __nv_bfloat16 *a_hat, const __nv_bfloat16 *w_hat, int64
         const int width = wide_pair_tile(M, N, K, d);
         if (width) return launch_tcw(a_hat, w_hat, M, N, K, width, bias, y, ldy, yq, d, st, et);
         return launch_tc2(a_hat, w_hat, M, N, K, bias, y, ldy, yq, d, st, et);
+    }
+    if (tb.count == 1 && M > 128) {
+        const int width = one_round_width(M, N, d);
+        if (width) return launch_tcw(a_hat, w_hat, M, N, K, width, bias, y, ldy, yq, d, st, et);
     }
     if (may_split && tb.count == 1) {
         int split = 0;

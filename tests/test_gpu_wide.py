@@ -83,3 +83,18 @@ def test_every_width_has_the_bits_of_narrow_calls(M, N, K, width):
 def test_exponents_at_the_ends_of_the_range_on_wide_tiles():
     from tests.test_gpu_dec import check_ends_of_the_range
     check_ends_of_the_range(414, 1040, 9686, 16, 4)
+
+
+# one round of tiles narrower than 256 columns: 224, 192 and 160 on 148 SMs, ragged in M, N and K
+@pytest.mark.parametrize("M,N,K", [(1237, 3002, 2080), (760, 4600, 1040), (1530, 1900, 528), (250, 11008, 1040)])
+def test_one_round_of_narrow_pair_tiles_has_the_bits_of_narrow_calls(M, N, K):
+    g, x, fa, wm, we, fw = _operands(M, N, K, M + N)
+    bias = torch.randn(N, generator=g, device="cuda")
+    y = torch.full((M, N + 5), -3.0, device="cuda")
+    mxb.mx_linear(x, fa, wm, we, fw, N, bias=bias, y=y[:, :N], algo=mxb.MX_ALGO_TCGEN05)
+    for n in range(0, N, 512):
+        cols = min(512, N - n)
+        assert torch.equal(y[:, n:n + cols], mxb.mx_linear(x, fa, wm[n:n + cols], we[n:n + cols], fw, cols, bias=bias[n:n + cols].clone(),
+                                                           algo=mxb.MX_ALGO_TCGEN05))
+    assert (y[:, N:] == -3.0).all()
+    assert mxb.mx_poll_status() == 0
