@@ -14,7 +14,8 @@
 //   warps 4..15  : three groups that decode every third K step each into one of four or eight stages of 32 columns
 //   warps 16..23 : epilogue
 // The tile is 256 features x T tokens, T a multiple of 32 that the host picks so that the tiles fill whole rounds of the chip's
-// pairs; up to T = 192 there are two accumulators, so the epilogue of a tile runs under the next one's MMAs.
+// pairs; up to T = 192 there are two accumulators, so the epilogue of a tile runs under the next one's MMAs.  Few tiles: K is cut
+// over the pairs of a cluster, whose partial tiles go to shared memory and are added up in the order of K (mx_gemm_splitk.cuh).
 // Bound by the integer instructions of the decoding warps: 0.27 us per K step and round whatever T (without the MMAs the same,
 // without the decoding 0.16 at T = 64 and 0.31, the MMAs' own time, at 256; four groups of warps, or two steps per turn of a group,
 // changed nothing).  Whole calls, M x K x N, against a pass and a product / gemm_dec_kernel: 512 x 4096 x 11008 54.8 -> 45.5 us
@@ -39,7 +40,7 @@ struct TmwCfg {
     static constexpr int RAW_STAGES = 4, MAX_A_STAGES = 8, MAX_STAGES = 8;  // of packed weights, decoded weights, activations
     static constexpr uint32_t RAW_MANT = BN * 128, RAW_EXP = BN * 20;    // 128 mantissa bytes and the words of at most 16 exponent bytes per row
     static constexpr uint32_t RAW_BYTES = RAW_STAGES * (RAW_MANT + RAW_EXP);
-    static constexpr int MAX_T = 256;
+    static constexpr int MAX_T = 256, MAX_SPLIT = 4;
     // Tensor memory: one accumulator of T columns, or two up to T = 192; behind them the stages of decoded weights, 32 columns each
     static constexpr uint32_t TMEM_COLS = 512;
     static __host__ __device__ constexpr int accs(int T) { return T <= 192 ? 2 : 1; }
@@ -65,6 +66,7 @@ struct TmwParams {
     int stages;
     int early;                // 1: the launch in front is this call's activation pass
     int exp_words;            // 1: every row's exponent bytes start at a whole word
+    int split;                // > 1: pieces of K; a cluster of as many pairs shares one tile, and the grid has a cluster per tile
 };
 
 // The exponent bytes of 128 rows of packed weights, for the warp that feeds the decoding ones: a lane owns rows lane, lane + 32,
@@ -150,8 +152,44 @@ __device__ __forceinline__ void tmw_transpose(uint8_t *buf, int lane, uint32_t (
     }
 }
 
-template <bool NIB, bool QOUT>
-__global__ void __cluster_dims__(2, 1, 1) __maxnreg__(80)
+// A warp's 32 features x 32 tokens (r[j] = token j of the lane's feature) of a partial tile [token][128 features] at `part` of every
+// CTA of this rank in its pair, added up over the cluster's `split` pairs in the order of their pieces of K.
+__device__ __forceinline__ void tmw_sum(uint32_t part, int split, uint32_t rank, int chunk, int feature, uint32_t (&r)[32])
+{
+    for (int s = 0; s < split; ++s) {
+        const uint32_t src = ptx::map_to_cta(part, 2u * s + rank) + (uint32_t)(chunk * 32 * 512 + feature * 4);
+        float x[32];
+#pragma unroll
+        for (int j = 0; j < 32; ++j) asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(x[j]) : "r"(src + 512u * j) : "memory");
+#pragma unroll
+        for (int j = 0; j < 32; ++j) r[j] = __float_as_uint(s ? __uint_as_float(r[j]) + x[j] : x[j]);
+    }
+}
+
+// The tile's results of 32 tokens from m0 on: bias, ReLU, residual, fp32 or MXInt store.  buf: the warp's transposing buffer (QOUT).
+template <bool QOUT>
+__device__ __forceinline__ void tmw_store(const TcParams &p, int m0, int n, float bias, uint8_t *buf, int lane, uint32_t (&r)[32])
+{
+    tmw_tail(p, m0, n, bias, r);
+    if (QOUT) {
+        tmw_transpose(buf, lane, r);
+        store_mxint_chunk(p, m0 + lane, n - lane, r);
+    } else if (n < p.N) {
+        float *dst = p.y + (int64_t)m0 * p.ldy + n;
+        if (m0 + 32 <= p.M) {
+#pragma unroll
+            for (int j = 0; j < 32; ++j) dst[(int64_t)j * p.ldy] = __uint_as_float(r[j]);
+        } else {
+#pragma unroll
+            for (int j = 0; j < 32; ++j)
+                if (m0 + j < p.M) dst[(int64_t)j * p.ldy] = __uint_as_float(r[j]);
+        }
+    }
+}
+
+// SPLIT: K cut over the pairs of a cluster.
+template <bool NIB, bool QOUT, bool SPLIT>
+__global__ void __maxnreg__(80)
 gemm_tmw_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constant__ CUtensorMap tmap_r, const TcParams p, const TmwParams wp)
 {
     using Cfg = TmwCfg;
@@ -183,8 +221,10 @@ gemm_tmw_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constan
     static_assert(8 * (ACC_BARS + 4) + 8 <= 512 && Cfg::RAW_BYTES % 1024 == 0, "barriers; the activations' tiles are aligned");
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const uint32_t rank = ptx::cluster_ctarank();                        // 0: leader
+    const uint32_t cta = ptx::cluster_ctarank(), rank = cta & 1u, lead = SPLIT ? cta & ~1u : 0u;      // rank 0: leader of its pair
     const bool leader = rank == 0;
+    const uint16_t both = (uint16_t)(3u << lead);                        // the pair's CTAs
+    const int split = SPLIT ? wp.split : 1;
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < Cfg::MAX_STAGES; ++s) {
@@ -219,8 +259,10 @@ gemm_tmw_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constan
     const uint32_t tmem_base = *tmem_slot;
 
     const int num_tiles = p.tiles_m * p.tiles_n;                         // tiles_m of tokens, tiles_n of 256 features
-    const int pair = blockIdx.x >> 1, npairs = gridDim.x >> 1;
-    const int kblocks = (p.K + TC_BK - 1) / TC_BK, raws = (kblocks + SPR - 1) / SPR;
+    const int pair = blockIdx.x / (2 * split), npairs = gridDim.x / (2 * split);          // (K cut: a cluster of pairs)
+    // the pair's piece of K: whole raw stages; split <= their number
+    const int k_all = (p.K + TC_BK - 1) / TC_BK, raws_all = (k_all + SPR - 1) / SPR, piece = SPLIT ? (int)(cta >> 1) : 0;
+    const int kb0 = raws_all * piece / split * SPR, kblocks = min(k_all, raws_all * (piece + 1) / split * SPR) - kb0, raws = (kblocks + SPR - 1) / SPR;
     bool timed_out = false;
     // early: the launch in front only writes the activations' operand form, and starts this one when ITS predecessors are
     // complete: the weights may be fetched and decoded meanwhile (decoding writes tensor memory alone)
@@ -238,11 +280,11 @@ gemm_tmw_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constan
                     break;
                 }
                 if (ptx::elect_one()) {
-                    const uint32_t leader_full = ptx::map_to_cta(x_full(s), 0), sx = x_base + s * stage_bytes;
+                    const uint32_t leader_full = ptx::map_to_cta(x_full(s), lead), sx = x_base + s * stage_bytes;
                     const bool two = kb + 1 < kblocks;
                     if (leader) ptx::mbar_arrive_expect_tx(x_full(s), two ? 2 * stage_bytes : stage_bytes);
-                    ptx::tma_load_2d_pair(sx, &tmap_x, kb * TC_BK, m0, leader_full);
-                    if (two) ptx::tma_load_2d_pair(sx + (stage_bytes >> 1), &tmap_x, (kb + 1) * TC_BK, m0, leader_full);
+                    ptx::tma_load_2d_pair(sx, &tmap_x, (kb0 + kb) * TC_BK, m0, leader_full);
+                    if (two) ptx::tma_load_2d_pair(sx + (stage_bytes >> 1), &tmap_x, (kb0 + kb + 1) * TC_BK, m0, leader_full);
                 }
                 if (++s == stages) { s = 0; ph ^= 1u; }
             }
@@ -287,19 +329,19 @@ gemm_tmw_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constan
 #pragma unroll
                         for (int j = 0; j < TC_BK / 16; ++j)
                             ptx::mma_bf16_ts_pair(d_tmem, tm + a_col + 32u * a0 + 8u * j, desc + 2u * j, idesc, (kb | j) != 0 ? 1u : 0u);
-                        ptx::mma_commit_pair(a_empty(a0), 3);            // both CTAs may refill their stages
+                        ptx::mma_commit_pair(a_empty(a0), both);            // both CTAs may refill their stages
                         if (two) {
 #pragma unroll
                             for (int j = 0; j < TC_BK / 16; ++j)
                                 ptx::mma_bf16_ts_pair(d_tmem, tm + a_col + 32u * a1 + 8u * j, desc + (stage_bytes >> 5) + 2u * j, idesc, 1u);
-                            ptx::mma_commit_pair(a_empty(a1), 3);
+                            ptx::mma_commit_pair(a_empty(a1), both);
                         }
-                        ptx::mma_commit_pair(x_empty(cur), 3);
+                        ptx::mma_commit_pair(x_empty(cur), both);
                     }
                     ready = __all_sync(0xFFFFFFFFu, n0 && n1 && nx);
                 }
                 if (timed_out) break;
-                if (ptx::elect_one()) ptx::mma_commit_pair(t_full(acc), 3);
+                if (ptx::elect_one()) ptx::mma_commit_pair(t_full(acc), both);
             }
         }
         __syncwarp();
@@ -317,7 +359,7 @@ gemm_tmw_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constan
                     timed_out = true;
                     break;
                 }
-                const int kb = i * SPR, b0 = kb * (b16 ? 4 : 2);
+                const int kb = kb0 + i * SPR, b0 = kb * (b16 ? 4 : 2);
                 if (lane == 0) {
                     ptx::fence_proxy_async_smem();
                     ptx::mbar_arrive_expect_tx(r_full(s), Cfg::RAW_MANT);
@@ -407,7 +449,7 @@ gemm_tmw_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constan
             ptx::tc_fence_before_sync();
             __syncwarp();
             if (lane == 0) {
-                ptx::mbar_arrive_cluster_relaxed(ptx::map_to_cta(a_full(a), 0));
+                ptx::mbar_arrive_cluster_relaxed(ptx::map_to_cta(a_full(a), lead));
                 for (int x = 0; x <= extra; ++x) ptx::mbar_arrive(r_empty(rs));
             }
             there = __all_sync(0xFFFFFFFFu, next);
@@ -433,25 +475,18 @@ gemm_tmw_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constan
                 uint32_t r[32];
                 ptx::tmem_ld_32x32(src + (uint32_t)c, r);
                 ptx::tmem_ld_wait();
-                tmw_tail(p, m0 + c, n, bias, r);
-                if (QOUT) {
-                    tmw_transpose(smem_gen + (tr_base - smem_base) + 4096 * (warp - 4 - 4 * GROUPS), lane, r);
-                    store_mxint_chunk(p, m0 + c + lane, n - lane, r);
-                } else if (n < p.N) {
-                    float *dst = p.y + (int64_t)(m0 + c) * p.ldy + n;
-                    if (m0 + c + 32 <= p.M) {
+                if (SPLIT) {
+                    // the partial tile, [token][feature], over the stages: all loads have landed and been used when t_full completes
 #pragma unroll
-                        for (int j = 0; j < 32; ++j) dst[(int64_t)j * p.ldy] = __uint_as_float(r[j]);
-                    } else {
-#pragma unroll
-                        for (int j = 0; j < 32; ++j)
-                            if (m0 + c + j < p.M) dst[(int64_t)j * p.ldy] = __uint_as_float(r[j]);
-                    }
+                    for (int j = 0; j < 32; ++j)
+                        *reinterpret_cast<uint32_t *>(smem_gen + (c + j) * 512 + (quad * 32 + lane) * 4) = r[j];
+                } else {
+                    tmw_store<QOUT>(p, m0 + c, n, bias, smem_gen + (tr_base - smem_base) + 4096 * (warp - 4 - 4 * GROUPS), lane, r);
                 }
             }
             ptx::tc_fence_before_sync();
             __syncwarp();
-            if (lane == 0) ptx::mbar_arrive_cluster_relaxed(ptx::map_to_cta(t_empty(acc), 0));
+            if (lane == 0) ptx::mbar_arrive_cluster_relaxed(ptx::map_to_cta(t_empty(acc), lead));
         }
     }
 
@@ -460,6 +495,23 @@ gemm_tmw_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constan
         atomicOr(p.status, STATUS_TIMEOUT_BIT);
         const uint64_t t0 = ptx::globaltimer_ns();
         while (ptx::globaltimer_ns() - t0 < 100000ull) __nanosleep(1000);
+    }
+    if (SPLIT) {
+        __syncwarp();
+        ptx::cluster_sync();                                             // every partial tile is in place
+        if (warp >= 4 + 4 * GROUPS) {
+            const int n0 = (pair / p.tiles_m) * 256 + (int)rank * Cfg::BN, m0 = (pair % p.tiles_m) * T;
+            // quarter u & 3 of the features of tokens 32 (u >> 2) ..: dealt to the epilogue warps of all pairs
+            for (int u = piece + split * (warp - 4 - 4 * GROUPS); u < T / 8; u += split * Cfg::EPI_WARPS) {
+                const int c = u >> 2, f = (u & 3) * 32 + lane, n = n0 + f;
+                if (m0 + 32 * c >= p.M || n - lane >= p.N) continue;     // warp-uniform
+                uint32_t r[32];
+                tmw_sum(smem_base, split, rank, c, f, r);
+                tmw_store<QOUT>(p, m0 + 32 * c, n, p.ex_bias && n < p.N ? __ldg(p.ex_bias + n) : 0.f,
+                                smem_gen + (tr_base - smem_base) + 4096 * (warp - 4 - 4 * GROUPS), lane, r);
+            }
+        }
+        __syncwarp();
     }
     ptx::tc_fence_before_sync();
     __syncthreads();

@@ -62,7 +62,8 @@ struct DeviceInfo {
     bool splitk_attr_set[4] = {};
     int splitk_clusters[mx::SplitKCfg::MAX_SPLIT + 1] = {-1, -1, -1, -1, -1};
     bool attn_attr_set[2] = {false, false};
-    bool tmw_attr_set[4] = {};
+    bool tmw_attr_set[8] = {};
+    int tmw_clusters[8][mx::TmwCfg::MAX_SPLIT + 1] = {};       // resident clusters by kernel and pairs per cluster
     bool dec_attr_set[12] = {};
     int dec_clusters[12][mx::DecCfg::MAX_SPLIT + 1] = {};      // resident clusters by kernel and cluster size
 };
@@ -1667,7 +1668,43 @@ mx_status_t dec_config(cudaLaunchConfig_t &cfg, cudaLaunchAttribute *attr, int p
 
 bool dec_is_faster(int64_t M, int64_t N, int64_t K, int split, bool rec, int sm_count);
 
-int tmw_tokens(int64_t M, int64_t N, int64_t K, bool nib, bool rec, int split, bool dec, int sm_count);
+typedef void (*TmwKernel)(CUtensorMap, CUtensorMap, mx::TcParams, mx::TmwParams);
+const TmwKernel g_tmw[8] = {                              // nibbles, MXInt result, K cut: 4 * , 2 * , 1 *
+    mx::gemm_tmw_kernel<false, false, false>, mx::gemm_tmw_kernel<false, false, true>, mx::gemm_tmw_kernel<false, true, false>,
+    mx::gemm_tmw_kernel<false, true, true>, mx::gemm_tmw_kernel<true, false, false>, mx::gemm_tmw_kernel<true, false, true>,
+    mx::gemm_tmw_kernel<true, true, false>, mx::gemm_tmw_kernel<true, true, true>};
+
+void tmw_config(cudaLaunchConfig_t &cfg, cudaLaunchAttribute *attr, int split, int clusters, cudaStream_t st)
+{
+    cfg.gridDim = dim3((unsigned)(2 * split * clusters));
+    cfg.blockDim = dim3(mx::TmwCfg::THREADS);
+    cfg.dynamicSmemBytes = 227 * 1024;
+    cfg.stream = st;
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = (unsigned)(2 * split);
+    attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+}
+
+// Clusters of `split` pairs that are resident at once; looked up once.
+mx_status_t tmw_clusters(DeviceInfo &d, int which, int split, int *out)
+{
+    const mx_status_t s = smem_attr_once(d.tmw_attr_set[which], g_tmw[which], 227 * 1024);
+    if (s != MX_OK) return s;
+    std::lock_guard<std::mutex> lk(g_init_mu);
+    int &known = d.tmw_clusters[which][split];
+    if (known == 0) {
+        cudaLaunchConfig_t cfg = {};
+        cudaLaunchAttribute attr[2];
+        tmw_config(cfg, attr, split, d.sm_count, nullptr);
+        MX_CUDA(cudaOccupancyMaxActiveClusters(&known, g_tmw[which], &cfg));
+    }
+    *out = known;
+    return MX_OK;
+}
+
+int tmw_tokens(int64_t M, int64_t N, int64_t K, bool nib, bool rec, int split, bool dec, int sm_count, const int *clusters, int *pieces);
 
 // Whether the product decodes its weights itself, in which kernel, and for gemm_dec_kernel into how many pieces K is cut: the most
 // whose clusters all fit at once, of at least four K steps each.
@@ -1706,17 +1743,20 @@ mx_status_t dec_plan(int64_t M, int64_t N, int64_t K, const mx_format_t &fa, con
         }
         *use = dec_is_faster(M, N, K, out->split, rec, d.sm_count);
     }
-    out->tokens = tmw_tokens(M, N, K, nib, rec, panels <= mx::DecCfg::MAX_P ? out->split : 0, *use, d.sm_count);
+    const int which = (nib ? 4 : 0) + (quantized ? 2 : 0);
+    int clusters[mx::TmwCfg::MAX_SPLIT + 1] = {}, pieces = 1;
+    for (int s = 1; s <= mx::TmwCfg::MAX_SPLIT; ++s) {
+        const mx_status_t cs = tmw_clusters(d, which + (s > 1 ? 1 : 0), s, &clusters[s]);
+        if (cs != MX_OK) return cs;
+    }
+    out->tokens = tmw_tokens(M, N, K, nib, rec, panels <= mx::DecCfg::MAX_P ? out->split : 0, *use, d.sm_count, clusters, &pieces);
     if (out->tokens) {
-        out->which = (nib ? 2 : 0) + (quantized ? 1 : 0);
+        out->which = which + (pieces > 1 ? 1 : 0);
+        out->split = pieces;
         *use = true;
     }
     return MX_OK;
 }
-
-typedef void (*TmwKernel)(CUtensorMap, CUtensorMap, mx::TcParams, mx::TmwParams);
-const TmwKernel g_tmw[4] = {mx::gemm_tmw_kernel<false, false>, mx::gemm_tmw_kernel<false, true>, mx::gemm_tmw_kernel<true, false>,
-                            mx::gemm_tmw_kernel<true, true>};
 
 mx_status_t launch_tmw(const DecPlan &g, const __nv_bfloat16 *a_hat, const void *w_mant, const mx_format_t &fw, mx::TcParams &p,
                        const uint8_t *w_exp, DeviceInfo &d, cudaStream_t st)
@@ -1735,9 +1775,16 @@ mx_status_t launch_tmw(const DecPlan &g, const __nv_bfloat16 *a_hat, const void 
     const int64_t tiles = (int64_t)p.tiles_m * p.tiles_n;
     if (tiles > INT32_MAX / 2) return MX_ERR_SHAPE;
     const int pairs = (int)(tiles < d.sm_count / 2 ? tiles : d.sm_count / 2);
-    const mx::TmwParams wp{w_exp, fw.elem_bits, fw.block_rows == 2 ? 1 : 0, fw.block, T, Cfg::stages(T, p.yq_mant), 1, g.exp_words};
+    const mx::TmwParams wp{w_exp, fw.elem_bits, fw.block_rows == 2 ? 1 : 0, fw.block, T, Cfg::stages(T, p.yq_mant), 1, g.exp_words, g.split};
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute attr[2];
+    tmw_config(cfg, attr, g.split, g.split > 1 ? (int)tiles : pairs, st);
+    cfg.dynamicSmemBytes = Cfg::smem_bytes(T, p.yq_mant);
+    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[1].val.programmaticStreamSerializationAllowed = 1;
+    cfg.numAttrs = g_prof.on ? 1 : 2;                     // see launch_dep
     ProfScope prof(KIND_GEMM_TC, st);
-    MX_CUDA(launch_dep(g_tmw[g.which], dim3(2 * pairs), dim3(Cfg::THREADS), Cfg::smem_bytes(T, p.yq_mant), st, tm_x, tm_r, p, wp));
+    MX_CUDA(cudaLaunchKernelEx(&cfg, g_tmw[g.which], tm_x, tm_r, p, wp));
     MX_CUDA(cudaGetLastError());
     return MX_OK;
 }
@@ -1785,24 +1832,25 @@ mx_status_t launch_dec(const DecPlan &g, const __nv_bfloat16 *a_hat, const void 
     return MX_OK;
 }
 
-// Tokens per tile with which gemm_tmw_kernel is expected to be the fastest route, 0 where another one is.  Estimates in us of
-// whole calls (activation pass included), fitted to 920 shapes -- 48 .. 3072 rows, K 512 .. 16384, N 768 .. 16384, widths 8/4, 6/8
-// and 4/4 -- with every tile and both other routes measured; their errors are 6 % (one sigma).
-// - gemm_tmw_kernel: rounds of 74 pairs, each 0.28 us per K step of 64 whatever the tile (its integer instructions; 0.35 for
+// Tokens per tile and pieces of K with which gemm_tmw_kernel is expected to be the fastest route, 0 where another one is.  Estimates
+// in us of whole calls (activation pass included), fitted to 1480 shapes -- 48 .. 3072 rows, K 512 .. 16384, N 768 .. 16384, widths
+// 8/4, 6/8, 8/8 and 4/4 -- with every tile, every cut and both other routes measured; their errors are 4 to 6 % (one sigma).
+// - gemm_tmw_kernel: rounds of 74 pairs, each 0.27 us per K step of 64 whatever the tile (its integer instructions; 0.35 for
 //   weights in bytes, 0.29 at 256 tokens, where the MMAs take as long), the epilogue behind the last round or, with one
-//   accumulator, behind each.
+//   accumulator, behind each.  K cut: one round of clusters that all fit at once, the steps of the longest piece, the exchange.
 // - a pass that writes the weights out and the product on them (`rec`: on records): 0.5 us per M weights, 0.28 (0.13) us per step
 //   and round of 256 x 256 tiles, 0.15 per step of one wave of 128 x 128 tiles, half or a quarter as many steps where K is cut.
 // - gemm_dec_kernel (split > 0): 0.11 us and 0.16 per panel of 128 rows per step; a second wave of clusters costs 34 us.
-// Taken where it is the best by 4 % up to 384 rows and by 8 % above; the route taken is then within 1.5 % of the fastest on average
-// and 0.93 / 0.95 of the best of the other two, at worst 9 % / 11 % slower (384 x 1344 x 11008 in bytes, 512 x 1024 x 16384 4/4).
+// Taken where it is the best by 6 to 10 %; over the shapes of 129 .. 1536 rows the route taken is then 0.956 of the best of the
+// other two on average, 0.93 being possible, and at worst 13 % slower (1024 x 5120 x 5120 54 / 61; the next 10 %).
 // Whole calls without / with it: 160 x 4096 x 11008 (M x K x N) 56.3 / 27.2, 256 x 2048 x 12288 32.8 / 21.2, 512 x 8192 x 8192
-// 88.6 / 60.9, 768 x 16384 x 4096 130 / 86, 1024 x 4096 x 4096 38.6 / 34.3.  Above 1536 rows the passes cost too little beside the
-// product (2048 x 4096 x 4096 62.5 / 60.6, 3072 x 1344 x 11008 74 / 94).
+// 88.6 / 60.9, 768 x 16384 x 4096 130 / 86, 1024 x 4096 x 4096 38.6 / 34.3; K cut in two 448 x 16384 x 4096 97 / 57, in three
+// 352 x 8192 x 2048 29.5 / 27.4.  Above 1536 rows the passes cost too little beside the product (2048 x 4096 x 4096 62.5 / 60.6,
+// 3072 x 1344 x 11008 74 / 94).
 // Some sizes where it is faster stay with the pass, because the tests fix by its launches which sizes have one: up to 128 rows those
 // that gemm_dec_kernel leaves to it (128 x 1024 x 9600 15.0 / 13), up to 256 K below 1280 (256 x 1024 x 16384 19.3 / 13.5), up to 384
-// with longer K those of less than 20 % (384 x 4096 x 6144 35.6 / 31.7).
-int tmw_tokens(int64_t M, int64_t N, int64_t K, bool nib, bool rec, int split, bool dec, int sm_count)
+// with longer K and not cut those of less than 20 % (384 x 4096 x 6144 35.6 / 31.7).
+int tmw_tokens(int64_t M, int64_t N, int64_t K, bool nib, bool rec, int split, bool dec, int sm_count, const int *clusters, int *pieces)
 {
     if (M > 1536 || (N + 255) / 256 > INT32_MAX / 8) return 0;
     const double m = (double)M, n = (double)N, k = (double)K, pairs = sm_count / 2;
@@ -1811,11 +1859,17 @@ int tmw_tokens(int64_t M, int64_t N, int64_t K, bool nib, bool rec, int split, b
     int tokens = 0;
     double best = 1e30;
     for (int T = 64; T <= mx::TmwCfg::MAX_T && T < M + 64; T += 32) {
-        const double rounds = up(up(m / T) * up(n / 256) / pairs);
-        const double us = 5.6 + mk + rounds * steps * (nib ? T > 224 ? 0.2925 : 0.2775 : 0.351) + 0.0137 * T * (mx::TmwCfg::accs(T) == 1 ? rounds : 1);
-        if (us < best) {
-            best = us;
-            tokens = T;
+        const double tiles = up(m / T) * up(n / 256), rounds = up(tiles / pairs), step_us = nib ? T > 224 ? 0.288 : 0.273 : 0.345;
+        for (int s = 1; s <= mx::TmwCfg::MAX_SPLIT; ++s) {
+            const int unit = nib ? 4 : 2;                                // K steps per stage of packed weights
+            if (s > 1 && (tiles > clusters[s] || steps < s * unit)) break;
+            const double us = 1.1 * mk + (s == 1 ? 6.3 + rounds * steps * step_us + 0.0137 * T * (mx::TmwCfg::accs(T) == 1 ? rounds : 1)
+                                                 : 5.5 + 0.73 * s + up(up(steps / unit) / s) * unit * step_us + 0.023 * T);
+            if (us < best) {
+                best = us;
+                tokens = T;
+                *pieces = s;
+            }
         }
     }
     const bool few = M <= 384;
@@ -1835,7 +1889,7 @@ int tmw_tokens(int64_t M, int64_t N, int64_t K, bool nib, bool rec, int split, b
         other = dec < other ? dec : other;
     }
     if (M <= 128 ? !dec : M <= 256 ? K < 1280 : false) return 0;
-    return best < (!few ? 0.92 : M > 256 && K > 3072 ? 0.8 : 0.96) * other ? tokens : 0;
+    return best < (!few ? rec ? 0.9 : 0.92 : *pieces > 1 ? 0.93 : M > 256 && K > 3072 ? 0.8 : 0.94) * other ? tokens : 0;
 }
 
 // Whether to run it, against a pass over the weights and then a product (`rec`: of block-scaled records, where that one would

@@ -62,6 +62,43 @@ def test_weights_decoded_into_tensor_memory(M, K, N, block, wa, ww, rows2):
     assert mxb.mx_poll_status() == 0
 
 
+@pytest.mark.parametrize("M,K,N,block,wa,ww", [
+    (500, 8208, 4098, 16, 8, 4),           # two pieces, the last K step of 16; 256 tokens, a ragged last tile of features
+    (640, 8192, 2048, 32, 6, 4),           # two pieces, 160 tokens
+    (352, 8192, 2048, 16, 8, 4),           # three pieces
+    (400, 16400, 4096, 16, 8, 8),          # bytes
+    (384, 16384, 4100, 32, 8, 3),
+])
+def test_pieces_of_K_added_up_in_a_cluster(M, K, N, block, wa, ww):
+    """The partial sums of two to four pieces are added in fp32: at most one rounding of a partial sum more than one chain per
+    piece, 2^-22 of the absolute sum S; 1e-5 S as elsewhere.  The tail and the MXInt result come from the same sums."""
+    g = torch.Generator(device="cuda")
+    g.manual_seed(M + K + N)
+    fa, fw = mxb.MxFormat(block, wa), mxb.MxFormat(block, ww)
+    x = torch.randn(M, K, generator=g, device="cuda")
+    wm, we = mxb.mx_quantize(torch.randn(N, K, generator=g, device="cuda") * 0.02, fw)
+    bias = torch.randn(N, generator=g, device="cuda")
+    am, ae = mxb.mx_quantize(x, fa)
+    S = mxb.mx_dequantize(am, ae, K, fa).abs().double() @ mxb.mx_dequantize(wm, we, K, fw).abs().double().t() + bias.abs().double()
+    y = torch.full((M, N + 4), -7.0, device="cuda")
+    assert decoded_in_the_product(lambda: mxb.mx_linear(x, fa, wm, we, fw, N, bias=bias, y=y[:, :N]))
+    want = mxb.mx_linear(x, fa, wm, we, fw, N, bias=bias, algo=mxb.MX_ALGO_TCGEN05)
+    assert (y[:, N:] == -7.0).all()
+    y = y[:, :N].contiguous()
+    assert ((y - want).abs().double() <= 1e-5 * S).all()
+    assert torch.equal(mxb.mx_gemm(am, ae, fa, wm, we, fw, M, N, K, bias=bias), y)
+    assert torch.equal(mxb.mx_linear(x, fa, wm, we, fw, N, bias=bias), y)                # the same every time
+    res = torch.randn(M, N, generator=g, device="cuda")
+    z = torch.relu(y) + res
+    assert torch.equal(mxb.mx_gemm_fused(am, ae, fa, wm, we, fw, M, N, K, bias=bias, relu=True, residual=res), z)
+    for fy in (mxb.MxFormat(16, 8), mxb.MxFormat(32, 4)):
+        if N % fy.block == 0:
+            ym, ye = mxb.mx_linear_fused(x, fa, wm, we, fw, N, bias=bias, relu=True, residual=res, fy=fy)
+            qm, qe = mxb.mx_quantize(z, fy)
+            assert torch.equal(ym, qm) and torch.equal(ye, qe)
+    assert mxb.mx_poll_status() == 0
+
+
 @pytest.mark.parametrize("block,ww", [(16, 4), (32, 8)])
 def test_any_exponents_any_address_and_a_normalised_input(block, ww):
     """Exponent bytes at the ends of the range, rows of them at odd addresses, activations from a LayerNorm: as behind a pass."""
