@@ -6,17 +6,18 @@
 // -- P panels of 128, an accumulator in tensor memory each -- and a piece of K (a cluster shares the tile, the partial tiles are
 // added through distributed shared memory as in mx_gemm_splitk.cuh); per K step of 64 it fetches P * 16 KB of A and 4 (8) KB of
 // packed weights, whose decoded tile serves all P panels.
-//   warp 0      : A tiles by TMA (one lane)
-//   warp 1      : tensor-memory allocation, MMA issue (one lane)
+//   warp 0      : A tiles by TMA
+//   warp 1      : tensor-memory allocation, MMA issue
 //   warp 2      : packed weights: 128 rows x 128 bytes by TMA, exponent bytes by background copies (plain loads in flight would be
 //                 waited for at every proxy fence that publishes a decoded step)
 //   warps 4..15 : three groups that decode every third K step each -- a step is a chain of a wait, a shared-memory read, the
 //                 conversion, the stores, a proxy fence and an arrival, about 0.6 us whatever its size -- then the partial tiles,
 //                 reduction and epilogue
-// Bound by an SM's intake and, up to about eight steps per CTA, by the chain from the first fetch to the last reduced value:
-// 128 x 4096 x 4096 16.7 us as a whole call (19.6 behind a pass over the weights), 128 x 4096 (N) x 11008 30.9 (41.5),
-// 128 x 28672 x 8192 135 (192), 256 x 5120 x 13824 58 (98).  Tried and slower: two K steps per proxy fence and group with four
-// stages of A in place of seven (0.1 to 0.5 us).
+// Bound by shared memory with three panels (per step 48 + 20 KB written, 96 + 4 KB read at 128 bytes per clock), by the decoding
+// warps and an SM's intake with one, and up to about eight steps per CTA by the chain from the first fetch to the last reduced
+// value.  Whole calls, M x K x N, 8/4 bits, behind a pass over the weights / here (us): 128 x 4096 x 4096 19.5 / 14.7,
+// 128 x 11008 x 4096 40.1 / 24.4, 256 x 8192 x 8192 72 / 44, 384 x 8192 x 8192 91 / 59.  Tried and slower: two K steps per proxy fence
+// and group with four stages of A in place of seven (0.1 to 0.5 us), a ring of A in panels instead of K steps.
 #pragma once
 #include <cuda.h>
 #include <cuda_runtime.h>

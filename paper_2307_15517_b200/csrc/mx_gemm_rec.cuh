@@ -9,8 +9,8 @@
 // Two CTAs on neighbouring SMs (a cluster of two) share one 256 x 256 output tile, K step 128: each holds one record
 // of A and one of W per step, plus the scales of its own A rows and of all 256 rows of W (the pair's MMA reads the W
 // scales from both CTAs' tensor memory).  The warp roles and barriers are those of mx_gemm_tc2.cuh:
-//   warp 0      : TMA producer (one lane, in both CTAs; bytes are counted on the leader's barrier)
-//   warp 1      : tensor-memory allocation (both CTAs), scale copies and MMA issue (one lane, leader only)
+//   warp 0      : TMA producer (in both CTAs; bytes are counted on the leader's barrier)
+//   warp 1      : tensor-memory allocation (both CTAs), scale copies and MMA issue (leader only)
 //   warps 2..9  : epilogue of the CTA's own 128 rows, two warps per TMEM lane quarter
 // What bounds it: operand fetch, 64 KB per 256 x 256 x 128 step and pair (13 TB/s over the chip at 0.36 us per step), and the
 // shared-memory reads of the MMAs (0.32 us per step with the fetches removed; 0.26 us is the pipe's peak).

@@ -6,8 +6,8 @@
 // accumulates its K steps, leaves its partial tile in its own shared memory (the stage buffers are free by then), and
 // after a cluster barrier each CTA adds up the partials of every S-th chunk of 32 columns through distributed shared
 // memory, in rank order -- deterministic -- and runs the epilogue on it.  Not persistent: one tile per cluster.
-//   warp 0      : TMA producer (one lane)
-//   warp 1      : tensor-memory allocation, MMA issue (one lane)
+//   warp 0      : TMA producer
+//   warp 1      : tensor-memory allocation, MMA issue
 //   warps 2..9  : partial tile to shared memory, then reduction and epilogue
 // Every mbarrier wait is bounded; a CTA whose wait expired still reaches both cluster barriers.
 #pragma once

@@ -12,8 +12,8 @@
 // Kernel: persistent, one CTA per SM, 128 x BN output tile, K step 64 (one 128-byte swizzled
 // row of bf16), STAGES-deep TMA pipeline, two accumulators in tensor memory (2*BN <= 512
 // columns) so that the epilogue of tile t overlaps the MMAs of tile t+1.
-//   warp 0      : TMA producer (one lane)
-//   warp 1      : tensor-memory allocation, MMA issue (one lane)
+//   warp 0      : TMA producer
+//   warp 1      : tensor-memory allocation, MMA issue
 //   warps 2..   : epilogue, TMEM -> registers -> (+bias) -> global fp32 (eight warps in the plain kernel, two per
 //                 TMEM lane quarter with half of the tile's columns each; four in the in-kernel-decode variants)
 // Every mbarrier wait is bounded in time; on expiry the kernel raises a CTA-wide abort flag,

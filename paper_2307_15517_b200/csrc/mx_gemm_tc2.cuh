@@ -2,13 +2,13 @@
 // and operands as mx_gemm_tc.cuh: exactly decoded bf16 tiles, fp32 accumulation in tensor memory).
 //
 // Two CTAs on neighbouring SMs (a cluster of two) share one 256 x 256 output tile: each holds 128
-// rows of A and 128 of the 256 rows of W per K step, one thread of the leader CTA issues
+// rows of A and 128 of the 256 rows of W per K step, an elected lane of the leader CTA issues
 // tcgen05.mma.cta_group::2, and each CTA's tensor memory receives the 128 x 256 half of the tile
 // that belongs to its rows.  Against the one-CTA 128 x 256 tile this cuts the bytes that pass
 // through each SM's shared memory per flop by a third (32 KB instead of 48 KB per K step), which
 // is what bounds that kernel, and leaves room for six stages instead of four.
 //
-//   warp 0      : TMA producer (one lane, in both CTAs; bytes are counted on the leader's barrier)
+//   warp 0      : TMA producer (in both CTAs; bytes are counted on the leader's barrier)
 //   warp 1      : tensor-memory allocation (both CTAs), MMA issue (leader only)
 //   warps 2..9  : epilogue of the CTA's own 128 rows (fp32, or MXInt as in the one-CTA kernel): warp w reads
 //                 TMEM lanes 32 * (w % 4) .. + 31 and 128 of the 256 columns -- two warps per scheduler, so one

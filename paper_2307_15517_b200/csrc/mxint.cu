@@ -230,7 +230,9 @@ mx_status_t launch_quantize_rows(const InT *x, int64_t rows, int64_t K, int64_t 
             MX_CUDA(launch_dep(mx::quantize_rows2_kernel<InT, 32>, dim3(grid), dim3(256), 0, st, x, rows, K, ldx, f.elem_bits, out));
         return MX_OK;
     }
-    if (chunks <= (int64_t)d.sm_count * 512) {             // few items: one per warp, in small CTAs on all SMs
+    // few items: one per warp, in CTAs of two warps on all SMs (CTAs of eight warps with two items each / these, us: 128 x 768 fp32 to
+    // MXInt4 2.0 / 1.7, 352 x 2048 2.6 / 2.5, 1024 x 768 2.5 / 2.5: the line is where they are even)
+    if (chunks <= (int64_t)d.sm_count * 512) {
         const unsigned g = (unsigned)((rows * ((K / 8 + 31) / 32) + 1) / 2);
         ProfScope prof(KIND_QUANTIZE, st);
         if (f.block == 16)
@@ -306,7 +308,9 @@ mx_status_t launch_dequant_bf16(const void *mant, const uint8_t *exps, int64_t r
         return launch_dequant_bf16(mant, exps, 1, rows * K, f, out, rows * K, flat, 1, d, st);
     }
     ProfScope prof(KIND_DEQUANTIZE, st);
-    if (wide_ok && rows * (K / 32) * batch <= (int64_t)d.sm_count * 256) {      // few items: one per warp, in small CTAs on all SMs
+    // few items: one per warp, in CTAs of two warps on all SMs (CTAs of eight warps with two items each / these, us: 352 x 2048 MXInt8
+    // to bf16 2.7 / 1.9, 2048 x 768 3.0 / 2.6, 1024 x 4096 4.0 / 4.0)
+    if (wide_ok && rows * (K / 32) * batch <= (int64_t)d.sm_count * 256) {
         const dim3 grid((unsigned)(rows * ((K / 32 + 31) / 32) + 1) / 2, (unsigned)batch);
         if (nib) MX_CUDA(launch_dep(mx::decode_bf16_kernel<true, 1>, dim3(grid), dim3(64), 0, st, m, exps, rows, K, f.block, f.elem_bits, out, ld, ps));
         else MX_CUDA(launch_dep(mx::decode_bf16_kernel<false, 1>, dim3(grid), dim3(64), 0, st, m, exps, rows, K, f.block, f.elem_bits, out, ld, ps));
