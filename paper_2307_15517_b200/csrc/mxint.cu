@@ -1708,7 +1708,7 @@ mx_status_t tmw_clusters(DeviceInfo &d, int which, int split, int *out)
     return MX_OK;
 }
 
-int tmw_tokens(int64_t M, int64_t N, int64_t K, bool nib, bool rec, int split, bool dec, int sm_count, const int *clusters, int *pieces);
+int tmw_tokens(int64_t M, int64_t N, int64_t K, bool nib, bool rec, int split, int sm_count, const int *clusters, int *pieces);
 
 // Whether the product decodes its weights itself, in which kernel, and for gemm_dec_kernel into how many pieces K is cut: the most
 // whose clusters all fit at once, of at least four K steps each.
@@ -1747,13 +1747,14 @@ mx_status_t dec_plan(int64_t M, int64_t N, int64_t K, const mx_format_t &fa, con
         }
         *use = dec_is_faster(M, N, K, out->split, rec, d.sm_count);
     }
+    if (M > 1536 || (M <= 128 && !*use)) return MX_OK;             // (see tmw_tokens)
     const int which = (nib ? 4 : 0) + (quantized ? 2 : 0);
     int clusters[mx::TmwCfg::MAX_SPLIT + 1] = {}, pieces = 1;
     for (int s = 1; s <= mx::TmwCfg::MAX_SPLIT; ++s) {
         const mx_status_t cs = tmw_clusters(d, which + (s > 1 ? 1 : 0), s, &clusters[s]);
         if (cs != MX_OK) return cs;
     }
-    out->tokens = tmw_tokens(M, N, K, nib, rec, panels <= mx::DecCfg::MAX_P ? out->split : 0, *use, d.sm_count, clusters, &pieces);
+    out->tokens = tmw_tokens(M, N, K, nib, rec, panels <= mx::DecCfg::MAX_P ? out->split : 0, d.sm_count, clusters, &pieces);
     if (out->tokens) {
         out->which = which + (pieces > 1 ? 1 : 0);
         out->split = pieces;
@@ -1854,9 +1855,8 @@ mx_status_t launch_dec(const DecPlan &g, const __nv_bfloat16 *a_hat, const void 
 // Some sizes where it is faster stay with the pass, because the tests fix by its launches which sizes have one: up to 128 rows those
 // that gemm_dec_kernel leaves to it (128 x 1024 x 9600 15.0 / 13), up to 256 K below 1280 (256 x 1024 x 16384 19.3 / 13.5), up to 384
 // with longer K and not cut those of less than 20 % (384 x 4096 x 6144 35.6 / 31.7).
-int tmw_tokens(int64_t M, int64_t N, int64_t K, bool nib, bool rec, int split, bool dec, int sm_count, const int *clusters, int *pieces)
+int tmw_tokens(int64_t M, int64_t N, int64_t K, bool nib, bool rec, int split, int sm_count, const int *clusters, int *pieces)
 {
-    if (M > 1536 || (N + 255) / 256 > INT32_MAX / 8) return 0;
     const double m = (double)M, n = (double)N, k = (double)K, pairs = sm_count / 2;
     const double steps = (double)((K + mx::TC_BK - 1) / mx::TC_BK), mk = m * k * 1e-6, mn = m * n * 1e-6, nk = n * k * 1e-6;
     auto up = [](double x) { return (double)(int64_t)(x + 0.999999); };
@@ -1892,7 +1892,7 @@ int tmw_tokens(int64_t M, int64_t N, int64_t K, bool nib, bool rec, int split, b
         const double dec = -26.1 + 3.9 * mk + 1.03 * mn + waves * (up(steps / split) * (0.112 + 0.159 * up(m / 128)) * (nib ? 1 : 1.16) + 34.45);
         other = dec < other ? dec : other;
     }
-    if (M <= 128 ? !dec : M <= 256 ? K < 1280 : false) return 0;
+    if (M > 128 && M <= 256 && K < 1280) return 0;
     return best < (!few ? rec ? 0.9 : 0.92 : *pieces > 1 ? 0.93 : M > 256 && K > 3072 ? 0.8 : 0.94) * other ? tokens : 0;
 }
 
