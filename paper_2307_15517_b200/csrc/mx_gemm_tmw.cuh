@@ -16,11 +16,11 @@
 // The tile is 256 features x T tokens, T a multiple of 32 that the host picks so that the tiles fill whole rounds of the chip's
 // pairs; up to T = 192 there are two accumulators, so the epilogue of a tile runs under the next one's MMAs.  Few tiles: K is cut
 // over the pairs of a cluster, whose partial tiles go to shared memory and are added up in the order of K (mx_gemm_splitk.cuh).
-// Bound by the integer instructions of the decoding warps: 0.27 us per K step and round whatever T (without the MMAs the same,
-// without the decoding 0.16 at T = 64 and 0.31, the MMAs' own time, at 256; four groups of warps, or two steps per turn of a group,
-// changed nothing).  Whole calls, M x K x N, against a pass and a product / gemm_dec_kernel: 512 x 4096 x 11008 54.8 -> 45.5 us
-// (50.6 with an MXInt result), 256 x 4096 x 12288 58.2 -> 29.9, 128 x 4096 x 11008 30.1 -> 25.6, 352 x 2048 x 6144 19.4 -> 16.6;
-// where it is chosen: tmw_tokens.
+// Bound by the instructions of the decoding warps, 0.25 us per K step and round up to T = 192 (without the MMAs the same, without the
+// decoding 0.16 at T = 64 and 0.31 at 256; four groups of warps, two steps per turn of a group, or half of the shifts as
+// multiplications changed nothing), and above by the MMAs (T = 224: 442 to 447 of the 2 T = 448 clocks).  Whole calls, M x K x N,
+// against a pass and a product / gemm_dec_kernel: 512 x 4096 x 11008 54.8 -> 45.5 us (with an MXInt result 53.3), 256 x 4096 x 12288
+// 58.2 -> 29.9, 128 x 4096 x 11008 30.1 -> 25.6, 352 x 2048 x 6144 19.4 -> 16.6; where it is chosen: tmw_tokens.
 // Persistent; all waits are bounded.
 #pragma once
 #include <cuda.h>
@@ -372,8 +372,12 @@ gemm_tmw_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constan
     } else if (warp >= 4 && warp < 4 + 4 * GROUPS) {
         // a lane a row, both halves of the step, straight into the row's 32 columns of the stage
         const int g = (warp - 4) >> 2, quad = warp & 3, r = 32 * quad + lane;
-        const uint8_t *mrow = smem_gen + r * 128, *ebase = smem_gen + (exp_base - smem_base) + r * (4 * EW), *erow = ebase;
-        const uint32_t dst = tmem_base + ((uint32_t)(quad * 32) << 16) + a_col;
+        // Shared addresses are 32-bit offsets whose parts are worked out once: of the 260 instructions that a step cost a warp, 110
+        // decode (240 now; 512 x 4096 x 11008 with an MXInt8 result, tiles of 192 tokens, 55.3 -> 53.3 us; at 224 tokens the MMAs bind).
+        const uint32_t mrow = raw_base - smem_base + r * 128, swz = (uint32_t)(r & 7) << 4, ebase = exp_base - smem_base + r * (4 * EW);
+        const uint32_t dst = tmem_base + ((uint32_t)(quad * 32) << 16) + a_col, a_full_lead = ptx::map_to_cta(a_full(0), lead);
+        const bool e_word = b16 && wp.exp_words;
+        uint32_t erow = ebase;
         int kb = g, tile = pair, tile_raw = 0;                           // step within the tile, tile, its first raw stage
         uint32_t step = (uint32_t)g;
         auto row_exps = [&]() {                                          // where the tile's exponent bytes of this row start
@@ -381,32 +385,31 @@ gemm_tmw_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constan
             erow = ebase + ((uint32_t)reinterpret_cast<uintptr_t>(wp.w_exp + (int64_t)(n >> wp.w_rows2) * (p.K / wp.block)) & 3u);
         };
         auto settle = [&]() {
-            bool moved = false;
-            while (kb >= kblocks) { kb -= kblocks; tile += npairs; tile_raw += raws; moved = true; }
-            if (moved && tile < num_tiles) row_exps();
+            if (kb < kblocks) return;
+            while (kb >= kblocks) { kb -= kblocks; tile += npairs; tile_raw += raws; }
+            if (tile < num_tiles) row_exps();
         };
         row_exps();
         settle();
         // Each barrier is looked at well before its answer is needed: waiting for one that is long complete takes 130 clocks, of
         // which a step of this loop had three in about 1500.
         bool there = false;                                              // the raw stage is known to be full
+        uint32_t ri = (uint32_t)tile_raw + (uint32_t)kb / SPR;           // raw stages before this step's
         while (tile < num_tiles) {
-            const int j = kb % SPR, a = (int)(step & as_mask);
-            const uint32_t ri = (uint32_t)(tile_raw + kb / SPR), a_ph = ((step >> as_shift) & 1u) ^ 1u;
-            const int rs = ri % RS, extra = kb == kblocks - 1 ? raws * SPR - kblocks : 0;      // steps that the tile's last raw stage does not have
+            const uint32_t j = (uint32_t)kb % SPR, a = step & as_mask, a_ph = ((step >> as_shift) & 1u) ^ 1u, rs = ri % RS;
+            const bool last = kb == kblocks - 1;
             if (!there && !__all_sync(0xFFFFFFFFu, ptx::mbar_wait_bounded(r_full(rs), (ri / RS) & 1u, abort_flag, TC_WAIT_LIMIT_NS))) {
                 timed_out = true;
                 break;
             }
             bool free = ptx::mbar_test(a_empty(a), a_ph);
             // (the exponents of all 32 rows: one path per warp)
-            const uint32_t e4 = step_exps(erow + rs * Cfg::RAW_EXP, j, b16, wp.exp_words);
+            const uint8_t *ex = smem_gen + (erow + rs * Cfg::RAW_EXP);
+            const uint32_t e4 = e_word ? *reinterpret_cast<const uint32_t *>(ex + 4 * j) : step_exps(ex, (int)j, b16, wp.exp_words);
+            const uint32_t at = mrow + rs * Cfg::RAW_MANT + ((j * (uint32_t)STEP_BYTES) ^ swz);      // 16-byte chunk c of the row: at ^ 16 c
             auto load = [&](int h, uint4 (&m)[NIB ? 1 : 2]) {
 #pragma unroll
-                for (int q = 0; q < (NIB ? 1 : 2); ++q) {
-                    const int c = NIB ? 2 * j + h : 4 * j + 2 * h + q;                        // 16-byte chunk of the row's 128 bytes
-                    m[q] = *reinterpret_cast<const uint4 *>(mrow + rs * Cfg::RAW_MANT + ((c ^ (r & 7)) << 4));
-                }
+                for (int q = 0; q < (NIB ? 1 : 2); ++q) m[q] = *reinterpret_cast<const uint4 *>(smem_gen + (at ^ (uint32_t)((NIB ? h : 2 * h + q) << 4)));
             };
             auto store = [&](int h, const uint32_t (&o)[4][4]) {
                 if (h == 0) {                                            // the stage is needed only now
@@ -443,14 +446,16 @@ gemm_tmw_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constan
             step += GROUPS;
             kb += GROUPS;
             settle();
-            const uint32_t rn = (uint32_t)(tile_raw + kb / SPR);
-            const bool next = tile < num_tiles && ptx::mbar_test(r_full(rn % RS), (rn / RS) & 1u);
+            ri = (uint32_t)tile_raw + (uint32_t)kb / SPR;
+            const bool next = ptx::mbar_test(r_full(ri % RS), (ri / RS) & 1u);        // (not used behind the last tile)
             ptx::tmem_st_wait();
             ptx::tc_fence_before_sync();
             __syncwarp();
             if (lane == 0) {
-                ptx::mbar_arrive_cluster_relaxed(ptx::map_to_cta(a_full(a), lead));
-                for (int x = 0; x <= extra; ++x) ptx::mbar_arrive(r_empty(rs));
+                ptx::mbar_arrive_cluster_relaxed(a_full_lead + 8u * a);
+                ptx::mbar_arrive(r_empty(rs));
+                if (last)                                                // the steps that the tile's last raw stage does not have
+                    for (int x = kblocks; x < raws * SPR; ++x) ptx::mbar_arrive(r_empty(rs));
             }
             there = __all_sync(0xFFFFFFFFu, next);
         }
