@@ -1842,7 +1842,8 @@ mx_status_t launch_dec(const DecPlan &g, const __nv_bfloat16 *a_hat, const void 
 // 8/4, 6/8, 8/8 and 4/4 -- with every tile, every cut and both other routes measured; their errors are 4 to 6 % (one sigma).
 // - gemm_tmw_kernel: rounds of 74 pairs, each 0.27 us per K step of 64 whatever the tile (its decoding warps; 0.25 up to 192 tokens
 //   since a step has fewer instructions, which the estimate leaves out; 0.35 for weights in bytes, 0.29 at 256 tokens, where the
-//   MMAs take as long), the epilogue behind the last round or, with one accumulator, behind each.  K cut: one round of clusters that all fit at once, the steps of the longest piece, the exchange.
+//   MMAs take as long), the epilogue behind the last round or, with one accumulator, behind each.  K cut: one round of
+//   clusters that all fit at once, the steps of the longest piece, the exchange.
 // - a pass that writes the weights out and the product on them (`rec`: on records): 0.5 us per M weights, 0.28 (0.13) us per step
 //   and round of 256 x 256 tiles, 0.15 per step of one wave of 128 x 128 tiles, half or a quarter as many steps where K is cut.
 // - gemm_dec_kernel (split > 0): 0.11 us and 0.16 per panel of 128 rows per step; a second wave of clusters costs 34 us.
