@@ -30,6 +30,7 @@
 #include "mx_gemm_tc.cuh"
 #include "mx_gemv_mma.cuh"
 #include "mx_ptx.cuh"
+#include "mx_step_walk.h"
 
 namespace mx {
 
@@ -225,6 +226,8 @@ gemm_tmw_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constan
     const bool leader = rank == 0;
     const uint16_t both = (uint16_t)(3u << lead);                        // the pair's CTAs
     const int split = SPLIT ? wp.split : 1;
+    using Walk = StepWalk<SPR, GROUPS>;
+    static_assert(RS > GROUPS, "what the waits for raw stages rely on (see StepWalk)");
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < Cfg::MAX_STAGES; ++s) {
@@ -348,8 +351,13 @@ gemm_tmw_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constan
     } else if (warp == 2) {
         // raw stages: 128 rows x 128 mantissa bytes in one tiled load, their exponent bytes in the background (see gemm_dec_kernel)
         ExpFeed feed(wp.w_exp, p.K / wp.block, EB, 0, wp.exp_words);
+        const bool wait_last = Walk::waits_for_last(kblocks);            // (see StepWalk)
         uint32_t ri = 0;
         for (int t = pair; t < num_tiles && !timed_out; t += npairs) {
+            if (wait_last && ri && !__all_sync(0xFFFFFFFFu, ptx::mbar_wait_bounded(r_full((ri - 1) % RS), ((ri - 1) / RS) & 1u, abort_flag, TC_WAIT_LIMIT_NS))) {
+                timed_out = true;
+                break;
+            }
             const int n0 = (t / p.tiles_m) * 256 + (int)rank * Cfg::BN;
             feed.rows(wp.w_exp, n0, p.N, wp.w_rows2, lane);
             for (int i = 0; i < raws; ++i, ++ri) {
@@ -378,27 +386,27 @@ gemm_tmw_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constan
         const uint32_t dst = tmem_base + ((uint32_t)(quad * 32) << 16) + a_col, a_full_lead = ptx::map_to_cta(a_full(0), lead);
         const bool e_word = b16 && wp.exp_words;
         uint32_t erow = ebase;
-        int kb = g, tile = pair, tile_raw = 0;                           // step within the tile, tile, its first raw stage
-        uint32_t step = (uint32_t)g;
+        Walk at{g, pair, 0, (uint32_t)g};
         auto row_exps = [&]() {                                          // where the tile's exponent bytes of this row start
-            const int n = min((tile / p.tiles_m) * 256 + (int)rank * Cfg::BN + r, p.N - 1);
+            const int n = min((at.tile / p.tiles_m) * 256 + (int)rank * Cfg::BN + r, p.N - 1);
             erow = ebase + ((uint32_t)reinterpret_cast<uintptr_t>(wp.w_exp + (int64_t)(n >> wp.w_rows2) * (p.K / wp.block)) & 3u);
         };
         auto settle = [&]() {
-            if (kb < kblocks) return;
-            while (kb >= kblocks) { kb -= kblocks; tile += npairs; tile_raw += raws; }
-            if (tile < num_tiles) row_exps();
+            if (at.kb < kblocks) return;
+            at.settle(kblocks, raws, npairs);
+            if (at.tile < num_tiles) row_exps();
         };
         row_exps();
         settle();
         // Each barrier is looked at well before its answer is needed: waiting for one that is long complete takes 130 clocks, of
         // which a step of this loop had three in about 1500.
         bool there = false;                                              // the raw stage is known to be full
-        uint32_t ri = (uint32_t)tile_raw + (uint32_t)kb / SPR;           // raw stages before this step's
-        while (tile < num_tiles) {
-            const uint32_t j = (uint32_t)kb % SPR, a = step & as_mask, a_ph = ((step >> as_shift) & 1u) ^ 1u, rs = ri % RS;
-            const bool last = kb == kblocks - 1;
-            if (!there && !__all_sync(0xFFFFFFFFu, ptx::mbar_wait_bounded(r_full(rs), (ri / RS) & 1u, abort_flag, TC_WAIT_LIMIT_NS))) {
+        uint32_t ri = at.raw();                                          // raw stages before this step's
+        while (at.tile < num_tiles) {
+            const uint32_t j = (uint32_t)at.kb % SPR, a = at.step & as_mask, a_ph = ((at.step >> as_shift) & 1u) ^ 1u, rs = ri % RS;
+            const bool last = at.kb == kblocks - 1;
+            if (!there && !__all_sync(0xFFFFFFFFu, (!Walk::ASKS_EMPTY || ptx::mbar_wait_bounded(r_empty(rs), ((ri / RS) & 1u) ^ 1u, abort_flag, TC_WAIT_LIMIT_NS)) &&
+                                                   ptx::mbar_wait_bounded(r_full(rs), (ri / RS) & 1u, abort_flag, TC_WAIT_LIMIT_NS))) {
                 timed_out = true;
                 break;
             }
@@ -406,10 +414,10 @@ gemm_tmw_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constan
             // (the exponents of all 32 rows: one path per warp)
             const uint8_t *ex = smem_gen + (erow + rs * Cfg::RAW_EXP);
             const uint32_t e4 = e_word ? *reinterpret_cast<const uint32_t *>(ex + 4 * j) : step_exps(ex, (int)j, b16, wp.exp_words);
-            const uint32_t at = mrow + rs * Cfg::RAW_MANT + ((j * (uint32_t)STEP_BYTES) ^ swz);      // 16-byte chunk c of the row: at ^ 16 c
+            const uint32_t chunks = mrow + rs * Cfg::RAW_MANT + ((j * (uint32_t)STEP_BYTES) ^ swz);      // 16-byte chunk c of the row: chunks ^ 16 c
             auto load = [&](int h, uint4 (&m)[NIB ? 1 : 2]) {
 #pragma unroll
-                for (int q = 0; q < (NIB ? 1 : 2); ++q) m[q] = *reinterpret_cast<const uint4 *>(smem_gen + (at ^ (uint32_t)((NIB ? h : 2 * h + q) << 4)));
+                for (int q = 0; q < (NIB ? 1 : 2); ++q) m[q] = *reinterpret_cast<const uint4 *>(smem_gen + (chunks ^ (uint32_t)((NIB ? h : 2 * h + q) << 4)));
             };
             auto store = [&](int h, const uint32_t (&o)[4][4]) {
                 if (h == 0) {                                            // the stage is needed only now
@@ -443,11 +451,13 @@ gemm_tmw_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constan
                 timed_out = true;
                 break;
             }
-            step += GROUPS;
-            kb += GROUPS;
+            at.step += GROUPS;
+            at.kb += GROUPS;
             settle();
-            ri = (uint32_t)tile_raw + (uint32_t)kb / SPR;
-            const bool next = ptx::mbar_test(r_full(ri % RS), (ri / RS) & 1u);        // (not used behind the last tile)
+            ri = at.raw();
+            bool next = true;                                            // (not used behind the last tile)
+            if (Walk::ASKS_EMPTY) next = ptx::mbar_test(r_empty(ri % RS), ((ri / RS) & 1u) ^ 1u);
+            next = ptx::mbar_test(r_full(ri % RS), (ri / RS) & 1u) && next;
             ptx::tmem_st_wait();
             ptx::tc_fence_before_sync();
             __syncwarp();

@@ -29,6 +29,12 @@ def decoded_in_the_product(call):
     (500, 96, 16384, 32, 8, 4, 1),         # two K steps (one and a half), 128 tokens
     (600, 160, 14000, 32, 6, 8, 1),        # three K steps, 160 tokens
     (1400, 512, 11582, 16, 8, 4, 1),
+    (1500, 64, 16384, 16, 8, 4, 1),        # tiles of one step, each a stage of packed weights: a group passes two for one of its own
+    (1500, 32, 16384, 32, 4, 3, 1),
+    (1500, 48, 16384, 16, 8, 8, 1),
+    (1000, 96, 16000, 16, 8, 8, 1),        # two steps, one stage
+    (768, 4096, 11008, 32, 8, 8, 1),       # bytes, a group has no step in every third stage: 256 tokens, eight stages of decoded weights
+    (500, 1104, 8192, 16, 8, 6, 1),
 ])
 def test_weights_decoded_into_tensor_memory(M, K, N, block, wa, ww, rows2):
     g = torch.Generator(device="cuda")
