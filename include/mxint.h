@@ -425,6 +425,15 @@ MX_API mx_status_t mx_poll_status(void *stream);
  */
 MX_API mx_status_t mx_selftest_wait_expiry(uint32_t limit_us, void *stream);
 
+/*
+ * Self-test of the dispatch: the product kernel that mx_linear (quantized: mx_linear_q) takes for these sizes of more than 32 rows
+ * by MX_ALGO_AUTO or MX_ALGO_TCGEN05 on the current device.  route[0]: 1 weights decoded into shared memory, 2 into tensor memory,
+ * 3 block-scaled E4M3 operands; bf16 operands 4 with K cut over a cluster, 5 on one CTA per tile, 6 and 7 on CTA pairs (tiles of
+ * 256 columns, of other widths).  route[1]: tokens (2) or columns of a tile; route[2]: pieces of K.  Launches nothing.
+ */
+MX_API mx_status_t mx_selftest_route(int64_t M, int64_t N, int64_t K, mx_format_t fa, mx_format_t fw, int32_t quantized,
+                                     mx_algo_t algo, int32_t *route);
+
 /* ---- the layer with an MXInt result ------------------------------------------------------------
  *
  * Sec. 3.2 (software emulators): an operator's floating-point result is quantized again to the

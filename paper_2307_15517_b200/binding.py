@@ -131,6 +131,8 @@ def _load() -> C.CDLL:
     L.mx_poll_status.argtypes = [vp]
     L.mx_selftest_wait_expiry.argtypes = [C.c_uint32, vp]
     L.mx_selftest_wait_expiry.restype = i32
+    L.mx_selftest_route.argtypes = [i64, i64, i64, F, F, i32, i32, C.POINTER(C.c_int32)]
+    L.mx_selftest_route.restype = i32
     L.mx_gemm_batched_workspace_bytes.argtypes = [i64, i64, i64, i64]
     L.mx_gemm_batched_workspace_bytes.restype = sz
     L.mx_gemm_batched.argtypes = [vp, vp, F, i64, i64, vp, vp, F, i64, i64, i64, i64, i64, i64, vp, i64, i64,
@@ -682,6 +684,13 @@ def mx_poll_status(stream=None) -> int:
 def mx_selftest_wait_expiry(limit_us: int = 2000, stream=None) -> None:
     """Launches the library's bounded-wait self-test (a wait nobody satisfies, given up after limit_us)."""
     _check(lib.mx_selftest_wait_expiry(limit_us, _stream(stream)), "mx_selftest_wait_expiry")
+
+
+def mx_selftest_route(M: int, N: int, K: int, fa: MxFormat, fw: MxFormat, quantized: bool = False, algo: int = MX_ALGO_AUTO):
+    """(kernel, tokens or columns of a tile, pieces of K) of a layer of these sizes: see include/mxint.h."""
+    route = (C.c_int32 * 3)()
+    _check(lib.mx_selftest_route(M, N, K, fa, fw, int(quantized), algo, route), "mx_selftest_route")
+    return tuple(route)
 
 
 KERNEL_KINDS = ("quantize", "dequantize", "gemm_tc", "gemm_simt", "gemm_stream", "prep", "glue")

@@ -1198,40 +1198,55 @@ int one_round_width(int64_t M, int64_t N, const DeviceInfo &d)
     return w >= 160 && w <= 224 ? (int)w : 0;
 }
 
-// Pre-decoded bf16 weights (both operands fetched by TMA).  may_split: K may be cut (the sum is then not one chain).
+// Which product on bf16 operands a call takes (`count` products of one shape in one launch).  may_split: K may be cut (the sum is
+// then not one chain).
+// One wave of the smallest tile that gives one: a wave of 128 x 256 tiles takes 1.1 to 1.2 times as long as one of
+// 128 x 128, not twice (352 x 8192 x 2048, 192 or 96 tiles: 33.3 against 25.7 us per call; 352 x 6144 x 2048, 144 or 72:
+// 22.9 against 24.4).  Beyond that CTA pairs (a third less shared-memory traffic per flop: 512 x 11008 x 4096 74.3 against
+// 83.3 us, +14 % on 8192^3), but a ragged half pair is not worth a second wave (300 x 12288 x 4096: 144 tiles of
+// 128 x 256 62.1, 96 pair tiles 75.0).  Pairs also for one nearly full wave of long tiles (2048 x 2048 x 8192 product
+// 49.5 against 56.5 us); a short single wave starts faster on the one-CTA kernel (2048^3 call 23.8 against 24.7).
+enum TcKernel { TC_ONE = 5, TC_PAIR = 6, TC_PAIR_WIDE = 7, TC_CUT = 4 };     // (numbers: mx_selftest_route)
+struct TcRoute { TcKernel kernel; int width, split; };                      // columns of a tile; pieces of K
+
+mx_status_t tc_route(int64_t M, int64_t N, int64_t K, int count, bool may_split, DeviceInfo &d, TcRoute *out)
+{
+    const int64_t panels = (M + 127) / 128;
+    const int64_t pair_tiles = ((M + 255) / 256) * ((N + 255) / 256);
+    const int64_t tiles128 = panels * ((N + 127) / 128) * count, tiles256 = panels * ((N + 255) / 256) * count;
+    const int pairs = d.sm_count / 2;
+    const bool long_wave = K >= 4096 && pair_tiles <= pairs && 4 * pair_tiles >= 3 * pairs && (panels & 1) == 0;
+    *out = {TC_ONE, N > 128 && tiles128 > d.sm_count ? 256 : 128, 1};
+    if (count > 1) return MX_OK;
+    if (M > 128 && (tiles256 > d.sm_count || long_wave)) {
+        const int width = wide_pair_tile(M, N, K, d);
+        *out = {width ? TC_PAIR_WIDE : TC_PAIR, width ? width : 256, 1};
+        return MX_OK;
+    }
+    const int width = M > 128 ? one_round_width(M, N, d) : 0;
+    if (width) {
+        *out = {TC_PAIR_WIDE, width, 1};
+        return MX_OK;
+    }
+    int split = 0;
+    const mx_status_t s = may_split ? splitk_ways(M, N, K, d, &split) : MX_OK;
+    if (s == MX_OK && split) *out = {TC_CUT, 128, split};
+    return s;
+}
+
+// Pre-decoded bf16 weights (both operands fetched by TMA).
 mx_status_t run_tc(const __nv_bfloat16 *a_hat, const __nv_bfloat16 *w_hat, int64_t M, int64_t N,
                    int64_t K, const float *bias, float *y, int64_t ldy, DeviceInfo &d, cudaStream_t st,
                    const QuantizedOut *yq = nullptr, const TcBatch &tb = TcBatch(), const EpiTail &et = EpiTail(), bool may_split = true)
 {
     const PackedW none;
-    // One wave of the smallest tile that gives one: a wave of 128 x 256 tiles takes 1.1 to 1.2 times as long as one of
-    // 128 x 128, not twice (352 x 8192 x 2048, 192 or 96 tiles: 33.3 against 25.7 us per call; 352 x 6144 x 2048, 144 or 72:
-    // 22.9 against 24.4).  Beyond that CTA pairs (a third less shared-memory traffic per flop: 512 x 11008 x 4096 74.3 against
-    // 83.3 us, +14 % on 8192^3), but a ragged half pair is not worth a second wave (300 x 12288 x 4096: 144 tiles of
-    // 128 x 256 62.1, 96 pair tiles 75.0).  Pairs also for one nearly full wave of long tiles (2048 x 2048 x 8192 product
-    // 49.5 against 56.5 us); a short single wave starts faster on the one-CTA kernel (2048^3 call 23.8 against 24.7).
-    const int64_t panels = (M + 127) / 128;
-    const int64_t pair_tiles = ((M + 255) / 256) * ((N + 255) / 256);
-    const int64_t tiles128 = panels * ((N + 127) / 128) * tb.count, tiles256 = panels * ((N + 255) / 256) * tb.count;
-    const int pairs = d.sm_count / 2;
-    const bool long_wave = K >= 4096 && pair_tiles <= pairs && 4 * pair_tiles >= 3 * pairs && (panels & 1) == 0;
-    if (tb.count == 1 && M > 128 && (tiles256 > d.sm_count || long_wave)) {
-        const int width = wide_pair_tile(M, N, K, d);
-        if (width) return launch_tcw(a_hat, w_hat, M, N, K, width, bias, y, ldy, yq, d, st, et);
-        return launch_tc2(a_hat, w_hat, M, N, K, bias, y, ldy, yq, d, st, et);
-    }
-    if (tb.count == 1 && M > 128) {
-        const int width = one_round_width(M, N, d);
-        if (width) return launch_tcw(a_hat, w_hat, M, N, K, width, bias, y, ldy, yq, d, st, et);
-    }
-    if (may_split && tb.count == 1) {
-        int split = 0;
-        const mx_status_t s = splitk_ways(M, N, K, d, &split);
-        if (s != MX_OK) return s;
-        if (split) return launch_splitk(a_hat, w_hat, M, N, K, split, bias, y, ldy, yq, d, st, et);
-    }
-    if (N > 128 && tiles128 > d.sm_count)
-        return launch_tc<256, mx::W_BF16>(a_hat, w_hat, none, M, N, K, bias, y, ldy, yq, d, st, tb, et);
+    TcRoute r;
+    const mx_status_t s = tc_route(M, N, K, tb.count, may_split, d, &r);
+    if (s != MX_OK) return s;
+    if (r.kernel == TC_PAIR_WIDE) return launch_tcw(a_hat, w_hat, M, N, K, r.width, bias, y, ldy, yq, d, st, et);
+    if (r.kernel == TC_PAIR) return launch_tc2(a_hat, w_hat, M, N, K, bias, y, ldy, yq, d, st, et);
+    if (r.kernel == TC_CUT) return launch_splitk(a_hat, w_hat, M, N, K, r.split, bias, y, ldy, yq, d, st, et);
+    if (r.width == 256) return launch_tc<256, mx::W_BF16>(a_hat, w_hat, none, M, N, K, bias, y, ldy, yq, d, st, tb, et);
     return launch_tc<128, mx::W_BF16>(a_hat, w_hat, none, M, N, K, bias, y, ldy, yq, d, st, tb, et);
 }
 
@@ -3387,6 +3402,39 @@ mx_status_t mx_selftest_wait_expiry(uint32_t limit_us, void *stream)
     if (s != MX_OK) return s;
     wait_probe_kernel<<<1, 32, 0, static_cast<cudaStream_t>(stream)>>>(d->status, (uint64_t)limit_us * 1000ull);
     MX_CUDA(cudaGetLastError());
+    return MX_OK;
+}
+
+mx_status_t mx_selftest_route(int64_t M, int64_t N, int64_t K, mx_format_t fa, mx_format_t fw, int32_t quantized, mx_algo_t algo,
+                               int32_t *route)
+{
+    if (!route) return MX_ERR_NULL;
+    if (!format_ok_any(fa) || !format_ok_any(fw) || fa.block != fw.block || (algo != MX_ALGO_AUTO && algo != MX_ALGO_TCGEN05)) return MX_ERR_FORMAT;
+    if (M <= 32 || N <= 0 || K <= 0 || (K % fa.block) != 0 || M > INT32_MAX / 2 || N > INT32_MAX / 2 || K > INT32_MAX / 2) return MX_ERR_SHAPE;
+    DeviceInfo *d = nullptr;
+    mx_status_t s = device_info(&d);
+    if (s != MX_OK) return s;
+    bool dec = false, rec = false;
+    DecPlan plan;
+    const bool any = algo == MX_ALGO_AUTO;
+    if (any) s = dec_plan(M, N, K, fa, fw, nullptr, quantized != 0, *d, &plan, &dec);
+    if (s != MX_OK) return s;
+    if (dec) {
+        route[0] = plan.tokens ? 2 : 1;
+        route[1] = plan.tokens ? plan.tokens : mx::DecCfg::BN;
+        route[2] = plan.split;
+        return MX_OK;
+    }
+    if (any && rec_fits(fa, fw, M, N, K)) {
+        s = rec_is_faster(M, N, K, *d, &rec);
+        if (s != MX_OK) return s;
+    }
+    TcRoute r;
+    s = tc_route(M, N, K, 1, any, *d, &r);
+    if (s != MX_OK) return s;
+    route[0] = rec ? 3 : (int)r.kernel;
+    route[1] = rec ? 256 : r.width;
+    route[2] = rec ? 1 : r.split;
     return MX_OK;
 }
 

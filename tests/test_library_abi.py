@@ -124,6 +124,10 @@ def test_invalid_arguments_are_rejected_on_the_host(mxb):
     assert sq(fp=F(16, 8, 8, 2)) == -3
     assert sq(s=None) == -1 and sq(ld=66) == -4
     assert L.mx_selftest_wait_expiry(0, None) == -2
+    route = (C.c_int32 * 3)()
+    assert L.mx_selftest_route(32, 64, 64, mxb.MxFormat(16, 8), mxb.MxFormat(16, 4), 0, mxb.MX_ALGO_AUTO, route) == -2
+    assert L.mx_selftest_route(64, 64, 64, mxb.MxFormat(16, 8), mxb.MxFormat(16, 4), 0, mxb.MX_ALGO_SIMT, route) == -3
+    assert L.mx_selftest_route(64, 64, 64, mxb.MxFormat(16, 8), mxb.MxFormat(16, 4), 0, mxb.MX_ALGO_AUTO, None) == -1
     # fused attention: head dimension 128, whole query tiles, one-row container formats, aligned leading dimensions
     f8 = F(16, 8)
     at = lambda **kw: L.mx_attention(kw.get("q", fake), fake, fake, fake, kw.get("fqk", f8), fake, fake, f8,
