@@ -231,9 +231,12 @@ mx_status_t launch_quantize_rows(const InT *x, int64_t rows, int64_t K, int64_t 
         return MX_OK;
     }
     // few items: one per warp, in CTAs of two warps on all SMs (CTAs of eight warps with two items each / these, us: 128 x 768 fp32 to
-    // MXInt4 2.0 / 1.7, 352 x 2048 2.6 / 2.5, 1024 x 768 2.5 / 2.5: the line is where they are even)
-    if (chunks <= (int64_t)d.sm_count * 512) {
-        const unsigned g = (unsigned)((rows * ((K / 8 + 31) / 32) + 1) / 2);
+    // MXInt4 2.0 / 1.7, 352 x 2048 2.6 / 2.5, 1024 x 768 2.5 / 2.5: the line is where they are even).  Short rows are an item each: more
+    // items than are resident at once only while the others' CTAs, counted by elements, are few as well (16384 x 16 14.2 / 8.9,
+    // but 16384 x 32 7.8 / 8.9, 32768 x 16 14.2 / 17.5)
+    const int64_t items = rows * ((K / 8 + 31) / 32);
+    if (chunks <= (int64_t)d.sm_count * (items <= (int64_t)d.sm_count * 48 ? 512 : 352)) {
+        const unsigned g = (unsigned)((items + 1) / 2);
         ProfScope prof(KIND_QUANTIZE, st);
         if (f.block == 16)
             MX_CUDA(launch_dep(mx::quantize_rows_kernel<InT, 16, 1>, dim3(g), dim3(64), 0, st, x, rows, K, ldx, (int)f.elem_bits, out));

@@ -24,10 +24,11 @@ def test_blocks_along_the_slow_axis(rows, K, B, w, dtype):
     assert np.array_equal(mant.cpu().numpy(), orc.pack(q, w)) and np.array_equal(exps.cpu().numpy(), e) and int(cnt) == bad
 
 
-@pytest.mark.parametrize("rows,K", [(1, 32), (2, 992), (33, 352), (352, 1056), (147, 2048), (148, 4096), (149, 4128), (4097, 96)])
+@pytest.mark.parametrize("rows,K", [(1, 32), (2, 992), (33, 352), (352, 1056), (147, 2048), (148, 4096), (149, 4128), (4097, 96),
+                                    (7104, 64), (7105, 64), (13024, 32), (13025, 32)])
 @pytest.mark.parametrize("B,w,dtype", [(16, 4, torch.float32), (32, 8, torch.bfloat16)])
 def test_few_items(rows, K, B, w, dtype):
-    """Both sides of the lines: 148 x 512 chunks of 8 (quantizer) and 148 x 256 items of 32 (decoder) on 148 SMs."""
+    """Both sides of the lines: 148 x 512 chunks of 8, or of 148 x 48 rows and 148 x 352 chunks (quantizer) and 148 x 256 items of 32 (decoder) on 148 SMs."""
     g = torch.Generator().manual_seed(rows + K)
     x = (torch.randn(rows, K, generator=g) * torch.exp2(torch.randint(-20, 20, (rows, 1), generator=g).float())).to(dtype)
     f = mxb.MxFormat(B, w)
