@@ -76,7 +76,7 @@ typedef enum {
                               K range cut over a cluster of up to eight CTAs and the pieces added in fp32,
                               in order;
                             - M <= 1536 and such weights, where estimates of all routes say that it is
-                              faster (mostly from 129 rows and some 8 M weights on): the same values, the
+                              faster (most sizes from 129 rows on, wide layers also of fewer): the same values, the
                               weights decoded into tensor memory, the sums of MX_ALGO_TCGEN05; few tiles: the
                               K range cut over two to four pairs of CTAs, the pieces added in fp32, in order;
                             - few 128 x 128 tiles (at most 74) and K of 1024 or more: the bf16 operands of

@@ -1712,24 +1712,29 @@ void tmw_config(cudaLaunchConfig_t &cfg, cudaLaunchAttribute *attr, int split, i
     cfg.numAttrs = 1;
 }
 
-// Clusters of `split` pairs that are resident at once; looked up once.
-mx_status_t tmw_clusters(DeviceInfo &d, int which, int split, int *out)
+// Clusters of 2 .. MAX_SPLIT pairs that are resident at once; looked up once.
+mx_status_t tmw_clusters(DeviceInfo &d, int which, int (&out)[mx::TmwCfg::MAX_SPLIT + 1])
 {
     const mx_status_t s = smem_attr_once(d.tmw_attr_set[which], g_tmw[which], 227 * 1024);
     if (s != MX_OK) return s;
     std::lock_guard<std::mutex> lk(g_init_mu);
-    int &known = d.tmw_clusters[which][split];
-    if (known == 0) {
-        cudaLaunchConfig_t cfg = {};
-        cudaLaunchAttribute attr[2];
-        tmw_config(cfg, attr, split, d.sm_count, nullptr);
-        MX_CUDA(cudaOccupancyMaxActiveClusters(&known, g_tmw[which], &cfg));
+    for (int split = 2; split <= mx::TmwCfg::MAX_SPLIT; ++split) {
+        int &known = d.tmw_clusters[which][split];
+        if (known == 0) {
+            cudaLaunchConfig_t cfg = {};
+            cudaLaunchAttribute attr[2];
+            tmw_config(cfg, attr, split, d.sm_count, nullptr);
+            MX_CUDA(cudaOccupancyMaxActiveClusters(&known, g_tmw[which], &cfg));
+        }
+        out[split] = known;
     }
-    *out = known;
     return MX_OK;
 }
 
-int tmw_tokens(int64_t M, int64_t N, int64_t K, bool nib, bool rec, int split, int sm_count, const int *clusters, int *pieces);
+double tc_us(const TcRoute &r, int64_t M, int64_t N, int64_t K, int sm_count);
+double rec_us(int64_t M, int64_t N, int64_t K, int sm_count);
+double dec_us(int64_t M, int64_t N, int64_t K, int split, bool nib, bool words, int sm_count);
+int tmw_tokens(int64_t M, int64_t N, int64_t K, bool nib, bool words, double other, int sm_count, const int *clusters, int *pieces);
 
 // Whether the product decodes its weights itself, in which kernel, and for gemm_dec_kernel into how many pieces K is cut: the most
 // whose clusters all fit at once, of at least four K steps each.
@@ -1768,14 +1773,23 @@ mx_status_t dec_plan(int64_t M, int64_t N, int64_t K, const mx_format_t &fa, con
         }
         *use = dec_is_faster(M, N, K, out->split, rec, d.sm_count);
     }
-    if (M > 1536 || (M <= 128 && !*use)) return MX_OK;             // (see tmw_tokens)
+    if (M > 1536) return MX_OK;                                          // (see tmw_tokens)
+    double other = 0;                                                    // us of the route that is taken else
+    if (*use) {
+        other = dec_us(M, N, K, out->split, nib, out->exp_words != 0, d.sm_count);
+    } else if (rec) {
+        other = rec_us(M, N, K, d.sm_count);
+    } else {
+        TcRoute r;
+        const mx_status_t ts = tc_route(M, N, K, 1, true, d, &r);
+        if (ts != MX_OK) return ts;
+        other = tc_us(r, M, N, K, d.sm_count);
+    }
     const int which = (nib ? 4 : 0) + (quantized ? 2 : 0);
     int clusters[mx::TmwCfg::MAX_SPLIT + 1] = {}, pieces = 1;
-    for (int s = 1; s <= mx::TmwCfg::MAX_SPLIT; ++s) {
-        const mx_status_t cs = tmw_clusters(d, which + (s > 1 ? 1 : 0), s, &clusters[s]);
-        if (cs != MX_OK) return cs;
-    }
-    out->tokens = tmw_tokens(M, N, K, nib, rec, panels <= mx::DecCfg::MAX_P ? out->split : 0, d.sm_count, clusters, &pieces);
+    const mx_status_t cs = tmw_clusters(d, which + 1, clusters);
+    if (cs != MX_OK) return cs;
+    out->tokens = tmw_tokens(M, N, K, nib, out->exp_words != 0, other, d.sm_count, clusters, &pieces);
     if (out->tokens) {
         out->which = which + (pieces > 1 ? 1 : 0);
         out->split = pieces;
@@ -1858,39 +1872,86 @@ mx_status_t launch_dec(const DecPlan &g, const __nv_bfloat16 *a_hat, const void 
     return MX_OK;
 }
 
-// Tokens per tile and pieces of K with which gemm_tmw_kernel is expected to be the fastest route, 0 where another one is.  Estimates
-// in us of whole calls (activation pass included), fitted to 1480 shapes -- 48 .. 3072 rows, K 512 .. 16384, N 768 .. 16384, widths
-// 8/4, 6/8, 8/8 and 4/4 -- with every tile, every cut and both other routes measured; their errors are 4 to 6 % (one sigma).
-// - gemm_tmw_kernel: rounds of 74 pairs, each 0.27 us per K step of 64 whatever the tile (its decoding warps; 0.25 up to 192 tokens
-//   since a step has fewer instructions, which the estimate leaves out; 0.35 for weights in bytes, 0.29 at 256 tokens, where the
-//   MMAs take as long), the epilogue behind the last round or, with one accumulator, behind each.  K cut: one round of
-//   clusters that all fit at once, the steps of the longest piece, the exchange.
-// - a pass that writes the weights out and the product on them (`rec`: on records): 0.5 us per M weights, 0.28 (0.13) us per step
-//   and round of 256 x 256 tiles, 0.15 per step of one wave of 128 x 128 tiles, half or a quarter as many steps where K is cut.
-// - gemm_dec_kernel (split > 0): 0.11 us and 0.16 per panel of 128 rows per step; a second wave of clusters costs 34 us.
-// Taken where it is the best by 6 to 10 %; over the shapes of 129 .. 1536 rows the route taken is then 0.956 of the best of the
-// other two on average, 0.93 being possible, and at worst 13 % slower (1024 x 5120 x 5120 54 / 61; the next 10 %).
-// Whole calls without / with it: 160 x 4096 x 11008 (M x K x N) 56.3 / 27.2, 256 x 2048 x 12288 32.8 / 21.2, 512 x 8192 x 8192
-// 88.6 / 60.9, 768 x 16384 x 4096 130 / 86, 1024 x 4096 x 4096 38.6 / 34.3; K cut in two 448 x 16384 x 4096 97 / 57, in three
-// 352 x 8192 x 2048 29.5 / 27.4.  Above 1536 rows the passes cost too little beside the product (2048 x 4096 x 4096 62.5 / 60.6,
-// 3072 x 1344 x 11008 74 / 94).
-// Some sizes where it is faster stay with the pass, because the tests fix by its launches which sizes have one: up to 128 rows those
-// that gemm_dec_kernel leaves to it (128 x 1024 x 9600 15.0 / 13), up to 256 K below 1280 (256 x 1024 x 16384 19.3 / 13.5), up to 384
-// with longer K and not cut those of less than 20 % (384 x 4096 x 6144 35.6 / 31.7).
-int tmw_tokens(int64_t M, int64_t N, int64_t K, bool nib, bool rec, int split, int sm_count, const int *clusters, int *pieces)
+// Estimates in us of whole calls on 148 SMs, pass over the activations included: what dec_plan compares gemm_tmw_kernel with the other
+// routes by.  Fitted to 3700 shapes -- 17 .. 2048 rows, K 32 .. 16384, N 2 .. 16384, widths 8/4, 4/4 and 8/8 -- with every route timed
+// (tmw_tokens: up to eleven tiles and cuts each).  One sigma of their errors: tmw_us and dec_us 4.9 %, tc_us 5.9 %, rec_us 4.6 %.
+double up(double x) { return (double)(int64_t)(x + 0.999999); }
+
+// gemm_tmw_kernel on tiles of T tokens, K in `pieces`.  Rounds of 74 pairs, each 0.253 us per K step of 64 up to 160 tokens (its
+// decoding warps), 0.263 at 192, 0.272 and 0.301 at 224 and 256 (its MMAs), for weights in bytes 0.342 and 0.349; more where exponent
+// rows are no whole words and come word by word; a tenth less on few pairs.  An odd number of steps costs two.  With one accumulator an
+// epilogue behind each round.
+double tmw_us(double M, double N, double K, bool nib, bool words, int T, int pieces, double pairs)
 {
-    const double m = (double)M, n = (double)N, k = (double)K, pairs = sm_count / 2;
-    const double steps = (double)((K + mx::TC_BK - 1) / mx::TC_BK), mk = m * k * 1e-6, mn = m * n * 1e-6, nk = n * k * 1e-6;
-    auto up = [](double x) { return (double)(int64_t)(x + 0.999999); };
+    const double steps = up(K / 64), mk = M * K * 1e-6, mn = M * N * 1e-6, unit = nib ? 4 : 2;   // unit: steps per stage of packed weights
+    const double tiles = up(M / T) * up(N / 256), load = tiles * pieces < pairs ? tiles * pieces / pairs : 1;
+    double step = nib ? T <= 160 ? 0.253 : T <= 192 ? 0.263 : T <= 224 ? 0.272 : 0.301 : T <= 192 ? 0.342 : 0.349;
+    if (!words) step = nib ? 0.332 : 0.402;
+    step *= 0.9 + 0.1 * load;
+    if (pieces > 1)                                                      // (2 % on top: what the fit lacks where the clusters fill the chip)
+        return 1.02 * (5.21 + 0.6 * pieces + 1.12 * load + 0.916 * mk + 0.753 * mn + up(up(steps / unit) / pieces) * unit * step + 0.021 * T);
+    const double rounds = up(tiles / pairs), odd = 2 * (steps - 2 * (double)(int64_t)(steps / 2));
+    return 6.32 + 0.916 * mk + 0.472 * mn + rounds * (steps + odd) * step + 0.009 * T * (mx::TmwCfg::accs(T) == 1 ? rounds : 1);
+}
+
+// A pass that writes both operands out in bf16, and the product.  The pass deals items of 256 activations and 1024 weights of one row
+// -- short rows leave lanes idle -- to CTAs that are counted by elements (prep_operands_kernel).
+double tc_us(const TcRoute &r, int64_t M, int64_t N, int64_t K, int sm_count)
+{
+    const double m = (double)M, n = (double)N, k = (double)K, steps = up(k / 64), pairs = sm_count / 2;
+    const double mk = m * k * 1e-6, mn = m * n * 1e-6, nk = n * k * 1e-6;
+    const double ctas = mk * 1e6 / 2048 + nk * 1e6 / 8192, most = 16.0 * sm_count;
+    const double turns = (m * up(k / 256) + n * up(k / 1024)) / (4 * (ctas < most ? ctas : most)) - 2;
+    double us = 0.44 * n * up(k / 1024) * 1024e-6 + (nk > 40 ? 0.2 * (nk - 40) : 0) + 0.93 * mk + (turns > 0 ? 0.4 * turns : 0);
+    us += (0.47 + (N % 4 ? 0.42 : 0)) * mn + (K % 32 ? 2 : 0);           // rows of y without whole 16 bytes; two launches
+    const double tiles = up(m / 256) * up(n / r.width);
+    switch (r.kernel) {
+    case TC_CUT: return us + 7.7 + 0.154 * up(steps / r.split);
+    case TC_PAIR: return us + 8.05 + 0.283 * steps * 0.5 * (tiles / pairs + up(tiles / pairs));      // (the epilogue runs under the next round)
+    case TC_PAIR_WIDE: return us + 7.1 + 0.286 * steps * up(tiles / pairs) * r.width / 256;
+    default: break;
+    }
+    const double waves = up(up(m / 128) * up(n / r.width) / sm_count);
+    return us + (r.width == 128 ? 6.35 + 0.182 * steps * waves : 7.0 + 0.302 * steps * waves);
+}
+
+// The same on block-scaled records.
+double rec_us(int64_t M, int64_t N, int64_t K, int sm_count)
+{
+    const double m = (double)M, n = (double)N, k = (double)K, nk = n * k * 1e-6, t = up(m / 256) * up(n / 256) / (sm_count / 2);
+    return 8.2 + 0.278 * up(k / 128) * (t > 1 ? 0.5 * (t + up(t)) : 1) + 0.424 * nk + (nk > 40 ? 0.19 * (nk - 40) : 0) + 1.22 * m * k * 1e-6 +
+           (0.57 + (N % 4 ? 0.67 : 0)) * m * n * 1e-6;
+}
+
+// gemm_dec_kernel: waves of clusters.
+double dec_us(int64_t M, int64_t N, int64_t K, int split, bool nib, bool words, int sm_count)
+{
+    const double m = (double)M, k = (double)K, panels = up(m / 128), ctas = up((double)N / 128) * split, waves = up(ctas / sm_count);
+    const double load = ctas < sm_count ? ctas / sm_count : 1;
+    double step = (panels <= 1 ? 0.332 : panels <= 2 ? 0.449 : 0.634) * (nib ? 1 : 1.13);
+    if (!words && step < 0.4) step = 0.4;
+    return 5.85 + 1.8 * panels + 2.0 * m * k * 1e-6 + 0.51 * m * (double)N * 1e-6 + 0.02 * (split - 1) + 0.67 * load + 5 * (waves - 1) +
+           waves * up(up(k / 64) / split) * step * (0.9 + 0.1 * load);
+}
+
+// Tokens per tile and pieces of K with which gemm_tmw_kernel is expected to take at most 0.98 of `other`, else 0.  Over the shapes
+// measured the route taken is then 0.926 of the other one on average and 1.009 of the best; in 33 of 3400 it is more than 2 % slower
+// than the other one (in six by 8 to 15 %).  Whole calls without / with it: 160 x 4096 x 11008 (M x K x N)
+// 40.4 / 25.0, 128 x 4096 x 11008 30.0 / 25.0, 256 x 2048 x 12288 26.8 / 21.3, 256 x 1024 x 16384 20.1 / 16.7, 512 x 8192 x 8192
+// 80.5 / 53.0, 768 x 16384 x 4096 105 / 86, 1024 x 4096 x 4096 38.4 / 35.1; K cut in two 448 x 16384 x 4096 100 / 54.6, in three
+// 352 x 8192 x 2048 29.6 / 27.6; left alone 1237 x 2048 x 2048 18.8 / 20.1.  Above 1536 rows the passes cost too little beside the product
+// (2048 x 4096 x 4096 62.6 / 61.0, 3072 x 1344 x 11008 74 / 82).
+int tmw_tokens(int64_t M, int64_t N, int64_t K, bool nib, bool words, double other, int sm_count, const int *clusters, int *pieces)
+{
+    const double m = (double)M, n = (double)N, k = (double)K;
+    double best = 0.98 * other;
     int tokens = 0;
-    double best = 1e30;
+    if (N < 32) return 0;                                                // an eighth of a tile (1400 x 64 x 4 7.6 / 7.9)
     for (int T = 64; T <= mx::TmwCfg::MAX_T && T < M + 64; T += 32) {
-        const double tiles = up(m / T) * up(n / 256), rounds = up(tiles / pairs), step_us = nib ? T > 224 ? 0.288 : 0.273 : 0.345;
+        const double tiles = up(m / T) * up(n / 256);
         for (int s = 1; s <= mx::TmwCfg::MAX_SPLIT; ++s) {
-            const int unit = nib ? 4 : 2;                                // K steps per stage of packed weights
-            if (s > 1 && (tiles > clusters[s] || steps < s * unit)) break;
-            const double us = 1.1 * mk + (s == 1 ? 6.3 + rounds * steps * step_us + 0.0137 * T * (mx::TmwCfg::accs(T) == 1 ? rounds : 1)
-                                                 : 5.5 + 0.73 * s + up(up(steps / unit) / s) * unit * step_us + 0.023 * T);
+            if (s > 1 && (tiles > clusters[s] || up(k / 64) < s * (nib ? 4 : 2))) break;
+            const double us = tmw_us(m, n, k, nib, words, T, s, sm_count / 2);
             if (us < best) {
                 best = us;
                 tokens = T;
@@ -1898,44 +1959,27 @@ int tmw_tokens(int64_t M, int64_t N, int64_t K, bool nib, bool rec, int split, i
             }
         }
     }
-    const bool few = M <= 384;
-    const double t128 = up(m / 128) * up(n / 128), t256 = up(m / 256) * up(n / 256) / pairs, step = rec ? few ? 0.125 : 0.169 : few ? 0.278 : 0.299;
-    double product = (t256 > 1 ? 0.5 * (t256 + up(t256)) : 1) * steps * step + (few ? -10.4 : 2.5);
-    if (2 * t128 <= pairs * 2) {
-        const double cut = steps / (4 * t128 > pairs * 2 ? 2 : 4) * (few ? 0.152 : 0.164) + (few ? -9.9 : 2.9);
-        product = cut < product ? cut : product;
-    } else if (t128 <= pairs * 2) {
-        const double wave = steps * (few ? 0.152 : 0.164) + (few ? -10.4 : 2.5);
-        product = wave < product ? wave : product;
-    }
-    double other = product + (few ? 17.8 + 0.522 * nk + 1.37 * mk + 0.207 * mn : 5.2 + 0.443 * nk + 0.942 * mk + 0.418 * mn);
-    if (split) {
-        const double waves = up(up(n / 128) * split / sm_count);
-        const double dec = -26.1 + 3.9 * mk + 1.03 * mn + waves * (up(steps / split) * (0.112 + 0.159 * up(m / 128)) * (nib ? 1 : 1.16) + 34.45);
-        other = dec < other ? dec : other;
-    }
-    if (M > 128 && M <= 256 && K < 1280) return 0;
-    return best < (!few ? rec ? 0.9 : 0.92 : *pieces > 1 ? 0.93 : M > 256 && K > 3072 ? 0.8 : 0.94) * other ? tokens : 0;
+    return tokens;
 }
 
-// Whether to run it, against a pass over the weights and then a product (`rec`: of block-scaled records, where that one would
-// run, else of bf16).  Whole calls in a graph, us, without -> with it; 8-bit activations, 4-bit weights, blocks of 16 (records:
-// 4 bits), B200:
-//   rows    K x N         without -> with     records        rows    K x N         without -> with     records
-//   128     1024 x 4096    12.5 -> 10.7    13.1 -> 10.6      128     4096 x 22528   84.2 ->  76.6    73.9 -> 76.8
-//   128     2048 x 6144    17.4 -> 16.6    20.1 -> 16.4      128     2048 x 28672   52.0 ->  46.7    45.9 -> 46.5
-//   128     8192 x 2048    24.0 -> 19.5    24.0 -> 19.7      128     4096 x 32000  111.5 ->  77.8    94.2 -> 77.8
-//   128     4096 x 4096    19.5 -> 16.8    19.3 -> 16.8      256     2048 x 2560    13.7 ->  14.9    13.7 -> 14.9
-//   128     1024 x 9600    15.0 -> 16.4    16.2 -> 16.4      256     4096 x 4096    24.2 ->  21.9    24.0 -> 21.9
-//   64      1024 x 9600    14.5 -> 15.6    15.4 -> 15.6      256     11008 x 4096   54.1 ->  40.1    54.1 -> 39.9
-//   128     256 x 9600     13.1 -> 10.4    13.1 -> 10.4      256     1024 x 16384   19.3 ->  21.9    19.0 -> 21.9
-//   128     4096 x 9600    41.2 -> 39.7    35.4 -> 39.7      256     3072 x 14336   48.3 ->  42.2    34.8 -> 42.2
-//   128     1024 x 16384   17.2 -> 16.8    18.2 -> 16.8      256     4096 x 16384   63.9 ->  52.8    49.2 -> 52.8
-//   128     4096 x 16384   59.2 -> 39.9    47.3 -> 40.1      384     4096 x 3072    23.4 ->  24.8    23.2 -> 25.0
-//   128     1024 x 19072   20.5 -> 30.7    23.1 -> 30.5      384     4096 x 4096    31.3 ->  26.2    27.4 -> 26.4
-//   128     4096 x 19072   75.6 -> 76.0    65.9 -> 76.0      384     4096 x 6144    35.6 ->  37.7    31.3 -> 37.3
-//   128     1024 x 28672   24.4 -> 31.5    27.2 -> 31.3      384     6144 x 6144    52.2 ->  50.6    43.4 -> 50.2
-//   128     1344 x 28672   36.7 -> 36.3    35.0 -> 36.3      384     8192 x 8192    90.5 ->  63.1    63.1 -> 63.5
+// Whether gemm_dec_kernel beats a pass over the weights and then a product (`rec`: of block-scaled records, where that one would run,
+// else of bf16); tmw_tokens decides after it.  Whole calls in a graph, us, 8-bit activations (records: 4 bits), 4-bit weights, blocks
+// of 16; bf16 / records / gemm_dec_kernel / the best of gemm_tmw_kernel:
+//   rows     K x N        bf16    rec    dec    tmw      rows     K x N        bf16    rec    dec    tmw
+//   128   1024 x 4096    10.8   11.9    9.8   10.5      128   4096 x 22528   83.6   70.1   57.5   41.7
+//   128   2048 x 6144    16.5   18.7   13.9   14.5      128   2048 x 28672   51.8   45.4   37.9   26.4
+//   128   8192 x 2048    22.0   33.3   16.1   19.4      128   4096 x 32000  109.9   91.7   58.2   41.6
+//   128   4096 x 4096    19.6   24.2   14.6   17.2      256   2048 x 2560    12.4   15.9   14.1   14.1
+//   128   1024 x 9600    14.0   15.5   13.6   11.7      256   4096 x 4096    22.8   24.8   19.1   20.3
+//   64    1024 x 9600    13.6   14.4   12.8   10.7      256  11008 x 4096    50.6   58.2   34.7   35.7
+//   128    256 x 9600    12.7   10.4    9.5    8.7      256   1024 x 16384   20.1   18.9   20.7   16.7
+//   128   4096 x 9600    37.8   35.6   29.9   24.8      256   3072 x 14336   41.8   36.2   35.3   26.1
+//   128   1024 x 16384   17.1   18.0   14.0   12.4      256   4096 x 16384   63.3   48.8   43.3   31.8
+//   128   4096 x 16384   58.2   48.0   31.1   26.1      384   4096 x 3072    21.7   24.7   23.5   22.5
+//   128   1024 x 19072   21.5   22.8   25.7   16.2      384   4096 x 4096    26.7   26.2   25.2   23.6
+//   128   4096 x 19072   74.8   62.2   57.2   40.6      384   4096 x 6144    31.2   31.2   34.6   26.9
+//   128   1024 x 28672   26.7   27.6   27.5   17.9      384   6144 x 6144    46.2   43.6   46.5   34.9
+//   128   1344 x 28672   37.4   35.8   31.0   22.9      384   8192 x 8192    76.0   61.0   58.6   45.7
 // Up to 128 rows: while its CTAs make one wave that leaves at most three SMs in ten idle, wherever the weights are large.  A
 // second wave repeats ramp and exchange, which the other product overlaps with its loads: from K = 1344 on where it is full, from
 // 4096 on where not.  A single wave that is not full and not cut is worth it against bf16 only, for very short K or long.

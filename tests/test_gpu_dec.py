@@ -1,8 +1,8 @@
-"""Up to 384 rows with the packed weights decoded inside the product (gemm_dec_kernel), at the edges of its panels (128 rows),
-tiles (128 columns), pieces of K (pairs of 64) and stages, for every storage form of the weights: against the same product
-behind a pass over the weights.  Both add exact products up in fp32, in orders of their own: at most K/16 rounded additions
-of partial sums on either side, each within 2^-24 of the absolute sum S, for K <= 16384 2^-13 S at the very most; 1e-5 S as
-elsewhere.  The fused tail and the MXInt result come from the same sums."""
+"""Up to 384 rows with the packed weights decoded inside the product: gemm_dec_kernel (1) at the edges of its panels (128 rows), tiles
+(128 columns), pieces of K (pairs of 64) and stages, for every storage form of the weights, and sizes that gemm_tmw_kernel (2) takes:
+against the same product behind a pass over the weights.  Both add exact products up in fp32, in orders of their own: at most K/16
+rounded additions of partial sums on either side, each within 2^-24 of the absolute sum S, for K <= 16384 2^-13 S at the very most;
+1e-5 S as elsewhere.  The fused tail and the MXInt result come from the same sums."""
 import pytest
 import torch
 
@@ -11,29 +11,35 @@ from paper_2307_15517_b200 import binding as mxb
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("M,K,N,block,wa,ww,rows2", [
-    (17, 4096, 4112, 16, 8, 4, 1),         # one panel, K in four pieces
-    (33, 784, 3002, 16, 8, 8, 1),          # K % 64 == 16, exponent rows of 49 bytes, a ragged last tile; bytes
-    (128, 8224, 2050, 32, 7, 4, 2),        # odd K steps in eight pieces, weights in two-row blocks
-    (64, 96, 32000, 32, 6, 3, 1),          # two K steps, K not cut
-    (100, 2080, 2001, 16, 8, 2, 1),        # odd row length: stores of single values
-    (40, 4096, 2000, 16, 4, 4, 1),         # operands that could be records
-    (129, 3104, 4100, 16, 8, 4, 1),        # two panels
-    (256, 4096, 4096, 32, 8, 8, 1),
-    (256, 1040, 16200, 16, 8, 6, 1),       # K not cut
-    (257, 4112, 4090, 16, 8, 8, 2),        # three panels
-    (384, 8192, 4096, 16, 8, 4, 1),
-    (384, 4192, 4200, 32, 4, 4, 1),
-    (64, 160, 14400, 32, 6, 3, 1),         # three K steps, K not cut, one wave
-    (100, 1344, 28416, 16, 8, 4, 1),       # two waves
-    (96, 720, 130, 16, 8, 8, 1),           # few weights: twelve K steps in three pieces
-    (33, 960, 300, 32, 8, 4, 1),           # ... fifteen
-    (256, 3088, 16200, 16, 8, 6, 1),       # two panels, K not cut
+@pytest.mark.parametrize("M,K,N,block,wa,ww,rows2,kernel", [
+    (17, 4096, 4112, 16, 8, 4, 1, 0),      # one panel, K in four pieces (the query starts at 33 rows)
+    (33, 784, 3002, 16, 8, 8, 1, 1),       # K % 64 == 16, exponent rows of 49 bytes, a ragged last tile; bytes
+    (128, 8224, 2050, 32, 7, 4, 2, 1),     # odd K steps in eight pieces, weights in two-row blocks
+    (64, 96, 32000, 32, 6, 3, 1, 2),       # two K steps
+    (100, 2080, 2001, 16, 8, 2, 1, 1),     # odd row length: stores of single values
+    (40, 4096, 2000, 16, 4, 4, 1, 1),      # operands that could be records
+    (129, 3104, 4100, 16, 8, 4, 1, 1),     # two panels
+    (256, 4096, 4096, 32, 8, 8, 1, 1),
+    (256, 1040, 16200, 16, 8, 6, 1, 2),
+    (257, 4112, 4090, 16, 8, 8, 2, 0),     # (near the line between them)
+    (384, 8192, 4096, 16, 8, 4, 1, 2),
+    (384, 4192, 4200, 32, 4, 4, 1, 1),     # three panels
+    (64, 160, 14400, 32, 6, 3, 1, 2),      # three K steps
+    (100, 1344, 28416, 16, 8, 4, 1, 2),
+    (96, 720, 130, 16, 8, 8, 1, 1),        # few weights: twelve K steps in three pieces
+    (33, 960, 300, 32, 8, 4, 1, 1),        # ... fifteen
+    (256, 3088, 16200, 16, 8, 6, 1, 2),
+    (71, 288, 7760, 16, 8, 8, 1, 1),       # K not cut
+    (151, 5280, 2862, 32, 8, 4, 1, 1),     # two panels, K in five pieces
+    (264, 4512, 13286, 16, 8, 3, 1, 1),    # three panels, K not cut
+    (272, 4160, 29707, 32, 8, 8, 1, 1),    # two waves
+    (309, 9568, 1831, 16, 8, 6, 1, 1),     # three panels in eight pieces
 ])
-def test_weights_decoded_in_the_product(M, K, N, block, wa, ww, rows2):
+def test_weights_decoded_in_the_product(M, K, N, block, wa, ww, rows2, kernel):
     g = torch.Generator(device="cuda")
     g.manual_seed(M + K + N)
     fa, fw = mxb.MxFormat(block, wa), mxb.MxFormat(block, ww, block_rows=rows2)
+    assert not kernel or mxb.mx_selftest_route(M, N, K, fa, fw)[0] == kernel
     ld = -(-K // 8) * 8
     x = torch.randn(M, ld, generator=g, device="cuda")[:, :K]
     w = torch.randn(N, K, generator=g, device="cuda") * 0.02 * torch.exp2(torch.randint(-9, 9, (N, 1), generator=g, device="cuda").float())
@@ -97,22 +103,26 @@ def _launches(call):
     return {kind: n for kind, (_, n) in mxb.mx_profile_end().items()}
 
 
-@pytest.mark.parametrize("M,K,N,block,wa,ww,decoded", [
-    (64, 704, 512, 16, 8, 4, False), (64, 768, 512, 16, 8, 4, True), (33, 960, 256, 16, 8, 4, True), (33, 992, 256, 16, 8, 4, False),
-    (128, 768, 256, 16, 8, 4, False), (128, 768, 768, 16, 4, 4, True), (128, 896, 768, 16, 8, 4, False),
-    (128, 1024, 9600, 16, 8, 4, False), (64, 1024, 9600, 16, 8, 4, False), (128, 256, 9600, 16, 8, 4, True), (128, 4096, 9600, 16, 8, 4, True),
-    (128, 1024, 18944, 16, 8, 4, True), (128, 1024, 19072, 16, 8, 4, False), (128, 1024, 28672, 16, 8, 4, False),
-    (128, 1344, 28672, 16, 8, 4, True), (128, 4096, 19072, 16, 8, 4, True), (128, 2048, 19072, 16, 8, 4, False),
-    (256, 1024, 16384, 16, 8, 4, False), (256, 3072, 14336, 16, 8, 4, True), (384, 4096, 6144, 16, 8, 4, False),
-    (384, 4096, 4096, 16, 8, 4, True), (100, 2080, 3002, 16, 8, 4, True),
+@pytest.mark.parametrize("M,K,N,block,wa,ww,kernel", [
+    (64, 704, 512, 16, 8, 4, 5), (64, 768, 512, 16, 8, 4, 1), (33, 960, 256, 16, 8, 4, 1), (33, 992, 256, 16, 8, 4, 4),
+    (128, 768, 256, 16, 8, 4, 5), (128, 768, 768, 16, 4, 4, 1), (128, 896, 768, 16, 8, 4, 5),
+    (128, 1024, 9600, 16, 8, 4, 2), (64, 1024, 9600, 16, 8, 4, 2), (128, 256, 9600, 16, 8, 4, 2), (128, 4096, 9600, 16, 8, 4, 2),
+    (128, 1024, 18944, 16, 8, 4, 2), (128, 1024, 19072, 16, 8, 4, 2), (128, 1024, 28672, 16, 8, 4, 2),
+    (128, 1344, 28672, 16, 8, 4, 2), (128, 4096, 19072, 16, 8, 4, 2), (128, 2048, 19072, 16, 8, 4, 2),
+    (256, 1024, 16384, 16, 8, 4, 2), (256, 3072, 14336, 16, 8, 4, 2), (384, 4096, 6144, 16, 8, 4, 2),
+    (384, 4096, 4096, 16, 8, 4, 2), (100, 2080, 3002, 16, 8, 4, 1), (1237, 2080, 3002, 16, 6, 6, 7), (352, 2048, 1024, 16, 8, 4, 4),
+    (256, 4096, 4096, 32, 8, 8, 1), (1536, 4096, 11008, 16, 8, 4, 2), (1537, 4096, 11008, 16, 8, 4, 6), (1400, 768, 31, 16, 8, 4, 5),
 ])
-def test_sizes_at_which_the_weights_are_decoded_in_the_product(M, K, N, block, wa, ww, decoded):
-    """Either side of the lines of the rule, by the launches: with it a pass over the activations alone."""
+def test_sizes_at_which_the_weights_are_decoded_in_the_product(M, K, N, block, wa, ww, kernel):
+    """Sizes of every route, by the query and by the launches: with kernels 1 and 2 a pass over the activations alone."""
+    if torch.cuda.get_device_properties(0).multi_processor_count != 148:
+        pytest.skip("sizes for 148 SMs")
     fa, fw = mxb.MxFormat(block, wa), mxb.MxFormat(block, ww)
+    assert mxb.mx_selftest_route(M, N, K, fa, fw)[0] == kernel
     x = torch.randn(M, K, device="cuda")
     wm, we = mxb.mx_quantize(torch.randn(N, K, device="cuda"), fw)
     n = _launches(lambda: mxb.mx_linear(x, fa, wm, we, fw, N))
-    assert (n["quantize"] == 1 and n["prep"] == n["dequantize"] == 0) == decoded, n
+    assert (n["quantize"] == 1 and n["prep"] == n["dequantize"] == 0) == (kernel in (1, 2)), n
     assert n["gemm_tc"] == 1
 
 

@@ -10,43 +10,57 @@ from paper_2307_15517_b200 import binding as mxb
 pytestmark = pytest.mark.gpu
 
 
-def decoded_in_the_product(call):
-    mxb.mx_profile_begin()
-    call()
-    n = {kind: k for kind, (_, k) in mxb.mx_profile_end().items()}
-    return n["prep"] == 0 and n["gemm_tc"] == 1 and n["quantize"] == 1
+def runs(M, K, N, fa, fw, tokens, pieces):
+    """The kernel, and on 148 SMs its tile and its pieces of K, for the fp32 and the MXInt result."""
+    tile = torch.cuda.get_device_properties(0).multi_processor_count == 148
+    for quantized in (False, True):
+        route = mxb.mx_selftest_route(M, N, K, fa, fw, quantized)
+        assert route[0] == 2 and (not tile or route[1:] == (tokens, pieces)), route
 
 
-@pytest.mark.parametrize("M,K,N,block,wa,ww,rows2", [
-    (400, 784, 8200, 16, 8, 8, 1),         # K % 64 == 16, exponent rows of 49 bytes, 224 tokens: one accumulator
-    (385, 4128, 16200, 32, 6, 4, 1),       # two rounds of 224 tokens, a ragged last tile of features
-    (700, 592, 16001, 16, 7, 4, 1),        # 192 tokens, four rounds; rows of 37 exponent bytes; odd row length
-    (640, 4096, 4100, 16, 8, 3, 1),        # 160 tokens, one round
-    (900, 8192, 4102, 32, 8, 4, 2),        # 256 tokens; weights in two-row blocks
-    (513, 1344, 12290, 16, 8, 6, 1),       # a last token tile of 129, whole tiles of the second CTA outside
-    (257, 2080, 12290, 16, 8, 2, 1),       # 96 tokens, 33 K steps
-    (130, 1296, 16162, 16, 8, 8, 2),       # 21 K steps; bytes in two-row blocks
-    (500, 96, 16384, 32, 8, 4, 1),         # two K steps (one and a half), 128 tokens
-    (600, 160, 14000, 32, 6, 8, 1),        # three K steps, 160 tokens
-    (1400, 512, 11582, 16, 8, 4, 1),
-    (1500, 64, 16384, 16, 8, 4, 1),        # tiles of one step, each a stage of packed weights: a group passes two for one of its own
-    (1500, 32, 16384, 32, 4, 3, 1),
-    (1500, 48, 16384, 16, 8, 8, 1),
-    (1000, 96, 16000, 16, 8, 8, 1),        # two steps, one stage
-    (768, 4096, 11008, 32, 8, 8, 1),       # bytes, a group has no step in every third stage: 256 tokens, eight stages of decoded weights
-    (500, 1104, 8192, 16, 8, 6, 1),
+@pytest.mark.parametrize("M,K,N,block,wa,ww,rows2,tokens", [
+    (400, 784, 8200, 16, 8, 8, 1, 224),    # K % 64 == 16, exponent rows of 49 bytes; one accumulator
+    (385, 4128, 16200, 32, 6, 4, 1, 224),  # two rounds, a ragged last tile of features
+    (700, 592, 16001, 16, 7, 5, 1, 192),   # four rounds; rows of 37 exponent bytes; odd row length
+    (640, 4096, 4100, 16, 8, 3, 1, 160),   # one round
+    (900, 8192, 4102, 32, 8, 4, 2, 256),   # weights in two-row blocks
+    (513, 1344, 12290, 16, 8, 6, 1, 192),  # a last token tile of 129, whole tiles of the second CTA outside
+    (257, 2080, 12290, 16, 8, 2, 1, 96),   # 33 K steps
+    (130, 1296, 16162, 16, 8, 8, 2, 160),  # 21 K steps; bytes in two-row blocks
+    (500, 96, 16384, 32, 8, 4, 1, 192),    # two K steps (one and a half)
+    (600, 160, 14000, 32, 6, 8, 1, 160),   # three K steps
+    (1400, 512, 11582, 16, 8, 4, 1, 192),
+    (1500, 64, 16384, 16, 8, 4, 1, 192),   # tiles of one step, each a stage of packed weights, of which a group has every third
+    (1500, 32, 16384, 32, 4, 3, 1, 192),
+    (1500, 48, 16384, 16, 8, 8, 1, 192),
+    (1000, 96, 16000, 16, 8, 8, 1, 160),   # two steps, one stage
+    (768, 4096, 11008, 32, 8, 8, 1, 256),  # bytes: a group has no step in every third stage; eight stages of decoded weights
+    (500, 1104, 8192, 16, 8, 6, 1, 256),
+    (33, 32, 136, 32, 8, 3, 1, 64),        # the smallest: half a step, a token beyond the first CTA's
+    (170, 32, 9522, 16, 8, 3, 1, 64),      # two rounds
+    (152, 80, 10562, 16, 8, 6, 1, 64),
+    (245, 32, 10196, 16, 8, 8, 1, 96),
+    (198, 32, 11144, 32, 8, 4, 1, 96),
+    (524, 80, 6612, 16, 8, 6, 1, 128),
+    (485, 32, 6322, 32, 8, 4, 1, 128),
+    (275, 352, 13702, 32, 8, 3, 1, 160),
+    (1505, 272, 4630, 16, 8, 5, 1, 224),   # bytes, one accumulator, several rounds
+    (1098, 416, 6702, 16, 8, 4, 1, 224),
+    (483, 560, 13796, 16, 8, 7, 1, 256),
+    (984, 416, 9006, 16, 8, 2, 2, 256),
 ])
-def test_weights_decoded_into_tensor_memory(M, K, N, block, wa, ww, rows2):
+def test_weights_decoded_into_tensor_memory(M, K, N, block, wa, ww, rows2, tokens):
     g = torch.Generator(device="cuda")
     g.manual_seed(M + K + N)
     fa, fw = mxb.MxFormat(block, wa), mxb.MxFormat(block, ww, block_rows=rows2)
+    runs(M, K, N, fa, fw, tokens, 1)
     ld = -(-K // 8) * 8
     x = torch.randn(M, ld, generator=g, device="cuda")[:, :K]
     w = torch.randn(N, K, generator=g, device="cuda") * 0.02 * torch.exp2(torch.randint(-9, 9, (N, 1), generator=g, device="cuda").float())
     wm, we = mxb.mx_quantize(w, fw)
     bias = torch.randn(N, generator=g, device="cuda")
     y = torch.full((M, N + 4), -7.0, device="cuda")
-    assert decoded_in_the_product(lambda: mxb.mx_linear(x, fa, wm, we, fw, N, bias=bias, y=y[:, :N]))
+    mxb.mx_linear(x, fa, wm, we, fw, N, bias=bias, y=y[:, :N])
     want = mxb.mx_linear(x, fa, wm, we, fw, N, bias=bias, algo=mxb.MX_ALGO_TCGEN05)
     assert mxb.mx_poll_status() == 0
     assert (y[:, N:] == -7.0).all()
@@ -68,26 +82,43 @@ def test_weights_decoded_into_tensor_memory(M, K, N, block, wa, ww, rows2):
     assert mxb.mx_poll_status() == 0
 
 
-@pytest.mark.parametrize("M,K,N,block,wa,ww", [
-    (500, 8208, 4098, 16, 8, 4),           # two pieces, the last K step of 16; 256 tokens, a ragged last tile of features
-    (640, 8192, 2048, 32, 6, 4),           # two pieces, 160 tokens
-    (352, 8192, 2048, 16, 8, 4),           # three pieces
-    (400, 16400, 4096, 16, 8, 8),          # bytes
-    (384, 16384, 4100, 32, 8, 3),
+@pytest.mark.parametrize("M,K,N,block,wa,ww,tokens,pieces", [
+    (226, 3312, 6184, 16, 8, 6, 256, 2),   # the last K step of 48; a ragged last tile of features
+    (640, 8192, 2048, 32, 6, 4, 160, 2),
+    (352, 8192, 2048, 16, 8, 4, 192, 3),
+    (400, 16400, 4096, 16, 8, 8, 224, 2),  # bytes
+    (502, 4192, 2693, 32, 8, 4, 256, 3),   # pieces of unequal length, the last K step of 32; odd row length
+    (38, 464, 137, 16, 8, 6, 64, 2),       # a second piece of two stages of packed weights, half of the features outside
+    (36, 5920, 4273, 16, 8, 2, 64, 3),
+    (108, 848, 155, 16, 8, 5, 64, 4),
+    (137, 1376, 4077, 32, 8, 2, 96, 2),
+    (194, 1104, 1668, 16, 8, 7, 96, 3),
+    (207, 1232, 2919, 16, 8, 8, 128, 2),
+    (126, 8224, 4788, 16, 8, 2, 128, 3),
+    (104, 11104, 3807, 16, 8, 4, 128, 4),
+    (136, 1872, 2969, 16, 8, 6, 160, 3),
+    (139, 3552, 3196, 32, 8, 3, 160, 4),
+    (188, 1584, 5964, 16, 8, 5, 192, 2),
+    (171, 2352, 3573, 16, 8, 8, 192, 4),
+    (395, 3296, 2524, 32, 8, 3, 224, 3),
+    (210, 3216, 3300, 16, 8, 7, 224, 4),
+    (450, 2992, 2686, 16, 8, 7, 256, 3),
+    (239, 10528, 2543, 32, 8, 3, 256, 4),
 ])
-def test_pieces_of_K_added_up_in_a_cluster(M, K, N, block, wa, ww):
+def test_pieces_of_K_added_up_in_a_cluster(M, K, N, block, wa, ww, tokens, pieces):
     """The partial sums of two to four pieces are added in fp32: at most one rounding of a partial sum more than one chain per
     piece, 2^-22 of the absolute sum S; 1e-5 S as elsewhere.  The tail and the MXInt result come from the same sums."""
     g = torch.Generator(device="cuda")
     g.manual_seed(M + K + N)
     fa, fw = mxb.MxFormat(block, wa), mxb.MxFormat(block, ww)
+    runs(M, K, N, fa, fw, tokens, pieces)
     x = torch.randn(M, K, generator=g, device="cuda")
     wm, we = mxb.mx_quantize(torch.randn(N, K, generator=g, device="cuda") * 0.02, fw)
     bias = torch.randn(N, generator=g, device="cuda")
     am, ae = mxb.mx_quantize(x, fa)
     S = mxb.mx_dequantize(am, ae, K, fa).abs().double() @ mxb.mx_dequantize(wm, we, K, fw).abs().double().t() + bias.abs().double()
     y = torch.full((M, N + 4), -7.0, device="cuda")
-    assert decoded_in_the_product(lambda: mxb.mx_linear(x, fa, wm, we, fw, N, bias=bias, y=y[:, :N]))
+    mxb.mx_linear(x, fa, wm, we, fw, N, bias=bias, y=y[:, :N])
     want = mxb.mx_linear(x, fa, wm, we, fw, N, bias=bias, algo=mxb.MX_ALGO_TCGEN05)
     assert (y[:, N:] == -7.0).all()
     y = y[:, :N].contiguous()
@@ -108,7 +139,7 @@ def test_pieces_of_K_added_up_in_a_cluster(M, K, N, block, wa, ww):
 @pytest.mark.parametrize("block,ww", [(16, 4), (32, 8)])
 def test_any_exponents_any_address_and_a_normalised_input(block, ww):
     """Exponent bytes at the ends of the range, rows of them at odd addresses, activations from a LayerNorm: as behind a pass."""
-    M, K, N = 640, 4096, 4352
+    M, K, N = 448, 4096, 9216
     g = torch.Generator(device="cuda")
     g.manual_seed(ww)
     fa, fw = mxb.MxFormat(block, 8), mxb.MxFormat(block, ww)
@@ -116,8 +147,8 @@ def test_any_exponents_any_address_and_a_normalised_input(block, ww):
     wm, we = mxb.mx_quantize(torch.randn(N, K, generator=g, device="cuda") * 0.02, fw)
     for row, blk, e in ((3, 1, 0), (4, 2, 1), (5, 3, 226), (6, 0, 227), (7, 5, 150), (N - 1, K // block - 1, 255), (130, 4, 255)):
         we[row, blk] = e
-    y = torch.empty(M, N, device="cuda")
-    assert decoded_in_the_product(lambda: mxb.mx_linear(x, fa, wm, we, fw, N, y=y))
+    runs(M, K, N, fa, fw, 224, 1)
+    y = mxb.mx_linear(x, fa, wm, we, fw, N)
     want = mxb.mx_linear(x, fa, wm, we, fw, N, algo=mxb.MX_ALGO_TCGEN05)
     nan = torch.isnan(want)
     assert nan[:, N - 1].all() and nan[:, 130].all() and not nan[:, :130].any()
@@ -140,6 +171,7 @@ def test_weights_written_by_the_launch_in_front():
     g = torch.Generator(device="cuda")
     g.manual_seed(5)
     fa, fw = mxb.MxFormat(16, 8), mxb.MxFormat(16, 4)
+    runs(M, K, N, fa, fw, 160, 1)
     x = torch.randn(M, K, generator=g, device="cuda")
     ws = [torch.randn(N, K, generator=g, device="cuda") for _ in range(5)]
     want = [mxb.mx_linear(x, fa, *mxb.mx_quantize(w, fw), fw, N, algo=mxb.MX_ALGO_TCGEN05) for w in ws]
