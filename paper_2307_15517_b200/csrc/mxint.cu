@@ -1195,13 +1195,14 @@ int wide_pair_tile(int64_t M, int64_t N, int64_t K, const DeviceInfo &d)
 // many as the 128 x 128 tiles and gain nothing (1024 x 2048 x 2048, 128 columns, 16.1 / 16.9), 256 columns neither (24.1 / 24.6).
 // Not where tiles of 128 x 128 make one wave, which need 32 KB per step (19.6 / 22.1 at 384 x 2048 x 6144, 31.8 / 35.6 at 384 x 4096 x
 // 6144, 35.3 / 38.1 at 384 x 5120 x 5120), and not for fewer than five K steps, whose results leave in one burst at the end (640 x 256 x
-// 4096 12.4 / 13.6, 300 x 96 x 6464 17.0 / 23.8; of 300 shapes from K = 320 on none is more than 4 % slower).
-int one_round_width(int64_t M, int64_t N, const DeviceInfo &d)
+// 4096 12.4 / 13.6, 300 x 96 x 6464 17.0 / 23.8; of 300 shapes from K = 320 on none is more than 4 % slower), four of 160 columns
+// (2048 x 256 x 1408 11.5 / 10.0).
+int one_round_width(int64_t M, int64_t N, int64_t K, const DeviceInfo &d)
 {
     const int64_t rows = (M + 255) / 256, cols = d.sm_count / 2 / rows;
     if (!cols) return 0;
     const int64_t w = ((N + cols - 1) / cols + 31) / 32 * 32;
-    return w >= 160 && w <= 224 ? (int)w : 0;
+    return w >= 160 && w <= (K < 320 ? 160 : 224) ? (int)w : 0;
 }
 
 // Which product on bf16 operands a call takes (`count` products of one shape in one launch).  may_split: K may be cut (the sum is
@@ -1229,7 +1230,7 @@ mx_status_t tc_route(int64_t M, int64_t N, int64_t K, int count, bool may_split,
         *out = {width ? TC_PAIR_WIDE : TC_PAIR, width ? width : 256, 1};
         return MX_OK;
     }
-    const int width = M > 128 && K >= 320 && tiles128 > d.sm_count ? one_round_width(M, N, d) : 0;
+    const int width = M > 128 && K >= 256 && tiles128 > d.sm_count ? one_round_width(M, N, K, d) : 0;
     if (width) {
         *out = {TC_PAIR_WIDE, width, 1};
         return MX_OK;

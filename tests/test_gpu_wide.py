@@ -103,7 +103,8 @@ def test_one_round_of_narrow_pair_tiles_has_the_bits_of_narrow_calls(M, N, K):
 @pytest.mark.parametrize("M,N,K,kernel,width", [
     (384, 6144, 2048, 5, 128), (384, 6144, 4096, 5, 128), (384, 5120, 5120, 5, 128),       # 144 and 120 tiles of 128 x 128
     (385, 6144, 2048, 7, 192), (250, 11008, 1040, 7, 160), (256, 9472, 2048, 5, 128), (256, 9600, 2048, 7, 160),
-    (640, 4096, 256, 5, 256), (640, 4096, 320, 7, 192), (300, 6464, 96, 5, 256)])                # the same of 128 x 256; few K steps
+    (640, 4096, 256, 5, 256), (640, 4096, 320, 7, 192), (300, 6464, 96, 5, 256),                # few K steps
+    (2048, 1408, 256, 7, 160), (2048, 1408, 240, 5, 256)])
 def test_narrow_pair_tiles_only_where_they_are_faster(M, N, K, kernel, width):
     if torch.cuda.get_device_properties(0).multi_processor_count != 148:
         pytest.skip("sizes for 148 SMs")
