@@ -16,11 +16,12 @@
 // The tile is 256 features x T tokens, T a multiple of 32 that the host picks so that the tiles fill whole rounds of the chip's
 // pairs; up to T = 192 there are two accumulators, so the epilogue of a tile runs under the next one's MMAs.  Few tiles: K is cut
 // over the pairs of a cluster, whose partial tiles go to shared memory and are added up in the order of K (mx_gemm_splitk.cuh).
-// Bound by the instructions of the decoding warps, 0.25 us per K step and round up to T = 192 (without the MMAs the same, without the
-// decoding 0.16 at T = 64 and 0.31 at 256; four groups of warps, two steps per turn of a group, or half of the shifts as
-// multiplications changed nothing), and above by the MMAs (T = 224: 442 to 447 of the 2 T = 448 clocks).  Whole calls, M x K x N,
-// against a pass and a product / gemm_dec_kernel: 512 x 4096 x 11008 54.8 -> 45.5 us (with an MXInt result 53.3), 256 x 4096 x 12288
-// 58.2 -> 29.9, 128 x 4096 x 11008 30.1 -> 25.6, 352 x 2048 x 6144 19.4 -> 16.6; where it is chosen: tmw_tokens.
+// Bound by the instructions of the decoding warps, 0.25 us per K step and round up to T = 160 and 0.26 at 192 (without the MMAs the
+// same, without the decoding 0.16 at T = 64 and 0.31 at 256; four groups of warps, two steps per turn of a group, or half of the shifts
+// as multiplications changed nothing), and above by the MMAs (T = 224: 453 clocks per step by the counters, of which its MMAs need
+// 2 T = 448; 0.30 us at 256).
+// Whole calls, M x K x N, against a pass and a product / gemm_dec_kernel: 512 x 4096 x 11008 55.0 -> 45.6 us (with an MXInt result 53.3),
+// 256 x 4096 x 12288 42.5 -> 30.5, 128 x 4096 x 11008 30.0 -> 25.0, 352 x 2048 x 6144 19.2 -> 17.0; where it is chosen: tmw_tokens.
 // Persistent; all waits are bounded.
 #pragma once
 #include <cuda.h>
@@ -79,11 +80,11 @@ struct ExpFeed {
     int nb, bytes, words;     // exponent bytes of a row, per raw stage, and the words that hold the latter
     int unit;                 // 16, 8, 4: every piece is as wide and aligned; 0: by words
 
-    // the first stage starts at byte `start` of the rows, the others follow `bytes` apart
-    __device__ __forceinline__ ExpFeed(const uint8_t *w_exp, int nb_, int bytes_, int start, int exp_words)
+    // every stage starts a multiple of `bytes` into the rows (pieces of K are whole raw stages)
+    __device__ __forceinline__ ExpFeed(const uint8_t *w_exp, int nb_, int bytes_, int exp_words)
         : nb(nb_), bytes(bytes_), words((bytes_ >> 2) + (exp_words ? 0 : 1))
     {
-        const uint32_t all = (uint32_t)reinterpret_cast<uintptr_t>(w_exp) | (uint32_t)nb_ | (uint32_t)bytes_ | (uint32_t)start;
+        const uint32_t all = (uint32_t)reinterpret_cast<uintptr_t>(w_exp) | (uint32_t)nb_ | (uint32_t)bytes_;
         unit = !exp_words ? 0 : (all & 15u) == 0 ? 16 : (all & 7u) == 0 ? 8 : 4;
     }
     __device__ __forceinline__ void rows(const uint8_t *w_exp, int n0, int N, int shift, int lane)
@@ -350,7 +351,7 @@ gemm_tmw_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constan
         __syncwarp();
     } else if (warp == 2) {
         // raw stages: 128 rows x 128 mantissa bytes in one tiled load, their exponent bytes in the background (see gemm_dec_kernel)
-        ExpFeed feed(wp.w_exp, p.K / wp.block, EB, 0, wp.exp_words);
+        ExpFeed feed(wp.w_exp, p.K / wp.block, EB, wp.exp_words);
         const bool wait_last = Walk::waits_for_last(kblocks);            // (see StepWalk)
         uint32_t ri = 0;
         for (int t = pair; t < num_tiles && !timed_out; t += npairs) {
