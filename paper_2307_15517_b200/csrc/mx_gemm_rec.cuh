@@ -12,8 +12,8 @@
 //   warp 0      : TMA producer (in both CTAs; bytes are counted on the leader's barrier)
 //   warp 1      : tensor-memory allocation (both CTAs), scale copies and MMA issue (leader only)
 //   warps 2..9  : epilogue of the CTA's own 128 rows, two warps per TMEM lane quarter
-// What bounds it: operand fetch, 64 KB per 256 x 256 x 128 step and pair (13 TB/s over the chip at 0.36 us per step), and the
-// shared-memory reads of the MMAs (0.32 us per step with the fetches removed; 0.26 us is the pipe's peak).
+// What bounds it: the tensor pipe, 0.28 us per 256 x 256 x 128 step and pair against the pipe's own 0.26 (0.36 while one lane issued,
+// which was the bound then), with 64 KB of operands per step (17 TB/s over the chip); on few tiles per pair ramp and drain.
 //
 // Tensor memory: 512 columns cannot hold two accumulators of 256 and the scales.  The accumulators overlap by 32
 // columns ([0, 256) and [224, 480)), the last 32 columns hold two sets of scales.  The epilogue drains the shared

@@ -1085,11 +1085,13 @@ mx_status_t splitk_ways(int64_t M, int64_t N, int64_t K, DeviceInfo &d, int *out
 // - Where run_tc would cut K, a pair tile's 0.36 us per 128 of K, one tile after another, stand against the split's 0.2 us
 //   per 64 of a piece and its exchange, and against its operand form, which is twice as large.  The estimate below picks the
 //   faster side but for 4 % at most: 1 x 256 x 16384 55.5 / 27.3, 64 x 768 x 3072 18.1 / 12.9, 352 x 2048 x 8192 40.2 / 37.6,
-//   but 16 x 8192 x 8192 56.2 / 60.0 and 128 x 8192 x 16384 113 / 118.
+//   but 16 x 8192 x 8192 56.2 / 60.0 and 128 x 8192 x 16384 113 / 118.  (0.28 and 0.15 us since whole warps issue: the ratio, and
+//   the line, are the same.  Over 280 shapes of 17 to 1237 rows measured since, the side taken is 0.5 % off the faster one on average.)
 // - Otherwise records win from K = 2048 on (352 x 4096 x 4096 29.1 / 33.6, 768 x 2048 x 2048 19.1 / 19.3), and below that
 //   where the operands are large enough to pay for the pair tile's longer start and drain: 4096 x 2048 x 768 20.8 / 22.1,
 //   24 x 8192 x 512 11.7 / 12.5, but 1024 x 4096 x 768 15.9 / 14.7, 512 x 2048 x 1024 13.5 / 12.9.  Around the line the two
-//   differ by up to 12 % either way (128 x 12288 x 768 16.7 / 14.8).
+//   differ by up to 12 % either way (128 x 12288 x 768 16.7 / 14.8); short rows of wide layers are left on the slower side (448 x
+//   9536 x 256 11.8 / 17.3: their pass deals an item per row).
 mx_status_t rec_is_faster(int64_t M, int64_t N, int64_t K, DeviceInfo &d, bool *out)
 {
     int split = 0;
