@@ -1734,10 +1734,12 @@ mx_status_t tmw_clusters(DeviceInfo &d, int which, int (&out)[mx::TmwCfg::MAX_SP
     return MX_OK;
 }
 
-double tc_us(const TcRoute &r, int64_t M, int64_t N, int64_t K, int sm_count);
-double rec_us(int64_t M, int64_t N, int64_t K, int sm_count);
-double dec_us(int64_t M, int64_t N, int64_t K, int split, bool nib, bool words, int sm_count);
-int tmw_tokens(int64_t M, int64_t N, int64_t K, bool nib, bool words, double other, int sm_count, const int *clusters, int *pieces);
+enum ExpRows { EXP_WIDE, EXP_WORDS, EXP_BYTES };            // exponent rows: see tmw_us
+double tc_us(const TcRoute &r, int64_t M, int64_t N, int64_t K, bool quantized, int sm_count);
+double rec_us(int64_t M, int64_t N, int64_t K, bool quantized, int sm_count);
+double dec_us(int64_t M, int64_t N, int64_t K, int split, bool nib, bool words, bool quantized, int sm_count);
+int tmw_tokens(int64_t M, int64_t N, int64_t K, bool nib, int block, ExpRows rows, bool quantized, double other, int sm_count, const int *clusters,
+               int *pieces);
 
 // Whether the product decodes its weights itself, in which kernel, and for gemm_dec_kernel into how many pieces K is cut: the most
 // whose clusters all fit at once, of at least four K steps each.
@@ -1779,20 +1781,22 @@ mx_status_t dec_plan(int64_t M, int64_t N, int64_t K, const mx_format_t &fa, con
     if (M > 1536) return MX_OK;                                          // (see tmw_tokens)
     double other = 0;                                                    // us of the route that is taken else
     if (*use) {
-        other = dec_us(M, N, K, out->split, nib, out->exp_words != 0, d.sm_count);
+        other = dec_us(M, N, K, out->split, nib, out->exp_words != 0, quantized, d.sm_count);
     } else if (rec) {
-        other = rec_us(M, N, K, d.sm_count);
+        other = rec_us(M, N, K, quantized, d.sm_count);
     } else {
         TcRoute r;
         const mx_status_t ts = tc_route(M, N, K, 1, true, d, &r);
         if (ts != MX_OK) return ts;
-        other = tc_us(r, M, N, K, d.sm_count);
+        other = tc_us(r, M, N, K, quantized, d.sm_count);
     }
     const int which = (nib ? 4 : 0) + (quantized ? 2 : 0);
     int clusters[mx::TmwCfg::MAX_SPLIT + 1] = {}, pieces = 1;
     const mx_status_t cs = tmw_clusters(d, which + 1, clusters);
     if (cs != MX_OK) return cs;
-    out->tokens = tmw_tokens(M, N, K, nib, out->exp_words != 0, other, d.sm_count, clusters, &pieces);
+    const bool pairs_of_words = (((uint64_t)(K / fw.block) | reinterpret_cast<uintptr_t>(w_exp)) & 7u) == 0;
+    const ExpRows rows = !out->exp_words ? EXP_BYTES : pairs_of_words ? EXP_WIDE : EXP_WORDS;
+    out->tokens = tmw_tokens(M, N, K, nib, fw.block, rows, quantized, other, d.sm_count, clusters, &pieces);
     if (out->tokens) {
         out->which = which + (pieces > 1 ? 1 : 0);
         out->split = pieces;
@@ -1876,30 +1880,39 @@ mx_status_t launch_dec(const DecPlan &g, const __nv_bfloat16 *a_hat, const void 
 }
 
 // Estimates in us of whole calls on 148 SMs, pass over the activations included: what dec_plan compares gemm_tmw_kernel with the other
-// routes by.  Fitted to 3700 shapes -- 17 .. 2048 rows, K 32 .. 16384, N 2 .. 16384, widths 8/4, 4/4 and 8/8 -- with every route timed
-// (tmw_tokens: up to eleven tiles and cuts each).  One sigma of their errors: tmw_us and dec_us 4.9 %, tc_us 5.9 %, rec_us 4.6 %.
+// routes by.  Fitted to 5600 shapes -- 17 .. 2048 rows, K 32 .. 16384, N 2 .. 16384, widths 8/4, 4/4, 6/6 and 8/8, blocks of 16 and 32 --
+// with every route timed (tmw_tokens: up to eleven tiles and cuts each), 1900 of them with an MXInt result too.  One sigma of their
+// errors: tmw_us and dec_us 4.9 %, tc_us 5.9 %, rec_us 4.6 %; with an MXInt result (`quantized`) 5.7, 6.5, 5.5 and 11 %.
 double up(double x) { return (double)(int64_t)(x + 0.999999); }
 
 // gemm_tmw_kernel on tiles of T tokens, K in `pieces`.  Rounds of 74 pairs, each 0.253 us per K step of 64 up to 160 tokens (its
-// decoding warps), 0.263 at 192, 0.272 and 0.301 at 224 and 256 (its MMAs), for weights in bytes 0.342 and 0.349; more where exponent
-// rows are no whole words and come word by word; a tenth less on few pairs.  An odd number of steps costs two.  With one accumulator an
-// epilogue behind each round.
-double tmw_us(double M, double N, double K, bool nib, bool words, int T, int pieces, double pairs)
+// decoding warps), 0.263 at 192, 0.272 and 0.301 at 224 and 256 (its MMAs), for weights in bytes 0.342 and 0.349; a tenth less on few
+// pairs.  The exponent rows have to be copied in as well: by words (EXP_WORDS), of two pieces per K step of bytes in blocks of 16, they
+// take longer than the step, and so they do where they are no whole words (EXP_BYTES) and come by the words that hold them.  An odd
+// number of steps costs two.  An epilogue behind the last round, with one accumulator behind each; that of an MXInt result is long
+// enough to show under the next round's steps.
+double tmw_us(double M, double N, double K, bool nib, int block, ExpRows rows, bool quantized, int T, int pieces, double pairs)
 {
     const double steps = up(K / 64), mk = M * K * 1e-6, mn = M * N * 1e-6, unit = nib ? 4 : 2;   // unit: steps per stage of packed weights
     const double tiles = up(M / T) * up(N / 256), load = tiles * pieces < pairs ? tiles * pieces / pairs : 1;
     double step = nib ? T <= 160 ? 0.253 : T <= 192 ? 0.263 : T <= 224 ? 0.272 : 0.301 : T <= 192 ? 0.342 : 0.349;
-    if (!words) step = nib ? 0.332 : 0.402;
+    if (rows == EXP_BYTES) step = nib ? block == 16 ? 0.332 : 0.31 : block == 16 ? 0.46 : 0.415;
+    else if (rows == EXP_WORDS && !nib && block == 16) step = 0.4;
     step *= 0.9 + 0.1 * load;
     if (pieces > 1)                                                      // (2 % on top: what the fit lacks where the clusters fill the chip)
-        return 1.02 * (5.21 + 0.6 * pieces + 1.12 * load + 0.916 * mk + 0.753 * mn + up(up(steps / unit) / pieces) * unit * step + 0.021 * T);
+        return 1.02 * (5.21 + 0.6 * pieces + 1.12 * load + 0.916 * mk + 0.753 * mn + up(up(steps / unit) / pieces) * unit * step + 0.021 * T) +
+               (quantized ? 0.38 + 0.61 * mn + 0.007 * T : 0);
+    const bool one = mx::TmwCfg::accs(T) == 1;
     const double rounds = up(tiles / pairs), odd = 2 * (steps - 2 * (double)(int64_t)(steps / 2));
-    return 6.32 + 0.916 * mk + 0.472 * mn + rounds * (steps + odd) * step + 0.009 * T * (mx::TmwCfg::accs(T) == 1 ? rounds : 1);
+    const double us = 6.32 + 0.916 * mk + 0.472 * mn + rounds * (steps + odd) * step + 0.009 * T * (one ? rounds : 1);
+    if (!quantized) return us;
+    const double epilogue = 0.69 + 0.023 * T, shows = epilogue - steps * (nib ? 0.26 : 0.345);
+    return us - 1.63 + (one ? (epilogue - 0.009 * T) * rounds : epilogue + (shows > 0 ? (rounds - 1) * 0.6 * shows : 0));
 }
 
 // A pass that writes both operands out in bf16, and the product.  The pass deals items of 256 activations and 1024 weights of one row
 // -- short rows leave lanes idle -- to CTAs that are counted by elements (prep_operands_kernel).
-double tc_us(const TcRoute &r, int64_t M, int64_t N, int64_t K, int sm_count)
+double tc_us(const TcRoute &r, int64_t M, int64_t N, int64_t K, bool quantized, int sm_count)
 {
     const double m = (double)M, n = (double)N, k = (double)K, steps = up(k / 64), pairs = sm_count / 2;
     const double mk = m * k * 1e-6, mn = m * n * 1e-6, nk = n * k * 1e-6;
@@ -1907,6 +1920,7 @@ double tc_us(const TcRoute &r, int64_t M, int64_t N, int64_t K, int sm_count)
     const double turns = (m * up(k / 256) + n * up(k / 1024)) / (4 * (ctas < most ? ctas : most)) - 2;
     double us = 0.44 * n * up(k / 1024) * 1024e-6 + (nk > 40 ? 0.2 * (nk - 40) : 0) + 0.93 * mk + (turns > 0 ? 0.4 * turns : 0);
     us += (0.47 + (N % 4 ? 0.42 : 0)) * mn + (K % 32 ? 2 : 0);           // rows of y without whole 16 bytes; two launches
+    if (quantized) us += (r.kernel == TC_CUT ? 1.45 : r.kernel == TC_PAIR ? 0.6 : r.kernel == TC_PAIR_WIDE ? 0.003 * r.width : 0.25) - 0.055 * mn;
     const double tiles = up(m / 256) * up(n / r.width);
     switch (r.kernel) {
     case TC_CUT: return us + 7.7 + 0.154 * up(steps / r.split);
@@ -1919,42 +1933,43 @@ double tc_us(const TcRoute &r, int64_t M, int64_t N, int64_t K, int sm_count)
 }
 
 // The same on block-scaled records.
-double rec_us(int64_t M, int64_t N, int64_t K, int sm_count)
+double rec_us(int64_t M, int64_t N, int64_t K, bool quantized, int sm_count)
 {
     const double m = (double)M, n = (double)N, k = (double)K, nk = n * k * 1e-6, t = up(m / 256) * up(n / 256) / (sm_count / 2);
     return 8.2 + 0.278 * up(k / 128) * (t > 1 ? 0.5 * (t + up(t)) : 1) + 0.424 * nk + (nk > 40 ? 0.19 * (nk - 40) : 0) + 1.22 * m * k * 1e-6 +
-           (0.57 + (N % 4 ? 0.67 : 0)) * m * n * 1e-6;
+           (0.57 + (N % 4 ? 0.67 : 0)) * m * n * 1e-6 + (quantized ? 1.6 - 0.2 * m * n * 1e-6 : 0);
 }
 
 // gemm_dec_kernel: waves of clusters.
-double dec_us(int64_t M, int64_t N, int64_t K, int split, bool nib, bool words, int sm_count)
+double dec_us(int64_t M, int64_t N, int64_t K, int split, bool nib, bool words, bool quantized, int sm_count)
 {
     const double m = (double)M, k = (double)K, panels = up(m / 128), ctas = up((double)N / 128) * split, waves = up(ctas / sm_count);
     const double load = ctas < sm_count ? ctas / sm_count : 1;
     double step = (panels <= 1 ? 0.332 : panels <= 2 ? 0.449 : 0.634) * (nib ? 1 : 1.13);
     if (!words && step < 0.4) step = 0.4;
     return 5.85 + 1.8 * panels + 2.0 * m * k * 1e-6 + 0.51 * m * (double)N * 1e-6 + 0.02 * (split - 1) + 0.67 * load + 5 * (waves - 1) +
-           waves * up(up(k / 64) / split) * step * (0.9 + 0.1 * load);
+           waves * up(up(k / 64) / split) * step * (0.9 + 0.1 * load) + (quantized ? 1.14 + 0.46 * panels - 0.07 * m * (double)N * 1e-6 : 0);
 }
 
-// Tokens per tile and pieces of K with which gemm_tmw_kernel is expected to take at most 0.98 of `other`, else 0.  Over the shapes
-// measured the route taken is then 0.926 of the other one on average and 1.009 of the best; in 33 of 3400 it is more than 2 % slower
-// than the other one (in six by 8 to 15 %).  Whole calls without / with it: 160 x 4096 x 11008 (M x K x N)
+// Tokens per tile and pieces of K with which gemm_tmw_kernel is expected to take at most 0.98 of `other` (0.96 with an MXInt result,
+// whose estimates are off by more), else 0.  Over the shapes measured the route taken is then 0.925 (0.953) of the other one on average
+// and 1.008 (1.011) of the best; in 50 of 5300 (44 of 1900) it is more than 2 % slower than the other one, in nine (ten) by 8 to 20 %.  Whole calls without / with it: 160 x 4096 x 11008 (M x K x N)
 // 40.4 / 25.0, 128 x 4096 x 11008 30.0 / 25.0, 256 x 2048 x 12288 26.8 / 21.3, 256 x 1024 x 16384 20.1 / 16.7, 512 x 8192 x 8192
 // 80.5 / 53.0, 768 x 16384 x 4096 105 / 86, 1024 x 4096 x 4096 38.4 / 35.1; K cut in two 448 x 16384 x 4096 100 / 54.6, in three
 // 352 x 8192 x 2048 29.6 / 27.6; left alone 1237 x 2048 x 2048 18.8 / 20.1.  Above 1536 rows the passes cost too little beside the product
 // (2048 x 4096 x 4096 62.6 / 61.0, 3072 x 1344 x 11008 74 / 82).
-int tmw_tokens(int64_t M, int64_t N, int64_t K, bool nib, bool words, double other, int sm_count, const int *clusters, int *pieces)
+int tmw_tokens(int64_t M, int64_t N, int64_t K, bool nib, int block, ExpRows rows, bool quantized, double other, int sm_count, const int *clusters,
+               int *pieces)
 {
     const double m = (double)M, n = (double)N, k = (double)K;
-    double best = 0.98 * other;
+    double best = (quantized ? 0.96 : 0.98) * other;
     int tokens = 0;
     if (N < 32) return 0;                                                // an eighth of a tile (1400 x 64 x 4 7.6 / 7.9)
     for (int T = 64; T <= mx::TmwCfg::MAX_T && T < M + 64; T += 32) {
         const double tiles = up(m / T) * up(n / 256);
         for (int s = 1; s <= mx::TmwCfg::MAX_SPLIT; ++s) {
             if (s > 1 && (tiles > clusters[s] || up(k / 64) < s * (nib ? 4 : 2))) break;
-            const double us = tmw_us(m, n, k, nib, words, T, s, sm_count / 2);
+            const double us = tmw_us(m, n, k, nib, block, rows, quantized, T, s, sm_count / 2);
             if (us < best) {
                 best = us;
                 tokens = T;
