@@ -1882,7 +1882,7 @@ mx_status_t launch_dec(const DecPlan &g, const __nv_bfloat16 *a_hat, const void 
 // Estimates in us of whole calls on 148 SMs, pass over the activations included: what dec_plan compares gemm_tmw_kernel with the other
 // routes by.  Fitted to 5600 shapes -- 17 .. 2048 rows, K 32 .. 16384, N 2 .. 16384, widths 8/4, 4/4, 6/6 and 8/8, blocks of 16 and 32 --
 // with every route timed (tmw_tokens: up to eleven tiles and cuts each), 1900 of them with an MXInt result too.  One sigma of their
-// errors: tmw_us and dec_us 4.9 %, tc_us 5.9 %, rec_us 4.6 %; with an MXInt result (`quantized`) 5.7, 6.5, 5.5 and 11 %.
+// errors: tmw_us and dec_us 4.9 %, tc_us 5.9 %, rec_us 4.6 %; with an MXInt result (`quantized`) 4.4, 6.5, 5.5 and 11 %.
 double up(double x) { return (double)(int64_t)(x + 0.999999); }
 
 // gemm_tmw_kernel on tiles of T tokens, K in `pieces`.  Rounds of 74 pairs, each 0.253 us per K step of 64 up to 160 tokens (its
@@ -1901,13 +1901,13 @@ double tmw_us(double M, double N, double K, bool nib, int block, ExpRows rows, b
     step *= 0.9 + 0.1 * load;
     if (pieces > 1)                                                      // (2 % on top: what the fit lacks where the clusters fill the chip)
         return 1.02 * (5.21 + 0.6 * pieces + 1.12 * load + 0.916 * mk + 0.753 * mn + up(up(steps / unit) / pieces) * unit * step + 0.021 * T) +
-               (quantized ? 0.38 + 0.61 * mn + 0.007 * T : 0);
+               (quantized ? 0.35 + 0.75 * mn + 0.006 * T : 0);
     const bool one = mx::TmwCfg::accs(T) == 1;
     const double rounds = up(tiles / pairs), odd = 2 * (steps - 2 * (double)(int64_t)(steps / 2));
     const double us = 6.32 + 0.916 * mk + 0.472 * mn + rounds * (steps + odd) * step + 0.009 * T * (one ? rounds : 1);
     if (!quantized) return us;
-    const double epilogue = 0.69 + 0.023 * T, shows = epilogue - steps * (nib ? 0.26 : 0.345);
-    return us - 1.63 + (one ? (epilogue - 0.009 * T) * rounds : epilogue + (shows > 0 ? (rounds - 1) * 0.6 * shows : 0));
+    const double epilogue = 0.0131 * T, shows = one ? epilogue - 2.36 : 0.42 * (epilogue + 1.57 - steps * (nib ? 0.26 : 0.345));
+    return us - 0.27 + 0.315 * mn + epilogue + (one || shows > 0 ? (rounds - 1) * shows : 0);
 }
 
 // A pass that writes both operands out in bf16, and the product.  The pass deals items of 256 activations and 1024 weights of one row
@@ -1951,9 +1951,9 @@ double dec_us(int64_t M, int64_t N, int64_t K, int split, bool nib, bool words, 
            waves * up(up(k / 64) / split) * step * (0.9 + 0.1 * load) + (quantized ? 1.14 + 0.46 * panels - 0.07 * m * (double)N * 1e-6 : 0);
 }
 
-// Tokens per tile and pieces of K with which gemm_tmw_kernel is expected to take at most 0.98 of `other` (0.96 with an MXInt result,
-// whose estimates are off by more), else 0.  Over the shapes measured the route taken is then 0.925 (0.953) of the other one on average
-// and 1.008 (1.011) of the best; in 50 of 5300 (44 of 1900) it is more than 2 % slower than the other one, in nine (ten) by 8 to 20 %.  Whole calls without / with it: 160 x 4096 x 11008 (M x K x N)
+// Tokens per tile and pieces of K with which gemm_tmw_kernel is expected to take at most 0.98 of `other` (0.97 with an MXInt result,
+// whose estimates are off by more), else 0.  Over the shapes measured the route taken is then 0.925 (0.952) of the other one on average
+// and 1.008 (1.010) of the best; in 50 of 5300 (31 of 1900) it is more than 2 % slower than the other one, in nine (four) by 8 to 15 %.  Whole calls without / with it: 160 x 4096 x 11008 (M x K x N)
 // 40.4 / 25.0, 128 x 4096 x 11008 30.0 / 25.0, 256 x 2048 x 12288 26.8 / 21.3, 256 x 1024 x 16384 20.1 / 16.7, 512 x 8192 x 8192
 // 80.5 / 53.0, 768 x 16384 x 4096 105 / 86, 1024 x 4096 x 4096 38.4 / 35.1; K cut in two 448 x 16384 x 4096 100 / 54.6, in three
 // 352 x 8192 x 2048 29.6 / 27.6; left alone 1237 x 2048 x 2048 18.8 / 20.1.  Above 1536 rows the passes cost too little beside the product
@@ -1962,7 +1962,7 @@ int tmw_tokens(int64_t M, int64_t N, int64_t K, bool nib, int block, ExpRows row
                int *pieces)
 {
     const double m = (double)M, n = (double)N, k = (double)K;
-    double best = (quantized ? 0.96 : 0.98) * other;
+    double best = (quantized ? 0.97 : 0.98) * other;
     int tokens = 0;
     if (N < 32) return 0;                                                // an eighth of a tile (1400 x 64 x 4 7.6 / 7.9)
     for (int T = 64; T <= mx::TmwCfg::MAX_T && T < M + 64; T += 32) {

@@ -10,12 +10,11 @@ from paper_2307_15517_b200 import binding as mxb
 pytestmark = pytest.mark.gpu
 
 
-def runs(M, K, N, fa, fw, tokens, pieces):
-    """The kernel, and on 148 SMs its tile and its pieces of K, for the fp32 and the MXInt result."""
+def runs(M, K, N, fa, fw, tokens, pieces, quantized=False):
+    """The kernel, and on 148 SMs its tile and its pieces of K, for the fp32 or the MXInt result."""
+    route = mxb.mx_selftest_route(M, N, K, fa, fw, quantized)
     tile = torch.cuda.get_device_properties(0).multi_processor_count == 148
-    for quantized in (False, True):
-        route = mxb.mx_selftest_route(M, N, K, fa, fw, quantized)
-        assert route[0] == 2 and (not tile or route[1:] == (tokens, pieces)), route
+    assert route[0] == 2 and (not tile or route[1:] == (tokens, pieces)), route
 
 
 @pytest.mark.parametrize("M,K,N,block,wa,ww,rows2,tokens", [
@@ -38,15 +37,14 @@ def runs(M, K, N, fa, fw, tokens, pieces):
     (500, 1104, 8192, 16, 8, 6, 1, 256),
     (33, 32, 136, 32, 8, 3, 1, 64),        # the smallest: half a step, a token beyond the first CTA's
     (170, 32, 9522, 16, 8, 3, 1, 64),      # two rounds
-    (152, 80, 10562, 16, 8, 6, 1, 64),
-    (245, 32, 10196, 16, 8, 8, 1, 96),
+    (152, 80, 10562, 16, 8, 6, 1, 160),
+    (245, 32, 10196, 16, 8, 8, 1, 256),
     (198, 32, 11144, 32, 8, 4, 1, 96),
     (524, 80, 6612, 16, 8, 6, 1, 128),
     (485, 32, 6322, 32, 8, 4, 1, 128),
     (275, 352, 13702, 32, 8, 3, 1, 160),
     (1505, 272, 4630, 16, 8, 5, 1, 224),   # bytes, one accumulator, several rounds
     (1098, 416, 6702, 16, 8, 4, 1, 224),
-    (483, 560, 13796, 16, 8, 7, 1, 256),
     (984, 416, 9006, 16, 8, 2, 2, 256),
 ])
 def test_weights_decoded_into_tensor_memory(M, K, N, block, wa, ww, rows2, tokens):
@@ -90,19 +88,14 @@ def test_weights_decoded_into_tensor_memory(M, K, N, block, wa, ww, rows2, token
     (502, 4192, 2693, 32, 8, 4, 256, 3),   # pieces of unequal length, the last K step of 32; odd row length
     (38, 464, 137, 16, 8, 6, 64, 2),       # a second piece of two stages of packed weights, half of the features outside
     (36, 5920, 4273, 16, 8, 2, 64, 3),
-    (108, 848, 155, 16, 8, 5, 64, 4),
-    (137, 1376, 4077, 32, 8, 2, 96, 2),
     (194, 1104, 1668, 16, 8, 7, 96, 3),
     (207, 1232, 2919, 16, 8, 8, 128, 2),
     (126, 8224, 4788, 16, 8, 2, 128, 3),
     (104, 11104, 3807, 16, 8, 4, 128, 4),
-    (136, 1872, 2969, 16, 8, 6, 160, 3),
     (139, 3552, 3196, 32, 8, 3, 160, 4),
     (188, 1584, 5964, 16, 8, 5, 192, 2),
     (171, 2352, 3573, 16, 8, 8, 192, 4),
     (395, 3296, 2524, 32, 8, 3, 224, 3),
-    (210, 3216, 3300, 16, 8, 7, 224, 4),
-    (450, 2992, 2686, 16, 8, 7, 256, 3),
     (239, 10528, 2543, 32, 8, 3, 256, 4),
 ])
 def test_pieces_of_K_added_up_in_a_cluster(M, K, N, block, wa, ww, tokens, pieces):
@@ -133,6 +126,44 @@ def test_pieces_of_K_added_up_in_a_cluster(M, K, N, block, wa, ww, tokens, piece
             ym, ye = mxb.mx_linear_fused(x, fa, wm, we, fw, N, bias=bias, relu=True, residual=res, fy=fy)
             qm, qe = mxb.mx_quantize(z, fy)
             assert torch.equal(ym, qm) and torch.equal(ye, qe)
+    assert mxb.mx_poll_status() == 0
+
+
+@pytest.mark.parametrize("M,K,N,block,wa,ww,tokens,pieces", [
+    (36, 32, 128, 16, 8, 5, 64, 1), (164, 32, 10304, 32, 8, 6, 64, 1), (130, 32, 9568, 32, 8, 2, 64, 1),
+    (200, 32, 9664, 16, 8, 8, 96, 1), (200, 32, 9536, 16, 8, 2, 96, 1), (102, 32, 9536, 32, 8, 7, 128, 1), (296, 32, 9536, 32, 8, 7, 128, 1),
+    (306, 32, 9632, 32, 8, 2, 128, 1), (130, 32, 9952, 32, 8, 8, 160, 1), (388, 32, 9568, 32, 8, 6, 160, 1), (386, 32, 9600, 32, 8, 3, 160, 1),
+    (322, 32, 6240, 32, 8, 6, 192, 1), (484, 32, 9728, 32, 8, 8, 192, 1), (352, 160, 6208, 16, 8, 4, 192, 1), (516, 32, 9760, 32, 8, 4, 192, 1),
+    (388, 32, 7712, 16, 8, 6, 224, 1), (642, 32, 9664, 32, 8, 7, 224, 1), (202, 32, 12768, 32, 8, 4, 224, 1), (670, 32, 11328, 32, 8, 2, 224, 1),
+    (486, 144, 7264, 16, 8, 6, 256, 1), (730, 4960, 12256, 32, 8, 6, 256, 1), (240, 1056, 11424, 32, 8, 4, 256, 1), (766, 2208, 12480, 16, 8, 2, 256, 1),
+    (40, 400, 192, 16, 8, 7, 64, 2), (40, 1104, 128, 16, 8, 7, 64, 3), (38, 1296, 960, 16, 8, 7, 64, 4), (136, 2304, 3552, 32, 8, 4, 96, 2),
+    (148, 4544, 2592, 16, 8, 4, 96, 3), (224, 3328, 3744, 32, 8, 2, 128, 2), (158, 1200, 7104, 16, 8, 8, 160, 2), (140, 2080, 4416, 32, 8, 3, 160, 3),
+    (132, 3376, 3360, 16, 8, 6, 160, 4), (164, 2448, 5984, 16, 8, 5, 192, 2), (162, 2176, 5216, 32, 8, 5, 192, 3), (172, 5248, 3552, 16, 8, 3, 192, 4),
+    (212, 3248, 5952, 16, 8, 7, 224, 2), (202, 2208, 5504, 32, 8, 4, 224, 3), (222, 8224, 3648, 32, 8, 3, 224, 4), (238, 4432, 5920, 16, 8, 6, 256, 2),
+    (478, 5024, 2720, 32, 8, 2, 256, 3),
+])
+def test_MXInt_results_of_every_tile_and_cut(M, K, N, block, wa, ww, tokens, pieces):
+    """Uncut: the quantized sums of a product behind a pass.  Cut sums differ from those by 2^-22 of the absolute sum S at most (see
+    above), some 1600 steps of a code: a code next to a rounding boundary may move by one step, 8e-4 of them at the very most."""
+    g = torch.Generator(device="cuda")
+    g.manual_seed(M + K + N)
+    fa, fw = mxb.MxFormat(block, wa), mxb.MxFormat(block, ww)
+    runs(M, K, N, fa, fw, tokens, pieces, True)
+    x = torch.randn(M, K, generator=g, device="cuda")
+    wm, we = mxb.mx_quantize(torch.randn(N, K, generator=g, device="cuda") * 0.02, fw)
+    bias = torch.randn(N, generator=g, device="cuda")
+    y = mxb.mx_linear(x, fa, wm, we, fw, N, bias=bias, algo=mxb.MX_ALGO_TCGEN05)
+    for fy in (mxb.MxFormat(16, 8), mxb.MxFormat(32, 4), mxb.MxFormat(16, 5, block_rows=2)):
+        ym, ye = mxb.mx_linear_q(x, fa, wm, we, fw, N, fy, bias=bias)
+        qm, qe = mxb.mx_quantize(y, fy)
+        if pieces == 1:
+            assert torch.equal(ym, qm) and torch.equal(ye, qe)
+        else:
+            a, b = mxb.mx_dequantize(ym, ye, N, fy), mxb.mx_dequantize(qm, qe, N, fy)
+            step = b.abs().view(M, N // fy.block, fy.block).amax(2, keepdim=True).expand(-1, -1, fy.block).reshape(M, N) * 2.0 ** (3 - fy.elem_bits)
+            if fy.block_rows == 2:
+                step = step.view(M // 2, 2, N).amax(1, keepdim=True).expand(-1, 2, -1).reshape(M, N)
+            assert ((a - b).abs() <= step).all() and (a != b).float().mean() <= 1e-3
     assert mxb.mx_poll_status() == 0
 
 
