@@ -466,7 +466,60 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant
     const int kblocks = (p.K + TC_BK - 1) / TC_BK;
     bool timed_out = false;
 
-    if (warp == 0) {
+    // In the variants that decode weights the decoding warps are the bound, and whole warps that poll and vote take their issue slots:
+    // the two loops keep to one lane there (975 x 2432 x 9600 4-bit, M x K x N, whole warps / one lane 105 / 81 us, 282 x 5248 x 9408
+    // 78 / 62; over 240 shapes 1.7 % on average).
+    if (FUSED && warp == 0) {
+        if (lane == 0) {
+            int s = 0;
+            uint32_t ph = 0;
+            for (int t = blockIdx.x; t < num_tiles && !timed_out; t += gridDim.x) {
+                const int m0 = (t % p.tiles_m) * TC_BM;
+                for (int kb = 0; kb < kblocks; ++kb) {
+                    if (!ptx::mbar_wait_bounded(empty_bar(s), ph ^ 1u, abort_flag, TC_WAIT_LIMIT_NS)) {
+                        timed_out = true;
+                        break;
+                    }
+                    ptx::mbar_arrive_expect_tx(full_bar(s), Cfg::A_BYTES);
+                    ptx::tma_load_2d(smem_base + s * Cfg::STAGE_BYTES, &tmap_a, kb * TC_BK, m0, full_bar(s));
+                    if (++s == STAGES) { s = 0; ph ^= 1u; }
+                }
+            }
+        }
+        __syncwarp();
+    } else if (FUSED && warp == 1) {
+        if (lane == 0) {
+            constexpr uint32_t idesc = ptx::idesc_bf16_f32(TC_BM, BN);
+            int s = 0, it = 0;
+            uint32_t ph = 0;
+            for (int t = blockIdx.x; t < num_tiles && !timed_out; t += gridDim.x, ++it) {
+                const int acc = it & 1;
+                const uint32_t acc_ph = (uint32_t)(it >> 1) & 1u;
+                if (!ptx::mbar_wait_bounded(tempty_bar(acc), acc_ph ^ 1u, abort_flag, TC_WAIT_LIMIT_NS)) {
+                    timed_out = true;
+                    break;
+                }
+                ptx::tc_fence_after_sync();
+                const uint32_t d_tmem = tmem_base + (uint32_t)(acc * BN);
+                for (int kb = 0; kb < kblocks; ++kb) {
+                    if (!ptx::mbar_wait_bounded(full_bar(s), ph, abort_flag, TC_WAIT_LIMIT_NS)) {
+                        timed_out = true;
+                        break;
+                    }
+                    ptx::tc_fence_after_sync();
+                    const uint32_t sa = smem_base + s * Cfg::STAGE_BYTES, sw = sa + Cfg::A_BYTES;
+#pragma unroll
+                    for (int j = 0; j < TC_BK / 16; ++j)
+                        ptx::mma_bf16_ss(d_tmem, ptx::smem_desc_k_sw128(sa, j * 32), ptx::smem_desc_k_sw128(sw, j * 32), idesc, (kb | j) != 0 ? 1u : 0u);
+                    ptx::mma_commit(empty_bar(s));                           // stage free once these MMAs retire
+                    if (++s == STAGES) { s = 0; ph ^= 1u; }
+                }
+                if (timed_out) break;
+                ptx::mma_commit(tfull_bar(acc));                             // accumulator complete
+            }
+        }
+        __syncwarp();
+    } else if (warp == 0) {
         int s = 0;
         uint32_t ph = 0;
         for (int t = blockIdx.x; t < num_tiles && !timed_out; t += gridDim.x) {
@@ -478,14 +531,14 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant
                     break;
                 }
                 if (ptx::elect_one()) {
-                    ptx::mbar_arrive_expect_tx(full_bar(s), FUSED ? Cfg::A_BYTES : Cfg::STAGE_BYTES);
+                    ptx::mbar_arrive_expect_tx(full_bar(s), Cfg::STAGE_BYTES);
                     const uint32_t sa = smem_base + s * Cfg::STAGE_BYTES;
-                    if (!FUSED && p.batch > 1) {
+                    if (p.batch > 1) {
                         ptx::tma_load_3d(sa, &tmap_a, kb * TC_BK, m0, tb, full_bar(s));
                         ptx::tma_load_3d(sa + Cfg::A_BYTES, &tmap_w, kb * TC_BK, n0, tb, full_bar(s));
                     } else {
                         ptx::tma_load_2d(sa, &tmap_a, kb * TC_BK, m0, full_bar(s));
-                        if (!FUSED) ptx::tma_load_2d(sa + Cfg::A_BYTES, &tmap_w, kb * TC_BK, n0, full_bar(s));
+                        ptx::tma_load_2d(sa + Cfg::A_BYTES, &tmap_w, kb * TC_BK, n0, full_bar(s));
                     }
                 }
                 if (++s == STAGES) { s = 0; ph ^= 1u; }
