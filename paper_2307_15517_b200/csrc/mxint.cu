@@ -1198,7 +1198,9 @@ int wide_pair_tile(int64_t M, int64_t N, int64_t K, const DeviceInfo &d)
 // Not where tiles of 128 x 128 make one wave, which need 32 KB per step (19.6 / 22.1 at 384 x 2048 x 6144, 31.8 / 35.6 at 384 x 4096 x
 // 6144, 35.3 / 38.1 at 384 x 5120 x 5120), and not for fewer than five K steps, whose results leave in one burst at the end (640 x 256 x
 // 4096 12.4 / 13.6, 300 x 96 x 6464 17.0 / 23.8; of 300 shapes from K = 320 on none is more than 4 % slower), four of 160 columns
-// (2048 x 256 x 1408 11.5 / 10.0).
+// (2048 x 256 x 1408 11.5 / 10.0).  Behind a pass that decodes both operands only from
+// K = 512 on (of 224 shapes none slower by more than 1 %; 1490 x 256 x 1632 12.6 / 14.8, 1099 x 320 x 2240 12.4 / 14.2, 582 x 384 x 4160
+// 13.0 / 13.6).
 int one_round_width(int64_t M, int64_t N, int64_t K, const DeviceInfo &d)
 {
     const int64_t rows = (M + 255) / 256, cols = d.sm_count / 2 / rows;
@@ -1218,7 +1220,8 @@ int one_round_width(int64_t M, int64_t N, int64_t K, const DeviceInfo &d)
 enum TcKernel { TC_ONE = 5, TC_PAIR = 6, TC_PAIR_WIDE = 7, TC_CUT = 4 };     // (numbers: mx_selftest_route)
 struct TcRoute { TcKernel kernel; int width, split; };                      // columns of a tile; pieces of K
 
-mx_status_t tc_route(int64_t M, int64_t N, int64_t K, int count, bool may_split, DeviceInfo &d, TcRoute *out)
+// packed: the pass in front decodes both operands (launch_dequant_pair).
+mx_status_t tc_route(int64_t M, int64_t N, int64_t K, int count, bool may_split, DeviceInfo &d, TcRoute *out, bool packed = false)
 {
     const int64_t panels = (M + 127) / 128;
     const int64_t pair_tiles = ((M + 255) / 256) * ((N + 255) / 256);
@@ -1232,7 +1235,7 @@ mx_status_t tc_route(int64_t M, int64_t N, int64_t K, int count, bool may_split,
         *out = {width ? TC_PAIR_WIDE : TC_PAIR, width ? width : 256, 1};
         return MX_OK;
     }
-    const int width = M > 128 && K >= 256 && tiles128 > d.sm_count ? one_round_width(M, N, K, d) : 0;
+    const int width = M > 128 && K >= (packed ? 512 : 256) && tiles128 > d.sm_count ? one_round_width(M, N, K, d) : 0;
     if (width) {
         *out = {TC_PAIR_WIDE, width, 1};
         return MX_OK;
@@ -1246,11 +1249,11 @@ mx_status_t tc_route(int64_t M, int64_t N, int64_t K, int count, bool may_split,
 // Pre-decoded bf16 weights (both operands fetched by TMA).
 mx_status_t run_tc(const __nv_bfloat16 *a_hat, const __nv_bfloat16 *w_hat, int64_t M, int64_t N,
                    int64_t K, const float *bias, float *y, int64_t ldy, DeviceInfo &d, cudaStream_t st,
-                   const QuantizedOut *yq = nullptr, const TcBatch &tb = TcBatch(), const EpiTail &et = EpiTail(), bool may_split = true)
+                   const QuantizedOut *yq = nullptr, const TcBatch &tb = TcBatch(), const EpiTail &et = EpiTail(), bool may_split = true, bool packed = false)
 {
     const PackedW none;
     TcRoute r;
-    const mx_status_t s = tc_route(M, N, K, tb.count, may_split, d, &r);
+    const mx_status_t s = tc_route(M, N, K, tb.count, may_split, d, &r, packed);
     if (s != MX_OK) return s;
     if (r.kernel == TC_PAIR_WIDE) return launch_tcw(a_hat, w_hat, M, N, K, r.width, bias, y, ldy, yq, d, st, et);
     if (r.kernel == TC_PAIR) return launch_tc2(a_hat, w_hat, M, N, K, bias, y, ldy, yq, d, st, et);
@@ -2357,7 +2360,7 @@ mx_status_t mx_gemm_ex(const void *a_mant, const uint8_t *a_exp, mx_format_t fa,
     s = launch_dequant_pair(a_mant, a_exp, fa, M, w_mant, w_exp, fw, N, K, a_hat, w_hat, *d, st);
     if (s != MX_OK) return s;
     if (algo == MX_ALGO_TCGEN05_BLOCKWISE) return launch_tcx(a_hat, w_hat, M, N, K, fa.block, bias, y, ldy, *d, st);
-    return run_tc(a_hat, w_hat, M, N, K, bias, y, ldy, *d, st, nullptr, TcBatch(), EpiTail(), any_algo);
+    return run_tc(a_hat, w_hat, M, N, K, bias, y, ldy, *d, st, nullptr, TcBatch(), EpiTail(), any_algo, true);
 }
 
 mx_status_t mx_gemm(const void *a_mant, const uint8_t *a_exp, mx_format_t fa, const void *w_mant,
@@ -2533,8 +2536,8 @@ static mx_status_t gemm_tc_impl(const void *a_mant, const uint8_t *a_exp, mx_for
                             static_cast<uint8_t *>(workspace), *d, st, et);
     s = launch_dequant_pair(a_mant, a_exp, fa, M, w_mant, w_exp, fw, N, K, a_hat, w_hat, *d, st);
     if (s != MX_OK) return s;
-    if (y) return run_tc(a_hat, w_hat, M, N, K, bias, y, ldy, *d, st, nullptr, TcBatch(), et);
-    return run_tc(a_hat, w_hat, M, N, K, bias, nullptr, N, *d, st, &yq, TcBatch(), et);
+    if (y) return run_tc(a_hat, w_hat, M, N, K, bias, y, ldy, *d, st, nullptr, TcBatch(), et, true, true);
+    return run_tc(a_hat, w_hat, M, N, K, bias, nullptr, N, *d, st, &yq, TcBatch(), et, true, true);
 }
 
 // The same for the layer: activations quantized on the fly.
@@ -3356,7 +3359,7 @@ mx_status_t mx_alt_gemm(const uint8_t *a_codes, const uint8_t *a_shared, mx_alt_
     if (s != MX_OK) return s;
     s = alt_decode_any(w_codes, w_shared, N, K, fw, w_hat, MX_BF16, K, *d, st);
     if (s != MX_OK) return s;
-    return run_tc(a_hat, w_hat, M, N, K, bias, y, ldy, *d, st);
+    return run_tc(a_hat, w_hat, M, N, K, bias, y, ldy, *d, st, nullptr, TcBatch(), EpiTail(), true, true);
 }
 
 // ---- product without any allocation ---------------------------------------------------------
