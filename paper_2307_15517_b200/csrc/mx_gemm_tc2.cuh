@@ -204,7 +204,13 @@ gemm_tc2_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constan
             }
             ptx::tc_fence_before_sync();
             __syncwarp();
-            if (lane == 0) ptx::mbar_arrive_cluster_relaxed(ptx::map_to_cta(tempty_bar(acc), 0));
+            // Relaxed is enough (only tensor memory was read) and the faster form where the epilogue only stores; with the residual's
+            // reads between the stores release is: 2812 x 1152 x 11552 (M x K x N) with bias, ReLU and residual 162.8 us relaxed, 159.0
+            // released, without them 86.2 and 89.3.
+            if (lane == 0) {
+                if (TAIL) ptx::mbar_arrive_cluster(ptx::map_to_cta(tempty_bar(acc), 0));
+                else ptx::mbar_arrive_cluster_relaxed(ptx::map_to_cta(tempty_bar(acc), 0));
+            }
         }
         if (p.tma_store && lane == 0) ptx::bulk_wait_group<0>();
     }

@@ -254,6 +254,10 @@ __device__ __forceinline__ uint32_t map_to_cta(uint32_t addr, uint32_t rank)
     asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
     return r;
 }
+__device__ __forceinline__ void mbar_arrive_cluster(uint32_t cluster_addr)
+{
+    asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(cluster_addr) : "memory");
+}
 // Arrival and bounded wait that order nothing but tensor-memory accesses (with tcgen05.fence on either side) and the completion
 // of asynchronous copies and MMAs: what the pair's pipeline barriers are for.  Release and acquire at cluster scope also order
 // the thread's accesses to global and shared memory, which none of that needs and which costs the thread microseconds.
